@@ -7,6 +7,7 @@
 
 #include "model.cuh"
 #include "gemm.cuh"
+#include "gemm_pair.cuh"
 
 using namespace scd;
 
@@ -17,6 +18,7 @@ void count_launches(long long n) { g_launches.fetch_add(n, std::memory_order_rel
 
 namespace {
 
+constexpr int PREFILL_ROWS = PAIR_MAX_X_TILES * PAIR_ROWS;   // rows one pass over a prompt carries (bf16)
 constexpr int GENERATE_BLOCK = 64;      // iterations scd_generate enqueues between two looks at the counters
 
 inline bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
@@ -152,7 +154,7 @@ void free_session_memory(scd_session *s)
     void *ptrs[] = {s->kv_pool, s->page_table, s->n_known, s->n_total, s->shift, s->prev_lw, s->drafts,
                     s->n_commit, s->tokens, s->tokens_u, s->row_y, s->row_y_indep, s->ids_buf, s->iter,
                     s->done_count, s->accept_flags, s->xbuf[0], s->xbuf[1], s->stats[0], s->stats[1],
-                    s->dev_stats, s->finished, s->h, s->ss, s->xn, s->qkv, s->att, s->gu, s->act, s->logits, s->gemm_ws, s->stamps};
+                    s->dev_stats, s->finished, s->h, s->ss, s->xn, s->qkv, s->att, s->gu, s->act, s->logits, s->gemm_ws, s->gemm_scratch, s->stamps};
     for (void *p : ptrs) if (p) cudaFree(p);
     if (s->host_pinned) cudaFreeHost(s->host_pinned);
     if (s->gemm_state) gemm_session_release(s);
@@ -254,12 +256,16 @@ int scd_session_create(scd_model_t *m, const scd_decode_config_t *cfg, scd_sessi
     s->att_t5_min_ctx = 512;
     // rows one forward may carry per stream-sequence: the window, or a prefill chunk
     s->chunk = std::max(s->L, std::max(1, std::min(128, 256 / s->Q)));
-    s->rows_cap = s->Q * s->chunk;
-    if (c.dtype == SCD_BF16 && s->rows_cap > 1024) {
+    if (c.dtype == SCD_BF16 && s->Q * s->chunk > 1024) {
         set_last_error("bf16 sessions carry at most 1024 rows per forward (S*B*L = %d)", s->Q * s->L);
         delete s;
         return SCD_ERR_CAPACITY;
     }
+    // A pass over the prompt carries up to PREFILL_ROWS rows: from some hundred rows on the weights are read for
+    // less than the tensor cores take, and the more tiles the evener the split over the SMs.
+    s->prefill_chunk = s->chunk;
+    if (c.dtype == SCD_BF16) s->prefill_chunk = std::max(s->chunk, std::min(c.max_seq - 1, PREFILL_ROWS / s->Q));
+    s->rows_cap = s->Q * s->prefill_chunk;
     s->pages_per_seq = (c.max_seq + c.kv_page_tokens - 1) / c.kv_page_tokens;
     const size_t es = elem_size(c.dtype);
     const int d = c.d_model, dq = c.n_heads * c.head_dim, dkv = c.n_kv_heads * c.head_dim, F = c.d_ffn, V = c.vocab_out;
@@ -301,7 +307,7 @@ int scd_session_create(scd_model_t *m, const scd_decode_config_t *cfg, scd_sessi
     { char *p; TRY_ALLOC(dev_alloc(&p, wide * rows * d * es)); s->xn = p; }
     { char *p; TRY_ALLOC(dev_alloc(&p, wide * rows * (dq + 2 * dkv) * es)); s->qkv = p; }
     { char *p; TRY_ALLOC(dev_alloc(&p, wide * rows * dq * es)); s->att = p; }
-    { char *p; TRY_ALLOC(dev_alloc(&p, rows * 2 * F * es)); s->gu = p; }
+    if (c.dtype == SCD_F32) { char *p; TRY_ALLOC(dev_alloc(&p, rows * 2 * F * es)); s->gu = p; }
     { char *p; TRY_ALLOC(dev_alloc(&p, wide * rows * F * es)); s->act = p; }
     s->ss_parts_cap = c.dtype == SCD_BF16 && m->gemm_plan ? gemm_norm_parts_cap(s) : 1;
     TRY_ALLOC(dev_alloc(&s->ss, (size_t)s->ss_parts_cap * rows));
@@ -364,8 +370,10 @@ int scd_prefill(scd_session_t *s, const int32_t *prompt_ids, int32_t P, int32_t 
                                        (size_t)P * sizeof(int), s->B, cudaMemcpyHostToDevice, st));
     // chunks of the prompt (all but its last token) through the forward, no logits; the kernels read the
     // prompt from the token records just copied, so the chunks are enqueued back to back
-    for (int p0 = 0; p0 < P - 1; p0 += s->chunk) {
-        const int len = std::min(s->chunk, P - 1 - p0);
+    const int passes = (P - 1 + s->prefill_chunk - 1) / s->prefill_chunk;
+    const int per_pass = passes > 0 ? std::min(s->prefill_chunk, ((P - 1 + passes - 1) / passes + 127) / 128 * 128) : 0;
+    for (int p0 = 0; p0 < P - 1; p0 += per_pass) {
+        const int len = std::min(per_pass, P - 1 - p0);
         ForwardArgs a;
         a.ids = nullptr; a.Mq = len; a.pos_override = p0; a.want_logits = false; a.skip = nullptr;
         a.logits = nullptr; a.hidden = nullptr; a.prof = nullptr; a.lm_lo = 0; a.lm_hi = 0; a.lm_eol = -1;

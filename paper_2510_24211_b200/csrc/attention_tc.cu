@@ -50,6 +50,12 @@ struct AttnParams {
     const int *skip;                   // optional device flag: set = nothing to do, return at once
     long long row0_k, row0_v;          // pool row of (this layer, K | V, page 0, head 0, token 0)
     int B, Mq, H, Hkv, n_rep, pages_per_seq, page_tokens, page_shift, max_seq, pos_override;
+    // Query row i of stream-sequence q is row q * row_stride + row_off + i of qkv and out and sits row_off + i positions
+    // behind the first row of the forward (row_off > 0: a later part of more rows than one launch takes).
+    int row_stride, row_off;
+    // More rows than one CTA takes through the tcgen05 kernel: chunk_rows > 0 rows per stream-sequence, Mq of them per CTA, all keys
+    // (also the chunk's own, written by kv_write_kernel) from the cache under the causal mask.
+    int chunk_rows;
     int C, stages, stages_v, n_mtiles;   // (stages_v: the tcgen05 kernel's V ring; its K ring has `stages` slots)
     float qscale;                      // log2(e) / sqrt(dh)
     unsigned long long *stamp;         // optional [2][STAMP_CTAS]: %globaltimer at CTA entry and exit
@@ -363,7 +369,7 @@ __global__ void __launch_bounds__(256) attention_tc_kernel(const __grid_constant
 
     // n_known was written by the previous iteration, which is complete before any kernel of this
     // one starts; the cache entries below `base` are older still.
-    const int base = p.pos_override >= 0 ? p.pos_override : p.n_known[b] - 1;
+    const int base = (p.pos_override >= 0 ? p.pos_override : p.n_known[b] - 1) + p.row_off;
     const int ctx = min(max(base, 0), p.max_seq);
     const int n_tiles = (ctx + TK - 1) / TK;
     // The last CTA of the cluster also rotates, stores and attends to the window rows, which costs
@@ -394,12 +400,17 @@ __global__ void __launch_bounds__(256) attention_tc_kernel(const __grid_constant
             tma_load_2d(&p.kv_map, &full_bar[s], dst + tile_bytes + h * (TK * 128), h * 64, (int)(p.row0_v + r));
         }
     };
-    if (tid == 0) {
+    auto first_tiles = [&]() {
         const int pre = min(p.stages - 1, my_tiles);
         for (int t = 0; t < pre; ++t) issue(t);
-    }
+    };
+    if (tid == 0 && p.row_off == 0) first_tiles();
 
     pdl_wait();                                                   // Q, K, V of the window come from the GEMM in front
+    if (tid == 0 && p.row_off > 0) {                              // the launch in front wrote the part before this one into the cache
+        asm volatile("fence.proxy.async.global;" ::: "memory");
+        first_tiles();
+    }
 
     // ---- Q: rotate, scale, stage in shared memory (8 dims of both halves per item, 16-byte accesses) ---
     const size_t qstride = (size_t)(p.H + 2 * p.Hkv) * DH;
@@ -411,7 +422,7 @@ __global__ void __launch_bounds__(256) attention_tc_kernel(const __grid_constant
         if (rr < rows) {
             const int i = rr % Mq, g = rr / Mq;
             const int pos = min(max(base + i, 0), p.max_seq - 1);
-            const float *src = p.qkv + ((size_t)q * Mq + i) * qstride + (size_t)(kvh * p.n_rep + g) * DH;
+            const float *src = p.qkv + ((size_t)q * p.row_stride + p.row_off + i) * qstride + (size_t)(kvh * p.n_rep + g) * DH;
             rotate8(src + j0, src + j0 + half, p.rope + (size_t)pos * half + j0, p.qscale, lo, hi, &rlo, &rhi);
         }
         *(uint4 *)(q_s + sw_off(qrows_pad, rr, j0)) = lo;
@@ -485,7 +496,7 @@ __global__ void __launch_bounds__(256) attention_tc_kernel(const __grid_constant
                 uint4 klo = make_uint4(0u, 0u, 0u, 0u), khi = klo, vlo = klo, vhi = klo;
                 const int pos = base + i;
                 if (i < Mq && pos >= 0 && pos < p.max_seq) {
-                    const float *src = p.qkv + ((size_t)q * Mq + i) * qstride + (size_t)(p.H + kvh) * DH;
+                    const float *src = p.qkv + ((size_t)q * p.row_stride + p.row_off + i) * qstride + (size_t)(p.H + kvh) * DH;
                     const float *vs = src + (size_t)p.Hkv * DH;
                     vlo = round8(vs + j0);
                     vhi = round8(vs + j0 + half);
@@ -556,7 +567,7 @@ __global__ void __launch_bounds__(256) attention_tc_kernel(const __grid_constant
             if (fin && rr < rows) {
                 const int i = rr % Mq, gq = rr / Mq;
                 const float inv = w.l[h] > 0.f ? 1.0f / w.l[h] : 0.f;
-                __nv_bfloat16 *dst = p.out + ((size_t)q * Mq + i) * ostride + (size_t)(kvh * p.n_rep + gq) * DH;
+                __nv_bfloat16 *dst = p.out + ((size_t)q * p.row_stride + p.row_off + i) * ostride + (size_t)(kvh * p.n_rep + gq) * DH;
 #pragma unroll
                 for (int j = 0; j < DH / 8; ++j) {
                     const int col = j * 8 + 2 * (lane & 3);
@@ -625,7 +636,7 @@ __global__ void __launch_bounds__(256) attention_tc_kernel(const __grid_constant
                 acc.z += wp * part[peer].z; acc.w += wp * part[peer].w;
             }
             const int i = rr % Mq, gq = rr / Mq;
-            __nv_bfloat16 *dst = p.out + ((size_t)q * Mq + i) * ostride + (size_t)(kvh * p.n_rep + gq) * DH + col;
+            __nv_bfloat16 *dst = p.out + ((size_t)q * p.row_stride + p.row_off + i) * ostride + (size_t)(kvh * p.n_rep + gq) * DH + col;
             uint2 packed;
             packed.x = pack_bf16(acc.x, acc.y);
             packed.y = pack_bf16(acc.z, acc.w);
@@ -825,10 +836,16 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
     pdl_trigger();
     const uint32_t tmem_q = tmem_base_s, tmem_s = tmem_base_s + 128u, tmem_o = tmem_base_s + 256u, tmem_p = tmem_base_s + 384u;
 
-    const int C = p.C, rank = blockIdx.x % C, unit = blockIdx.x / C;
+    const int C = p.C, rank = blockIdx.x % C;
+    // prefill: the query tiles with the most keys first, so that the short ones fill the last wave
+    const bool prefill = p.chunk_rows > 0;
+    const int n_units = (int)gridDim.x / C, heads = prefill ? n_units / ((p.chunk_rows + p.Mq - 1) / p.Mq) : n_units;
+    const int unit = (int)(blockIdx.x / C) % heads;
+    const int q_tile = prefill ? n_units / heads - 1 - (int)(blockIdx.x / C) / heads : 0;
     const int q = unit / p.Hkv, kvh = unit % p.Hkv;
     const int b = q % p.B;
-    const int Mq = p.Mq, rows = Mq * p.n_rep;
+    const int Mq = prefill ? min(p.Mq, p.chunk_rows - q_tile * p.Mq) : p.Mq, rows = Mq * p.n_rep;
+    const size_t row_base = (size_t)q * p.row_stride + p.row_off + q_tile * p.Mq;
     constexpr int R = 128 / G;                                    // query rows a CTA can carry (rows <= R)
     constexpr int NC = TK / G;                                    // keys of a tile per thread
     constexpr int half = DH / 2;
@@ -841,11 +858,12 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
     uint8_t *q_st = vring + (size_t)NV * tile_bytes;              // two planes of [R][DH] bf16, rows 16 bytes apart in the banks;
     uint8_t *w_st = q_st;                                         // after that the window's K tiles, then its V tiles
 
-    const int base = p.pos_override >= 0 ? p.pos_override : p.n_known[b] - 1;
-    const int ctx = min(max(base, 0), p.max_seq);
+    const int base = (p.pos_override >= 0 ? p.pos_override : p.n_known[b] - 1) + q_tile * p.Mq;
+    // keys that come from the cache: the committed context, in a prefill chunk also the rows of the chunk so far
+    const int ctx = min(max(base + (prefill ? Mq : 0), 0), p.max_seq);
     const int n_tiles = (ctx + TK - 1) / TK;
-    const bool has_window = rank == C - 1;
-    const int per = (n_tiles + 3 + C - 1) / C;
+    const bool has_window = rank == C - 1 && !prefill;
+    const int per = prefill ? n_tiles : (n_tiles + 3 + C - 1) / C;
     const int t0 = min(n_tiles, rank * per);
     const int t1 = has_window ? n_tiles : min(n_tiles, (rank + 1) * per);
     const int my_tiles = t1 - t0;
@@ -873,11 +891,15 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
         for (int h = 0; h < DH / 64; ++h) tma_load_2d(&p.kv_map, bar, dst + h * (TK * 128), h * 64, row0 + tile_row[t]);
     };
     const int row0_k = (int)p.row0_k, row0_v = (int)p.row0_v;     // (the pool has fewer than 2^31 rows)
-    // the first tiles do not depend on the kernel in front: on their way while it drains
-    if (k_lane)
-        for (int t = 0; t < min(NK, my_tiles); ++t) issue(t, kring + (size_t)t * tile_bytes, &kfull[t], row0_k);
-    if (v_lane)
-        for (int t = 0; t < min(NV, my_tiles); ++t) issue(t, vring + (size_t)t * tile_bytes, &vfull[t], row0_v);
+    // the first tiles do not depend on the kernel in front: on their way while it drains (in a prefill chunk they may:
+    // kv_write_kernel has just written them)
+    auto first_tiles = [&]() {
+        if (k_lane)
+            for (int t = 0; t < min(NK, my_tiles); ++t) issue(t, kring + (size_t)t * tile_bytes, &kfull[t], row0_k);
+        if (v_lane)
+            for (int t = 0; t < min(NV, my_tiles); ++t) issue(t, vring + (size_t)t * tile_bytes, &vfull[t], row0_v);
+    };
+    if (!prefill) first_tiles();
 
     // softmax threads: lane = column group * R + query row
     const int grp = tid / R, row = tid % R;                       // (warps 0-3; R is a multiple of 32)
@@ -910,6 +932,11 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
         }
 
     pdl_wait();                                                   // the projections come from the GEMM in front
+    if (prefill) {
+        // the keys were written with plain stores by the kernel in front, the copies read them through the async proxy
+        asm volatile("fence.proxy.async.global;" ::: "memory");
+        first_tiles();
+    }
 
 #pragma unroll
     for (int k = 0; k < QI; ++k) {
@@ -918,7 +945,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
             uint4 lo = make_uint4(0u, 0u, 0u, 0u), hi = lo, rlo = lo, rhi = lo;
             if (rr < rows) {
                 const int i = rr % Mq, g = rr / Mq;
-                const float *src = p.qkv + ((size_t)q * Mq + i) * qstride + (size_t)(kvh * p.n_rep + g) * DH;
+                const float *src = p.qkv + (row_base + i) * qstride + (size_t)(kvh * p.n_rep + g) * DH;
                 rotate8(src + j0, src + j0 + half, q_rope[k], p.qscale, lo, hi, &rlo, &rhi);
             }
             uint8_t *d0 = q_st + (size_t)rr * QROW, *d1 = d0 + (size_t)R * QROW;
@@ -938,7 +965,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
             const int i = wt * TK + jr, pos = base + i;
             w_k[wt][k][0] = w_k[wt][k][1] = w_v[wt][k][0] = w_v[wt][k][1] = make_uint4(0u, 0u, 0u, 0u);
             if (wt < n_wt && e < TK * CH && i < Mq && pos >= 0 && pos < p.max_seq) {
-                const float *src = p.qkv + ((size_t)q * Mq + i) * qstride + (size_t)(p.H + kvh) * DH;
+                const float *src = p.qkv + (row_base + i) * qstride + (size_t)(p.H + kvh) * DH;
                 const float *vs = src + (size_t)p.Hkv * DH;
                 w_v[wt][k][0] = round8(vs + j0);
                 w_v[wt][k][1] = round8(vs + j0 + half);
@@ -1138,7 +1165,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
             softmax_tile(wt, live ? max(0, min(min(TK, klim), qi - wt * TK + 1)) : 0);
         }
         for (int t = 0; t < my_tiles; ++t)
-            softmax_tile(n_wt + t, live ? min(TK, ctx - (t0 + t) * TK) : 0);
+            softmax_tile(n_wt + t, live ? min(TK, (prefill ? min(base + qi + 1, ctx) : ctx) - (t0 + t) * TK) : 0);
     }
     if (t_done > 0) wait_on(&bar_o[(t_done - 1) & 1], (unsigned)((t_done - 1) >> 1) & 1u, 9);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -1185,7 +1212,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
             const float inv = L > 0.f ? 1.0f / L : 0.f;
             acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
             const int i = rr % Mq, gq = rr / Mq;
-            __nv_bfloat16 *dst = p.out + ((size_t)q * Mq + i) * ostride + (size_t)(kvh * p.n_rep + gq) * DH + col;
+            __nv_bfloat16 *dst = p.out + (row_base + i) * ostride + (size_t)(kvh * p.n_rep + gq) * DH + col;
             uint2 packed;
             packed.x = pack_bf16(acc.x, acc.y);
             packed.y = pack_bf16(acc.z, acc.w);
@@ -1238,7 +1265,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
                     acc.z += wp * part[peer].z; acc.w += wp * part[peer].w;
                 }
                 const int i = rr % Mq, gq = rr / Mq;
-                __nv_bfloat16 *dst = p.out + ((size_t)q * Mq + i) * ostride + (size_t)(kvh * p.n_rep + gq) * DH + col;
+                __nv_bfloat16 *dst = p.out + (row_base + i) * ostride + (size_t)(kvh * p.n_rep + gq) * DH + col;
                 uint2 packed;
                 packed.x = pack_bf16(acc.x, acc.y);
                 packed.y = pack_bf16(acc.z, acc.w);
@@ -1260,6 +1287,34 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
     if (p.stamp && tid == 0 && blockIdx.x < STAMP_CTAS) p.stamp[STAMP_CTAS + blockIdx.x] = global_timer_ns();
 }
 
+// Prefill chunks: rotated keys and values of all rows into the cache, in front of the attention of the chunk.
+// Bound by its loads (fp32 projections in, bf16 out): one CTA per row, a thread per 8 dims of both halves of a head.
+template <int DH>
+__global__ void __launch_bounds__(256) kv_write_kernel(const __grid_constant__ AttnParams p)
+{
+    constexpr int half = DH / 2, CH = half / 8;
+    pdl_trigger();
+    if (p.skip && *p.skip) return;
+    const int q = blockIdx.x / p.chunk_rows, i = blockIdx.x % p.chunk_rows;
+    const int pos = (p.pos_override >= 0 ? p.pos_override : p.n_known[q % p.B] - 1) + i;
+    if (pos < 0 || pos >= p.max_seq) return;
+    const int page = p.page_table[(size_t)q * p.pages_per_seq + (pos >> p.page_shift)];
+    const float *row = p.qkv + ((size_t)q * p.row_stride + p.row_off + i) * (size_t)(p.H + 2 * p.Hkv) * DH;
+    pdl_wait();
+    for (int e = threadIdx.x; e < p.Hkv * CH; e += blockDim.x) {
+        const int kvh = e / CH, j0 = (e % CH) * 8;
+        const float *src = row + (size_t)(p.H + kvh) * DH, *vs = src + (size_t)p.Hkv * DH;
+        const long long r = ((long long)page * p.Hkv + kvh) * p.page_tokens + (pos & (p.page_tokens - 1));
+        __nv_bfloat16 *kd = p.pool + (size_t)(p.row0_k + r) * DH, *vd = p.pool + (size_t)(p.row0_v + r) * DH;
+        uint4 klo, khi;
+        rotate8(src + j0, src + j0 + half, p.rope + (size_t)pos * half + j0, 1.0f, klo, khi);
+        *(uint4 *)(vd + j0) = round8(vs + j0);
+        *(uint4 *)(vd + j0 + half) = round8(vs + j0 + half);
+        *(uint4 *)(kd + j0) = klo;
+        *(uint4 *)(kd + j0 + half) = khi;
+    }
+}
+
 struct AttnPlan {
     CUtensorMap kv_map;
     int sm_count;
@@ -1272,27 +1327,9 @@ bool attention_tc_supported(const scd_session *s, int Mq)
 {
     const scd_model_config_t &c = s->model->cfg;
     const int n_rep = c.n_heads / c.n_kv_heads;
+    // (longer prefill chunks run in parts of 128 query rows per KV head)
     return c.dtype == SCD_BF16 && s->attn_plan != nullptr && (c.head_dim == 64 || c.head_dim == 128) &&
-           c.kv_page_tokens % TK == 0 && Mq * n_rep <= 128;
-}
-
-int attention_session_prepare(scd_session *s)
-{
-    const scd_model_config_t &c = s->model->cfg;
-    s->attn_plan = nullptr;
-    if (c.dtype != SCD_BF16 || !(c.head_dim == 64 || c.head_dim == 128) || c.kv_page_tokens % TK != 0) return SCD_OK;
-    AttnPlan *plan = new AttnPlan();
-    const unsigned long long total_rows = (unsigned long long)c.n_layers * 2ull * s->Q * s->pages_per_seq *
-                                          c.n_kv_heads * c.kv_page_tokens;
-    if (total_rows >= (1ull << 31)) { delete plan; return SCD_OK; }      // row coordinates are int32: keep the SIMT path
-    int rc = make_tensor_map_bf16_2d(&plan->kv_map, s->kv_pool, total_rows, (unsigned long long)c.head_dim, TK, 64);
-    if (rc != SCD_OK) { delete plan; return rc; }
-    int dev = 0;
-    cudaGetDevice(&dev);
-    plan->sm_count = 148;
-    cudaDeviceGetAttribute(&plan->sm_count, cudaDevAttrMultiProcessorCount, dev);
-    s->attn_plan = plan;
-    return SCD_OK;
+           c.kv_page_tokens % TK == 0 && (Mq * n_rep <= 128 || n_rep <= 128);
 }
 
 void attention_session_release(scd_session *s)
@@ -1327,18 +1364,14 @@ static T5Kernel t5_kernel(int dh, int rows, int *G_out)
                      : (G == 1 ? attention_t5_kernel<64, 1> : G == 2 ? attention_t5_kernel<64, 2> : attention_t5_kernel<64, 4>);
 }
 
-// The largest cluster the tcgen05 kernel may use for windows of `rows` query rows: one CTA per SM and one wave,
-// i.e. the device must hold one cluster per (sequence, KV head) at the same time. Any size up to 8 (the kernel
-// splits tiles and rows evenly). The answer depends on how the SMs are grouped, so the runtime is asked - once.
-static int t5_max_cluster(const scd_session *s, AttnPlan *plan, int rows)
+// the tcgen05 kernel's shared-memory opt-in, once per device
+static int t5_prepare()
 {
-    if (plan->t5_rows == rows) return plan->t5_C;
-    const scd_model_config_t &c = s->model->cfg;
-    const int units = s->Q * c.n_kv_heads;
     static DeviceOnce once;
     int dev = 0;
-    if (current_device(&dev) != SCD_OK) return 0;
-    const int rc = once.run(dev, [&]() -> int {
+    const int rc = current_device(&dev);
+    if (rc != SCD_OK) return rc;
+    return once.run(dev, []() -> int {
         SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<128, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
         SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<128, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
         SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<128, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
@@ -1347,7 +1380,17 @@ static int t5_max_cluster(const scd_session *s, AttnPlan *plan, int rows)
         SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<64, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
         return SCD_OK;
     });
-    if (rc != SCD_OK) return 0;
+}
+
+// The largest cluster the tcgen05 kernel may use for windows of `rows` query rows: one CTA per SM and one wave,
+// i.e. the device must hold one cluster per (sequence, KV head) at the same time. Any size up to 8 (the kernel
+// splits tiles and rows evenly). The answer depends on how the SMs are grouped, so the runtime is asked - once.
+static int t5_max_cluster(const scd_session *s, AttnPlan *plan, int rows)
+{
+    if (plan->t5_rows == rows) return plan->t5_C;
+    const scd_model_config_t &c = s->model->cfg;
+    const int units = s->Q * c.n_kv_heads;
+    if (t5_prepare() != SCD_OK) return 0;
     int G = 1;
     const T5Kernel fn = t5_kernel(c.head_dim, rows, &G);
     cudaLaunchConfig_t cfg;
@@ -1402,7 +1445,8 @@ int attention_tc_variant(const scd_session *s, int Mq, long long ctx)
 static int attention_t5(scd_session *s, AttnParams &p, int C, cudaStream_t st)
 {
     const scd_model_config_t &c = s->model->cfg;
-    const int dh = c.head_dim, units = s->Q * c.n_kv_heads;
+    const int dh = c.head_dim, q_tiles = p.chunk_rows > 0 ? (p.chunk_rows + p.Mq - 1) / p.Mq : 1;
+    const int units = s->Q * c.n_kv_heads * q_tiles;
     const int rows = p.Mq * p.n_rep;
     int G = 1;
     const T5Kernel fn = t5_kernel(dh, rows, &G);
@@ -1437,7 +1481,30 @@ static int attention_t5(scd_session *s, AttnParams &p, int C, cudaStream_t st)
     return SCD_OK;
 }
 
-int attention_tc(scd_session *s, int layer, int Mq, int pos_override, cudaStream_t st)
+// All rows of a forward of more than 128 query rows per KV head: keys and values into the cache, then one CTA per
+// (stream-sequence, KV head, 128 query rows), each over all the keys its rows may attend to.
+static int attention_chunk(scd_session *s, AttnParams &p, cudaStream_t st)
+{
+    const scd_model_config_t &c = s->model->cfg;
+    p.chunk_rows = p.Mq;
+    p.Mq = 128 / p.n_rep;
+    cudaLaunchConfig_t cfg;
+    std::memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)(s->Q * p.chunk_rows), 1, 1);
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (c.head_dim == 128) SCD_CUDA_TRY(cudaLaunchKernelEx(&cfg, kv_write_kernel<128>, p));
+    else SCD_CUDA_TRY(cudaLaunchKernelEx(&cfg, kv_write_kernel<64>, p));
+    count_launches(1);
+    return attention_t5(s, p, 1, st);
+}
+
+static int attention_part(scd_session *s, int layer, int Mq, int row_stride, int row_off, int pos_override, bool chunk, cudaStream_t st)
 {
     const scd_model_config_t &c = s->model->cfg;
     AttnPlan *plan = (AttnPlan *)s->attn_plan;
@@ -1461,9 +1528,14 @@ int attention_tc(scd_session *s, int layer, int Mq, int pos_override, cudaStream
     p.pages_per_seq = s->pages_per_seq; p.page_tokens = c.kv_page_tokens;
     p.page_shift = __builtin_ctz((unsigned)c.kv_page_tokens);
     p.max_seq = c.max_seq; p.pos_override = pos_override;
+    p.row_stride = row_stride; p.row_off = row_off;
     p.n_mtiles = (Mq * p.n_rep + 15) / 16;
     p.qscale = 1.4426950408889634f / sqrtf((float)c.head_dim);
-    const int variant = attention_tc_variant(s, Mq, pos_override >= 0 ? (long long)pos_override : s->ctx_floor);
+    if (chunk) {
+        const int rc = t5_prepare();
+        return rc == SCD_OK ? attention_chunk(s, p, st) : rc;
+    }
+    const int variant = attention_tc_variant(s, Mq, (pos_override >= 0 ? (long long)pos_override : s->ctx_floor) + row_off);
     if ((variant & 15) == 2) return attention_t5(s, p, variant >> 4, st);
     const int units = s->Q * c.n_kv_heads;
     // split-KV over a cluster: up to two CTAs per SM over the whole grid, a power of two (measured:
@@ -1532,6 +1604,41 @@ int attention_tc(scd_session *s, int layer, int Mq, int pos_override, cudaStream
         else SCD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attention_tc_kernel<64, 1>, p));
     }
     count_launches(1);
+    return SCD_OK;
+}
+
+int attention_session_prepare(scd_session *s)
+{
+    const scd_model_config_t &c = s->model->cfg;
+    s->attn_plan = nullptr;
+    if (c.dtype != SCD_BF16 || !(c.head_dim == 64 || c.head_dim == 128) || c.kv_page_tokens % TK != 0) return SCD_OK;
+    AttnPlan *plan = new AttnPlan();
+    const unsigned long long total_rows = (unsigned long long)c.n_layers * 2ull * s->Q * s->pages_per_seq *
+                                          c.n_kv_heads * c.kv_page_tokens;
+    if (total_rows >= (1ull << 31)) { delete plan; return SCD_OK; }      // row coordinates are int32: keep the SIMT path
+    int rc = make_tensor_map_bf16_2d(&plan->kv_map, s->kv_pool, total_rows, (unsigned long long)c.head_dim, TK, 64);
+    if (rc != SCD_OK) { delete plan; return rc; }
+    int dev = 0;
+    cudaGetDevice(&dev);
+    plan->sm_count = 148;
+    cudaDeviceGetAttribute(&plan->sm_count, cudaDevAttrMultiProcessorCount, dev);
+    s->attn_plan = plan;
+    // the launch shape of the session's window (asked from the runtime) now, not in the first iteration
+    attention_tc_variant(s, s->L, std::max(0ll, s->att_t5_min_ctx));
+    return SCD_OK;
+}
+
+int attention_tc(scd_session *s, int layer, int Mq, int pos_override, cudaStream_t st)
+{
+    const scd_model_config_t &c = s->model->cfg;
+    const int part = 128 / (c.n_heads / c.n_kv_heads);            // query positions of one launch's CTA
+    if (Mq <= part) return attention_part(s, layer, Mq, Mq, 0, pos_override, false, st);
+    if (s->att_t5_min_ctx >= 0 && (c.max_seq + TK - 1) / TK <= T5_MAX_TILES)
+        return attention_part(s, layer, Mq, Mq, 0, pos_override, true, st);
+    for (int off = 0; off < Mq; off += part) {                    // one part after the other: each finds the one before in the cache
+        const int rc = attention_part(s, layer, std::min(part, Mq - off), Mq, off, pos_override, false, st);
+        if (rc != SCD_OK) return rc;
+    }
     return SCD_OK;
 }
 

@@ -49,6 +49,8 @@
 #include <tuple>
 
 #include "gemm.cuh"
+#include "gemm_pair.cuh"
+#include "ptx.cuh"
 
 namespace scd {
 
@@ -60,9 +62,9 @@ constexpr int UMMA_K = 16;
 constexpr int MAX_SEG = 3;
 constexpr int MAX_STAGES = 12;
 constexpr int MAX_CLUSTER = 8;
-constexpr int MAX_ROWS = 256;        // window rows one GEMM may carry
+constexpr int MAX_ROWS = 256;        // window rows one launch may carry (scd_gemm_bf16)
+constexpr int WS_ROWS = 128;         // ... and up to which a session uses this kernel
 constexpr int GEMM_THREADS = 192;
-constexpr unsigned SPIN_LIMIT = 1u << 22;
 
 enum { EPI_BF16 = 0, EPI_F32 = 1, EPI_RESID = 2, EPI_SWIGLU = 3 };
 
@@ -99,110 +101,10 @@ struct GemmParams {
     unsigned long long *stamp;       // optional [2][STAMP_CTAS]: %globaltimer at CTA entry and exit
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, unsigned count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, unsigned bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-// Bounded wait: false when the limit ran out.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity)
-{
-    const uint32_t a = smem_u32(bar);
-    for (unsigned i = 0; i < SPIN_LIMIT; ++i) {
-        unsigned ok;
-        asm volatile("{\n\t.reg .pred p;\n\t"
-                     "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                     "selp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(ok) : "r"(a), "r"(parity) : "memory");
-        if (ok) return true;
-    }
-    return false;
-}
-
-__device__ __forceinline__ void tma_load_2d(const CUtensorMap *map, uint64_t *bar, void *dst, int x, int y,
-                                            uint64_t policy)
-{
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-                 " [%0], [%1, {%3, %4}], [%2], %5;"
-                 ::"r"(smem_u32(dst)), "l"((uint64_t)map), "r"(smem_u32(bar)), "r"(x), "r"(y), "l"(policy)
-                 : "memory");
-}
-__device__ __forceinline__ void tma_load_3d(const CUtensorMap *map, uint64_t *bar, void *dst, int x, int y, int z,
-                                            uint64_t policy)
-{
-    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-                 " [%0], [%1, {%3, %4, %5}], [%2], %6;"
-                 ::"r"(smem_u32(dst)), "l"((uint64_t)map), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z), "l"(policy)
-                 : "memory");
-}
-__device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap *map)
-{
-    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)map) : "memory");
-}
-
-__device__ __forceinline__ void cluster_sync_all()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 __device__ __forceinline__ void epilogue_bar_sync()          // the four epilogue warps only
 {
     asm volatile("bar.sync 1, 128;" ::: "memory");
 }
-__device__ __forceinline__ float ld_peer_f32(uint32_t local_smem_addr, uint32_t peer)
-{
-    uint32_t remote;
-    float v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local_smem_addr), "r"(peer));
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote) : "memory");
-    return v;
-}
-
-// K-major, 128-byte-swizzled operand tile: rows of 128 bytes, 8-row groups 1024 bytes apart.
-__device__ __forceinline__ uint64_t umma_desc(uint32_t smem_addr)
-{
-    return (uint64_t)((smem_addr >> 4) & 0x3FFFu) | (1ull << 16) | (64ull << 32) | (1ull << 46) | (2ull << 61);
-}
-
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc)
-{
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                 ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(acc) : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint64_t *bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                 ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v)
-{
-    uint32_t r[32];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-                 : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v)
-{
-    uint32_t r[16];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-                 "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                 : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 __device__ __forceinline__ float4 ld_peer_f32x4(uint32_t local_smem_addr, uint32_t peer)
 {
     uint32_t remote;
@@ -675,15 +577,14 @@ int make_map(CUtensorMap *map, const void *ptr, uint64_t rows, uint64_t K, uint3
     return make_tensor_map_bf16_2d(map, ptr, rows, K, box_rows, BLOCK_K);
 }
 
-// Two-plane activation buffer [2][rows][K] bf16: box = 64 (K) x box_rows x both planes, 128-byte swizzle.
-// (rows: rows of a plane that the map covers from ptr on; plane_rows: rows from one plane to the other)
-int make_map_planes(CUtensorMap *map, const void *ptr, uint64_t rows, uint64_t plane_rows, uint64_t K, uint32_t box_rows)
+// Two-plane activation buffer [2][rows][K] bf16: box = 64 (K) x box_rows x box_planes, 128-byte swizzle.
+int make_map_planes(CUtensorMap *map, const void *ptr, uint64_t rows, uint64_t K, uint32_t box_rows, uint32_t box_planes)
 {
     EncodeTiledFn fn = encode_fn();
     SCD_REQUIRE(fn, SCD_ERR_CUDA, "cuTensorMapEncodeTiled entry point not found");
     cuuint64_t dims[3] = {K, rows, 2};
-    cuuint64_t strides[2] = {K * 2, plane_rows * K * 2};
-    cuuint32_t box[3] = {BLOCK_K, box_rows, 2};
+    cuuint64_t strides[2] = {K * 2, rows * K * 2};
+    cuuint32_t box[3] = {BLOCK_K, box_rows, box_planes};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(ptr), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -696,6 +597,7 @@ int make_map_planes(CUtensorMap *map, const void *ptr, uint64_t rows, uint64_t p
 struct GemmPlan {                    // per model: weight-side tensor maps, built on first use
     std::map<std::tuple<const void *, int, int, int>, CUtensorMap> wmaps;   // (matrix, rows, K, box rows)
     int sm_count;
+    int pairs;                       // CTA pairs that fit the device at once
     int kind_splits[GEMM_KINDS];     // K slices per GEMM kind chosen by gemm_set_kind_splits (0: the rule)
     int forced_splits, forced_stages; // scd_model_gemm_tune (0: the rule)
 };
@@ -792,17 +694,31 @@ struct SessionGemm {                 // activation-side tensor maps of a session
     std::map<std::tuple<const void *, int, int>, CUtensorMap> xmaps;
 };
 
-// (planes = 2: both planes of an activation buffer in one map; 1: its hi plane alone; m0: first row the map covers)
-int x_map(scd_session *s, const void *buf, int K, int nbox, int planes, int m0, CUtensorMap *out)
+// (planes = 2: both planes of an activation buffer in one map; 1: its hi plane alone)
+int x_map(scd_session *s, const void *buf, int K, int nbox, int planes, CUtensorMap *out)
 {
     SessionGemm *sg = (SessionGemm *)s->gemm_state;
-    buf = (const __nv_bfloat16 *)buf + (size_t)m0 * K;
     auto key = std::make_tuple(buf, K, nbox * 4 + planes);
     auto it = sg->xmaps.find(key);
     if (it == sg->xmaps.end()) {
         CUtensorMap m;
-        int rc = planes == 2 ? make_map_planes(&m, buf, (uint64_t)(s->rows_cap - m0), (uint64_t)s->rows_cap, (uint64_t)K, (uint32_t)nbox)
-                             : make_map(&m, buf, (uint64_t)(s->rows_cap - m0), (uint64_t)K, (uint32_t)nbox);
+        int rc = planes == 2 ? make_map_planes(&m, buf, (uint64_t)s->rows_cap, (uint64_t)K, (uint32_t)nbox, 2)
+                             : make_map(&m, buf, (uint64_t)s->rows_cap, (uint64_t)K, (uint32_t)nbox);
+        if (rc != SCD_OK) return rc;
+        it = sg->xmaps.emplace(key, m).first;
+    }
+    *out = it->second;
+    return SCD_OK;
+}
+// (for the CTA-pair kernel: 128 rows of one plane per copy)
+int x_map_pair(scd_session *s, const void *buf, int K, CUtensorMap *out)
+{
+    SessionGemm *sg = (SessionGemm *)s->gemm_state;
+    auto key = std::make_tuple(buf, K, 0);
+    auto it = sg->xmaps.find(key);
+    if (it == sg->xmaps.end()) {
+        CUtensorMap m;
+        int rc = make_map_planes(&m, buf, (uint64_t)s->rows_cap, (uint64_t)K, 128, 1);
         if (rc != SCD_OK) return rc;
         it = sg->xmaps.emplace(key, m).first;
     }
@@ -813,8 +729,6 @@ int x_map(scd_session *s, const void *buf, int K, int nbox, int planes, int m0, 
 
 struct NormIn { const float *ss; int parts; };                 // statistics of the x rows
 struct NormOut { const void *gain; void *xg; float *ss; };     // what a residual GEMM leaves behind
-
-int g_last_tiles = 0;                 // weight tiles of the most recent GEMM launch
 
 int w_map(GemmPlan *plan, const Segment &sg, int box_rows, CUtensorMap *out)
 {
@@ -830,12 +744,67 @@ int w_map(GemmPlan *plan, const Segment &sg, int box_rows, CUtensorMap *out)
     return SCD_OK;
 }
 
+// Forwards of more than 128 rows go to the CTA-pair kernel, whatever the shape: there the tensor cores bound the
+// GEMM, and at 256 rows this file's kernel has a ring of two slots.
+int run_gemm_pair(scd_session *s, const Segment *segs, int n_seg, int epi, const void *x, int K, int rows, void *out, int ldo,
+                  const NormIn *nin, const NormOut *nout, int x_planes, int *parts_out, cudaStream_t st)
+{
+    GemmPlan *plan = (GemmPlan *)s->model->gemm_plan;
+    const bool pair = epi == EPI_SWIGLU;
+    PairParams p;
+    std::memset(&p, 0, sizeof(p));
+    int t0 = 0;
+    for (int i = 0; i < n_seg; ++i) {
+        int rc = w_map(plan, segs[i], 128, &p.tmap_w[i]);
+        if (rc != SCD_OK) return rc;
+        p.seg_row0[i] = segs[i].row0;
+        p.seg_end[i] = segs[i].row_end;
+        p.seg_col0[i] = segs[i].col0;
+        p.seg_tile0[i] = t0;
+        if (!pair) t0 += (segs[i].row_end - segs[i].row0 + PAIR_COLS - 1) / PAIR_COLS;
+    }
+    p.n_seg = pair ? 1 : n_seg;
+    p.w_tiles = pair ? (segs[0].row_end + 127) / 128 : t0;
+    p.seg_tile0[p.n_seg] = p.w_tiles;
+    p.rows = rows;
+    p.x_tiles = (rows + PAIR_ROWS - 1) / PAIR_ROWS;
+    p.planes = x_planes;
+    p.k_blocks = K / BLOCK_K;
+    p.epi = epi == EPI_RESID ? PAIR_EPI_RESID : pair ? PAIR_EPI_SWIGLU : PAIR_EPI_F32;
+    p.out = out;
+    p.ldo = ldo;
+    p.out_plane = (long long)s->rows_cap * ldo;
+    p.ss_stride = s->rows_cap;
+    if (nin && nin->ss) {
+        p.ss_in = nin->ss; p.ss_parts = nin->parts;
+        p.inv_k = 1.0f / (float)K; p.eps = s->model->cfg.rms_eps;
+    }
+    if (nout && nout->xg) {
+        const int parts = (ldo + PAIR_UNIT - 1) / PAIR_UNIT;
+        SCD_REQUIRE(parts <= s->ss_parts_cap, SCD_ERR_SHAPE, "norm statistics: %d parts > %d", parts, s->ss_parts_cap);
+        p.gain_next = (const __nv_bfloat16 *)nout->gain;
+        p.xg_out = (__nv_bfloat16 *)nout->xg;
+        p.ss_out = nout->ss;
+        *parts_out = parts;
+    }
+    int rc = x_map_pair(s, x, K, &p.tmap_x);
+    if (rc != SCD_OK) return rc;
+    SCD_REQUIRE(pair_counter_count(p.w_tiles, p.x_tiles) <= s->gemm_counters, SCD_ERR_SHAPE, "GEMM: too many tiles");
+    p.scratch = s->gemm_scratch;
+    p.err = (int *)s->gemm_ws;
+    p.counters = (unsigned *)s->gemm_ws + 64;
+    p.skip = s->skip_now;
+    p.stamp = take_stamp_slot();
+    return launch_gemm_pair(p, plan->pairs, st);
+}
+
 // x_planes: 2 = multiply with both planes of x, 1 = with its hi plane alone (where the output is rounded to
 // bf16 right away - Q, K, V - or is the last stage - the logits - the remainder plane buys nothing)
-// (the window rows m0 .. m0 + rows - 1, at most 256: one accumulator holds all rows of a weight tile)
-int run_gemm_rows(scd_session *s, int kind, const Segment *segs, int n_seg, int epi, const void *x, int K, int m0, int rows,
-                  void *out, int ldo, const NormIn *nin, const NormOut *nout, int x_planes, cudaStream_t st)
+// *parts_out: partial sums of squares per row that a residual GEMM left
+int run_gemm(scd_session *s, int kind, const Segment *segs, int n_seg, int epi, const void *x, int K, int rows,
+             void *out, int ldo, const NormIn *nin, const NormOut *nout, int x_planes, int *parts_out, cudaStream_t st)
 {
+    if (rows > WS_ROWS) return run_gemm_pair(s, segs, n_seg, epi, x, K, rows, out, ldo, nin, nout, x_planes, parts_out, st);
     GemmPlan *plan = (GemmPlan *)s->model->gemm_plan;
     const bool pair = epi == EPI_SWIGLU;
     GemmParams p;
@@ -862,39 +831,26 @@ int run_gemm_rows(scd_session *s, int kind, const Segment *segs, int n_seg, int 
     p.stages = choose_stages(p.nbox, p.x_planes, (p.k_blocks + p.k_splits - 1) / p.k_splits,
                              tiles * p.k_splits <= 2 * plan->sm_count, plan->forced_stages);
     p.epi = epi;
-    // everything indexed by window row starts at row m0
-    const size_t out_elem = (epi == EPI_BF16 || epi == EPI_SWIGLU) ? 2 : 4;
-    p.out = (char *)out + (size_t)m0 * ldo * out_elem;
+    p.out = out;
     p.ldo = ldo;
     p.ss_stride = s->rows_cap;
     if (nin && nin->ss) {
-        p.ss_in = nin->ss + m0; p.ss_parts = nin->parts;
+        p.ss_in = nin->ss; p.ss_parts = nin->parts;
         p.inv_k = 1.0f / (float)K; p.eps = s->model->cfg.rms_eps;
     }
     if (nout && nout->xg) {
         SCD_REQUIRE(tiles <= s->ss_parts_cap, SCD_ERR_SHAPE, "norm statistics: %d tiles > %d", tiles, s->ss_parts_cap);
         p.gain_next = (const __nv_bfloat16 *)nout->gain;
-        p.xg_out = (__nv_bfloat16 *)nout->xg + (size_t)m0 * ldo;
-        p.ss_out = nout->ss + m0;
+        p.xg_out = (__nv_bfloat16 *)nout->xg;
+        p.ss_out = nout->ss;
+        *parts_out = tiles;                                // one partial sum of squares per output tile
     }
-    int rc = x_map(s, x, K, p.nbox, p.x_planes, m0, &p.tmap_x);
+    int rc = x_map(s, x, K, p.nbox, p.x_planes, &p.tmap_x);
     if (rc != SCD_OK) return rc;
     p.err = (int *)s->gemm_ws;
     p.skip = s->skip_now;
     p.stamp = take_stamp_slot();
-    g_last_tiles = tiles;
     return launch(p, tiles, st);
-}
-
-// More than 256 window rows: one pass over the weights per block of 256 rows.
-int run_gemm(scd_session *s, int kind, const Segment *segs, int n_seg, int epi, const void *x, int K, int rows,
-             void *out, int ldo, const NormIn *nin, const NormOut *nout, int x_planes, cudaStream_t st)
-{
-    for (int m0 = 0; m0 < rows; m0 += 256) {
-        const int rc = run_gemm_rows(s, kind, segs, n_seg, epi, x, K, m0, std::min(256, rows - m0), out, ldo, nin, nout, x_planes, st);
-        if (rc != SCD_OK) return rc;
-    }
-    return SCD_OK;
 }
 
 }  // namespace
@@ -911,6 +867,22 @@ int gemm_plan_create(scd_model *m)
         delete plan;
         return cuda_fail(cudaGetLastError(), "cudaDeviceGetAttribute");
     }
+    int rc = pair_grid_limit(&plan->pairs);
+    // the maps of all weights now, for both kernels: a session's first window pays for none of them
+    const scd_model_config_t &c = m->cfg;
+    const int d = c.d_model, dq = c.n_heads * c.head_dim, dkv = c.n_kv_heads * c.head_dim;
+    CUtensorMap unused;
+    auto add = [&](const void *w, int rows, int K, int box) { if (rc == SCD_OK) rc = w_map(plan, Segment{w, rows, K, 0, rows, 0}, box, &unused); };
+    for (int l = 0; l < c.n_layers; ++l) {
+        add(m->wq[l], dq, d, 128);
+        add(m->wk[l], dkv, d, 128);
+        add(m->wv[l], dkv, d, 128);
+        add(m->wo[l], d, dq, 128);
+        for (int box = 64; box <= 128; box += 64) { add(m->w_gate[l], c.d_ffn, d, box); add(m->w_up[l], c.d_ffn, d, box); }
+        add(m->w_down[l], d, c.d_ffn, 128);
+    }
+    add(m->lm_head, c.vocab_out, d, 128);
+    if (rc != SCD_OK) { delete plan; return rc; }
     m->gemm_plan = plan;
     return SCD_OK;
 }
@@ -930,7 +902,7 @@ int gemm_tc_qkv(scd_session *s, int l, int rows, int ss_parts, cudaStream_t st)
     const Segment segs[3] = {{m->wq[l], dq, d, 0, dq, 0}, {m->wk[l], dkv, d, 0, dkv, dq}, {m->wv[l], dkv, d, 0, dkv, dq + dkv}};
     const NormIn nin = {s->ss, ss_parts};
     // fp32 out: the attention kernel rotates Q and K in fp32 and rounds each of Q, K, V to bf16 once
-    return run_gemm(s, GEMM_QKV, segs, 3, EPI_F32, s->xn, d, rows, s->qkv, dq + 2 * dkv, &nin, nullptr, 1, st);
+    return run_gemm(s, GEMM_QKV, segs, 3, EPI_F32, s->xn, d, rows, s->qkv, dq + 2 * dkv, &nin, nullptr, 1, nullptr, st);
 }
 
 int gemm_tc_residual(scd_session *s, int l, int which, int rows, const void *gain_next, int *parts_out,
@@ -942,11 +914,8 @@ int gemm_tc_residual(scd_session *s, int l, int which, int rows, const void *gai
     const int K = which == 0 ? dq : c.d_ffn;
     const Segment segs[1] = {{which == 0 ? m->wo[l] : m->w_down[l], c.d_model, K, 0, c.d_model, 0}};
     const NormOut nout = {gain_next, s->xn, s->ss};
-    const int rc = run_gemm(s, which == 0 ? GEMM_O : GEMM_DOWN, segs, 1, EPI_RESID, which == 0 ? s->att : s->act, K, rows,
-                            s->h, c.d_model, nullptr,
-                            &nout, 2, st);
-    *parts_out = g_last_tiles;                          // one partial sum of squares per output tile
-    return rc;
+    return run_gemm(s, which == 0 ? GEMM_O : GEMM_DOWN, segs, 1, EPI_RESID, which == 0 ? s->att : s->act, K, rows,
+                    s->h, c.d_model, nullptr, &nout, 2, parts_out, st);
 }
 
 int gemm_tc_gate_up(scd_session *s, int l, int rows, int ss_parts, cudaStream_t st)
@@ -955,7 +924,7 @@ int gemm_tc_gate_up(scd_session *s, int l, int rows, int ss_parts, cudaStream_t 
     const scd_model_config_t &c = m->cfg;
     const Segment segs[2] = {{m->w_gate[l], c.d_ffn, c.d_model, 0, c.d_ffn, 0}, {m->w_up[l], c.d_ffn, c.d_model, 0, c.d_ffn, 0}};
     const NormIn nin = {s->ss, ss_parts};
-    return run_gemm(s, GEMM_GATE_UP, segs, 2, EPI_SWIGLU, s->xn, c.d_model, rows, s->act, c.d_ffn, &nin, nullptr, 2, st);
+    return run_gemm(s, GEMM_GATE_UP, segs, 2, EPI_SWIGLU, s->xn, c.d_model, rows, s->act, c.d_ffn, &nin, nullptr, 2, nullptr, st);
 }
 
 // Logits of the ids [lo, hi) and, when eol >= 0, of id eol; other columns of `logits` are left
@@ -970,7 +939,7 @@ int gemm_tc_lm_head(scd_session *s, int rows, float *logits, int lo, int hi, int
     if (eol >= 0 && !(eol >= lo8 && eol < hi))
         segs[n++] = {s->model->lm_head, c.vocab_out, c.d_model, eol & ~7, std::min(c.vocab_out, (eol & ~7) + 8), 0};
     const NormIn nin = {s->ss, ss_parts};
-    return run_gemm(s, GEMM_LM_HEAD, segs, n, EPI_F32, s->xn, c.d_model, rows, logits, c.vocab_out, &nin, nullptr, 1, st);
+    return run_gemm(s, GEMM_LM_HEAD, segs, n, EPI_F32, s->xn, c.d_model, rows, logits, c.vocab_out, &nin, nullptr, 1, nullptr, st);
 }
 
 void gemm_set_kind_splits(scd_model *m, int kind, int k_splits)
@@ -979,16 +948,24 @@ void gemm_set_kind_splits(scd_model *m, int kind, int k_splits)
     if (plan && kind >= 0 && kind < GEMM_KINDS) plan->kind_splits[kind] = std::max(0, std::min(k_splits, MAX_CLUSTER));
 }
 
-// Upper bound of the partial sums of squares a residual GEMM leaves per row (= its output tiles).
-int gemm_norm_parts_cap(const scd_session *s) { return std::max(1024, (s->model->cfg.d_model + 7) / 8); }
+// Upper bound of the partial sums of squares a residual GEMM leaves per row (one per 32 columns).
+int gemm_norm_parts_cap(const scd_session *s) { return (s->model->cfg.d_model + PAIR_UNIT - 1) / PAIR_UNIT; }
 
-// Per-session state: the activation-side tensor maps and the device error word.
+// Per-session state: the activation-side tensor maps, the device error word and, when a forward can have more
+// rows than one weight-streaming launch takes, the CTA-pair kernel's tile counters and partial tiles.
 int gemm_session_prepare(scd_session *s)
 {
     s->gemm_state = new SessionGemm();
-    SCD_CUDA_TRY(cudaMalloc(&s->gemm_ws, 256));
-    SCD_CUDA_TRY(cudaMemset(s->gemm_ws, 0, 256));
     s->gemm_ws_bytes = 256;
+    if (s->rows_cap > WS_ROWS) {
+        const scd_model_config_t &c = s->model->cfg;
+        const int widest = std::max(std::max((c.n_heads + 2 * c.n_kv_heads) * c.head_dim, 2 * c.d_ffn), std::max(c.vocab_out, c.d_model));
+        s->gemm_counters = pair_counter_count(widest / PAIR_COLS + PAIR_MAX_SEG + 1, (s->rows_cap + PAIR_ROWS - 1) / PAIR_ROWS);
+        s->gemm_ws_bytes += s->gemm_counters * sizeof(unsigned);
+        SCD_CUDA_TRY(cudaMalloc(&s->gemm_scratch, pair_scratch_bytes(((GemmPlan *)s->model->gemm_plan)->pairs)));
+    }
+    SCD_CUDA_TRY(cudaMalloc(&s->gemm_ws, s->gemm_ws_bytes));
+    SCD_CUDA_TRY(cudaMemset(s->gemm_ws, 0, s->gemm_ws_bytes));
     return SCD_OK;
 }
 

@@ -18,8 +18,9 @@ struct scd_session {
     scd_model *model;
     scd_decode_config_t cfg;
     int B, S, Q, L;           // sequences, streams per sequence, stream-sequences, window rows
-    int chunk;                // rows per stream-sequence that one forward may carry
-    int rows_cap;             // Q * chunk
+    int chunk;                // rows per stream-sequence that one explicit forward may carry
+    int prefill_chunk;        // ... that one pass over the prompt carries (>= chunk)
+    int rows_cap;             // Q * prefill_chunk
     int pages_per_seq;
     int prompt_len, n_new;
     bool prefilled;
@@ -51,8 +52,9 @@ struct scd_session {
     int att_variant;          // attention variant the captured iteration was built with
     long long att_t5_min_ctx; // known context from which the tcgen05 attention kernel is used (< 0: never)
     void *stamps;             // device time stamps of scd_step_timeline (allocated on first use)
-    void *gemm_ws;            // device error word of the tcgen05 GEMM
-    size_t gemm_ws_bytes;
+    void *gemm_ws;            // device error word of the tcgen05 kernels, then the CTA-pair GEMM's tile counters
+    size_t gemm_ws_bytes, gemm_counters;
+    float *gemm_scratch;      // partial tiles of the CTA-pair GEMM
     void *gemm_state;         // activation-side tensor maps
     void *attn_plan;          // tensor map of the KV pool for the tensor-core attention (bf16 sessions)
 

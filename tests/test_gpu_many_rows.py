@@ -1,0 +1,64 @@
+"""GPU parity of forwards of more than 128 rows (prefill chunks, large batches): the CTA-pair GEMM and the
+attention over chunks of several query tiles, against the oracle's forward. Bound: 3e-2 in max-relative error, the
+parity bound of the bf16 path."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2510_24211_b200 import binding as scd
+from test_gpu_session import MID_BF16_D64, MID_BF16_D128_GQA, SMALL_BF16, _models, _rel
+
+pytestmark = pytest.mark.gpu
+
+WIDE_GQA4 = dict(n_layers=2, d_model=576, n_heads=8, n_kv_heads=2, head_dim=64, d_ffn=832, vocab_out=1000,
+                 vocab_in=1010, dtype="bf16", rope_base=10000.0, rms_eps=1e-5)   # tiles of 256 that end inside a run of 32
+
+
+@pytest.mark.parametrize("shape,page,P,B,M,min_ctx", [
+    (MID_BF16_D64, 64, 130, 1, 3, 512),        # 129 prompt rows: one more than the weight-streaming kernel takes
+    (MID_BF16_D64, 64, 258, 1, 129, 512),      # 257 rows: a second x tile with one row; a window of two query tiles
+    (MID_BF16_D64, 128, 258, 1, 129, -1),      # the same through the mma.sync attention kernel, part after part
+    (MID_BF16_D128_GQA, 64, 700, 1, 65, 512),  # two query heads per KV head: 64 positions per query tile
+    (WIDE_GQA4, 64, 161, 3, 43, 512),          # 480 prompt rows, 129 window rows of three sequences
+    (WIDE_GQA4, 128, 2700, 1, 5, 512),         # two passes over the prompt (2560 rows at most), the second over a context
+    (SMALL_BF16, 16, 150, 2, 70, 512),         # head_dim 32: no tensor-core attention
+])
+def test_many_rows_match_oracle(shape, page, P, B, M, min_ctx):
+    gm, om = _models(shape, max_seq=P + M + 9, seed=17, std=0.06, page=page, n_streams=B)
+    rng = np.random.default_rng(P)
+    prompt = rng.integers(0, shape["vocab_in"], size=(B, P)).astype(np.int32)
+    sess = scd.Session(gm, scd.decode_config(batch=B, window_L=M, allowed_hi=shape["vocab_out"]))
+    sess.scd_session_attention_min_ctx(min_ctx)
+    sess.scd_prefill(prompt, n_new=M + 4)
+    ids = np.concatenate([prompt[:, -1:], rng.integers(0, shape["vocab_in"], size=(B, M - 1))], axis=1).astype(np.int32)
+    logits, hidden = sess.scd_forward_window(torch.from_numpy(ids).cuda(), want_hidden=True)
+    for b in range(B):
+        om.forward(prompt[b, :-1], 0, stream=b)
+        ref_logits, ref_hidden = om.forward(ids[b], P - 1, stream=b, want_hidden=True)
+        assert _rel(hidden[b].cpu().numpy(), ref_hidden) <= 3e-2
+        assert _rel(logits[b].cpu().numpy(), ref_logits) <= 3e-2
+    again = sess.scd_forward_window(torch.from_numpy(ids).cuda())
+    assert torch.equal(again, logits)          # cut tiles are added up in a fixed order
+
+
+def test_step_of_many_rows_reads_only_the_sampled_ids():
+    """A decoding step of 160 rows computes the logits of the allowed ids and of the end-of-row id alone; they are
+    those of the explicit forward over the whole vocabulary. Only where a tile's sum over K is cut differs: fp32
+    sums of 576 terms in another order, 1e-5 of the largest logit."""
+    shape, B, L, P = WIDE_GQA4, 5, 16, 40
+    gm, _ = _models(shape, max_seq=P + 80, seed=5, std=0.06, page=64)
+    rng = np.random.default_rng(2)
+    cond = rng.integers(0, shape["vocab_in"], size=(B, P)).astype(np.int32)
+    cfg = scd.decode_config(batch=B, window_L=L, top_k=50, cfg_lambda=1.0, seed=4, allowed_lo=100, allowed_hi=613,
+                            row_period=9, eol_id=901)
+    sess = scd.Session(gm, cfg)
+    prompts = np.concatenate([cond, np.full_like(cond, 1)])
+    sess.scd_prefill(prompts, n_new=60)
+    drafts = sess.scd_debug_read("drafts").copy()
+    ids = np.concatenate([prompts[:, -1:], np.tile(drafts[:, :L - 1], (2, 1))], axis=1).astype(np.int32)
+    want = sess.scd_forward_window(torch.from_numpy(np.ascontiguousarray(ids)).cuda()).cpu().numpy()
+    sess.scd_step()
+    got = sess.scd_debug_read("logits")
+    for lo, hi in ((100, 613), (901, 902)):
+        assert _rel(got[:, :, lo:hi], want[:, :, lo:hi]) <= 1e-5
