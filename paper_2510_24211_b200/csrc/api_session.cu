@@ -154,7 +154,7 @@ void free_session_memory(scd_session *s)
     void *ptrs[] = {s->kv_pool, s->page_table, s->n_known, s->n_total, s->shift, s->prev_lw, s->drafts,
                     s->n_commit, s->tokens, s->tokens_u, s->row_y, s->row_y_indep, s->ids_buf, s->iter,
                     s->done_count, s->accept_flags, s->xbuf[0], s->xbuf[1], s->stats[0], s->stats[1],
-                    s->dev_stats, s->finished, s->h, s->ss, s->xn, s->qkv, s->att, s->gu, s->act, s->logits, s->gemm_ws, s->gemm_scratch, s->stamps};
+                    s->dev_stats, s->finished, s->h, s->ss, s->xn, s->qkv, s->att, s->act, s->logits, s->gemm_ws, s->gemm_scratch, s->stamps};
     for (void *p : ptrs) if (p) cudaFree(p);
     if (s->host_pinned) cudaFreeHost(s->host_pinned);
     if (s->gemm_state) gemm_session_release(s);
@@ -307,7 +307,6 @@ int scd_session_create(scd_model_t *m, const scd_decode_config_t *cfg, scd_sessi
     { char *p; TRY_ALLOC(dev_alloc(&p, wide * rows * d * es)); s->xn = p; }
     { char *p; TRY_ALLOC(dev_alloc(&p, wide * rows * (dq + 2 * dkv) * es)); s->qkv = p; }
     { char *p; TRY_ALLOC(dev_alloc(&p, wide * rows * dq * es)); s->att = p; }
-    if (c.dtype == SCD_F32) { char *p; TRY_ALLOC(dev_alloc(&p, rows * 2 * F * es)); s->gu = p; }
     { char *p; TRY_ALLOC(dev_alloc(&p, wide * rows * F * es)); s->act = p; }
     s->ss_parts_cap = c.dtype == SCD_BF16 && m->gemm_plan ? gemm_norm_parts_cap(s) : 1;
     TRY_ALLOC(dev_alloc(&s->ss, (size_t)s->ss_parts_cap * rows));

@@ -44,7 +44,7 @@ struct scd_session {
 
     // activations (device)
     float *h;                 // residual stream [rows][d]
-    void *xn, *qkv, *att, *gu, *act;
+    void *xn, *qkv, *att, *act;
     float *ss;                // bf16 sessions: partial sums of squares of h, [ss_parts_cap][rows_cap]
     int ss_parts_cap;
     float *logits;            // [rows_cap_logits][V]

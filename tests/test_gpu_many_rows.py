@@ -62,3 +62,34 @@ def test_step_of_many_rows_reads_only_the_sampled_ids():
     got = sess.scd_debug_read("logits")
     for lo, hi in ((100, 613), (901, 902)):
         assert _rel(got[:, :, lo:hi], want[:, :, lo:hi]) <= 1e-5
+
+
+TINY_F32 = dict(n_layers=2, d_model=128, n_heads=4, n_kv_heads=2, head_dim=32, d_ffn=208, vocab_out=300, vocab_in=310,
+                dtype="f32", rope_base=10000.0, rms_eps=1e-5)
+
+
+@pytest.mark.parametrize("over,P,B,M", [
+    (dict(), 5, 1, 1),                                                       # one row
+    (dict(head_dim=96, n_heads=2, n_kv_heads=1), 40, 1, 17),                 # a second tile with one row
+    (dict(d_model=130, d_ffn=206), 37, 2, 16),                               # K not a multiple of four: scalar loads
+    (dict(d_model=1100, d_ffn=1030, head_dim=64, n_heads=4, n_kv_heads=4), 20, 1, 19),   # rows longer than one piece in shared memory
+    (dict(head_dim=128, n_heads=3, n_kv_heads=3, d_ffn=600), 300, 1, 33),    # ten key tiles over eight warps
+    (dict(d_ffn=2048, vocab_out=5000), 130, 2, 64),                          # enough columns for four per warp
+])
+def test_fp32_layers_match_oracle(over, P, B, M):
+    """The fp32 path against the oracle. Bound 2e-5 of the largest value: fp32 sums of up to 2048 terms, two layers
+    (one sum's error is about sqrt(2048) 2^-24 = 3e-6 of its magnitude)."""
+    shape = dict(TINY_F32, **over)
+    gm, om = _models(shape, max_seq=P + M + 9, seed=19, std=0.05, n_streams=B)
+    rng = np.random.default_rng(P)
+    prompt = rng.integers(0, shape["vocab_in"], size=(B, P)).astype(np.int32)
+    sess = scd.Session(gm, scd.decode_config(batch=B, window_L=M, allowed_hi=shape["vocab_out"]))
+    sess.scd_prefill(prompt, n_new=M + 4)
+    ids = np.concatenate([prompt[:, -1:], rng.integers(0, shape["vocab_in"], size=(B, M - 1))], axis=1).astype(np.int32)
+    logits, hidden = sess.scd_forward_window(torch.from_numpy(ids).cuda(), want_hidden=True)
+    for b in range(B):
+        if P > 1:
+            om.forward(prompt[b, :-1], 0, stream=b)
+        ref_logits, ref_hidden = om.forward(ids[b], P - 1, stream=b, want_hidden=True)
+        assert _rel(hidden[b].cpu().numpy(), ref_hidden) <= 2e-5
+        assert _rel(logits[b].cpu().numpy(), ref_logits) <= 2e-5
