@@ -223,7 +223,7 @@ int scd_verify(const scd_decode_config_t *cfg, int32_t V, const float *p_logits,
  *     pool and outside any stream capture; from the second call on nothing is allocated. The address
  *     is cached per device ordinal for the life of the process (cudaDeviceReset invalidates it).
  *   - All calls on a device share the one buffer, which keeps whatever the previous call left
- *     in it; the part that must start at zero is cleared on `stream` before the kernel. Two
+ *     in it; nothing in it is read before it is written. Two
  *     calls that can overlap on the GPU (different streams, no ordering between them) race on
  *     the buffer: order them, or give one of them scd_verify with its own workspace. */
 int64_t scd_verify_noalloc_max_bytes(void);

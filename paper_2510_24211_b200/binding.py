@@ -198,9 +198,9 @@ def scd_verify(cfg: DecodeConfig, p_logits, q_logits, draft_ids, positions, iter
     if workspace is None:
         workspace = torch.empty(scd_verify_workspace_bytes(cfg, V), dtype=torch.uint8, device=dev)
     n_commit = torch.empty(B, dtype=torch.int32, device=dev)
-    committed = torch.zeros(B, L, dtype=torch.int32, device=dev)
+    committed = torch.empty(B, L, dtype=torch.int32, device=dev)
     next_drafts = torch.empty(B, L, dtype=torch.int32, device=dev)
-    flags = torch.zeros(B, L, dtype=torch.uint8, device=dev)
+    flags = torch.empty(B, L, dtype=torch.uint8, device=dev)
     _check(lib().scd_verify(C.byref(cfg), V, _ptr(p_logits), _ptr(q_logits), _ptr(draft_ids),
                             _ptr(positions), iteration, _ptr(n_commit), _ptr(committed),
                             _ptr(next_drafts), _ptr(flags), _ptr(workspace), _stream(stream)))

@@ -73,7 +73,6 @@ void session_verify_params(scd_session *s, VerifyParams &p)
     p.tokens = s->tokens; p.token_stride = s->model->cfg.max_seq;
     p.accept_flags = s->accept_flags;
     p.row_y = s->row_y; p.row_y_indep = s->row_y_indep;
-    p.done_count = s->done_count;
     p.dev_stats = s->dev_stats;
     p.finished = s->finished;
 }
@@ -92,7 +91,6 @@ int enqueue_step(scd_session *s, cudaStream_t st, StepProfiler *prof = nullptr)
     VerifyParams p;
     session_verify_params(s, p);
     if (prof) prof->mark(PROF_VERIFY);
-    count_launches(1);
     return launch_verify(p, st);
 }
 
@@ -153,7 +151,7 @@ void free_session_memory(scd_session *s)
     if (s->step_graph) cudaGraphExecDestroy(s->step_graph);
     void *ptrs[] = {s->kv_pool, s->page_table, s->n_known, s->n_total, s->shift, s->prev_lw, s->drafts,
                     s->n_commit, s->tokens, s->tokens_u, s->row_y, s->row_y_indep, s->ids_buf, s->iter,
-                    s->done_count, s->accept_flags, s->xbuf[0], s->xbuf[1], s->stats[0], s->stats[1],
+                    s->accept_flags, s->xbuf[0], s->xbuf[1], s->stats[0], s->stats[1],
                     s->dev_stats, s->finished, s->h, s->ss, s->xn, s->qkv, s->att, s->act, s->logits, s->gemm_ws, s->gemm_scratch, s->stamps};
     for (void *p : ptrs) if (p) cudaFree(p);
     if (s->host_pinned) cudaFreeHost(s->host_pinned);
@@ -287,7 +285,6 @@ int scd_session_create(scd_model_t *m, const scd_decode_config_t *cfg, scd_sessi
     TRY_ALLOC(dev_alloc(&s->prev_lw, s->B));
     TRY_ALLOC(dev_alloc(&s->n_commit, s->B));
     TRY_ALLOC(dev_alloc(&s->iter, s->B));
-    TRY_ALLOC(dev_alloc(&s->done_count, s->B));
     TRY_ALLOC(dev_alloc(&s->drafts, wrows));
     TRY_ALLOC(dev_alloc(&s->row_y, wrows));
     TRY_ALLOC(dev_alloc(&s->row_y_indep, 2 * wrows));
@@ -323,7 +320,6 @@ int scd_session_create(scd_model_t *m, const scd_decode_config_t *cfg, scd_sessi
 #undef TRY_ALLOC
     const int np = s->Q * s->pages_per_seq;
     identity_pages_kernel<<<(np + 255) / 256, 256>>>(s->page_table, np);
-    cudaMemset(s->done_count, 0, s->B * sizeof(unsigned));
     cudaMemset(s->dev_stats, 0, sizeof(VerifyStatsDev));
     cudaMemset(s->kv_pool, 0, s->kv_layer_stride * c.n_layers * es);
     cudaMemset(s->logits, 0, (size_t)s->Q * s->L * V * sizeof(float));

@@ -77,7 +77,7 @@ void fill_verify_params(VerifyParams &p, const scd_decode_config_t *cfg, int V)
 static inline int64_t align256(int64_t x) { return (x + 255) & ~(int64_t)255; }
 
 struct VerifyWorkspace {
-    int64_t xbuf, stats0, stats1, row_y, row_y_indep, done, total;
+    int64_t xbuf, stats0, stats1, row_y, row_y_indep, total;
 };
 
 static VerifyWorkspace verify_layout(int B, int L, int V)
@@ -90,7 +90,7 @@ static VerifyWorkspace verify_layout(int B, int L, int V)
     w.stats1 = off;      off = align256(off + rows * (int64_t)sizeof(RowStats));
     w.row_y = off;       off = align256(off + rows * 4);
     w.row_y_indep = off; off = align256(off + rows * 8);
-    w.done = off;        off = align256(off + (int64_t)B * 4);
+    off = align256(off + (int64_t)B * 4);              // (spare: the size that callers know)
     w.total = off;
     return w;
 }
@@ -175,9 +175,6 @@ int scd_verify(const scd_decode_config_t *cfg, int32_t V, const float *p_logits,
     p.accept_flags = accept_flags;
     p.row_y = (int *)(ws + w.row_y);
     p.row_y_indep = (int *)(ws + w.row_y_indep);
-    p.done_count = (unsigned *)(ws + w.done);
-    SCD_CUDA_TRY(cudaMemsetAsync(p.done_count, 0, (size_t)p.B * 4, st));
-    count_launches(1);
     return launch_verify(p, st);
 }
 
@@ -240,8 +237,7 @@ int scd_verify_noalloc(const scd_decode_config_t *cfg, int32_t V, const float *p
         return SCD_OK;
     });
     if (rc != SCD_OK) return rc;
-    // scd_verify zeroes the part of the workspace that must start at zero (the per-sequence
-    // tickets) on `stream` before the kernel; everything else is written before it is read
+    // everything in the workspace is written before it is read
     return scd_verify(cfg, V, p_logits, q_logits, draft_ids, positions, iteration, n_commit, committed_ids,
                       next_draft_ids, accept_flags, g_noalloc_scratch_addr[dev], stream);
 }

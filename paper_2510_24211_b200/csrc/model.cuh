@@ -34,7 +34,7 @@ struct scd_session {
     // window state (device)
     int *n_known, *n_total, *shift, *prev_lw, *drafts, *n_commit, *tokens, *tokens_u;
     int *row_y, *row_y_indep, *ids_buf;
-    unsigned *iter, *done_count;
+    unsigned *iter;
     unsigned char *accept_flags;
     float *xbuf[2];
     scd::RowStats *stats[2];

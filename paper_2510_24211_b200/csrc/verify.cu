@@ -1,12 +1,10 @@
-// Fused verify-and-redraft kernel: logits -> CFG mix -> temperature -> top-k -> integer weights
-// -> accept / reject -> residual sample -> first rejection -> commit -> coupled redraft.
+// Fused verify-and-redraft kernel for rows of more than 131072 ids (shorter ones: verify_rows.cu): logits -> CFG
+// mix -> temperature -> top-k -> integer weights -> accept / reject -> residual sample -> redraft.
 //
-// One CTA per window row (Algorithm 6 evaluates ALL rows, with no break; Algorithm 1 per row).
-// The CTA that finishes last for a sequence ("last block done" ticket, no spinning) runs the
-// only serial part, the first-rejection index (the Accept step of Algorithm 6), commits the accepted
-// prefix and builds the next window: a row that survives keeps its MRS output as draft and its
-// target distribution as draft distribution, which is the maximal coupling of Algorithm 3
-// at no extra cost (Sec. 4.3).
+// One CTA per window row (Algorithm 6 evaluates ALL rows, with no break; Algorithm 1 per row). The kernel behind
+// finds the first rejection (the Accept step of Algorithm 6), commits the accepted prefix and builds the next
+// window: a row that survives keeps its MRS output as draft and its target distribution as draft distribution,
+// which is the maximal coupling of Algorithm 3 at no extra cost (Sec. 4.3).
 //
 // Redraft rules besides the maximal coupling: the independent redraw of Algorithm 2 (SJD), its
 // alpha-mixture with the coupling (Algorithm 5), and the Gumbel-sharing coupling (Algorithms 4
@@ -374,18 +372,6 @@ __device__ int block_search(const F &f, int lo, int hi, unsigned U, Smem &sm)
     return res;
 }
 
-// ---- Gumbel race (Algorithm 4, in the exponential-race form of its proof) ----------------------
-// Candidate v finishes at E_v / W_v, E_v = -log2 u_v in fixed point; the earliest wins. Times are
-// compared by cross-multiplication in 128 bits and ties go to the smaller id: a strict total
-// order, so the winner does not depend on how the candidates are dealt to threads.
-struct Racer { unsigned long long T; unsigned W; int v; };       // v < 0: nobody yet
-__device__ __forceinline__ bool race_before(const Racer &a, const Racer &b)
-{
-    if (a.v < 0) return false;
-    if (b.v < 0) return true;
-    const u128 l = (u128)a.T * b.W, r = (u128)b.T * a.W;
-    return l < r || (l == r && a.v < b.v);
-}
 // argmin over ids [lo, hi) with weight(v) > 0; the noise of id v at a position is the same in
 // every iteration (the coupling shares it between the draft and the target distribution).
 template <class F>
@@ -399,14 +385,7 @@ __device__ int block_race(const F &weight, int lo, int hi, const VerifyParams &p
         const Racer c = {neglog2_q40(noise_u24(p.seed, NOISE_GUMBEL, (unsigned)b, pos, 0u, (unsigned)v)), W, v};
         if (race_before(c, best)) best = c;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        Racer other;
-        other.T = __shfl_xor_sync(FULL, best.T, o);
-        other.W = __shfl_xor_sync(FULL, best.W, o);
-        other.v = __shfl_xor_sync(FULL, best.v, o);
-        if (race_before(other, best)) best = other;
-    }
+    best = warp_racer(best);
     if (lane == 0) { sm.red_lo[warp] = best.T; sm.red_hi[warp] = ((unsigned long long)best.W << 32) | (unsigned)best.v; }
     __syncthreads();
     Racer r = {0ull, 0u, -1};
@@ -416,6 +395,22 @@ __device__ int block_race(const F &weight, int lo, int hi, const VerifyParams &p
     }
     __syncthreads();
     return r.v;
+}
+
+// argmin under equal weights
+__device__ int block_fresh_race(int lo, int hi, const VerifyParams &p, int b, long long pos, Smem &sm)
+{
+    unsigned long long best = 0;
+    for (int v = lo + (int)threadIdx.x; v < hi; v += VT) best = max(best, fresh_key(p, b, pos, v));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_xor_sync(FULL, best, o));
+    if ((threadIdx.x & 31) == 0) sm.red_lo[threadIdx.x >> 5] = best;
+    __syncthreads();
+    best = sm.red_lo[0];
+#pragma unroll
+    for (int i = 1; i < NW; ++i) best = max(best, sm.red_lo[i]);
+    __syncthreads();
+    return fresh_key_id(best);
 }
 
 // Rows are staged in shared memory when they fit (stage_cap floats per row; stage_q: a second
@@ -656,11 +651,11 @@ __global__ void __launch_bounds__(VT, 1) verify_kernel(const VerifyParams p, int
                 if (Y < 0) Y = X;
             }
             bool indep = p.mode == SCD_MODE_SJD;
+            Yi = Y;
             if (p.mode == SCD_MODE_ALPHA) {
                 // Algorithm 5: keep the coupled redraft with probability alpha, b = (Ub + 1) / 2^24
                 const unsigned Ub = noise_u24(p.seed, NOISE_ALPHA, (unsigned)b, pos, w.t, 0);
                 indep = !((double)(Ub + 1u) <= (double)p.alpha * 16777216.0);
-                Yi = Y;
             }
             if (p.mode == SCD_MODE_SCD_GS) {
                 // Algorithm 7: beyond the committed prefix the next draft is the Gumbel-max sample
@@ -673,7 +668,7 @@ __global__ void __launch_bounds__(VT, 1) verify_kernel(const VerifyParams p, int
                 const long long posf = w.pos0 + L + k;
                 int flo, fhi;
                 allowed_range(p, posf, flo, fhi);
-                Yf = block_race([](int) -> unsigned { return 1u; }, flo, fhi, p, b, posf, sm);
+                Yf = block_fresh_race(flo, fhi, p, b, posf, sm);
             }
             if (indep) {
                 // Algorithm 2 (its redraw step): the next draft is an independent draw from p
@@ -690,92 +685,29 @@ __global__ void __launch_bounds__(VT, 1) verify_kernel(const VerifyParams p, int
             if (p.mode == SCD_MODE_SCD_GS) p.row_y_indep[(size_t)p.B * L + row] = Yf;
         }
     }
-
-    // ---- last CTA of the sequence: first rejection, commit, next window ----------------------
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) {
-        const unsigned ticket = atomicAdd(&p.done_count[b], 1u);
-        sm.flag = (ticket == gridDim.x - 1) ? 1 : 0;
-    }
-    __syncthreads();
-    if (!sm.flag) return;
-    __threadfence();
-
-    if (w.Lw == 0) {
-        if (tid == 0) { p.n_commit[b] = 0; p.done_count[b] = 0; }
-        return;
-    }
-    if (tid == 0) sm.result = w.Lw;
-    __syncthreads();
-    if (tid < w.Lw && __ldcg(&p.accept_flags[(size_t)b * L + tid]) == 0) atomicMin(&sm.result, tid);
-    __syncthreads();
-    const int kstar = sm.result;
-    const int a = kstar < w.Lw ? kstar + 1 : w.Lw;     // the rejected row's residual sample is committed
-
-    for (int kk = tid; kk < L; kk += VT) {
-        const size_t row = (size_t)b * L + kk;
-        if (kk < a) {
-            const int y = __ldcg(&p.row_y[row]);
-            if (p.committed_ids) p.committed_ids[row] = y;
-            if (p.tokens) p.tokens[(size_t)b * p.token_stride + w.pos0 + kk] = y;
-        }
-        if (p.mode != SCD_MODE_AR) {
-            const int src = kk + a;
-            int nd;
-            if (src < w.Lw)
-                nd = p.mode != SCD_MODE_SCD_MC ? __ldcg(&p.row_y_indep[(size_t)b * L + src])
-                                               : __ldcg(&p.row_y[(size_t)b * L + src]);
-            else if (p.mode == SCD_MODE_SCD_GS && src >= L)
-                nd = __ldcg(&p.row_y_indep[(size_t)p.B * L + (size_t)b * L + (src - L)]);   // position pos0 + src
-            else
-                nd = fresh_draft(p, b, w.pos0 + a + kk, w.t + 1u);
-            // every row CTA of this sequence has passed its ticket, so draft_in is no longer read
-            p.draft_out[row] = nd;
-        }
-    }
-    if (tid == 0) {
-        p.n_commit[b] = a;
-        if (p.n_known) {
-            p.n_known[b] = (int)w.pos0 + a;
-            p.iter[b] = w.t + 1u;
-            p.shift[b] = a;
-            p.prev_lw[b] = w.Lw;
-            // this iteration completed the sequence (it was live: Lw > 0): the last of the batch raises the flag
-            if (p.finished && (int)w.pos0 + a >= p.n_total[b] && atomicAdd(&p.finished[0], 1) == p.B - 1) p.finished[1] = 1;
-        }
-        if (p.dev_stats) {
-            atomicMax(&p.dev_stats->forwards, (unsigned long long)w.t + 1ull);   // iterations in which a sequence was live
-            atomicAdd(&p.dev_stats->committed, (unsigned long long)a);
-            atomicAdd(&p.dev_stats->accept_hist[a], 1ull);
-        }
-        p.done_count[b] = 0;
-    }
 }
 
-// Window initialisation after prefill: every row fresh.
-__global__ void init_window_kernel(const VerifyParams p)
+// Window initialisation after prefill: every row fresh. Gumbel: a CTA per row.
+__global__ void __launch_bounds__(VT) init_window_kernel(const VerifyParams p)
 {
     __shared__ Smem sm;
-    const int b = blockIdx.x;
+    const int b = blockIdx.y;
     const long long pos0 = p.n_known[b];
     if (p.mode == SCD_MODE_SCD_GS) {
-        for (int k = 0; k < p.L; ++k) {
-            int lo, hi;
-            allowed_range(p, pos0 + k, lo, hi);
-            const int d = block_race([](int) -> unsigned { return 1u; }, lo, hi, p, b, pos0 + k, sm);
-            if (threadIdx.x == 0) p.draft_out[(size_t)b * p.L + k] = d;
-        }
+        const int k = blockIdx.x;
+        int lo, hi;
+        allowed_range(p, pos0 + k, lo, hi);
+        const int d = block_fresh_race(lo, hi, p, b, pos0 + k, sm);
+        if (threadIdx.x == 0) p.draft_out[(size_t)b * p.L + k] = d;
     } else {
         for (int k = threadIdx.x; k < p.L; k += blockDim.x)
             p.draft_out[(size_t)b * p.L + k] = fresh_draft(p, b, pos0 + k, 0u);
     }
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && blockIdx.x == 0) {
         p.iter[b] = 0u;
         p.shift[b] = 0;
         p.prev_lw[b] = 0;
         p.n_commit[b] = 0;
-        p.done_count[b] = 0u;
     }
 }
 
@@ -783,9 +715,12 @@ __global__ void init_window_kernel(const VerifyParams p)
 
 int launch_verify(const VerifyParams &p, cudaStream_t stream)
 {
-    // a cluster per row wherever it applies; this kernel keeps the Gumbel race, the nucleus truncation
-    // and rows too long for a cluster's registers
-    if (verify_cluster_supported(p)) return launch_verify_cluster(p, stream);
+    count_launches(2);
+    // a cluster per row; this kernel keeps the rows that are too long for one
+    if (verify_rows_supported(p)) {
+        const int rc = launch_verify_rows(p, stream);
+        return rc == SCD_OK ? launch_commit(p, stream) : rc;
+    }
     dim3 grid((unsigned)p.L, (unsigned)p.B);
     // shared-memory staging: both rows if they fit, else the target row alone, else none
     const int n = p.allowed_hi - p.allowed_lo;
@@ -805,12 +740,12 @@ int launch_verify(const VerifyParams &p, cudaStream_t stream)
     if (rc != SCD_OK) return rc;
     verify_kernel<<<grid, VT, smem, stream>>>(p, stage_cap, stage_q);
     SCD_CUDA_TRY(cudaGetLastError());
-    return SCD_OK;
+    return launch_commit(p, stream);
 }
 
 int launch_init_window(const VerifyParams &p, cudaStream_t stream)
 {
-    init_window_kernel<<<p.B, VT, 0, stream>>>(p);
+    init_window_kernel<<<dim3(p.mode == SCD_MODE_SCD_GS ? p.L : 1, p.B), VT, 0, stream>>>(p);
     SCD_CUDA_TRY(cudaGetLastError());
     return SCD_OK;
 }

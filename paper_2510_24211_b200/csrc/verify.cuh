@@ -60,8 +60,7 @@ struct VerifyParams {
     int token_stride;
     unsigned char *accept_flags;  // [B][L] out (k_j of every row)
     int *row_y;                   // [B][L] scratch: per-row output token Y_j
-    int *row_y_indep;             // [2][B][L] scratch: redraft beyond the prefix (SJD, alpha, Gumbel); fresh rows (Gumbel)
-    unsigned int *done_count;     // [B] scratch, zero on entry, zero again on exit
+    int *row_y_indep;             // [2][B][L] scratch: redraft of a row that stays in the window; rows entering it (Gumbel)
     VerifyStatsDev *dev_stats;    // session counters (or NULL)
     int *finished;                // session: [0] sequences that reached their final length, [1] = 1 once all B have
                                   // (the forward kernels of an iteration enqueued after that return at once)   (or NULL)
@@ -130,10 +129,44 @@ __device__ __forceinline__ WindowState load_state(const VerifyParams &p, int b)
     return w;
 }
 
+// ---- Gumbel race (Algorithm 4, in the exponential-race form of its proof) ----------------------------
+// Candidate v finishes at E_v / W_v, E_v = -log2 u_v in fixed point; the earliest wins. Times are compared by
+// cross-multiplication in 128 bits and ties go to the smaller id: a strict total order, so the winner does not
+// depend on how the candidates are dealt to threads. The noise of id v at a position is the same in every iteration.
+struct Racer { unsigned long long T; unsigned W; int v; };       // v < 0: nobody yet
+__device__ __forceinline__ bool race_before(const Racer &a, const Racer &b)
+{
+    if (a.v < 0) return false;
+    if (b.v < 0) return true;
+    const u128 l = (u128)a.T * b.W, r = (u128)b.T * a.W;
+    return l < r || (l == r && a.v < b.v);
+}
+__device__ __forceinline__ Racer warp_racer(Racer best)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        Racer other;
+        other.T = __shfl_xor_sync(0xffffffffu, best.T, o);
+        other.W = __shfl_xor_sync(0xffffffffu, best.W, o);
+        other.v = __shfl_xor_sync(0xffffffffu, best.v, o);
+        if (race_before(other, best)) best = other;
+    }
+    return best;
+}
+// With equal weights the winner has the smallest E_v. Neighbouring variates are 2^-24 / ln 2 apart in -log2 u and
+// more, E_v is exact to 2^-39: it strictly falls with U, so the winner is the largest U, the smallest id among equals.
+__device__ __forceinline__ unsigned long long fresh_key(const VerifyParams &p, int b, long long pos, int v)
+{
+    return ((unsigned long long)noise_u24(p.seed, NOISE_GUMBEL, (unsigned)b, pos, 0u, (unsigned)v) << 32) | (0xFFFFFFFFu - (unsigned)v);
+}
+__device__ __forceinline__ int fresh_key_id(unsigned long long key) { return (int)(0xFFFFFFFFu - (unsigned)key); }
+
+// the rows' kernel, then commit_kernel
 int launch_verify(const VerifyParams &p, cudaStream_t stream);
-// the kernel that gives every window row a thread-block cluster (verify_cluster.cu)
-bool verify_cluster_supported(const VerifyParams &p);
-int launch_verify_cluster(const VerifyParams &p, cudaStream_t stream);
+// the kernel that gives every window row a thread-block cluster (verify_rows.cu); rows of up to 131072 ids
+bool verify_rows_supported(const VerifyParams &p);
+int launch_verify_rows(const VerifyParams &p, cudaStream_t stream);
+int launch_commit(const VerifyParams &p, cudaStream_t stream);
 int launch_init_window(const VerifyParams &p, cudaStream_t stream);
 
 }  // namespace scd

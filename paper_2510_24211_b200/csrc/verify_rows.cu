@@ -1,0 +1,955 @@
+// Fused verify-and-redraft, one thread-block cluster of C CTAs per window row (Algorithm 6 evaluates all rows,
+// Algorithm 1 per row). The row's ids are dealt to CTAs and warps in contiguous ranges.
+//
+// By bytes a row is nothing; a kernel over a few rows is bound by its chain of row-wide exchanges, one over many
+// rows by issue slots. So the passes over ALL ids do as little as possible per id, and everything dear - the
+// exponential, 128-bit products, noise - runs on the ids that survive the truncation (2000 of 16384 with the image
+// settings), packed densely:
+//   1. x = post-processed logit (guidance mix, temperature); row maximum m                          -> exchange
+//   2. top-k: histogram of the live ids (x >= m - 22: only they have a weight) over NB equal steps of m - x;
+//      the step that holds the k-th largest id. Nucleus alone: weights W = trunc(scd_exp(x - m) 2^30) and the mass per
+//      NB logarithmic steps of W; the step in which the mass from the top reaches top_p of the row   -> exchange
+//   3. the ids of that step and the steps above go to a list per warp, in id order, with their x
+//   4. on the lists: top-k: mass above the step; the candidates OF the step, over the cluster, and by counting the
+//      exact k-th largest                                                                             -> exchange
+//      nucleus: the selected step is divided again, NB ways, until it is one value of W              -> 2 exchanges, mostly
+//   5. accept test in 128-bit integers; on rejection the residual masses max(0, Wp_v Zq - Wq_v Zp)   -> exchange
+//      and the inverse-CDF walk in the one warp that holds the target
+// Rows of up to 256 ids per warp stay in registers over passes 1-3 (REG); longer ones are read again from L2.
+// A warp whose list would overflow (a row that hardly is truncated) works on its whole range instead, reading x
+// again: entry e is then simply its e-th id. commit_kernel, one CTA per sequence behind this grid, does the
+// only serial part: first rejection, commit, next window.
+//
+// us per scd_verify call on a B200, before (an exponential per id, four byte-wise passes over the cluster for the nucleus,
+// tickets for the commit, the race on one CTA per row) and now: 1 x 32 rows of 16384 ids, top-k 2000: 32.8, 28.7;
+// 8 x 32 with guidance: 107.8, 67.1; 64 rows of 64000 ids, top-p 0.8: 279, 90; 2 x 32 of 16384, Gumbel: 234, 42.
+//
+// Gumbel race (Algorithm 4): the winner is the smallest E_v / W_v of integers that take 40 squarings each. An fp32
+// estimate of every ratio first, the integers only for ids within RACE_SLACK of the smallest estimate. A row that
+// may enter the window races under equal weights, which is the largest variate (see fresh_key).
+//
+// Exactness: sums are integers, thresholds are exact selections, every decision is an integer inequality: nothing
+// depends on how ids are dealt to threads or CTAs. No thread spins: the only waits are hardware barriers that
+// every CTA of a cluster reaches the same number of times (branches that hold one are taken on values that all
+// CTAs of the cluster compute from the same data).
+#include <algorithm>
+
+#include "verify.cuh"
+
+namespace scd {
+
+namespace {
+
+constexpr int CT = 512;
+constexpr int NWARP = CT / 32;
+constexpr int NB = 1024;           // steps of a histogram
+constexpr int MAXC = 8;
+constexpr int MAXJ = 32;           // ids of a lane at most: a CTA takes up to 16384 ids
+constexpr int CAND_CAP = 1024;     // candidates of a row that are selected by counting
+constexpr int WCAP_REG = 256;      // list entries of a warp: its whole range, or
+constexpr int WCAP_LONG = 448;     // ... of up to 1024 ids (two CTAs share an SM's memory)
+constexpr float LIVE_SPAN = 22.0f; // scd_exp(x) = 0 below -22
+constexpr unsigned W_TAIL = 1u << 14;   // nucleus: lighter ids are summed first and looked at one by one only if need be
+constexpr float RACE_SLACK = 2e-4f;
+constexpr unsigned FULLM = 0xffffffffu;
+
+// Code that runs on the target row and, when the draft row arrives as raw logits, on the draft row too: the
+// index is a compile-time constant inside, so that per-thread values stay in registers.
+template <int A> struct RowIndex { static constexpr int value = A; };
+#define EACH_ROW(...) do { auto fn_ = __VA_ARGS__; fn_(RowIndex<0>{}); if (NA > 1) fn_(RowIndex<1>{}); } while (0)
+
+struct Xchg {                                  // read by the peers through distributed shared memory
+    unsigned hist[2][2][NB];                   // [row]: counts, or masses in two parts (low 15 bits of the weights, the rest);
+                                               // once the peers have read them: the row's candidates
+    uint2 cand[2][CAND_CAP];                   // (order-preserving key of x, W) of the ids in the selected step
+    unsigned long long u64[4];
+    unsigned long long racer[2], fresh;        // (T, W : id) of this CTA's best racer; its largest fresh key
+    float f32[2];
+    unsigned cand_n[2];
+};
+
+struct Local {
+    float red_f[2][NWARP];
+    unsigned long long red_a[NWARP], red_b[NWARP];   // per-warp values of a block reduction
+    unsigned long long scan[2][NWARP / 2];
+    unsigned long long peer[4][MAXC];
+    unsigned peer_n[2][MAXC];
+    int sel[2];
+    unsigned sel_k[2], tau_key[2];
+    unsigned long long above[2], kept[2], total[2];
+};
+
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t peer_addr(uint32_t local, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ unsigned ld_peer_u32(const void *local, uint32_t rank)
+{
+    unsigned v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(peer_addr(smem_addr(local), rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned long long ld_peer_u64(const void *local, uint32_t rank)
+{
+    unsigned long long v;
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(peer_addr(smem_addr(local), rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint4 ld_peer_u32x4(const void *local, uint32_t rank)
+{
+    uint4 v;
+    asm volatile("ld.shared::cluster.v4.u32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(peer_addr(smem_addr(local), rank)) : "memory");
+    return v;
+}
+
+// step of the live range an id falls into: 0 at the maximum, NB - 1 at m - 22; -1: not live
+__device__ __forceinline__ int live_step(float x, float m)
+{
+    const float dlt = __fsub_rn(m, x);                 // = -(x - m) exactly
+    if (!(dlt <= LIVE_SPAN)) return -1;
+    return min(max(__float2int_rd(__fmul_rn(dlt, (float)NB / 22.5f)), 0), NB - 1);
+}
+// logarithmic step of a weight, heaviest first: exponent and five more bits (W >= 1, monotone)
+__device__ __forceinline__ int weight_step(unsigned w)
+{
+    const int e = 31 - __clz(w);
+    return NB - 1 - ((e << 5) | (int)(((w << (31 - e)) >> 26) & 31u));
+}
+__device__ __forceinline__ unsigned weight_step_lo(int step)         // smallest weight of a step
+{
+    const int s = NB - 1 - step, e = s >> 5;
+    const unsigned long long f = (32ull | (unsigned)(s & 31)) << e;  // in units of 2^-5, rounded up
+    return (unsigned)((f + 31) >> 5);
+}
+
+// residual mass of one id: max(0, Wp Zq - Wq Zp)
+__device__ __forceinline__ u128 residual_of(unsigned wp, unsigned wq, unsigned long long Zp, unsigned long long Zq)
+{
+    if (wp == 0u) return (u128)0;
+    const u128 a = mul_32x64(wp, Zq), b = mul_32x64(wq, Zp);
+    return a > b ? a - b : (u128)0;
+}
+
+// Whether row (b, pos) of iteration t is redrawn independently (Algorithm 2 always, Algorithm 5 by its coin).
+__device__ __forceinline__ bool redraw_independent(const VerifyParams &p, int b, long long pos, unsigned t)
+{
+    if (p.mode == SCD_MODE_SJD) return true;
+    if (p.mode != SCD_MODE_ALPHA) return false;
+    const unsigned Ub = noise_u24(p.seed, NOISE_ALPHA, (unsigned)b, pos, t, 0);
+    return !((double)(Ub + 1u) <= (double)p.alpha * 16777216.0);
+}
+
+// fp32 estimate of -log2((U + 1/2) / 2^24). Both arguments are exact (below 1/2 and above, 24 bits each), log2f and
+// log1pf err by an ulp or two.
+__device__ __forceinline__ float neglog2_estimate(unsigned U)
+{
+    if (U < (1u << 23)) return -log2f((float)(2u * U + 1u) * 0x1p-25f);
+    return -log1pf(-((float)(2u * (0xFFFFFFu - U) + 1u) * 0x1p-25f)) * 0x1.715476p+0f;
+}
+
+template <bool REG>
+__global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p, int C, int J)
+{
+    constexpr int WCAP = REG ? WCAP_REG : WCAP_LONG;   // entries of a warp's list
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ __align__(16) Xchg xc;
+    __shared__ Local lc;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = blockIdx.x % C;                   // = rank in the cluster (cluster dims (C, 1, 1))
+    const int k = blockIdx.x / C, b = blockIdx.y;
+    pdl_trigger();
+    // (in a session this grid may have started early: up to pdl_wait() it reads only what earlier iterations left
+    // behind - the window counters, the draft ids, the drafts' stored weights)
+    const WindowState w = load_state(p, b);
+    if (k >= w.Lw) { pdl_wait(); return; }             // (all CTAs of the cluster; no kernel ends before the one in front)
+    const int L = p.L, V = p.V;
+    const size_t row = (size_t)b * L + k;
+    const long long pos = w.pos0 + k;
+    int lo, hi;
+    allowed_range(p, pos, lo, hi);
+    const int wbase = lo + (rank * NWARP + warp) * (32 * J);         // this warp's ids: wbase + 32 j + lane, j < J
+    const bool mix = p.S == 2, div = p.temperature != 1.0f;
+    const bool use_topk = p.top_k > 0 && p.top_k < hi - lo;
+    const int qk = k + w.shift;
+    const bool fresh = !(qk < w.prev_lw);
+    const bool rawq = !fresh && p.q_is_raw;            // draft distribution from raw logits, built here
+    const int NA = rawq ? 2 : 1;
+    const bool mrs = p.mode != SCD_MODE_AR;
+    const float *c = p.p_logits + row * V;
+    const float *u = mix ? p.p_logits + ((size_t)(p.B + b) * L + k) * V : nullptr;
+    const float *qr = fresh ? nullptr : p.xbuf[w.parity ^ 1] + ((size_t)b * L + qk) * V;
+    float *list_x = (float *)dyn + (size_t)warp * WCAP;              // [row][warp][WCAP], then the target row's ids
+    unsigned short *list_id = (unsigned short *)(dyn + (size_t)2 * NWARP * WCAP * sizeof(float)) + (size_t)warp * WCAP;
+
+    auto csync = [&]() {                               // barrier of the cluster
+        if (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        else __syncthreads();
+    };
+    auto post_p = [&](float a, float bu) -> float {
+        if (mix) a = __fsub_rn(__fmul_rn(p.one_plus_lam, a), __fmul_rn(p.lam, bu));
+        return div ? __fdiv_rn(a, p.temperature) : a;
+    };
+    // (the target logits are read through L2: this kernel may have started before they were written, and the
+    // non-coherent load path then served stale lines of the previous iteration)
+    auto load_p = [&](int v) -> float { return post_p(__ldcg(c + v), mix ? __ldcg(u + v) : 0.f); };
+    auto load_q = [&](int v) -> float { const float x = qr[v]; return div ? __fdiv_rn(x, p.temperature) : x; };
+
+    float xr[2][8];
+    auto load8 = [&](auto A_, int j0) {                // x of ids j0 .. j0 + 7 of this lane, all loads in flight
+        constexpr int a = decltype(A_)::value;
+        float t[8], s[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int v = wbase + 32 * (j0 + i) + lane;
+            const bool in = j0 + i < J && v < hi;
+            t[i] = !in ? 0.f : a == 0 ? __ldcg(c + v) : qr[v];
+            s[i] = a == 0 && mix && in ? __ldcg(u + v) : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) xr[a][i] = a == 0 ? post_p(t[i], s[i]) : div ? __fdiv_rn(t[i], p.temperature) : t[i];
+    };
+    // body(id, exists, x) over this lane's ids, warp-uniformly
+    auto sweep = [&](auto A_, bool first, auto body) {
+        constexpr int a = decltype(A_)::value;
+#pragma unroll 1
+        for (int j0 = 0; j0 < J; j0 += 8) {
+            if (!REG || first) load8(A_, j0);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int v = wbase + 32 * (j0 + i) + lane;
+                body(v, j0 + i < J && v < hi, xr[a][i]);
+            }
+        }
+    };
+    auto warp_sum64 = [&](unsigned long long x) -> unsigned long long {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(FULLM, x, o);
+        return x;
+    };
+    auto all_cand = [&](int a) -> uint2 * { return (uint2 *)&xc.hist[a][0][0]; };
+    static_assert(sizeof(uint2) * CAND_CAP <= sizeof(xc.hist[0]), "the candidates reuse the histograms");
+    auto zero_hist = [&]() {
+        for (int i = tid; i < 2 * 2 * NB / 4; i += CT) ((uint4 *)&xc.hist[0][0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
+    };
+
+    // ---- pass 1: maximum ---------------------------------------------------------------------------------------
+    const int X = p.draft_in[row];
+    const bool x_in = X >= lo && X < hi;
+    const float xq_raw = qr && x_in ? qr[X] : 0.f;     // raw logit, or stored integer weight (bit pattern), of the draft
+    const unsigned long long Zq_stored = !fresh && !rawq ? p.stats[w.parity ^ 1][(size_t)b * L + qk].Z : 0ull;
+    zero_hist();
+    if (tid < 2) { xc.cand_n[tid] = 0u; lc.sel[tid] = -1; }
+    float m[2] = {-INFINITY, 0.f};
+    if (rawq) {                                        // (older than the kernel in front)
+        float t = -INFINITY;
+        sweep(RowIndex<1>{}, true, [&](int, bool in, float x) { if (in) t = fmaxf(t, x); });
+        t = warp_max(t);
+        if (lane == 0) lc.red_f[1][warp] = t;
+    }
+    pdl_wait();                                        // the target logits come from the kernel in front
+    const float xX = x_in ? load_p(X) : 0.f;           // the draft's own logit: every CTA weighs X itself
+    {
+        float t = -INFINITY;
+        sweep(RowIndex<0>{}, true, [&](int, bool in, float x) { if (in) t = fmaxf(t, x); });
+        t = warp_max(t);
+        if (lane == 0) lc.red_f[0][warp] = t;
+    }
+    __syncthreads();
+    if (warp < NA) {
+        const float t = warp_max(lane < NWARP ? lc.red_f[warp][lane] : -INFINITY);
+        if (lane == 0) xc.f32[warp] = t;
+    }
+    csync();                                                                          // ---- exchange: maxima
+    // (what every thread needs from every peer is fetched once per CTA, one lane per peer: distributed shared
+    // memory is for few, wide requests)
+    if (warp < NA) {
+        const float t = warp_max(lane < C ? __uint_as_float(ld_peer_u32(&xc.f32[warp], (uint32_t)lane)) : -INFINITY);
+        if (lane == 0) lc.red_f[warp][0] = t;
+    }
+    __syncthreads();
+    m[0] = lc.red_f[0][0];
+    if (rawq) m[1] = lc.red_f[1][0];
+
+    // merges the C histograms: threads 0..255 take the target row, 256..511 the draft row; each owns four steps. Scans
+    // them and leaves the step in which the running sum (from `base` on) reaches top_k (counts) or top_p of the mass Z (0:
+    // of all steps and lc.peer[row][0]) in lc.sel, the sum above it in lc.above and up to it in lc.kept, the sum of all
+    // steps in lc.total.
+    auto select_step = [&](bool mass, unsigned long long Z0, unsigned long long Z1, unsigned long long base0, unsigned long long base1) {
+        const int a = tid >> 8, t = tid & 255, wi = warp & 7;
+        unsigned long long s[4] = {0ull, 0ull, 0ull, 0ull}, mine = 0, inc = 0;
+        if (a < NA) {
+#pragma unroll
+            for (int part = 0; part < 2; ++part) {
+                if (part && !mass) break;
+                uint4 t4[MAXC];
+#pragma unroll
+                for (int r = 0; r < MAXC; ++r) t4[r] = r < C ? ld_peer_u32x4(&xc.hist[a][part][4 * t], (uint32_t)r) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                for (int r = 0; r < MAXC; ++r) {
+                    const int sh = part ? 15 : 0;
+                    s[0] += (unsigned long long)t4[r].x << sh; s[1] += (unsigned long long)t4[r].y << sh;
+                    s[2] += (unsigned long long)t4[r].z << sh; s[3] += (unsigned long long)t4[r].w << sh;
+                }
+            }
+            mine = s[0] + s[1] + s[2] + s[3];
+            inc = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long v = __shfl_up_sync(FULLM, inc, o);
+                if (lane >= o) inc += v;
+            }
+            if (lane == 31) lc.scan[a][wi] = inc;
+        }
+        __syncthreads();
+        if (a < NA) {
+            unsigned long long acc = (a ? base1 : base0) + inc - mine, tot = 0, want = a ? Z1 : Z0;
+#pragma unroll
+            for (int i = 0; i < NWARP / 2; ++i) {
+                if (i < wi) acc += lc.scan[a][i];
+                tot += lc.scan[a][i];
+            }
+            if (t == 0) lc.total[a] = tot;
+            if (mass && want == 0ull) want = tot + lc.peer[a][0];
+            const u128 need = (u128)p.top_p24 * want;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const bool hit = mass ? ((u128)(acc + s[j]) << 24) >= need && ((u128)acc << 24) < need
+                                      : acc < (unsigned)p.top_k && (unsigned)p.top_k <= acc + s[j];
+                if (hit) { lc.sel[a] = 4 * t + j; lc.above[a] = acc; lc.kept[a] = acc + s[j]; }
+                acc += s[j];
+            }
+        }
+        __syncthreads();
+    };
+    auto add_mass = [&](int a, int step, unsigned wv) {
+        atomicAdd(&xc.hist[a][0][step], wv & 0x7FFFu);
+        atomicAdd(&xc.hist[a][1][step], wv >> 15);
+    };
+
+    // ---- pass 2: the step of the threshold -------------------------------------------------------------------------
+    unsigned long long Zall[2] = {0ull, 0ull};         // normaliser
+    if (use_topk) {
+        EACH_ROW([&](auto A_) {
+            constexpr int a = decltype(A_)::value;
+            sweep(A_, false, [&](int, bool in, float x) {
+                const int s = in ? live_step(x, m[a]) : -1;
+                if (s >= 0) atomicAdd(&xc.hist[a][0][s], 1u);
+            });
+        });
+        csync();                                                                      // ---- exchange: histograms
+        select_step(false, 0ull, 0ull, 0ull, 0ull);
+        // (no step: fewer than top_k live ids. The k-th largest then has weight 0, and so has everything below it: the
+        // threshold is dropped, the weights are those of the definition)
+        if (tid < 2) lc.sel_k[tid] = (unsigned)p.top_k - (unsigned)lc.above[tid];
+    } else if (p.top_p24) {
+        for (unsigned cut = W_TAIL;; cut = 1u) {       // a second time, with every weight, if the light ids decide
+            EACH_ROW([&](auto A_) {
+                constexpr int a = decltype(A_)::value;
+                unsigned long long tail = 0;
+                sweep(A_, false, [&](int, bool in, float x) {
+                    const unsigned wv = in ? weight_of(x, m[a], -INFINITY) : 0u;
+                    if (wv >= cut) add_mass(a, weight_step(wv), wv);
+                    else tail += wv;
+                });
+                tail = warp_sum64(tail);
+                if (lane == 0) (a ? lc.red_b : lc.red_a)[warp] = tail;
+            });
+            __syncthreads();
+            if (warp < NA) {
+                const unsigned long long t = warp_sum64(lane < NWARP ? (warp ? lc.red_b : lc.red_a)[lane] : 0ull);
+                if (lane == 0) xc.u64[warp] = t;
+            }
+            csync();                                                                  // ---- exchange: histograms, tails
+            if (warp < NA) {
+                const unsigned long long t = warp_sum64(lane < C ? ld_peer_u64(&xc.u64[warp], (uint32_t)lane) : 0ull);
+                if (lane == 0) lc.peer[warp][0] = t;
+            }
+            __syncthreads();
+            select_step(true, 0ull, 0ull, 0ull, 0ull);
+            Zall[0] = lc.total[0] + lc.peer[0][0];
+            if (rawq) Zall[1] = lc.total[1] + lc.peer[1][0];
+            const bool again = cut > 1u && (lc.sel[0] < 0 || (rawq && lc.sel[1] < 0));
+            csync();                                   // every peer has read these tables
+            if (tid < 2 && again) lc.sel[tid] = -1;
+            zero_hist();
+            __syncthreads();
+            if (!again) break;
+        }
+    }
+
+    // ---- pass 3: the lists -------------------------------------------------------------------------------------------
+    int sb[2] = {lc.sel[0], lc.sel[1]};
+    int n_list[2] = {0, 0};                            // (warp-uniform)
+    unsigned *wstore = p.keep_x ? (unsigned *)(p.xbuf[w.parity] + row * V) : nullptr;
+    EACH_ROW([&](auto A_) {
+        constexpr int a = decltype(A_)::value;
+        int n = 0;
+        sweep(A_, false, [&](int v, bool in, float x) {
+            bool keep = false;
+            if (in) {
+                const int s = live_step(x, m[a]);
+                if (use_topk) keep = s >= 0 && (sb[a] < 0 || s <= sb[a]);
+                else if (p.top_p24 && s >= 0) { const unsigned wv = weight_of(x, m[a], -INFINITY); keep = wv != 0u && (sb[a] < 0 || weight_step(wv) <= sb[a]); }
+                else keep = s >= 0;
+            }
+            const unsigned vote = __ballot_sync(FULLM, keep);
+            const int at = n + __popc(vote & ((1u << lane) - 1u));
+            if (keep && at < WCAP) {
+                list_x[a * NWARP * WCAP + at] = x;
+                if (a == 0) list_id[at] = (unsigned short)(v - wbase);
+            }
+            if (a == 0 && wstore && in && !keep) wstore[v] = 0u;
+            n += __popc(vote);
+        });
+        n_list[a] = n;
+    });
+    __syncwarp();
+    // entry e of this warp: its list, or its whole range when the list did not fit
+    const bool whole[2] = {n_list[0] > WCAP, n_list[1] > WCAP};
+    const int n_e[2] = {whole[0] ? 32 * J : n_list[0], whole[1] ? 32 * J : n_list[1]};
+    auto entry_x = [&](auto A_, int e, bool &in) -> float {          // x of entry e (in: it exists)
+        constexpr int a = decltype(A_)::value;
+        in = e < n_e[a] && (!whole[a] || wbase + e < hi);
+        if (!in) return -INFINITY;
+        if (!whole[a]) return list_x[a * NWARP * WCAP + e];
+        return a == 0 ? load_p(wbase + e) : load_q(wbase + e);
+    };
+    auto entry_id = [&](int e) -> int { return wbase + (whole[0] ? e : (int)list_id[e]); };
+
+    float tau[2] = {-INFINITY, -INFINITY};
+    unsigned theta[2] = {0u, 0u};
+    if (use_topk || !p.top_p24) {
+        // ---- mass above the selected step, its candidates, the exact threshold, the normaliser ------------------------
+        EACH_ROW([&](auto A_) {
+            constexpr int a = decltype(A_)::value;
+            unsigned long long z = 0;
+            for (int e0 = 0; e0 < n_e[a]; e0 += 32) {
+                bool in;
+                const float x = entry_x(A_, e0 + lane, in);
+                const int s = in ? live_step(x, m[a]) : -1;
+                if (s < 0) continue;
+                if (sb[a] >= 0 && s > sb[a]) continue;
+                const unsigned wv = weight_of(x, m[a], -INFINITY);
+                if (sb[a] < 0 || s < sb[a]) z += wv;
+                else {
+                    const unsigned at = atomicAdd(&xc.cand_n[a], 1u);
+                    if (at < CAND_CAP) xc.cand[a][at] = make_uint2(float_key(x), wv);
+                }
+            }
+            z = warp_sum64(z);
+            if (lane == 0) (a ? lc.red_b : lc.red_a)[warp] = z;
+        });
+        __syncthreads();
+        if (warp < NA) {
+            const unsigned long long t = warp_sum64(lane < NWARP ? (warp ? lc.red_b : lc.red_a)[lane] : 0ull);
+            if (lane == 0) xc.u64[warp] = t;
+        }
+        csync();                                                                      // ---- exchange: masses, candidates
+        if (warp < 2 * NA) {                           // warps 0, 1: the target row's mass and counts; 2, 3: the draft row's
+            const int a = warp >> 1;
+            if (warp & 1) { if (lane < MAXC) lc.peer_n[a][lane] = lane < C && lc.sel[a] >= 0 ? ld_peer_u32(&xc.cand_n[a], (uint32_t)lane) : 0u; }
+            else {
+                const unsigned long long t = warp_sum64(lane < C ? ld_peer_u64(&xc.u64[a], (uint32_t)lane) : 0ull);
+                if (lane == 0) lc.total[a] = t;
+            }
+        }
+        __syncthreads();
+        unsigned n_all[2] = {0u, 0u};
+        EACH_ROW([&](auto A_) {
+            constexpr int a = decltype(A_)::value;
+            Zall[a] = lc.total[a];
+#pragma unroll
+            for (int r = 0; r < MAXC; ++r) n_all[a] += lc.peer_n[a][r];
+            if (sb[a] < 0 || n_all[a] > CAND_CAP) return;
+            unsigned off = 0;
+            for (int r = 0; r < C; ++r) {              // gather (the order does not matter)
+                const unsigned n = lc.peer_n[a][r];
+                for (unsigned e = tid; e < n; e += CT) {
+                    const unsigned long long kw = ld_peer_u64(&xc.cand[a][e], (uint32_t)r);
+                    all_cand(a)[off + e] = make_uint2((unsigned)kw, (unsigned)(kw >> 32));
+                }
+                off += n;
+            }
+        });
+        __syncthreads();
+        EACH_ROW([&](auto A_) {                        // the sel_k-th largest key of the list, by counting
+            constexpr int a = decltype(A_)::value;
+            if (sb[a] < 0 || n_all[a] > CAND_CAP) return;
+            const unsigned kk = lc.sel_k[a];
+            for (unsigned j = tid; j < n_all[a]; j += CT) {
+                const unsigned key = all_cand(a)[j].x;
+                unsigned gt = 0, ge = 0;
+                for (unsigned i = 0; i < n_all[a]; ++i) {
+                    const unsigned o = all_cand(a)[i].x;
+                    gt += o > key ? 1u : 0u;
+                    ge += o >= key ? 1u : 0u;
+                }
+                if (gt < kk && kk <= ge) lc.tau_key[a] = key;        // (equal keys write the same value)
+            }
+        });
+        __syncthreads();
+        EACH_ROW([&](auto A_) {
+            constexpr int a = decltype(A_)::value;
+            if (sb[a] < 0) return;
+            if (n_all[a] <= CAND_CAP) {
+                const unsigned tk = lc.tau_key[a];
+                tau[a] = key_float(tk);
+                unsigned long long add = 0;            // the candidates that stay (every warp sums the list for itself)
+                for (unsigned i = lane; i < n_all[a]; i += 32)
+                    if (all_cand(a)[i].x >= tk) add += all_cand(a)[i].y;
+                Zall[a] += warp_sum64(add);
+                return;
+            }
+            // long runs of equal or nearly equal logits: radix selection over the cluster, 8 bits of the key per pass,
+            // among the ids of the step; then the normaliser from scratch
+            unsigned prefix = 0, mask = 0, kk = lc.sel_k[a];
+            for (int pass = 0; pass < 4; ++pass) {
+                const int shift = 24 - 8 * pass;
+                csync();                               // (nobody still reads the counters)
+                for (int i = tid; i < 256; i += CT) xc.hist[a][0][i] = 0u;
+                __syncthreads();
+                for (int e0 = 0; e0 < n_e[a]; e0 += 32) {
+                    bool in;
+                    const float x = entry_x(A_, e0 + lane, in);
+                    if (!in || live_step(x, m[a]) != sb[a]) continue;
+                    const unsigned key = float_key(x);
+                    if ((key & mask) == prefix) atomicAdd(&xc.hist[a][0][(key >> shift) & 255u], 1u);
+                }
+                csync();
+                if (warp == 0) {                       // lane l owns the values 8 l .. 8 l + 7
+                    unsigned cnt[8], mine = 0;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        cnt[j] = 0;
+                        for (int r = 0; r < C; ++r) cnt[j] += ld_peer_u32(&xc.hist[a][0][8 * lane + j], (uint32_t)r);
+                        mine += cnt[j];
+                    }
+                    unsigned suf = mine;               // sum over lanes >= lane
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const unsigned t = __shfl_down_sync(FULLM, suf, o);
+                        if (lane + o < 32) suf += t;
+                    }
+                    unsigned acc = suf - mine;
+#pragma unroll
+                    for (int j = 7; j >= 0; --j) {
+                        if (acc < kk && kk <= acc + cnt[j]) { lc.tau_key[a] = 8u * lane + j; lc.sel_k[a] = kk - acc; }
+                        acc += cnt[j];
+                    }
+                }
+                __syncthreads();
+                prefix |= lc.tau_key[a] << shift;
+                mask |= 0xFFu << shift;
+                kk = lc.sel_k[a];
+            }
+            tau[a] = key_float(prefix);
+            unsigned long long z = 0;
+            for (int e0 = 0; e0 < n_e[a]; e0 += 32) {
+                bool in;
+                const float x = entry_x(A_, e0 + lane, in);
+                if (in) z += weight_of(x, m[a], tau[a]);
+            }
+            z = warp_sum64(z);
+            if (lane == 0) lc.red_a[warp] = z;
+            __syncthreads();
+            if (warp == 0) {
+                const unsigned long long t = warp_sum64(lane < NWARP ? lc.red_a[lane] : 0ull);
+                if (lane == 0) xc.u64[2 + a] = t;
+            }
+            csync();
+            if (warp == 0) {
+                const unsigned long long t = warp_sum64(lane < C ? ld_peer_u64(&xc.u64[2 + a], (uint32_t)lane) : 0ull);
+                if (lane == 0) lc.total[a] = t;
+            }
+            __syncthreads();
+            Zall[a] = lc.total[a];
+        });
+    }
+    // ---- nucleus: theta = the largest weight whose ids {W >= theta} hold at least top_p of the mass. The selected step
+    // is a range [range_lo, range_lo + 2^bits) of weights, divided NB ways until it is one value. -------------------
+    if (p.top_p24) {
+        unsigned range_lo[2] = {0u, 0u};
+        int bits[2] = {0, 0};
+        unsigned long long above[2] = {0ull, 0ull};    // mass of the weights above the range
+        auto level = [&](auto step_of) {               // one division: step_of(a, W) = step of NB, heaviest first, or -1
+            EACH_ROW([&](auto A_) {
+                constexpr int a = decltype(A_)::value;
+                for (int e0 = 0; e0 < n_e[a]; e0 += 32) {
+                    bool in;
+                    const float x = entry_x(A_, e0 + lane, in);
+                    const unsigned wv = in ? weight_of(x, m[a], tau[a]) : 0u;
+                    const int s = wv != 0u ? step_of(a, wv) : -1;
+                    if (s >= 0) add_mass(a, s, wv);
+                }
+            });
+            csync();
+            select_step(true, Zall[0], Zall[1], above[0], above[1]);
+            EACH_ROW([&](auto A_) {
+                constexpr int a = decltype(A_)::value;
+                sb[a] = lc.sel[a];
+                above[a] = lc.above[a];
+            });
+            csync();                                   // every peer has read these tables
+            zero_hist();
+            __syncthreads();
+        };
+        if (use_topk) {                                // (the histogram tables hold the counts of top-k)
+            csync();
+            zero_hist();
+            __syncthreads();
+            level([&](int, unsigned wv) { return weight_step(wv); });
+        } else {
+            above[0] = lc.above[0];
+            above[1] = lc.above[1];
+        }
+        EACH_ROW([&](auto A_) {
+            constexpr int a = decltype(A_)::value;
+            range_lo[a] = weight_step_lo(sb[a]);
+            bits[a] = max(0, ((NB - 1 - sb[a]) >> 5) - 5);           // a step is 2^(e - 5) weights wide
+        });
+        while (bits[0] > 0 || (rawq && bits[1] > 0)) {
+            const int sh[2] = {max(0, bits[0] - 10), max(0, bits[1] - 10)};
+            level([&](int a, unsigned wv) -> int {
+                const unsigned d = (wv - range_lo[a]) >> sh[a];
+                return wv >= range_lo[a] && ((wv - range_lo[a]) >> bits[a]) == 0u ? NB - 1 - (int)d : -1;
+            });
+            EACH_ROW([&](auto A_) {
+                constexpr int a = decltype(A_)::value;
+                range_lo[a] += (unsigned)(NB - 1 - sb[a]) << sh[a];
+                bits[a] = sh[a];
+            });
+        }
+        EACH_ROW([&](auto A_) {
+            constexpr int a = decltype(A_)::value;
+            theta[a] = range_lo[a];
+            Zall[a] = lc.kept[a];
+        });
+    }
+    const unsigned long long Zp = Zall[0];
+    const unsigned long long Zq = rawq ? Zall[1] : fresh ? (unsigned long long)(hi - lo) : Zq_stored;
+    auto weight_p = [&](int e, bool &in) -> unsigned {
+        const float x = entry_x(RowIndex<0>{}, e, in);
+        return in ? weight_of(x, m[0], tau[0], theta[0]) : 0u;
+    };
+    if (wstore) {
+        for (int e = lane; e < n_e[0]; e += 32) {
+            bool in;
+            const unsigned wv = weight_p(e, in);
+            if (in) wstore[entry_id(e)] = wv;
+        }
+    }
+    if (rank == 0 && tid == 0) {
+        RowStats st; st.m = m[0]; st.tau = tau[0]; st.Z = Zp; st.theta = theta[0]; st.pad_ = 0u;
+        p.stats[w.parity][row] = st;
+    }
+
+    // Sum of `mass` over the row's entries, and the entry in which a running sum in id order first exceeds
+    // (U * sum) >> 24. found(id) runs in one lane of the cluster; returns the sum.
+    auto draw = [&](unsigned U, auto mass, auto found) -> u128 {
+        Limbs s = {0ull, 0ull};
+        for (int e0 = 0; e0 < n_e[0]; e0 += 32) s.add(mass(e0 + lane));
+        s = warp_sum(s);
+        __syncthreads();                               // (an earlier user of these is done)
+        if (lane == 0) { lc.red_a[warp] = s.lo; lc.red_b[warp] = s.hi; }
+        __syncthreads();
+        if (warp < 2) {
+            const unsigned long long t = warp_sum64(lane < NWARP ? (warp ? lc.red_b : lc.red_a)[lane] : 0ull);
+            if (lane == 0) xc.u64[2 + warp] = t;
+        }
+        csync();                                                                      // ---- exchange: masses
+        if (warp < 2 && lane < MAXC) lc.peer[warp][lane] = lane < C ? ld_peer_u64(&xc.u64[2 + warp], (uint32_t)lane) : 0ull;
+        __syncthreads();
+        u128 total = 0, run = 0;
+#pragma unroll
+        for (int r = 0; r < MAXC; ++r) {
+            const u128 t = ((u128)lc.peer[1][r] << 40) + lc.peer[0][r];
+            if (r < rank) run += t;
+            total += t;
+        }
+        for (int i = 0; i < warp; ++i) run += ((u128)lc.red_b[i] << 40) + lc.red_a[i];
+        const u128 target = ((u128)U * total) >> 24;
+        if (total != 0 && run <= target && target < run + s.value()) {               // (one warp of the cluster)
+            for (int e0 = 0; e0 < n_e[0]; e0 += 32) {
+                Limbs r = {0ull, 0ull};
+                r.add(mass(e0 + lane));
+                const Limbs inc = warp_scan_inclusive(r, lane);
+                const unsigned hit = __ballot_sync(FULLM, run + inc.value() > target);
+                if (hit) {
+                    if (lane == __ffs(hit) - 1) found(entry_id(e0 + lane));
+                    break;
+                }
+                Limbs tot;
+                tot.lo = __shfl_sync(FULLM, inc.lo, 31);
+                tot.hi = __shfl_sync(FULLM, inc.hi, 31);
+                run += tot.value();
+            }
+        }
+        csync();                                       // every peer has read the slots
+        return total;
+    };
+
+    // ---- Algorithm 1 on (p, q, X) -----------------------------------------------------------------------------------
+    // row_y: the row's output; row_y_indep: what becomes of it if the row stays in the window
+    const bool indep = mrs && redraw_independent(p, b, pos, w.t);
+    const bool race = p.mode == SCD_MODE_SCD_GS;
+    int *const redraft = indep || race ? nullptr : p.row_y_indep + row;
+    const bool first = rank == 0 && tid == 0;
+    if (mrs) {
+        const unsigned WpX = x_in ? weight_of(xX, m[0], tau[0], theta[0]) : 0u;
+        const unsigned WqX = !x_in ? 0u : rawq ? weight_of(div ? __fdiv_rn(xq_raw, p.temperature) : xq_raw, m[1], tau[1], theta[1])
+                                  : fresh ? 1u : __float_as_uint(xq_raw);
+        const unsigned Ua = noise_u24(p.seed, NOISE_ACCEPT, (unsigned)b, pos, w.t, 0);
+        // u <= min(1, p(X)/q(X)) with u = (Ua+1)/2^24  <=>  (Ua+1) Wq[X] Zp <= Wp[X] Zq 2^24;
+        // a draft without mass under p is rejected
+        const u128 lhs = (u128)(Ua + 1u) * WqX * Zp;
+        const u128 rhs = ((u128)WpX * Zq) << 24;
+        const bool accept = WpX != 0u && lhs <= rhs;
+        if (first) p.accept_flags[row] = accept ? 1 : 0;
+        bool keep_x = accept;
+        if (!accept) {
+            // Y ~ norm(max(0, p - q))
+            const unsigned Ur = noise_u24(p.seed, NOISE_RESIDUAL, (unsigned)b, pos, w.t, 0);
+            const u128 total = draw(Ur, [&](int e) -> u128 {
+                bool in;
+                const unsigned wp = weight_p(e, in);
+                if (wp == 0u) return (u128)0;
+                const int v = entry_id(e);
+                const unsigned wq = rawq ? weight_of(load_q(v), m[1], tau[1], theta[1]) : fresh ? 1u : __float_as_uint(qr[v]);
+                return residual_of(wp, wq, Zp, Zq);
+            }, [&](int y) {
+                p.row_y[row] = y;
+                if (redraft) *redraft = y;
+            });
+            keep_x = total == 0;
+        }
+        if (keep_x && first) {
+            p.row_y[row] = X;
+            if (redraft) *redraft = X;
+        }
+    }
+    // ---- an independent draw from p: the token of vanilla AR, the redraft of Algorithm 2 ------------------------------
+    if (indep || !mrs) {
+        const unsigned Ui = noise_u24(p.seed, NOISE_INDEP, (unsigned)b, pos, mrs ? w.t : 0u, 0);
+        int *const dst = mrs ? p.row_y_indep + row : p.row_y + row;
+        const u128 total = draw(Ui, [&](int e) -> u128 { bool in; return (u128)weight_p(e, in); }, [&](int y) { *dst = y; });
+        if (first) {
+            if (total == 0) *dst = lo;
+            if (!mrs) p.accept_flags[row] = 1;
+        }
+    }
+    // ---- Algorithm 7: the redraft is the Gumbel-max sample of p under this position's shared noise; the row that may enter
+    // the window at position pos0 + L + k starts from the race under the uniform draft distribution --------------------
+    if (race) {
+        float best = INFINITY;
+        auto ratio = [&](int e, unsigned wv) -> float {
+            return __fdividef(neglog2_estimate(noise_u24(p.seed, NOISE_GUMBEL, (unsigned)b, pos, 0u, (unsigned)entry_id(e))), (float)wv);
+        };
+        for (int e = lane; e < n_e[0]; e += 32) {
+            bool in;
+            const unsigned wv = weight_p(e, in);
+            if (wv != 0u) best = fminf(best, ratio(e, wv));
+        }
+        const long long posf = w.pos0 + L + k;
+        int flo, fhi;
+        allowed_range(p, posf, flo, fhi);
+        unsigned long long fk = 0;
+        for (int v = flo + rank * CT + tid; v < fhi; v += C * CT) fk = max(fk, fresh_key(p, b, posf, v));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) fk = max(fk, __shfl_xor_sync(FULLM, fk, o));
+        const float wbest = -warp_max(-best);
+        if (lane == 0) { lc.red_f[0][warp] = wbest; lc.red_a[warp] = fk; }
+        __syncthreads();
+        if (warp == 0) {
+            const float t = -warp_max(lane < NWARP ? -lc.red_f[0][lane] : -INFINITY);
+            unsigned long long f = lane < NWARP ? lc.red_a[lane] : 0ull;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) f = max(f, __shfl_xor_sync(FULLM, f, o));
+            if (lane == 0) { xc.f32[0] = t; xc.fresh = f; }
+        }
+        csync();                                                                      // ---- exchange: smallest estimate
+        if (warp == 0) {
+            const float t = -warp_max(lane < C ? -__uint_as_float(ld_peer_u32(&xc.f32[0], (uint32_t)lane)) : -INFINITY);
+            if (lane == 0) lc.red_f[1][0] = t;
+        }
+        __syncthreads();
+        // The integers T carry up to 2^-39 of truncation, 4e-5 of the smallest variate there is, and the estimate
+        // errs by less than 2e-6: the winner's estimate is within RACE_SLACK of the smallest one.
+        const float bound = lc.red_f[1][0] * (1.0f + RACE_SLACK);
+        Racer mine = {0ull, 0u, -1};
+        if (best <= bound) {
+            for (int e = lane; e < n_e[0]; e += 32) {
+                bool in;
+                const unsigned wv = weight_p(e, in);
+                if (wv == 0u || !(ratio(e, wv) <= bound)) continue;
+                const int v = entry_id(e);
+                const Racer r = {neglog2_q40(noise_u24(p.seed, NOISE_GUMBEL, (unsigned)b, pos, 0u, (unsigned)v)), wv, v};
+                if (race_before(r, mine)) mine = r;
+            }
+        }
+        __syncwarp();
+        mine = warp_racer(mine);
+        if (lane == 0) { lc.red_a[warp] = mine.T; lc.red_b[warp] = ((unsigned long long)mine.W << 32) | (unsigned)mine.v; }
+        __syncthreads();
+        if (warp == 0) {
+            Racer r = {0ull, 0u, -1};
+            if (lane < NWARP) { r.T = lc.red_a[lane]; r.W = (unsigned)(lc.red_b[lane] >> 32); r.v = (int)(unsigned)lc.red_b[lane]; }
+            r = warp_racer(r);
+            if (lane == 0) { xc.racer[0] = r.T; xc.racer[1] = ((unsigned long long)r.W << 32) | (unsigned)r.v; }
+        }
+        csync();                                                                      // ---- exchange: racers
+        if (rank == 0 && warp == 0) {
+            Racer r = {0ull, 0u, -1};
+            unsigned long long f = 0;
+            if (lane < C) {
+                const unsigned long long wv = ld_peer_u64(&xc.racer[1], (uint32_t)lane);
+                r.T = ld_peer_u64(&xc.racer[0], (uint32_t)lane);
+                r.W = (unsigned)(wv >> 32);
+                r.v = (int)(unsigned)wv;
+                f = ld_peer_u64(&xc.fresh, (uint32_t)lane);
+            }
+            r = warp_racer(r);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) f = max(f, __shfl_xor_sync(FULLM, f, o));
+            if (lane == 0) {
+                p.row_y_indep[row] = r.v < 0 ? lo : r.v;
+                p.row_y_indep[(size_t)p.B * L + row] = fresh_key_id(f);
+            }
+        }
+    }
+    csync();                                           // nobody leaves while a peer may still read its shared memory
+}
+
+// First rejection, commit, next window: one CTA per sequence, a thread per row.
+__global__ void __launch_bounds__(256) commit_kernel(const VerifyParams p)
+{
+    __shared__ int redraft[256], entering_s[256], first_s;
+    const int b = blockIdx.x, k = threadIdx.x, L = p.L;
+    const WindowState w = load_state(p, b);
+    if (k == 0) first_s = w.Lw;
+    pdl_wait();                                        // the rows come from the grid in front
+    const size_t row = (size_t)b * L + k;
+    const bool live = k < w.Lw;
+    const int y = live ? __ldcg(&p.row_y[row]) : 0;
+    const int flag = live ? __ldcg(&p.accept_flags[row]) : 1;
+    entering_s[k] = p.mode == SCD_MODE_SCD_GS && live ? __ldcg(&p.row_y_indep[(size_t)p.B * L + row]) : 0;
+    redraft[k] = live && p.mode != SCD_MODE_AR ? __ldcg(&p.row_y_indep[row]) : 0;
+    __syncthreads();
+    if (flag == 0) atomicMin(&first_s, k);
+    __syncthreads();
+    if (w.Lw == 0) {
+        if (k == 0) p.n_commit[b] = 0;
+        return;
+    }
+    const int a = min(first_s + 1, w.Lw);              // the rejected row's residual sample is committed
+    if (k < L) {
+        if (k < a && p.tokens) p.tokens[(size_t)b * p.token_stride + w.pos0 + k] = y;
+        if (p.committed_ids) p.committed_ids[row] = k < a ? y : 0;
+        if (p.mode != SCD_MODE_AR) {
+            const int src = k + a;
+            p.draft_out[row] = src < w.Lw ? redraft[src]
+                             : p.mode == SCD_MODE_SCD_GS && src >= L ? entering_s[src - L]
+                                                                     : fresh_draft(p, b, w.pos0 + src, w.t + 1u);
+        }
+    }
+    if (k == 0) {
+        p.n_commit[b] = a;
+        if (p.n_known) {
+            p.n_known[b] = (int)w.pos0 + a;
+            p.iter[b] = w.t + 1u;
+            p.shift[b] = a;
+            p.prev_lw[b] = w.Lw;
+            // this iteration completed the sequence (it was live: Lw > 0): the last of the batch raises the flag
+            if (p.finished && (int)w.pos0 + a >= p.n_total[b] && atomicAdd(&p.finished[0], 1) == p.B - 1) p.finished[1] = 1;
+        }
+        if (p.dev_stats) {
+            atomicMax(&p.dev_stats->forwards, (unsigned long long)w.t + 1ull);   // iterations in which a sequence was live
+            atomicAdd(&p.dev_stats->committed, (unsigned long long)a);
+            atomicAdd(&p.dev_stats->accept_hist[a], 1ull);
+        }
+    }
+}
+
+// Cluster size and ids per lane for rows of at most n ids. One CTA per SM while that leaves a lane at most eight ids
+// (then they stay in registers), else two: a grid of one wave.
+bool choose_cluster(int n, int rows, int sm_count, int *C_out, int *J_out)
+{
+    auto ids_per_lane = [&](int C) { return (n + C * CT - 1) / (C * CT); };
+    int C = 1;
+    while (C < MAXC && ids_per_lane(C) > 4 && (rows * C * 2 <= sm_count || (rows * C * 2 <= 2 * sm_count && ids_per_lane(C) > 8))) C *= 2;
+    while (C < MAXC && ids_per_lane(C) > MAXJ) C *= 2;
+    *C_out = C;
+    *J_out = std::max(1, ids_per_lane(C));
+    return ids_per_lane(C) <= MAXJ;
+}
+
+template <class K, class... A>
+cudaError_t launch_ex(bool dependent, K kernel, dim3 grid, int threads, size_t smem, int C, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    int n = 0;
+    if (C > 0) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = (unsigned)C;
+        attr[n].val.clusterDim.y = 1;
+        attr[n++].val.clusterDim.z = 1;
+    }
+    if (dependent) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = n;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+}  // namespace
+
+bool verify_rows_supported(const VerifyParams &p)
+{
+    int C, J;
+    return choose_cluster(p.allowed_hi - p.allowed_lo, p.L * p.B, 148, &C, &J);
+}
+
+int launch_verify_rows(const VerifyParams &p, cudaStream_t stream)
+{
+    constexpr size_t SMEM_REG = (size_t)NWARP * WCAP_REG * 10, SMEM_LONG = (size_t)NWARP * WCAP_LONG * 10;   // two x lists, one of ids
+    int dev = 0, sms = 148;
+    int rc = current_device(&dev);
+    if (rc != SCD_OK) return rc;
+    static int sm_count[DeviceOnce::kSlots];
+    static DeviceOnce once;
+    rc = once.run(dev, [&]() -> int {
+        SCD_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        if (dev >= 0 && dev < DeviceOnce::kSlots) sm_count[dev] = sms;
+        SCD_CUDA_TRY(cudaFuncSetAttribute(verify_rows_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_REG));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(verify_rows_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LONG));
+        return SCD_OK;
+    });
+    if (rc != SCD_OK) return rc;
+    if (dev >= 0 && dev < DeviceOnce::kSlots) sms = sm_count[dev];
+    int C = 1, J = 1;
+    SCD_REQUIRE(choose_cluster(p.allowed_hi - p.allowed_lo, p.L * p.B, sms, &C, &J), SCD_ERR_SHAPE,
+                "verify: rows of %d ids do not fit a cluster", p.allowed_hi - p.allowed_lo);
+    // (the stand-alone call takes its inputs from the caller's kernels: only a session's grid may start early)
+    const dim3 grid((unsigned)(p.L * C), (unsigned)p.B, 1);
+    if (J <= 8) SCD_CUDA_TRY(launch_ex(p.n_known != nullptr, verify_rows_kernel<true>, grid, CT, SMEM_REG, C, stream, p, C, J));
+    else SCD_CUDA_TRY(launch_ex(p.n_known != nullptr, verify_rows_kernel<false>, grid, CT, SMEM_LONG, C, stream, p, C, J));
+    return SCD_OK;
+}
+
+int launch_commit(const VerifyParams &p, cudaStream_t stream)
+{
+    SCD_CUDA_TRY(launch_ex(true, commit_kernel, dim3((unsigned)p.B, 1, 1), (p.L + 31) / 32 * 32, 0, 0, stream, p));
+    return SCD_OK;
+}
+
+}  // namespace scd

@@ -182,3 +182,20 @@ def test_verify_draft_without_mass_is_rejected():
     assert (got[3][:, 0] == 0).all() and (got[0] == 1).all()         # row 0 of both sequences rejects
     for b in range(B):
         assert got[1][b, 0] == want["committed"][b, 0] and got[1][b, 0] != drafts[b, 0].item()
+
+
+@pytest.mark.parametrize("mode,B,L,V,kw", [
+    ("scd", 2, 80, 9000, dict(top_k=900)),                               # one CTA per row, read again from L2; short lists
+    ("scd", 2, 80, 9000, dict(top_k=3000, quantise=8.0)),                # lists and candidates overflow (ties)
+    ("sjd", 2, 80, 9000, dict()),                                        # no truncation: warps work on their whole ranges
+    ("alpha", 2, 80, 9000, dict(top_p=0.9, quantise=2.0, alpha=0.4)),    # nucleus among ties
+    ("scd", 2, 80, 9000, dict(top_p=0.9999999)),                         # the nucleus ends among the lightest weights
+    ("scd", 1, 5, 9000, dict(top_p=0.7, top_k=1500, lam=2.0, temperature=1.3)),   # both truncations, guidance, clusters of 8
+    ("gs", 2, 80, 5000, dict(top_k=300, lo=7, hi=4901)),
+    ("gs", 1, 3, 16385, dict()),                                         # a race over every id
+    ("ar", 3, 1, 65536, dict(top_k=2000)),
+    ("scd", 1, 3, 131073, dict(top_k=500)),                              # rows too long for a cluster
+    ("gs", 1, 3, 131073, dict(top_p=0.6)),
+])
+def test_verify_rows_at_the_edges_of_the_dispatch(mode, B, L, V, kw):
+    _run_case(mode, B, L, V, iteration=2, seed=21, **kw)
