@@ -150,11 +150,11 @@ def _check(rc):
 
 def _stream(stream=None):
     s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    return s.cuda_stream
 
 
 def _ptr(t):
-    return C.c_void_p(0) if t is None else C.c_void_p(t.data_ptr())
+    return 0 if t is None else t.data_ptr()
 
 
 def scd_strerror(code: int) -> str:

@@ -5,24 +5,30 @@
 // rows by issue slots. So the passes over ALL ids do as little as possible per id, and everything dear - the
 // exponential, 128-bit products, noise - runs on the ids that survive the truncation (2000 of 16384 with the image
 // settings), packed densely:
-//   1. x = post-processed logit (guidance mix, temperature); row maximum m                          -> exchange
-//   2. top-k: histogram of the live ids (x >= m - 22: only they have a weight) over NB equal steps of m - x;
-//      the step that holds the k-th largest id. Nucleus alone: weights W = trunc(scd_exp(x - m) 2^30) and the mass per
-//      NB logarithmic steps of W; the step in which the mass from the top reaches top_p of the row   -> exchange
-//   3. the ids of that step and the steps above go to a list per warp, in id order, with their x
-//   4. on the lists: top-k: mass above the step; the candidates OF the step, over the cluster, and by counting the
-//      exact k-th largest                                                                             -> exchange
-//      nucleus: the selected step is divided again, NB ways, until it is one value of W              -> 2 exchanges, mostly
+//   1. x = post-processed logit (guidance mix, temperature), of a sample of 1024 ids per CTA first: a bound that some
+//      more ids than top_k should exceed
+//   2. one sweep over the ids: row maximum m, and the ids at or above the bound go to a list per warp, in id order,
+//      with their x                                                                                   -> exchange
+//   3. on the lists: histogram over NB equal steps of m - x (live ids: x >= m - 22, only they have a weight
+//      W = trunc(scd_exp(x - m) 2^30)); the step that holds the k-th largest. If the bound of any CTA lies in that
+//      step or above it, the lists are built once more without one                                    -> exchange
+//   4. mass above the step; the candidates OF the step, over the cluster, and by counting the exact k-th largest
+//                                                                                                     -> exchange
+//      Nucleus without top-k: maximum and weights take a sweep each; the bound is one on W, from a sample as well, the
+//      mass below it is only summed. The step (logarithmic, of W) in which the mass from the top reaches top_p of the
+//      row is divided again, NB ways, until it is one value of W.
 //   5. accept test in 128-bit integers; on rejection the residual masses max(0, Wp_v Zq - Wq_v Zp)   -> exchange
 //      and the inverse-CDF walk in the one warp that holds the target
-// Rows of up to 256 ids per warp stay in registers over passes 1-3 (REG); longer ones are read again from L2.
+// Rows of up to 256 ids per warp stay in registers (REG): there the histogram counts every id and the lists come after
+// it, without a sample (28.9 us against 30.7 for 32 rows of 16384 ids). Longer ones are read again from L2 where a sweep
+// repeats (three sweeps, one for the histogram: 63.7 us against 53.8 for 256 rows of 16384 ids).
 // A warp whose list would overflow (a row that hardly is truncated) works on its whole range instead, reading x
 // again: entry e is then simply its e-th id. commit_kernel, one CTA per sequence behind this grid, does the
 // only serial part: first rejection, commit, next window.
 //
 // us per scd_verify call on a B200, before (an exponential per id, four byte-wise passes over the cluster for the nucleus,
-// tickets for the commit, the race on one CTA per row) and now: 1 x 32 rows of 16384 ids, top-k 2000: 32.8, 28.7;
-// 8 x 32 with guidance: 107.8, 67.1; 64 rows of 64000 ids, top-p 0.8: 279, 90; 2 x 32 of 16384, Gumbel: 234, 42.
+// tickets for the commit, the race on one CTA per row) and now: 1 x 32 rows of 16384 ids, top-k 2000: 32.8, 26.9;
+// 8 x 32 with guidance: 107.8, 53.4; 64 rows of 64000 ids, top-p 0.8: 279, 84; 2 x 32 of 16384, Gumbel: 234, 39.
 //
 // Gumbel race (Algorithm 4): the winner is the smallest E_v / W_v of integers that take 40 squarings each. An fp32
 // estimate of every ratio first, the integers only for ids within RACE_SLACK of the smallest estimate. A row that
@@ -49,7 +55,8 @@ constexpr int CAND_CAP = 1024;     // candidates of a row that are selected by c
 constexpr int WCAP_REG = 256;      // list entries of a warp: its whole range, or
 constexpr int WCAP_LONG = 448;     // ... of up to 1024 ids (two CTAs share an SM's memory)
 constexpr float LIVE_SPAN = 22.0f; // scd_exp(x) = 0 below -22
-constexpr unsigned W_TAIL = 1u << 14;   // nucleus: lighter ids are summed first and looked at one by one only if need be
+constexpr unsigned W_TAIL = 1u << 14;   // nucleus: lighter ids are only summed at first
+constexpr float LIST_SHARE = 0.28f;     // ... and so are those beyond this share of the ids (a list takes 448 of 1024)
 constexpr float RACE_SLACK = 2e-4f;
 constexpr unsigned FULLM = 0xffffffffu;
 
@@ -62,9 +69,9 @@ struct Xchg {                                  // read by the peers through dist
     unsigned hist[2][2][NB];                   // [row]: counts, or masses in two parts (low 15 bits of the weights, the rest);
                                                // once the peers have read them: the row's candidates
     uint2 cand[2][CAND_CAP];                   // (order-preserving key of x, W) of the ids in the selected step
-    unsigned long long u64[4];
+    unsigned long long u64[8];
     unsigned long long racer[2], fresh;        // (T, W : id) of this CTA's best racer; its largest fresh key
-    float f32[2];
+    float f32[4];                              // maxima, bounds
     unsigned cand_n[2];
 };
 
@@ -75,6 +82,7 @@ struct Local {
     unsigned long long peer[4][MAXC];
     unsigned peer_n[2][MAXC];
     int sel[2];
+    float bound[2];
     unsigned sel_k[2], tau_key[2];
     unsigned long long above[2], kept[2], total[2];
 };
@@ -199,31 +207,42 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
     auto load_q = [&](int v) -> float { const float x = qr[v]; return div ? __fdiv_rn(x, p.temperature) : x; };
 
     float xr[2][8];
-    auto load8 = [&](auto A_, int j0) {                // x of ids j0 .. j0 + 7 of this lane, all loads in flight
-        constexpr int a = decltype(A_)::value;
+    auto load8 = [&](int j0) {                         // x of ids j0 .. j0 + 7 of this lane, of both rows, all loads in flight
         float t[8], s[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int v = wbase + 32 * (j0 + i) + lane;
             const bool in = j0 + i < J && v < hi;
-            t[i] = !in ? 0.f : a == 0 ? __ldcg(c + v) : qr[v];
-            s[i] = a == 0 && mix && in ? __ldcg(u + v) : 0.f;
+            xr[1][i] = rawq && in ? qr[v] : 0.f;
+            t[i] = in ? __ldcg(c + v) : 0.f;
+            s[i] = mix && in ? __ldcg(u + v) : 0.f;
         }
 #pragma unroll
-        for (int i = 0; i < 8; ++i) xr[a][i] = a == 0 ? post_p(t[i], s[i]) : div ? __fdiv_rn(t[i], p.temperature) : t[i];
+        for (int i = 0; i < 8; ++i) {
+            xr[0][i] = post_p(t[i], s[i]);
+            if (div) xr[1][i] = __fdiv_rn(xr[1][i], p.temperature);
+        }
     };
-    // body(id, exists, x) over this lane's ids, warp-uniformly
-    auto sweep = [&](auto A_, bool first, auto body) {
-        constexpr int a = decltype(A_)::value;
+    // body(row, id, exists, x) over this lane's ids, warp-uniformly
+    bool loaded = false;
+    auto sweep = [&](auto body) {
 #pragma unroll 1
         for (int j0 = 0; j0 < J; j0 += 8) {
-            if (!REG || first) load8(A_, j0);
+            if (!REG || !loaded) load8(j0);
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const int v = wbase + 32 * (j0 + i) + lane;
-                body(v, j0 + i < J && v < hi, xr[a][i]);
+                body(RowIndex<0>{}, v, j0 + i < J && v < hi, xr[0][i]);
+            }
+            if (rawq) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int v = wbase + 32 * (j0 + i) + lane;
+                    body(RowIndex<1>{}, v, j0 + i < J && v < hi, xr[1][i]);
+                }
             }
         }
+        loaded = true;
     };
     auto warp_sum64 = [&](unsigned long long x) -> unsigned long long {
 #pragma unroll
@@ -236,48 +255,124 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         for (int i = tid; i < 2 * 2 * NB / 4; i += CT) ((uint4 *)&xc.hist[0][0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
     };
 
-    // ---- pass 1: maximum ---------------------------------------------------------------------------------------
     const int X = p.draft_in[row];
     const bool x_in = X >= lo && X < hi;
     const float xq_raw = qr && x_in ? qr[X] : 0.f;     // raw logit, or stored integer weight (bit pattern), of the draft
     const unsigned long long Zq_stored = !fresh && !rawq ? p.stats[w.parity ^ 1][(size_t)b * L + qk].Z : 0ull;
     zero_hist();
-    if (tid < 2) { xc.cand_n[tid] = 0u; lc.sel[tid] = -1; }
-    float m[2] = {-INFINITY, 0.f};
-    if (rawq) {                                        // (older than the kernel in front)
-        float t = -INFINITY;
-        sweep(RowIndex<1>{}, true, [&](int, bool in, float x) { if (in) t = fmaxf(t, x); });
-        t = warp_max(t);
-        if (lane == 0) lc.red_f[1][warp] = t;
-    }
+    if (tid < 2) { xc.cand_n[tid] = 0u; lc.sel[tid] = -1; lc.bound[tid] = -INFINITY; }
+    __syncthreads();
     pdl_wait();                                        // the target logits come from the kernel in front
     const float xX = x_in ? load_p(X) : 0.f;           // the draft's own logit: every CTA weighs X itself
-    {
-        float t = -INFINITY;
-        sweep(RowIndex<0>{}, true, [&](int, bool in, float x) { if (in) t = fmaxf(t, x); });
-        t = warp_max(t);
-        if (lane == 0) lc.red_f[0][warp] = t;
-    }
-    __syncthreads();
-    if (warp < NA) {
-        const float t = warp_max(lane < NWARP ? lc.red_f[warp][lane] : -INFINITY);
-        if (lane == 0) xc.f32[warp] = t;
-    }
-    csync();                                                                          // ---- exchange: maxima
-    // (what every thread needs from every peer is fetched once per CTA, one lane per peer: distributed shared
-    // memory is for few, wide requests)
-    if (warp < NA) {
-        const float t = warp_max(lane < C ? __uint_as_float(ld_peer_u32(&xc.f32[warp], (uint32_t)lane)) : -INFINITY);
-        if (lane == 0) lc.red_f[warp][0] = t;
-    }
-    __syncthreads();
-    m[0] = lc.red_f[0][0];
-    if (rawq) m[1] = lc.red_f[1][0];
+    unsigned *wstore = p.keep_x ? (unsigned *)(p.xbuf[w.parity] + row * V) : nullptr;
+    const bool nucleus = p.top_p24 != 0u && !use_topk; // the nucleus is taken of the whole row
+    float m[2] = {-INFINITY, 0.f};
+
+    // maxima (and bounds) of the CTAs -> of the row
+    auto exchange_max = [&](float m0, float m1) {
+        m0 = warp_max(m0);
+        m1 = warp_max(m1);
+        if (lane == 0) { lc.red_f[0][warp] = m0; lc.red_f[1][warp] = m1; }
+        __syncthreads();
+        if (warp < 2) {
+            const float t = warp_max(lane < NWARP ? lc.red_f[warp][lane] : -INFINITY);
+            if (lane == 0) { xc.f32[warp] = t; xc.f32[2 + warp] = lc.bound[warp]; }
+        }
+        csync();
+        // (what every thread needs from every peer is fetched once per CTA, one lane per peer: distributed shared
+        // memory is for few, wide requests)
+        if (warp < 4) {
+            const float t = warp_max(lane < C ? __uint_as_float(ld_peer_u32(&xc.f32[warp], (uint32_t)lane)) : -INFINITY);
+            if (lane == 0) { if (warp < 2) lc.red_f[warp][0] = t; else lc.bound[warp - 2] = t; }
+        }
+        __syncthreads();
+        m[0] = lc.red_f[0][0];
+        if (rawq) m[1] = lc.red_f[1][0];
+    };
+    // Two ids per lane of each row, spread over the warp's range.
+    auto sample = [&](auto body) {
+        const int ja = J / 4, jb = J - 1 - J / 4;
+        if (REG) {
+            if (!loaded) { load8(0); loaded = true; }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int v = wbase + 32 * i + lane;
+                if ((i == ja || i == jb) && i < J && v < hi) { body(0, xr[0][i]); if (rawq) body(1, xr[1][i]); }
+            }
+        } else {
+            const int va = wbase + 32 * ja + lane, vb = wbase + 32 * jb + lane;
+            const float pa = va < hi ? load_p(va) : 0.f, pb = vb < hi ? load_p(vb) : 0.f;
+            const float qa = rawq && va < hi ? load_q(va) : 0.f, qb = rawq && vb < hi ? load_q(vb) : 0.f;
+            if (va < hi) { body(0, pa); if (rawq) body(1, qa); }
+            if (vb < hi) { body(0, pb); if (rawq) body(1, qb); }
+        }
+    };
+    // After a sample's histogram (2 NB bins per row in the tables of the masses, the smallest sample in bin 0): the highest
+    // bin from which on at least `want(samples)` of them lie, if there is one. Thread t of row a looks at 8 bins.
+    auto sample_bin = [&](auto want, auto found) {
+        const int a = tid >> 8, t = tid & 255, wi = warp & 7;
+        unsigned cnt[8], mine = 0, inc = 0;
+        const unsigned *h = &xc.hist[a][0][0] + 2 * NB - 8 - 8 * t;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) { cnt[j] = h[j]; mine += cnt[j]; }
+        inc = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned v = __shfl_up_sync(FULLM, inc, o);
+            if (lane >= o) inc += v;
+        }
+        if (lane == 31) lc.scan[a][wi] = inc;
+        __syncthreads();
+        unsigned acc = inc - mine, all = 0;
+#pragma unroll
+        for (int i = 0; i < NWARP / 2; ++i) {
+            if (i < wi) acc += (unsigned)lc.scan[a][i];
+            all += (unsigned)lc.scan[a][i];
+        }
+        const unsigned need = want(all);
+#pragma unroll
+        for (int j = 7; j >= 0; --j) {
+            if (acc < need && need <= acc + cnt[j]) found(a, 2 * NB - 8 - 8 * t + j);
+            acc += cnt[j];
+        }
+        __syncthreads();
+        zero_hist();
+        __syncthreads();
+    };
+
+    // the lists (and the sweep that fills them): ids that `keep` names
+    int n_list[2] = {0, 0};                            // (warp-uniform)
+    auto append = [&](auto A_, int v, bool in, float x, bool keep) {
+        constexpr int a = decltype(A_)::value;
+        const unsigned vote = __ballot_sync(FULLM, keep);
+        const int at = n_list[a] + __popc(vote & ((1u << lane) - 1u));
+        if (keep && at < WCAP) {
+            list_x[a * NWARP * WCAP + at] = x;
+            if (a == 0) list_id[at] = (unsigned short)(v - wbase);
+        }
+        if (a == 0 && wstore && in && !keep) wstore[v] = 0u;
+        n_list[a] += __popc(vote);
+    };
+    // entry e of this warp: of its list, or of its whole range when the list did not fit
+    bool whole[2] = {false, false};
+    int n_e[2] = {0, 0};
+    auto close_lists = [&]() {
+        __syncwarp();
+#pragma unroll
+        for (int a = 0; a < 2; ++a) { whole[a] = n_list[a] > WCAP; n_e[a] = whole[a] ? 32 * J : n_list[a]; }
+    };
+    auto entry_x = [&](auto A_, int e, bool &in) -> float {          // x of entry e (in: it exists)
+        constexpr int a = decltype(A_)::value;
+        in = e < n_e[a] && (!whole[a] || wbase + e < hi);
+        if (!in) return -INFINITY;
+        if (!whole[a]) return list_x[a * NWARP * WCAP + e];
+        return a == 0 ? load_p(wbase + e) : load_q(wbase + e);
+    };
+    auto entry_id = [&](int e) -> int { return wbase + (whole[0] ? e : (int)list_id[e]); };
 
     // merges the C histograms: threads 0..255 take the target row, 256..511 the draft row; each owns four steps. Scans
-    // them and leaves the step in which the running sum (from `base` on) reaches top_k (counts) or top_p of the mass Z (0:
-    // of all steps and lc.peer[row][0]) in lc.sel, the sum above it in lc.above and up to it in lc.kept, the sum of all
-    // steps in lc.total.
+    // them and leaves the step in which the running sum (from `base` on) reaches top_k (counts) or top_p of the mass Z
+    // in lc.sel, the sum above it in lc.above and up to it in lc.kept.
     auto select_step = [&](bool mass, unsigned long long Z0, unsigned long long Z1, unsigned long long base0, unsigned long long base1) {
         const int a = tid >> 8, t = tid & 255, wi = warp & 7;
         unsigned long long s[4] = {0ull, 0ull, 0ull, 0ull}, mine = 0, inc = 0;
@@ -306,15 +401,9 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         }
         __syncthreads();
         if (a < NA) {
-            unsigned long long acc = (a ? base1 : base0) + inc - mine, tot = 0, want = a ? Z1 : Z0;
-#pragma unroll
-            for (int i = 0; i < NWARP / 2; ++i) {
-                if (i < wi) acc += lc.scan[a][i];
-                tot += lc.scan[a][i];
-            }
-            if (t == 0) lc.total[a] = tot;
-            if (mass && want == 0ull) want = tot + lc.peer[a][0];
-            const u128 need = (u128)p.top_p24 * want;
+            unsigned long long acc = (a ? base1 : base0) + inc - mine;
+            for (int i = 0; i < wi; ++i) acc += lc.scan[a][i];
+            const u128 need = (u128)p.top_p24 * (a ? Z1 : Z0);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const bool hit = mass ? ((u128)(acc + s[j]) << 24) >= need && ((u128)acc << 24) < need
@@ -330,99 +419,157 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         atomicAdd(&xc.hist[a][1][step], wv >> 15);
     };
 
-    // ---- pass 2: the step of the threshold -------------------------------------------------------------------------
+    int sb[2] = {-1, -1};                              // selected step
     unsigned long long Zall[2] = {0ull, 0ull};         // normaliser
-    if (use_topk) {
-        EACH_ROW([&](auto A_) {
-            constexpr int a = decltype(A_)::value;
-            sweep(A_, false, [&](int, bool in, float x) {
-                const int s = in ? live_step(x, m[a]) : -1;
-                if (s >= 0) atomicAdd(&xc.hist[a][0][s], 1u);
+    if (!nucleus) {
+        // ---- top-k, or no truncation ------------------------------------------------------------------------------
+        if (use_topk && !REG) {
+            sample([&](int a, float x) { atomicAdd(&xc.hist[a][0][0] + (float_key(x) >> 21), 1u); });
+            __syncthreads();
+            // (a share of top_k / n of the samples lies above the k-th largest, give or take; four deviations more are
+            // listed. Without that many samples the list takes everything.)
+            const float share = (float)p.top_k / (float)(hi - lo);
+            sample_bin([&](unsigned all) { const float e = share * (float)all; return (unsigned)(e + 4.0f * sqrtf(e)) + 4u; },
+                       [&](int a, int bin) {
+                           const float t = key_float((unsigned)bin << 21);
+                           lc.bound[a] = t > -INFINITY ? t : -INFINITY;      // (the bin of -inf begins among the NaNs)
+                       });
+        }
+        for (bool again = false;; again = true) {
+            const float bound[2] = {again ? -INFINITY : lc.bound[0], again ? -INFINITY : lc.bound[1]};
+            float mx[2] = {-INFINITY, -INFINITY};
+            n_list[0] = n_list[1] = 0;
+            sweep([&](auto A_, int v, bool in, float x) {
+                constexpr int a = decltype(A_)::value;
+                if (in) mx[a] = fmaxf(mx[a], x);
+                if (!REG) append(A_, v, in, x, in && x >= bound[a]);
             });
-        });
-        csync();                                                                      // ---- exchange: histograms
-        select_step(false, 0ull, 0ull, 0ull, 0ull);
-        // (no step: fewer than top_k live ids. The k-th largest then has weight 0, and so has everything below it: the
-        // threshold is dropped, the weights are those of the definition)
-        if (tid < 2) lc.sel_k[tid] = (unsigned)p.top_k - (unsigned)lc.above[tid];
-    } else if (p.top_p24) {
-        for (unsigned cut = W_TAIL;; cut = 1u) {       // a second time, with every weight, if the light ids decide
+            close_lists();
+            if (!again) exchange_max(mx[0], mx[1]);                                   // ---- exchange: maxima
+            if (use_topk) {
+                auto count = [&](int a, bool in, float x) {
+                    const int s = in ? live_step(x, a ? m[1] : m[0]) : -1;
+                    if (s >= 0) atomicAdd(&xc.hist[a][0][s], 1u);
+                };
+                if (REG) {
+                    sweep([&](auto A_, int, bool in, float x) { count(decltype(A_)::value, in, x); });
+                } else {
+                    EACH_ROW([&](auto A_) {
+                        constexpr int a = decltype(A_)::value;
+                        for (int e0 = 0; e0 < n_e[a]; e0 += 32) {
+                            bool in;
+                            const float x = entry_x(A_, e0 + lane, in);
+                            count(a, in, x);
+                        }
+                    });
+                }
+                csync();                                                              // ---- exchange: histograms
+                select_step(false, 0ull, 0ull, 0ull, 0ull);
+                // (no step: fewer than top_k live ids. The k-th largest then has weight 0, and so has everything below
+                // it: the threshold is dropped, the weights are those of the definition)
+                sb[0] = lc.sel[0];
+                sb[1] = lc.sel[1];
+            }
+            if (REG) {                                 // the ids are in registers: the lists come last
+                sweep([&](auto A_, int v, bool in, float x) {
+                    constexpr int a = decltype(A_)::value;
+                    const int s = in ? live_step(x, m[a]) : -1;
+                    append(A_, v, in, x, s >= 0 && (sb[a] < 0 || s <= sb[a]));
+                });
+                close_lists();
+            }
+            if (!use_topk) break;
+            bool complete = true;                      // every id of the step and above it is in the lists
             EACH_ROW([&](auto A_) {
                 constexpr int a = decltype(A_)::value;
-                unsigned long long tail = 0;
-                sweep(A_, false, [&](int, bool in, float x) {
+                const int s = live_step(lc.bound[a], m[a]);          // (a bound above m would be in step 0)
+                if (s >= 0 && (sb[a] < 0 || s <= sb[a])) complete = false;
+            });
+            if (complete || again) {
+                if (tid < 2) lc.sel_k[tid] = (unsigned)p.top_k - (unsigned)lc.above[tid];
+                break;
+            }
+            csync();                                   // every peer has read these tables
+            if (tid < 2) lc.sel[tid] = -1;
+            zero_hist();
+            __syncthreads();
+        }
+    } else {
+        // ---- nucleus of the whole row ---------------------------------------------------------------------------------
+        {
+            float mx[2] = {-INFINITY, -INFINITY};
+            sweep([&](auto A_, int, bool in, float x) { constexpr int a = decltype(A_)::value; if (in) mx[a] = fmaxf(mx[a], x); });
+            exchange_max(mx[0], mx[1]);                                               // ---- exchange: maxima
+        }
+        sample([&](int a, float x) {
+            const unsigned wv = weight_of(x, a ? m[1] : m[0], -INFINITY);
+            atomicAdd(&xc.hist[a][0][0] + (wv ? NB - 1 - weight_step(wv) : 0), 1u);
+        });
+        if (tid < 2) lc.bound[tid] = (float)W_TAIL;
+        __syncthreads();
+        sample_bin([&](unsigned all) { return (unsigned)(LIST_SHARE * (float)all) + 1u; },
+                   [&](int a, int bin) { lc.bound[a] = fmaxf((float)W_TAIL, bin > 0 ? (float)weight_step_lo(NB - 1 - bin) : 0.f); });
+        for (bool again = false;; again = true) {
+            // (a bound is the smallest weight of a step: exact in fp32)
+            const unsigned cut[2] = {again ? 1u : (unsigned)lc.bound[0], again ? 1u : (unsigned)lc.bound[1]};
+            unsigned long long z[2] = {0ull, 0ull};
+            n_list[0] = n_list[1] = 0;
+            sweep([&](auto A_, int v, bool in, float x) {
+                constexpr int a = decltype(A_)::value;
+                const unsigned wv = in ? weight_of(x, m[a], -INFINITY) : 0u;
+                z[a] += wv;
+                append(A_, v, in, x, wv >= cut[a]);
+            });
+            close_lists();
+            EACH_ROW([&](auto A_) {
+                constexpr int a = decltype(A_)::value;
+                const unsigned long long t = warp_sum64(z[a]);
+                if (lane == 0) (a ? lc.red_b : lc.red_a)[warp] = t;
+                for (int e0 = 0; e0 < n_e[a]; e0 += 32) {
+                    bool in;
+                    const float x = entry_x(A_, e0 + lane, in);
                     const unsigned wv = in ? weight_of(x, m[a], -INFINITY) : 0u;
-                    if (wv >= cut) add_mass(a, weight_step(wv), wv);
-                    else tail += wv;
-                });
-                tail = warp_sum64(tail);
-                if (lane == 0) (a ? lc.red_b : lc.red_a)[warp] = tail;
+                    if (wv >= cut[a]) add_mass(a, weight_step(wv), wv);
+                }
             });
             __syncthreads();
             if (warp < NA) {
                 const unsigned long long t = warp_sum64(lane < NWARP ? (warp ? lc.red_b : lc.red_a)[lane] : 0ull);
-                if (lane == 0) xc.u64[warp] = t;
+                if (lane == 0) { xc.u64[warp] = t; xc.f32[2 + warp] = (float)cut[warp]; }
             }
-            csync();                                                                  // ---- exchange: histograms, tails
-            if (warp < NA) {
-                const unsigned long long t = warp_sum64(lane < C ? ld_peer_u64(&xc.u64[warp], (uint32_t)lane) : 0ull);
-                if (lane == 0) lc.peer[warp][0] = t;
+            csync();                                                                  // ---- exchange: histograms, sums, bounds
+            if (warp < 2 * NA) {
+                const int a = warp >> 1;
+                if (warp & 1) {
+                    const float t = warp_max(lane < C ? __uint_as_float(ld_peer_u32(&xc.f32[2 + a], (uint32_t)lane)) : 0.f);
+                    if (lane == 0) lc.red_f[a][0] = t;
+                } else {
+                    const unsigned long long t = warp_sum64(lane < C ? ld_peer_u64(&xc.u64[a], (uint32_t)lane) : 0ull);
+                    if (lane == 0) lc.peer[a][0] = t;
+                }
             }
             __syncthreads();
-            select_step(true, 0ull, 0ull, 0ull, 0ull);
-            Zall[0] = lc.total[0] + lc.peer[0][0];
-            if (rawq) Zall[1] = lc.total[1] + lc.peer[1][0];
-            const bool again = cut > 1u && (lc.sel[0] < 0 || (rawq && lc.sel[1] < 0));
+            Zall[0] = lc.peer[0][0];
+            if (rawq) Zall[1] = lc.peer[1][0];
+            select_step(true, Zall[0], Zall[1], 0ull, 0ull);
+            bool complete = true;                      // every id of the step and above it is in the lists
+            EACH_ROW([&](auto A_) {
+                constexpr int a = decltype(A_)::value;
+                sb[a] = lc.sel[a];
+                if (sb[a] < 0 || (float)weight_step_lo(sb[a]) < lc.red_f[a][0]) complete = false;
+            });
             csync();                                   // every peer has read these tables
-            if (tid < 2 && again) lc.sel[tid] = -1;
             zero_hist();
             __syncthreads();
-            if (!again) break;
+            if (complete || again) break;
+            if (tid < 2) lc.sel[tid] = -1;
+            __syncthreads();
         }
     }
 
-    // ---- pass 3: the lists -------------------------------------------------------------------------------------------
-    int sb[2] = {lc.sel[0], lc.sel[1]};
-    int n_list[2] = {0, 0};                            // (warp-uniform)
-    unsigned *wstore = p.keep_x ? (unsigned *)(p.xbuf[w.parity] + row * V) : nullptr;
-    EACH_ROW([&](auto A_) {
-        constexpr int a = decltype(A_)::value;
-        int n = 0;
-        sweep(A_, false, [&](int v, bool in, float x) {
-            bool keep = false;
-            if (in) {
-                const int s = live_step(x, m[a]);
-                if (use_topk) keep = s >= 0 && (sb[a] < 0 || s <= sb[a]);
-                else if (p.top_p24 && s >= 0) { const unsigned wv = weight_of(x, m[a], -INFINITY); keep = wv != 0u && (sb[a] < 0 || weight_step(wv) <= sb[a]); }
-                else keep = s >= 0;
-            }
-            const unsigned vote = __ballot_sync(FULLM, keep);
-            const int at = n + __popc(vote & ((1u << lane) - 1u));
-            if (keep && at < WCAP) {
-                list_x[a * NWARP * WCAP + at] = x;
-                if (a == 0) list_id[at] = (unsigned short)(v - wbase);
-            }
-            if (a == 0 && wstore && in && !keep) wstore[v] = 0u;
-            n += __popc(vote);
-        });
-        n_list[a] = n;
-    });
-    __syncwarp();
-    // entry e of this warp: its list, or its whole range when the list did not fit
-    const bool whole[2] = {n_list[0] > WCAP, n_list[1] > WCAP};
-    const int n_e[2] = {whole[0] ? 32 * J : n_list[0], whole[1] ? 32 * J : n_list[1]};
-    auto entry_x = [&](auto A_, int e, bool &in) -> float {          // x of entry e (in: it exists)
-        constexpr int a = decltype(A_)::value;
-        in = e < n_e[a] && (!whole[a] || wbase + e < hi);
-        if (!in) return -INFINITY;
-        if (!whole[a]) return list_x[a * NWARP * WCAP + e];
-        return a == 0 ? load_p(wbase + e) : load_q(wbase + e);
-    };
-    auto entry_id = [&](int e) -> int { return wbase + (whole[0] ? e : (int)list_id[e]); };
-
     float tau[2] = {-INFINITY, -INFINITY};
     unsigned theta[2] = {0u, 0u};
-    if (use_topk || !p.top_p24) {
+    if (!nucleus) {
         // ---- mass above the selected step, its candidates, the exact threshold, the normaliser ------------------------
         EACH_ROW([&](auto A_) {
             constexpr int a = decltype(A_)::value;
@@ -464,17 +611,24 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
             Zall[a] = lc.total[a];
 #pragma unroll
             for (int r = 0; r < MAXC; ++r) n_all[a] += lc.peer_n[a][r];
-            if (sb[a] < 0 || n_all[a] > CAND_CAP) return;
-            unsigned off = 0;
-            for (int r = 0; r < C; ++r) {              // gather (the order does not matter)
-                const unsigned n = lc.peer_n[a][r];
-                for (unsigned e = tid; e < n; e += CT) {
-                    const unsigned long long kw = ld_peer_u64(&xc.cand[a][e], (uint32_t)r);
-                    all_cand(a)[off + e] = make_uint2((unsigned)kw, (unsigned)(kw >> 32));
-                }
-                off += n;
-            }
         });
+        {                                              // gather: half the threads per row, entry e of the peers' lists in turn
+            const int a = tid >> 8;
+            const unsigned n = a < NA ? n_all[a] : 0u;
+            if (n <= CAND_CAP) {
+                for (unsigned e = tid & 255; e < n; e += CT / 2) {
+                    unsigned off = 0;
+                    int rr = 0;
+#pragma unroll
+                    for (int r = 0; r < MAXC - 1; ++r) {
+                        const unsigned end = off + lc.peer_n[a][r];
+                        if (rr == r && e >= end) { off = end; rr = r + 1; }
+                    }
+                    const unsigned long long kw = ld_peer_u64(&xc.cand[a][e - off], (uint32_t)rr);
+                    all_cand(a)[e] = make_uint2((unsigned)kw, (unsigned)(kw >> 32));
+                }
+            }
+        }
         __syncthreads();
         EACH_ROW([&](auto A_) {                        // the sel_k-th largest key of the list, by counting
             constexpr int a = decltype(A_)::value;
@@ -648,8 +802,8 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
     }
 
     // Sum of `mass` over the row's entries, and the entry in which a running sum in id order first exceeds
-    // (U * sum) >> 24. found(id) runs in one lane of the cluster; returns the sum.
-    auto draw = [&](unsigned U, auto mass, auto found) -> u128 {
+    // (U * sum) >> 24. found(id) runs in one lane of the cluster; returns the sum. slot: of xc.u64, one per call.
+    auto draw = [&](int slot, unsigned U, auto mass, auto found) -> u128 {
         Limbs s = {0ull, 0ull};
         for (int e0 = 0; e0 < n_e[0]; e0 += 32) s.add(mass(e0 + lane));
         s = warp_sum(s);
@@ -658,10 +812,10 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         __syncthreads();
         if (warp < 2) {
             const unsigned long long t = warp_sum64(lane < NWARP ? (warp ? lc.red_b : lc.red_a)[lane] : 0ull);
-            if (lane == 0) xc.u64[2 + warp] = t;
+            if (lane == 0) xc.u64[slot + warp] = t;
         }
         csync();                                                                      // ---- exchange: masses
-        if (warp < 2 && lane < MAXC) lc.peer[warp][lane] = lane < C ? ld_peer_u64(&xc.u64[2 + warp], (uint32_t)lane) : 0ull;
+        if (warp < 2 && lane < MAXC) lc.peer[warp][lane] = lane < C ? ld_peer_u64(&xc.u64[slot + warp], (uint32_t)lane) : 0ull;
         __syncthreads();
         u128 total = 0, run = 0;
 #pragma unroll
@@ -688,7 +842,6 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
                 run += tot.value();
             }
         }
-        csync();                                       // every peer has read the slots
         return total;
     };
 
@@ -713,7 +866,7 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         if (!accept) {
             // Y ~ norm(max(0, p - q))
             const unsigned Ur = noise_u24(p.seed, NOISE_RESIDUAL, (unsigned)b, pos, w.t, 0);
-            const u128 total = draw(Ur, [&](int e) -> u128 {
+            const u128 total = draw(4, Ur, [&](int e) -> u128 {
                 bool in;
                 const unsigned wp = weight_p(e, in);
                 if (wp == 0u) return (u128)0;
@@ -735,7 +888,7 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
     if (indep || !mrs) {
         const unsigned Ui = noise_u24(p.seed, NOISE_INDEP, (unsigned)b, pos, mrs ? w.t : 0u, 0);
         int *const dst = mrs ? p.row_y_indep + row : p.row_y + row;
-        const u128 total = draw(Ui, [&](int e) -> u128 { bool in; return (u128)weight_p(e, in); }, [&](int y) { *dst = y; });
+        const u128 total = draw(6, Ui, [&](int e) -> u128 { bool in; return (u128)weight_p(e, in); }, [&](int y) { *dst = y; });
         if (first) {
             if (total == 0) *dst = lo;
             if (!mrs) p.accept_flags[row] = 1;

@@ -199,3 +199,27 @@ def test_verify_draft_without_mass_is_rejected():
 ])
 def test_verify_rows_at_the_edges_of_the_dispatch(mode, B, L, V, kw):
     _run_case(mode, B, L, V, iteration=2, seed=21, **kw)
+
+
+@pytest.mark.parametrize("V,L,B,top_k,top_p", [(9000, 80, 2, 700, 0.0), (9000, 80, 2, 0, 0.8), (4000, 6, 1, 300, 0.0)])
+def test_verify_bound_from_an_unlucky_sample(V, L, B, top_k, top_p):
+    """The bound that the lists start from is estimated from ids at fixed places of each warp's range: here exactly those
+    hold the largest logits, so that the bound is above the threshold and the lists are built again."""
+    p, q = synth.verify_logits(3, 1, B, L, V, device="cuda")
+    C = 1 if B * L > 74 else 8
+    J = -(-V // (C * 512))
+    j = torch.arange(V, device="cuda") // 32 % J
+    sampled = (j == J // 4) | (j == J - 1 - J // 4)
+    p[..., sampled] += 6.0
+    q[..., sampled] += 6.0
+    p[..., 0], q[..., 0] = float("-inf"), float("-inf")
+    drafts = synth.draft_ids_from_logits(q, top_k, 5)
+    positions = torch.arange(B, device="cuda", dtype=torch.int64) + 9
+    cfg = scd.decode_config(mode=scd.SCD_MODE_SCD_MC, batch=B, window_L=L, top_k=top_k, top_p=top_p, seed=8, allowed_hi=V)
+    n_commit, committed, next_drafts, flags = [t.cpu().numpy() for t in scd.scd_verify(cfg, p, q, drafts, positions, 4)]
+    want = oracle_verify("scd", p.cpu().numpy(), q.cpu().numpy(), drafts.cpu().numpy(), positions.cpu().numpy(), 4, 8,
+                         top_k=top_k, top_p=top_p)
+    assert np.array_equal(n_commit, want["n_commit"]) and np.array_equal(flags, want["flags"])
+    assert np.array_equal(next_drafts, want["next_drafts"])
+    for b in range(B):
+        assert np.array_equal(committed[b, :n_commit[b]], want["committed"][b, :n_commit[b]])
