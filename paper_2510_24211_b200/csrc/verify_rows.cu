@@ -864,15 +864,32 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         if (first) p.accept_flags[row] = accept ? 1 : 0;
         bool keep_x = accept;
         if (!accept) {
-            // Y ~ norm(max(0, p - q))
+            // Y ~ norm(max(0, p - q)). The draft's weights of the listed ids first: four gathers in flight, into the draft
+            // row's list, which is done with (one at a time, and again in the walk, they were 10 to 15 us of a row)
+            unsigned *const list_wq = (unsigned *)list_x + (size_t)NWARP * WCAP;
+            auto weight_q = [&](int v) -> unsigned {
+                return rawq ? weight_of(load_q(v), m[1], tau[1], theta[1]) : fresh ? 1u : __float_as_uint(qr[v]);
+            };
+            if (!whole[0] && !fresh) {
+                __syncwarp();
+                for (int e0 = lane; e0 < n_e[0]; e0 += 128) {
+                    float t[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) t[i] = e0 + 32 * i < n_e[0] ? qr[wbase + (int)list_id[e0 + 32 * i]] : 0.f;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        if (rawq && div) t[i] = __fdiv_rn(t[i], p.temperature);
+                        if (e0 + 32 * i < n_e[0]) list_wq[e0 + 32 * i] = rawq ? weight_of(t[i], m[1], tau[1], theta[1]) : __float_as_uint(t[i]);
+                    }
+                }
+                __syncwarp();
+            }
             const unsigned Ur = noise_u24(p.seed, NOISE_RESIDUAL, (unsigned)b, pos, w.t, 0);
             const u128 total = draw(4, Ur, [&](int e) -> u128 {
                 bool in;
                 const unsigned wp = weight_p(e, in);
                 if (wp == 0u) return (u128)0;
-                const int v = entry_id(e);
-                const unsigned wq = rawq ? weight_of(load_q(v), m[1], tau[1], theta[1]) : fresh ? 1u : __float_as_uint(qr[v]);
-                return residual_of(wp, wq, Zp, Zq);
+                return residual_of(wp, fresh ? 1u : whole[0] ? weight_q(wbase + e) : list_wq[e], Zp, Zq);
             }, [&](int y) {
                 p.row_y[row] = y;
                 if (redraft) *redraft = y;
