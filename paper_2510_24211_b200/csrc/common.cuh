@@ -126,7 +126,8 @@ __device__ __forceinline__ float scd_exp(float x)
     if (!(x >= -22.0f)) return 0.0f;
     if (x > 0.0f) x = 0.0f;
     const float t = __fmul_rn(x, 0x1.715476p+0f);
-    const float n = rintf(t);
+    const float big = __fadd_rn(t, 0x1.8p23f);     // rint(t) in the low bits (|t| < 2^22): conversions run at a quarter rate
+    const float n = __fsub_rn(big, 0x1.8p23f);
     float r = __fmaf_rn(n, -0x1.62e400p-1f, x);
     r = __fmaf_rn(n, -0x1.7f7d1cp-20f, r);
     float p = 0x1.6c16c2p-10f;
@@ -136,7 +137,7 @@ __device__ __forceinline__ float scd_exp(float x)
     p = __fmaf_rn(p, r, 0.5f);
     p = __fmaf_rn(p, r, 1.0f);
     p = __fmaf_rn(p, r, 1.0f);
-    const float scale = __int_as_float(((int)n + 127) << 23);
+    const float scale = __int_as_float((__float_as_int(big) - 0x4B400000 + 127) << 23);
     return __fmul_rn(p, scale);
 }
 
@@ -145,8 +146,9 @@ __device__ __forceinline__ float scd_exp(float x)
 __device__ __forceinline__ uint32_t weight_of(float x, float m, float tau)
 {
     if (!(x >= tau)) return 0u;
-    const float e = scd_exp(__fsub_rn(x, m));
-    return (uint32_t)__fmul_rn(e, 1073741824.0f);
+    // trunc(e 2^30) for 0 <= e < 2 by shifting the significand, 2^30 in its leading place (e = 0: shifted out)
+    const uint32_t e = __float_as_uint(scd_exp(__fsub_rn(x, m)));
+    return ((e << 7 & 0x3FFFFFFFu) | 0x40000000u) >> min(127u - (e >> 23), 31u);
 }
 // ... and 0 below the nucleus threshold theta (theta = 0: no top-p)
 __device__ __forceinline__ uint32_t weight_of(float x, float m, float tau, uint32_t theta)

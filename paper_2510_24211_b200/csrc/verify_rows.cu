@@ -27,8 +27,8 @@
 // only serial part: first rejection, commit, next window.
 //
 // us per scd_verify call on a B200, before (an exponential per id, four byte-wise passes over the cluster for the nucleus,
-// tickets for the commit, the race on one CTA per row) and now: 1 x 32 rows of 16384 ids, top-k 2000: 32.8, 26.9;
-// 8 x 32 with guidance: 107.8, 53.4; 64 rows of 64000 ids, top-p 0.8: 279, 84; 2 x 32 of 16384, Gumbel: 234, 39.
+// tickets for the commit, the race on one CTA per row) and now: 1 x 32 rows of 16384 ids, top-k 2000: 32.8, 26.6;
+// 8 x 32 with guidance: 107.8, 49.3; 64 rows of 64000 ids, top-p 0.8: 279, 78; 2 x 32 of 16384, Gumbel: 234, 39.
 //
 // Gumbel race (Algorithm 4): the winner is the smallest E_v / W_v of integers that take 40 squarings each. An fp32
 // estimate of every ratio first, the integers only for ids within RACE_SLACK of the smallest estimate. A row that
@@ -50,13 +50,12 @@ constexpr int CT = 512;
 constexpr int NWARP = CT / 32;
 constexpr int NB = 1024;           // steps of a histogram
 constexpr int MAXC = 8;
-constexpr int MAXJ = 32;           // ids of a lane at most: a CTA takes up to 16384 ids
+constexpr int MAXG = 4;            // groups of 256 ids per warp: a CTA takes up to 16384 ids
 constexpr int CAND_CAP = 1024;     // candidates of a row that are selected by counting
-constexpr int WCAP_REG = 256;      // list entries of a warp: its whole range, or
-constexpr int WCAP_LONG = 448;     // ... of up to 1024 ids (two CTAs share an SM's memory)
+constexpr int WCAP_LONG = 384;     // list entries of a warp of up to 1024 ids (two CTAs share an SM's memory)
 constexpr float LIVE_SPAN = 22.0f; // scd_exp(x) = 0 below -22
 constexpr unsigned W_TAIL = 1u << 14;   // nucleus: lighter ids are only summed at first
-constexpr float LIST_SHARE = 0.28f;     // ... and so are those beyond this share of the ids (a list takes 448 of 1024)
+constexpr float LIST_SHARE = 0.28f;     // ... and so are those beyond this share of the ids (a list takes 384 of 1024)
 constexpr float RACE_SLACK = 2e-4f;
 constexpr unsigned FULLM = 0xffffffffu;
 
@@ -68,7 +67,7 @@ template <int A> struct RowIndex { static constexpr int value = A; };
 struct Xchg {                                  // read by the peers through distributed shared memory
     unsigned hist[2][2][NB];                   // [row]: counts, or masses in two parts (low 15 bits of the weights, the rest);
                                                // once the peers have read them: the row's candidates
-    uint2 cand[2][CAND_CAP];                   // (order-preserving key of x, W) of the ids in the selected step
+    uint2 cand[2][CAND_CAP];                   // (order-preserving key of x, W) of the ids in the selected step ...
     unsigned long long u64[8];
     unsigned long long racer[2], fresh;        // (T, W : id) of this CTA's best racer; its largest fresh key
     float f32[4];                              // maxima, bounds
@@ -76,6 +75,7 @@ struct Xchg {                                  // read by the peers through dist
 };
 
 struct Local {
+    unsigned short cand_at[2][CAND_CAP];       // ... and where they are in this CTA's lists
     float red_f[2][NWARP];
     unsigned long long red_a[NWARP], red_b[NWARP];   // per-warp values of a block reduction
     unsigned long long scan[2][NWARP / 2];
@@ -159,10 +159,22 @@ __device__ __forceinline__ float neglog2_estimate(unsigned U)
     return -log1pf(-((float)(2u * (0xFFFFFFu - U) + 1u) * 0x1p-25f)) * 0x1.715476p+0f;
 }
 
-template <bool REG>
-__global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p, int C, int J)
+// post-processed logit of one id (u: unconditional row or null), off the main path
+__device__ __noinline__ float post_logit(const float *c, const float *u, int v, float one_plus_lam, float lam, float T)
 {
-    constexpr int WCAP = REG ? WCAP_REG : WCAP_LONG;   // entries of a warp's list
+    float x = __ldcg(c + v);
+    if (u) x = __fsub_rn(__fmul_rn(one_plus_lam, x), __fmul_rn(lam, __ldcg(u + v)));
+    return T != 1.0f ? __fdiv_rn(x, T) : x;
+}
+
+// A warp's ids come in groups of NS x 128: lane l holds ids 4 l .. 4 l + 3 of each 128 (16-byte loads where rows are
+// aligned). REG: one group, which stays in registers.
+template <int NS, bool REG>
+__global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p, int C, int G)
+{
+    constexpr int N = 4 * NS;                          // ids per lane and group
+    constexpr int WCAP = REG ? 32 * N : WCAP_LONG;     // entries of a warp's list
+    const int range = 32 * N * G;                      // ids of a warp
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ __align__(16) Xchg xc;
     __shared__ Local lc;
@@ -179,7 +191,9 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
     const long long pos = w.pos0 + k;
     int lo, hi;
     allowed_range(p, pos, lo, hi);
-    const int wbase = lo + (rank * NWARP + warp) * (32 * J);         // this warp's ids: wbase + 32 j + lane, j < J
+    // rows that are 16-byte aligned throughout are dealt from an aligned id on
+    const bool vec = (V & 3) == 0 && ((uintptr_t)p.p_logits & 15) == 0 && ((uintptr_t)p.xbuf[w.parity ^ 1] & 15) == 0;
+    const int wbase = (vec ? lo & ~3 : lo) + (rank * NWARP + warp) * range;
     const bool mix = p.S == 2, div = p.temperature != 1.0f;
     const bool use_topk = p.top_k > 0 && p.top_k < hi - lo;
     const int qk = k + w.shift;
@@ -190,57 +204,66 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
     const float *c = p.p_logits + row * V;
     const float *u = mix ? p.p_logits + ((size_t)(p.B + b) * L + k) * V : nullptr;
     const float *qr = fresh ? nullptr : p.xbuf[w.parity ^ 1] + ((size_t)b * L + qk) * V;
-    float *list_x = (float *)dyn + (size_t)warp * WCAP;              // [row][warp][WCAP], then the target row's ids
-    unsigned short *list_id = (unsigned short *)(dyn + (size_t)2 * NWARP * WCAP * sizeof(float)) + (size_t)warp * WCAP;
+    // the lists [warp][WCAP]: value (x, later the weight) and id of the target row's entries, values of the draft row's
+    uint2 *const list_p = (uint2 *)dyn + (size_t)warp * WCAP;
+    unsigned *const list_q = (unsigned *)((uint2 *)dyn + (size_t)NWARP * WCAP) + (size_t)warp * WCAP;
 
     auto csync = [&]() {                               // barrier of the cluster
         if (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
         else __syncthreads();
     };
-    auto post_p = [&](float a, float bu) -> float {
-        if (mix) a = __fsub_rn(__fmul_rn(p.one_plus_lam, a), __fmul_rn(p.lam, bu));
-        return div ? __fdiv_rn(a, p.temperature) : a;
-    };
     // (the target logits are read through L2: this kernel may have started before they were written, and the
     // non-coherent load path then served stale lines of the previous iteration)
-    auto load_p = [&](int v) -> float { return post_p(__ldcg(c + v), mix ? __ldcg(u + v) : 0.f); };
-    auto load_q = [&](int v) -> float { const float x = qr[v]; return div ? __fdiv_rn(x, p.temperature) : x; };
+    auto load_p = [&](int v) -> float { return post_logit(c, u, v, p.one_plus_lam, p.lam, p.temperature); };
+    auto load_q = [&](int v) -> float { return post_logit(qr, nullptr, v, 0.f, 0.f, p.temperature); };
 
-    float xr[2][8];
-    auto load8 = [&](int j0) {                         // x of ids j0 .. j0 + 7 of this lane, of both rows, all loads in flight
-        float t[8], s[8];
+    auto load4 = [&](const float *src, int v, float *x) {            // ids v .. v + 3, at least the first of them below hi
+        if (vec) {
+            const float4 t = __ldcg((const float4 *)(src + v));
+            x[0] = t.x; x[1] = t.y; x[2] = t.z; x[3] = t.w;
+        } else {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int v = wbase + 32 * (j0 + i) + lane;
-            const bool in = j0 + i < J && v < hi;
-            xr[1][i] = rawq && in ? qr[v] : 0.f;
-            t[i] = in ? __ldcg(c + v) : 0.f;
-            s[i] = mix && in ? __ldcg(u + v) : 0.f;
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            xr[0][i] = post_p(t[i], s[i]);
-            if (div) xr[1][i] = __fdiv_rn(xr[1][i], p.temperature);
+            for (int i = 0; i < 4; ++i) x[i] = v + i >= hi ? 0.f : p.n_known ? __ldcg(src + v + i) : src[v + i];
         }
     };
-    // body(row, id, exists, x) over this lane's ids, warp-uniformly
+    auto has = [&](int v) { return v >= lo && v < hi; };
+    float xr[2][N];
     bool loaded = false;
+    // body(v): this lane's x of group g are in xr[row], its ids in v + 128 h + i
     auto sweep = [&](auto body) {
 #pragma unroll 1
-        for (int j0 = 0; j0 < J; j0 += 8) {
-            if (!REG || !loaded) load8(j0);
+        for (int g = 0; g < G; ++g) {
+            const int v = wbase + g * 32 * N + 4 * lane;
+            if (!REG || !loaded) {                     // both rows, all loads in flight
+                float t[N], s[N];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int v = wbase + 32 * (j0 + i) + lane;
-                body(RowIndex<0>{}, v, j0 + i < J && v < hi, xr[0][i]);
-            }
-            if (rawq) {
+                for (int j = 0; j < N; ++j) t[j] = s[j] = xr[1][j] = 0.f;
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int v = wbase + 32 * (j0 + i) + lane;
-                    body(RowIndex<1>{}, v, j0 + i < J && v < hi, xr[1][i]);
+                for (int h = 0; h < NS; ++h) {
+                    if (v + 128 * h >= hi) continue;
+                    if (rawq) load4(qr, v + 128 * h, &xr[1][4 * h]);
+                    load4(c, v + 128 * h, &t[4 * h]);
+                    if (mix) load4(u, v + 128 * h, &s[4 * h]);
+                }
+                if (mix) {
+#pragma unroll
+                    for (int j = 0; j < N; ++j) t[j] = __fsub_rn(__fmul_rn(p.one_plus_lam, t[j]), __fmul_rn(p.lam, s[j]));
+                }
+                if (div) {
+#pragma unroll
+                    for (int j = 0; j < N; ++j) { t[j] = __fdiv_rn(t[j], p.temperature); xr[1][j] = __fdiv_rn(xr[1][j], p.temperature); }
+                }
+#pragma unroll
+                for (int j = 0; j < N; ++j) xr[0][j] = t[j];
+                // ids that do not exist: NaN, which no comparison below takes
+                const int v0 = wbase + g * 32 * N;
+                if (v0 < lo || v0 + 32 * N > hi) {
+#pragma unroll
+                    for (int j = 0; j < N; ++j)
+                        if (!has(v + 128 * (j >> 2) + (j & 3))) xr[0][j] = xr[1][j] = __int_as_float(0x7FC00000);
                 }
             }
+            body(v);
         }
         loaded = true;
     };
@@ -289,22 +312,20 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         m[0] = lc.red_f[0][0];
         if (rawq) m[1] = lc.red_f[1][0];
     };
-    // Two ids per lane of each row, spread over the warp's range.
+    // Two ids per lane of each row, spread over the warp's range (REG: of the registers).
     auto sample = [&](auto body) {
-        const int ja = J / 4, jb = J - 1 - J / 4;
         if (REG) {
-            if (!loaded) { load8(0); loaded = true; }
+            const int v = wbase + 4 * lane;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int v = wbase + 32 * i + lane;
-                if ((i == ja || i == jb) && i < J && v < hi) { body(0, xr[0][i]); if (rawq) body(1, xr[1][i]); }
-            }
+            for (int j = 0; j < N; j += N - 1)
+                if (has(v + 128 * (j >> 2) + (j & 3))) { body(0, xr[0][j]); if (rawq) body(1, xr[1][j]); }
         } else {
-            const int va = wbase + 32 * ja + lane, vb = wbase + 32 * jb + lane;
-            const float pa = va < hi ? load_p(va) : 0.f, pb = vb < hi ? load_p(vb) : 0.f;
-            const float qa = rawq && va < hi ? load_q(va) : 0.f, qb = rawq && vb < hi ? load_q(vb) : 0.f;
-            if (va < hi) { body(0, pa); if (rawq) body(1, qa); }
-            if (vb < hi) { body(0, pb); if (rawq) body(1, qb); }
+            const int n = range / 128, va = wbase + 128 * (n / 4) + 4 * lane + 1, vb = wbase + 128 * (n - 1 - n / 4) + 4 * lane + 2;
+            const bool ia = has(va), ib = has(vb);
+            const float pa = ia ? load_p(va) : 0.f, pb = ib ? load_p(vb) : 0.f;
+            const float qa = rawq && ia ? load_q(va) : 0.f, qb = rawq && ib ? load_q(vb) : 0.f;
+            if (ia) { body(0, pa); if (rawq) body(1, qa); }
+            if (ib) { body(0, pb); if (rawq) body(1, qb); }
         }
     };
     // After a sample's histogram (2 NB bins per row in the tables of the masses, the smallest sample in bin 0): the highest
@@ -340,18 +361,48 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         __syncthreads();
     };
 
-    // the lists (and the sweep that fills them): ids that `keep` names
-    int n_list[2] = {0, 0};                            // (warp-uniform)
-    auto append = [&](auto A_, int v, bool in, float x, bool keep) {
-        constexpr int a = decltype(A_)::value;
-        const unsigned vote = __ballot_sync(FULLM, keep);
-        const int at = n_list[a] + __popc(vote & ((1u << lane) - 1u));
-        if (keep && at < WCAP) {
-            list_x[a * NWARP * WCAP + at] = x;
-            if (a == 0) list_id[at] = (unsigned short)(v - wbase);
+    // The lists: of the group at v (see sweep), the ids that `keep` has a bit for (bit 4 h + i of row a), with their value
+    // (x, or the weight's bit pattern). One scan over the warp for both rows: counts of up to 128 in bytes.
+    int n_list[2] = {0, 0};                            // (warp-uniform; above WCAP once a list has overflowed)
+    auto append = [&](int v, const unsigned (&keep)[2], const float (&val)[2][N]) {
+        unsigned packed = 0;
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int h = 0; h < NS; ++h) packed |= (unsigned)__popc(keep[a] >> (4 * h) & 15u) << (8 * (a * NS + h));
+        unsigned inc = packed;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned t = __shfl_up_sync(FULLM, inc, o);
+            if (lane >= o) inc += t;
         }
-        if (a == 0 && wstore && in && !keep) wstore[v] = 0u;
-        n_list[a] += __popc(vote);
+        const unsigned all = __shfl_sync(FULLM, inc, 31);
+        inc -= packed;
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            if (a && !rawq) break;
+            int n = n_list[a];
+#pragma unroll
+            for (int h = 0; h < NS; ++h) n_list[a] += (int)(all >> (8 * (a * NS + h)) & 255u);
+            if (n_list[a] > WCAP) continue;
+#pragma unroll
+            for (int h = 0; h < NS; ++h) {
+                int at = n + (int)(inc >> (8 * (a * NS + h)) & 255u);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (!(keep[a] >> (4 * h + i) & 1u)) continue;
+                    if (a == 0) list_p[at] = make_uint2(__float_as_uint(val[a][4 * h + i]), (unsigned)(v + 128 * h + i));
+                    else list_q[at] = __float_as_uint(val[a][4 * h + i]);
+                    ++at;
+                }
+                n += (int)(all >> (8 * (a * NS + h)) & 255u);
+            }
+        }
+        if (wstore) {
+#pragma unroll
+            for (int j = 0; j < N; ++j)
+                if (!(keep[0] >> j & 1u) && has(v + 128 * (j >> 2) + (j & 3))) wstore[v + 128 * (j >> 2) + (j & 3)] = 0u;
+        }
     };
     // entry e of this warp: of its list, or of its whole range when the list did not fit
     bool whole[2] = {false, false};
@@ -359,16 +410,25 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
     auto close_lists = [&]() {
         __syncwarp();
 #pragma unroll
-        for (int a = 0; a < 2; ++a) { whole[a] = n_list[a] > WCAP; n_e[a] = whole[a] ? 32 * J : n_list[a]; }
+        for (int a = 0; a < 2; ++a) { whole[a] = n_list[a] > WCAP; n_e[a] = whole[a] ? range : n_list[a]; }
     };
-    auto entry_x = [&](auto A_, int e, bool &in) -> float {          // x of entry e (in: it exists)
+    float tau[2] = {-INFINITY, -INFINITY};
+    unsigned theta[2] = {0u, 0u};
+    auto entry_in = [&](int a, int e) -> bool { return e < n_e[a] && (!whole[a] || has(wbase + e)); };
+    auto entry_x = [&](auto A_, int e, bool &in) -> float {          // x of entry e (in: it exists), while the lists hold x
         constexpr int a = decltype(A_)::value;
-        in = e < n_e[a] && (!whole[a] || wbase + e < hi);
+        in = entry_in(a, e);
         if (!in) return -INFINITY;
-        if (!whole[a]) return list_x[a * NWARP * WCAP + e];
+        if (!whole[a]) return __uint_as_float(a == 0 ? list_p[e].x : list_q[e]);
         return a == 0 ? load_p(wbase + e) : load_q(wbase + e);
     };
-    auto entry_id = [&](int e) -> int { return wbase + (whole[0] ? e : (int)list_id[e]); };
+    auto entry_w = [&](auto A_, int e) -> unsigned {                 // its weight (0: none), once they hold weights
+        constexpr int a = decltype(A_)::value;
+        if (!entry_in(a, e)) return 0u;
+        if (!whole[a]) return a == 0 ? list_p[e].x : list_q[e];
+        return weight_of(a == 0 ? load_p(wbase + e) : load_q(wbase + e), m[a], tau[a]);
+    };
+    auto entry_id = [&](int e) -> int { return whole[0] ? wbase + e : (int)list_p[e].y; };
 
     // merges the C histograms: threads 0..255 take the target row, 256..511 the draft row; each owns four steps. Scans
     // them and leaves the step in which the running sum (from `base` on) reaches top_k (counts) or top_p of the mass Z
@@ -439,10 +499,18 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
             const float bound[2] = {again ? -INFINITY : lc.bound[0], again ? -INFINITY : lc.bound[1]};
             float mx[2] = {-INFINITY, -INFINITY};
             n_list[0] = n_list[1] = 0;
-            sweep([&](auto A_, int v, bool in, float x) {
-                constexpr int a = decltype(A_)::value;
-                if (in) mx[a] = fmaxf(mx[a], x);
-                if (!REG) append(A_, v, in, x, in && x >= bound[a]);
+            sweep([&](int v) {
+                unsigned keep[2] = {0u, 0u};
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+#pragma unroll
+                    for (int a = 0; a < 2; ++a) {
+                        mx[a] = fmaxf(mx[a], xr[a][j]);
+                        if (xr[a][j] >= bound[a]) keep[a] |= 1u << j;
+                    }
+                }
+                if (!rawq) keep[1] = 0u;
+                if (!REG) append(v, keep, xr);
             });
             close_lists();
             if (!again) exchange_max(mx[0], mx[1]);                                   // ---- exchange: maxima
@@ -452,7 +520,13 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
                     if (s >= 0) atomicAdd(&xc.hist[a][0][s], 1u);
                 };
                 if (REG) {
-                    sweep([&](auto A_, int, bool in, float x) { count(decltype(A_)::value, in, x); });
+                    sweep([&](int) {
+#pragma unroll
+                        for (int j = 0; j < N; ++j) {
+                            count(0, true, xr[0][j]);
+                            if (rawq) count(1, true, xr[1][j]);
+                        }
+                    });
                 } else {
                     EACH_ROW([&](auto A_) {
                         constexpr int a = decltype(A_)::value;
@@ -471,10 +545,18 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
                 sb[1] = lc.sel[1];
             }
             if (REG) {                                 // the ids are in registers: the lists come last
-                sweep([&](auto A_, int v, bool in, float x) {
-                    constexpr int a = decltype(A_)::value;
-                    const int s = in ? live_step(x, m[a]) : -1;
-                    append(A_, v, in, x, s >= 0 && (sb[a] < 0 || s <= sb[a]));
+                sweep([&](int v) {
+                    unsigned keep[2] = {0u, 0u};
+#pragma unroll
+                    for (int j = 0; j < N; ++j) {
+#pragma unroll
+                        for (int a = 0; a < 2; ++a) {
+                            const int s = live_step(xr[a][j], m[a]);
+                            if (s >= 0 && (sb[a] < 0 || s <= sb[a])) keep[a] |= 1u << j;
+                        }
+                    }
+                    if (!rawq) keep[1] = 0u;
+                    append(v, keep, xr);
                 });
                 close_lists();
             }
@@ -498,7 +580,10 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         // ---- nucleus of the whole row ---------------------------------------------------------------------------------
         {
             float mx[2] = {-INFINITY, -INFINITY};
-            sweep([&](auto A_, int, bool in, float x) { constexpr int a = decltype(A_)::value; if (in) mx[a] = fmaxf(mx[a], x); });
+            sweep([&](int) {
+#pragma unroll
+                for (int j = 0; j < N; ++j) { mx[0] = fmaxf(mx[0], xr[0][j]); mx[1] = fmaxf(mx[1], xr[1][j]); }
+            });
             exchange_max(mx[0], mx[1]);                                               // ---- exchange: maxima
         }
         sample([&](int a, float x) {
@@ -514,21 +599,29 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
             const unsigned cut[2] = {again ? 1u : (unsigned)lc.bound[0], again ? 1u : (unsigned)lc.bound[1]};
             unsigned long long z[2] = {0ull, 0ull};
             n_list[0] = n_list[1] = 0;
-            sweep([&](auto A_, int v, bool in, float x) {
-                constexpr int a = decltype(A_)::value;
-                const unsigned wv = in ? weight_of(x, m[a], -INFINITY) : 0u;
-                z[a] += wv;
-                append(A_, v, in, x, wv >= cut[a]);
+            sweep([&](int v) {
+                unsigned keep[2] = {0u, 0u};
+                float val[2][N];
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+#pragma unroll
+                    for (int a = 0; a < 2; ++a) {
+                        if (a && !rawq) break;
+                        const unsigned wv = weight_of(xr[a][j], m[a], -INFINITY);
+                        z[a] += wv;
+                        if (wv >= cut[a]) keep[a] |= 1u << j;
+                        val[a][j] = __uint_as_float(wv);
+                    }
+                }
+                append(v, keep, val);
             });
             close_lists();
             EACH_ROW([&](auto A_) {
                 constexpr int a = decltype(A_)::value;
                 const unsigned long long t = warp_sum64(z[a]);
                 if (lane == 0) (a ? lc.red_b : lc.red_a)[warp] = t;
-                for (int e0 = 0; e0 < n_e[a]; e0 += 32) {
-                    bool in;
-                    const float x = entry_x(A_, e0 + lane, in);
-                    const unsigned wv = in ? weight_of(x, m[a], -INFINITY) : 0u;
+                for (int e = lane; e < n_e[a]; e += 32) {
+                    const unsigned wv = entry_w(A_, e);
                     if (wv >= cut[a]) add_mass(a, weight_step(wv), wv);
                 }
             });
@@ -567,26 +660,28 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         }
     }
 
-    float tau[2] = {-INFINITY, -INFINITY};
-    unsigned theta[2] = {0u, 0u};
     if (!nucleus) {
         // ---- mass above the selected step, its candidates, the exact threshold, the normaliser ------------------------
         EACH_ROW([&](auto A_) {
             constexpr int a = decltype(A_)::value;
             unsigned long long z = 0;
-            for (int e0 = 0; e0 < n_e[a]; e0 += 32) {
+            for (int e = lane; e < n_e[a]; e += 32) {
                 bool in;
-                const float x = entry_x(A_, e0 + lane, in);
+                const float x = entry_x(A_, e, in);
                 const int s = in ? live_step(x, m[a]) : -1;
-                if (s < 0) continue;
-                if (sb[a] >= 0 && s > sb[a]) continue;
-                const unsigned wv = weight_of(x, m[a], -INFINITY);
-                if (sb[a] < 0 || s < sb[a]) z += wv;
-                else {
+                const bool above = s >= 0 && (sb[a] < 0 || s < sb[a]), cand = s >= 0 && s == sb[a];
+                const unsigned wv = above || cand ? weight_of(x, m[a], -INFINITY) : 0u;
+                if (above) z += wv;
+                if (!whole[a]) { if (a == 0) list_p[e].x = wv; else list_q[e] = wv; }   // the lists hold weights from here on
+                if (cand) {
                     const unsigned at = atomicAdd(&xc.cand_n[a], 1u);
-                    if (at < CAND_CAP) xc.cand[a][at] = make_uint2(float_key(x), wv);
+                    if (at < CAND_CAP) {
+                        xc.cand[a][at] = make_uint2(float_key(x), wv);
+                        lc.cand_at[a][at] = (unsigned short)(whole[a] ? 0xFFFF : warp * WCAP + e);
+                    }
                 }
             }
+            __syncwarp();
             z = warp_sum64(z);
             if (lane == 0) (a ? lc.red_b : lc.red_a)[warp] = z;
         });
@@ -652,6 +747,10 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
             if (n_all[a] <= CAND_CAP) {
                 const unsigned tk = lc.tau_key[a];
                 tau[a] = key_float(tk);
+                for (unsigned i = tid; i < xc.cand_n[a]; i += CT) {  // candidates below the threshold lose their weight
+                    const unsigned at = lc.cand_at[a][i];
+                    if (xc.cand[a][i].x < tk && at != 0xFFFFu) { if (a == 0) ((uint2 *)dyn)[at].x = 0u; else (list_q - (size_t)warp * WCAP)[at] = 0u; }
+                }
                 unsigned long long add = 0;            // the candidates that stay (every warp sums the list for itself)
                 for (unsigned i = lane; i < n_all[a]; i += 32)
                     if (all_cand(a)[i].x >= tk) add += all_cand(a)[i].y;
@@ -659,7 +758,10 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
                 return;
             }
             // long runs of equal or nearly equal logits: radix selection over the cluster, 8 bits of the key per pass,
-            // among the ids of the step; then the normaliser from scratch
+            // among the ids of the step; then the normaliser from scratch. The warps work on their whole ranges from here
+            // on (their lists hold weights that the threshold does not know).
+            whole[a] = true;
+            n_e[a] = range;
             unsigned prefix = 0, mask = 0, kk = lc.sel_k[a];
             for (int pass = 0; pass < 4; ++pass) {
                 const int shift = 24 - 8 * pass;
@@ -722,6 +824,7 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
             __syncthreads();
             Zall[a] = lc.total[a];
         });
+        __syncthreads();                               // (weights of other warps' entries were cleared)
     }
     // ---- nucleus: theta = the largest weight whose ids {W >= theta} hold at least top_p of the mass. The selected step
     // is a range [range_lo, range_lo + 2^bits) of weights, divided NB ways until it is one value. -------------------
@@ -732,10 +835,8 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         auto level = [&](auto step_of) {               // one division: step_of(a, W) = step of NB, heaviest first, or -1
             EACH_ROW([&](auto A_) {
                 constexpr int a = decltype(A_)::value;
-                for (int e0 = 0; e0 < n_e[a]; e0 += 32) {
-                    bool in;
-                    const float x = entry_x(A_, e0 + lane, in);
-                    const unsigned wv = in ? weight_of(x, m[a], tau[a]) : 0u;
+                for (int e = lane; e < n_e[a]; e += 32) {
+                    const unsigned wv = entry_w(A_, e);
                     const int s = wv != 0u ? step_of(a, wv) : -1;
                     if (s >= 0) add_mass(a, s, wv);
                 }
@@ -785,16 +886,13 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
     }
     const unsigned long long Zp = Zall[0];
     const unsigned long long Zq = rawq ? Zall[1] : fresh ? (unsigned long long)(hi - lo) : Zq_stored;
-    auto weight_p = [&](int e, bool &in) -> unsigned {
-        const float x = entry_x(RowIndex<0>{}, e, in);
-        return in ? weight_of(x, m[0], tau[0], theta[0]) : 0u;
+    auto weight_p = [&](int e) -> unsigned {
+        const unsigned wv = entry_w(RowIndex<0>{}, e);
+        return wv >= theta[0] ? wv : 0u;
     };
     if (wstore) {
-        for (int e = lane; e < n_e[0]; e += 32) {
-            bool in;
-            const unsigned wv = weight_p(e, in);
-            if (in) wstore[entry_id(e)] = wv;
-        }
+        for (int e = lane; e < n_e[0]; e += 32)
+            if (entry_in(0, e)) wstore[entry_id(e)] = weight_p(e);
     }
     if (rank == 0 && tid == 0) {
         RowStats st; st.m = m[0]; st.tau = tau[0]; st.Z = Zp; st.theta = theta[0]; st.pad_ = 0u;
@@ -866,7 +964,6 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         if (!accept) {
             // Y ~ norm(max(0, p - q)). The draft's weights of the listed ids first: four gathers in flight, into the draft
             // row's list, which is done with (one at a time, and again in the walk, they were 10 to 15 us of a row)
-            unsigned *const list_wq = (unsigned *)list_x + (size_t)NWARP * WCAP;
             auto weight_q = [&](int v) -> unsigned {
                 return rawq ? weight_of(load_q(v), m[1], tau[1], theta[1]) : fresh ? 1u : __float_as_uint(qr[v]);
             };
@@ -875,21 +972,20 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
                 for (int e0 = lane; e0 < n_e[0]; e0 += 128) {
                     float t[4];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) t[i] = e0 + 32 * i < n_e[0] ? qr[wbase + (int)list_id[e0 + 32 * i]] : 0.f;
+                    for (int i = 0; i < 4; ++i) t[i] = e0 + 32 * i < n_e[0] ? qr[list_p[e0 + 32 * i].y] : 0.f;
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         if (rawq && div) t[i] = __fdiv_rn(t[i], p.temperature);
-                        if (e0 + 32 * i < n_e[0]) list_wq[e0 + 32 * i] = rawq ? weight_of(t[i], m[1], tau[1], theta[1]) : __float_as_uint(t[i]);
+                        if (e0 + 32 * i < n_e[0]) list_q[e0 + 32 * i] = rawq ? weight_of(t[i], m[1], tau[1], theta[1]) : __float_as_uint(t[i]);
                     }
                 }
                 __syncwarp();
             }
             const unsigned Ur = noise_u24(p.seed, NOISE_RESIDUAL, (unsigned)b, pos, w.t, 0);
             const u128 total = draw(4, Ur, [&](int e) -> u128 {
-                bool in;
-                const unsigned wp = weight_p(e, in);
+                const unsigned wp = weight_p(e);
                 if (wp == 0u) return (u128)0;
-                return residual_of(wp, fresh ? 1u : whole[0] ? weight_q(wbase + e) : list_wq[e], Zp, Zq);
+                return residual_of(wp, fresh ? 1u : whole[0] ? weight_q(wbase + e) : list_q[e], Zp, Zq);
             }, [&](int y) {
                 p.row_y[row] = y;
                 if (redraft) *redraft = y;
@@ -905,7 +1001,7 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
     if (indep || !mrs) {
         const unsigned Ui = noise_u24(p.seed, NOISE_INDEP, (unsigned)b, pos, mrs ? w.t : 0u, 0);
         int *const dst = mrs ? p.row_y_indep + row : p.row_y + row;
-        const u128 total = draw(6, Ui, [&](int e) -> u128 { bool in; return (u128)weight_p(e, in); }, [&](int y) { *dst = y; });
+        const u128 total = draw(6, Ui, [&](int e) -> u128 { return (u128)weight_p(e); }, [&](int y) { *dst = y; });
         if (first) {
             if (total == 0) *dst = lo;
             if (!mrs) p.accept_flags[row] = 1;
@@ -919,8 +1015,7 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
             return __fdividef(neglog2_estimate(noise_u24(p.seed, NOISE_GUMBEL, (unsigned)b, pos, 0u, (unsigned)entry_id(e))), (float)wv);
         };
         for (int e = lane; e < n_e[0]; e += 32) {
-            bool in;
-            const unsigned wv = weight_p(e, in);
+            const unsigned wv = weight_p(e);
             if (wv != 0u) best = fminf(best, ratio(e, wv));
         }
         const long long posf = w.pos0 + L + k;
@@ -952,8 +1047,7 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         Racer mine = {0ull, 0u, -1};
         if (best <= bound) {
             for (int e = lane; e < n_e[0]; e += 32) {
-                bool in;
-                const unsigned wv = weight_p(e, in);
+                const unsigned wv = weight_p(e);
                 if (wv == 0u || !(ratio(e, wv) <= bound)) continue;
                 const int v = entry_id(e);
                 const Racer r = {neglog2_q40(noise_u24(p.seed, NOISE_GUMBEL, (unsigned)b, pos, 0u, (unsigned)v)), wv, v};
@@ -1043,17 +1137,18 @@ __global__ void __launch_bounds__(256) commit_kernel(const VerifyParams p)
     }
 }
 
-// Cluster size and ids per lane for rows of at most n ids. One CTA per SM while that leaves a lane at most eight ids
+// Cluster size and ids per warp for rows of at most n ids. One CTA per SM while that leaves a warp at most 256 ids
 // (then they stay in registers), else two: a grid of one wave.
-bool choose_cluster(int n, int rows, int sm_count, int *C_out, int *J_out)
+bool choose_cluster(const VerifyParams &p, int sm_count, int *C_out, int *ids_out)
 {
-    auto ids_per_lane = [&](int C) { return (n + C * CT - 1) / (C * CT); };
+    const int n = p.allowed_hi - p.allowed_lo + (p.allowed_lo & 3), rows = p.L * p.B;
+    auto ids = [&](int C) { return (std::max(n, 4) + C * NWARP - 1) / (C * NWARP); };
     int C = 1;
-    while (C < MAXC && ids_per_lane(C) > 4 && (rows * C * 2 <= sm_count || (rows * C * 2 <= 2 * sm_count && ids_per_lane(C) > 8))) C *= 2;
-    while (C < MAXC && ids_per_lane(C) > MAXJ) C *= 2;
+    while (C < MAXC && ids(C) > 128 && (rows * C * 2 <= sm_count || (rows * C * 2 <= 2 * sm_count && ids(C) > 256))) C *= 2;
+    while (C < MAXC && ids(C) > 256 * MAXG) C *= 2;
     *C_out = C;
-    *J_out = std::max(1, ids_per_lane(C));
-    return ids_per_lane(C) <= MAXJ;
+    *ids_out = ids(C);
+    return ids(C) <= 256 * MAXG;
 }
 
 template <class K, class... A>
@@ -1085,13 +1180,13 @@ cudaError_t launch_ex(bool dependent, K kernel, dim3 grid, int threads, size_t s
 
 bool verify_rows_supported(const VerifyParams &p)
 {
-    int C, J;
-    return choose_cluster(p.allowed_hi - p.allowed_lo, p.L * p.B, 148, &C, &J);
+    int C, ids;
+    return choose_cluster(p, 148, &C, &ids);
 }
 
 int launch_verify_rows(const VerifyParams &p, cudaStream_t stream)
 {
-    constexpr size_t SMEM_REG = (size_t)NWARP * WCAP_REG * 10, SMEM_LONG = (size_t)NWARP * WCAP_LONG * 10;   // two x lists, one of ids
+    auto lists = [](int wcap) { return NWARP * wcap * 12; };         // values and ids of one row, values of the other
     int dev = 0, sms = 148;
     int rc = current_device(&dev);
     if (rc != SCD_OK) return rc;
@@ -1100,19 +1195,21 @@ int launch_verify_rows(const VerifyParams &p, cudaStream_t stream)
     rc = once.run(dev, [&]() -> int {
         SCD_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         if (dev >= 0 && dev < DeviceOnce::kSlots) sm_count[dev] = sms;
-        SCD_CUDA_TRY(cudaFuncSetAttribute(verify_rows_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_REG));
-        SCD_CUDA_TRY(cudaFuncSetAttribute(verify_rows_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LONG));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(verify_rows_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lists(128)));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(verify_rows_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lists(256)));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(verify_rows_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lists(WCAP_LONG)));
         return SCD_OK;
     });
     if (rc != SCD_OK) return rc;
     if (dev >= 0 && dev < DeviceOnce::kSlots) sms = sm_count[dev];
-    int C = 1, J = 1;
-    SCD_REQUIRE(choose_cluster(p.allowed_hi - p.allowed_lo, p.L * p.B, sms, &C, &J), SCD_ERR_SHAPE,
-                "verify: rows of %d ids do not fit a cluster", p.allowed_hi - p.allowed_lo);
+    int C = 1, ids = 1;
+    SCD_REQUIRE(choose_cluster(p, sms, &C, &ids), SCD_ERR_SHAPE, "verify: rows of %d ids do not fit a cluster", p.allowed_hi - p.allowed_lo);
     // (the stand-alone call takes its inputs from the caller's kernels: only a session's grid may start early)
+    const bool dep = p.n_known != nullptr;
     const dim3 grid((unsigned)(p.L * C), (unsigned)p.B, 1);
-    if (J <= 8) SCD_CUDA_TRY(launch_ex(p.n_known != nullptr, verify_rows_kernel<true>, grid, CT, SMEM_REG, C, stream, p, C, J));
-    else SCD_CUDA_TRY(launch_ex(p.n_known != nullptr, verify_rows_kernel<false>, grid, CT, SMEM_LONG, C, stream, p, C, J));
+    if (ids <= 128) SCD_CUDA_TRY(launch_ex(dep, verify_rows_kernel<1, true>, grid, CT, (size_t)lists(128), C, stream, p, C, 1));
+    else if (ids <= 256) SCD_CUDA_TRY(launch_ex(dep, verify_rows_kernel<2, true>, grid, CT, (size_t)lists(256), C, stream, p, C, 1));
+    else SCD_CUDA_TRY(launch_ex(dep, verify_rows_kernel<2, false>, grid, CT, (size_t)lists(WCAP_LONG), C, stream, p, C, (ids + 255) / 256));
     return SCD_OK;
 }
 

@@ -201,15 +201,15 @@ def test_verify_rows_at_the_edges_of_the_dispatch(mode, B, L, V, kw):
     _run_case(mode, B, L, V, iteration=2, seed=21, **kw)
 
 
-@pytest.mark.parametrize("V,L,B,top_k,top_p", [(9000, 80, 2, 700, 0.0), (9000, 80, 2, 0, 0.8), (4000, 6, 1, 300, 0.0)])
+@pytest.mark.parametrize("V,L,B,top_k,top_p", [(9000, 80, 2, 700, 0.0), (9000, 80, 2, 0, 0.8), (9001, 80, 2, 300, 0.0), (4000, 6, 1, 300, 0.0)])
 def test_verify_bound_from_an_unlucky_sample(V, L, B, top_k, top_p):
     """The bound that the lists start from is estimated from ids at fixed places of each warp's range: here exactly those
     hold the largest logits, so that the bound is above the threshold and the lists are built again."""
     p, q = synth.verify_logits(3, 1, B, L, V, device="cuda")
     C = 1 if B * L > 74 else 8
-    J = -(-V // (C * 512))
-    j = torch.arange(V, device="cuda") // 32 % J
-    sampled = (j == J // 4) | (j == J - 1 - J // 4)
+    n = 2 * -(-V // (C * 16 * 256))                    # pieces of 128 ids per warp
+    v = torch.arange(V, device="cuda")
+    sampled = ((v // 128 % n == n // 4) & (v % 4 == 1)) | ((v // 128 % n == n - 1 - n // 4) & (v % 4 == 2))
     p[..., sampled] += 6.0
     q[..., sampled] += 6.0
     p[..., 0], q[..., 0] = float("-inf"), float("-inf")
