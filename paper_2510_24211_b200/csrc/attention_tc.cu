@@ -370,6 +370,7 @@ __global__ void __launch_bounds__(256) attention_tc_kernel(const __grid_constant
     // n_known was written by the previous iteration, which is complete before any kernel of this
     // one starts; the cache entries below `base` are older still.
     const int base = (p.pos_override >= 0 ? p.pos_override : p.n_known[b] - 1) + p.row_off;
+    const size_t row_base = (size_t)q * p.row_stride + p.row_off;
     const int ctx = min(max(base, 0), p.max_seq);
     const int n_tiles = (ctx + TK - 1) / TK;
     // The last CTA of the cluster also rotates, stores and attends to the window rows, which costs
@@ -422,7 +423,7 @@ __global__ void __launch_bounds__(256) attention_tc_kernel(const __grid_constant
         if (rr < rows) {
             const int i = rr % Mq, g = rr / Mq;
             const int pos = min(max(base + i, 0), p.max_seq - 1);
-            const float *src = p.qkv + ((size_t)q * p.row_stride + p.row_off + i) * qstride + (size_t)(kvh * p.n_rep + g) * DH;
+            const float *src = p.qkv + (row_base + i) * qstride + (size_t)(kvh * p.n_rep + g) * DH;
             rotate8(src + j0, src + j0 + half, p.rope + (size_t)pos * half + j0, p.qscale, lo, hi, &rlo, &rhi);
         }
         *(uint4 *)(q_s + sw_off(qrows_pad, rr, j0)) = lo;
@@ -496,7 +497,7 @@ __global__ void __launch_bounds__(256) attention_tc_kernel(const __grid_constant
                 uint4 klo = make_uint4(0u, 0u, 0u, 0u), khi = klo, vlo = klo, vhi = klo;
                 const int pos = base + i;
                 if (i < Mq && pos >= 0 && pos < p.max_seq) {
-                    const float *src = p.qkv + ((size_t)q * p.row_stride + p.row_off + i) * qstride + (size_t)(p.H + kvh) * DH;
+                    const float *src = p.qkv + (row_base + i) * qstride + (size_t)(p.H + kvh) * DH;
                     const float *vs = src + (size_t)p.Hkv * DH;
                     vlo = round8(vs + j0);
                     vhi = round8(vs + j0 + half);
@@ -567,7 +568,7 @@ __global__ void __launch_bounds__(256) attention_tc_kernel(const __grid_constant
             if (fin && rr < rows) {
                 const int i = rr % Mq, gq = rr / Mq;
                 const float inv = w.l[h] > 0.f ? 1.0f / w.l[h] : 0.f;
-                __nv_bfloat16 *dst = p.out + ((size_t)q * p.row_stride + p.row_off + i) * ostride + (size_t)(kvh * p.n_rep + gq) * DH;
+                __nv_bfloat16 *dst = p.out + (row_base + i) * ostride + (size_t)(kvh * p.n_rep + gq) * DH;
 #pragma unroll
                 for (int j = 0; j < DH / 8; ++j) {
                     const int col = j * 8 + 2 * (lane & 3);
@@ -636,7 +637,7 @@ __global__ void __launch_bounds__(256) attention_tc_kernel(const __grid_constant
                 acc.z += wp * part[peer].z; acc.w += wp * part[peer].w;
             }
             const int i = rr % Mq, gq = rr / Mq;
-            __nv_bfloat16 *dst = p.out + ((size_t)q * p.row_stride + p.row_off + i) * ostride + (size_t)(kvh * p.n_rep + gq) * DH + col;
+            __nv_bfloat16 *dst = p.out + (row_base + i) * ostride + (size_t)(kvh * p.n_rep + gq) * DH + col;
             uint2 packed;
             packed.x = pack_bf16(acc.x, acc.y);
             packed.y = pack_bf16(acc.z, acc.w);
@@ -787,7 +788,9 @@ __device__ __forceinline__ void t5_st32(uint32_t taddr, const float *v)
                  : "memory");
 }
 
-template <int DH, int G>
+// PRE: a prefill chunk, many query tiles per head (a parameter of its own: as a runtime switch it cost the window forward
+// 1 % at 2300 tokens of context and 1.5 % at 9000, 4210 and 3078 us of the whole forward against 4162 and 3034).
+template <int DH, int G, bool PRE>
 __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __grid_constant__ AttnParams p)
 {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -838,14 +841,17 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
 
     const int C = p.C, rank = blockIdx.x % C;
     // prefill: the query tiles with the most keys first, so that the short ones fill the last wave
-    const bool prefill = p.chunk_rows > 0;
-    const int n_units = (int)gridDim.x / C, heads = prefill ? n_units / ((p.chunk_rows + p.Mq - 1) / p.Mq) : n_units;
-    const int unit = (int)(blockIdx.x / C) % heads;
-    const int q_tile = prefill ? n_units / heads - 1 - (int)(blockIdx.x / C) / heads : 0;
+    int unit = blockIdx.x / C, q_tile = 0, Mq = p.Mq;
+    if constexpr (PRE) {
+        const int q_tiles = (p.chunk_rows + p.Mq - 1) / p.Mq, heads = (int)gridDim.x / C / q_tiles;
+        q_tile = q_tiles - 1 - unit / heads;
+        unit %= heads;
+        Mq = min(p.Mq, p.chunk_rows - q_tile * p.Mq);
+    }
     const int q = unit / p.Hkv, kvh = unit % p.Hkv;
     const int b = q % p.B;
-    const int Mq = prefill ? min(p.Mq, p.chunk_rows - q_tile * p.Mq) : p.Mq, rows = Mq * p.n_rep;
-    const size_t row_base = (size_t)q * p.row_stride + p.row_off + q_tile * p.Mq;
+    const int rows = Mq * p.n_rep;
+    const size_t row_base = (size_t)q * (PRE ? p.chunk_rows : Mq) + q_tile * p.Mq;
     constexpr int R = 128 / G;                                    // query rows a CTA can carry (rows <= R)
     constexpr int NC = TK / G;                                    // keys of a tile per thread
     constexpr int half = DH / 2;
@@ -858,12 +864,12 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
     uint8_t *q_st = vring + (size_t)NV * tile_bytes;              // two planes of [R][DH] bf16, rows 16 bytes apart in the banks;
     uint8_t *w_st = q_st;                                         // after that the window's K tiles, then its V tiles
 
-    const int base = (p.pos_override >= 0 ? p.pos_override : p.n_known[b] - 1) + q_tile * p.Mq;
+    const int base = (p.pos_override >= 0 ? p.pos_override : p.n_known[b] - 1) + (PRE ? q_tile * p.Mq : 0);
     // keys that come from the cache: the committed context, in a prefill chunk also the rows of the chunk so far
-    const int ctx = min(max(base + (prefill ? Mq : 0), 0), p.max_seq);
+    const int ctx = min(max(base + (PRE ? Mq : 0), 0), p.max_seq);
     const int n_tiles = (ctx + TK - 1) / TK;
-    const bool has_window = rank == C - 1 && !prefill;
-    const int per = prefill ? n_tiles : (n_tiles + 3 + C - 1) / C;
+    const bool has_window = !PRE && rank == C - 1;
+    const int per = PRE ? n_tiles : (n_tiles + 3 + C - 1) / C;
     const int t0 = min(n_tiles, rank * per);
     const int t1 = has_window ? n_tiles : min(n_tiles, (rank + 1) * per);
     const int my_tiles = t1 - t0;
@@ -899,7 +905,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
         if (v_lane)
             for (int t = 0; t < min(NV, my_tiles); ++t) issue(t, vring + (size_t)t * tile_bytes, &vfull[t], row0_v);
     };
-    if (!prefill) first_tiles();
+    if (!PRE) first_tiles();
 
     // softmax threads: lane = column group * R + query row
     const int grp = tid / R, row = tid % R;                       // (warps 0-3; R is a multiple of 32)
@@ -932,7 +938,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
         }
 
     pdl_wait();                                                   // the projections come from the GEMM in front
-    if (prefill) {
+    if (PRE) {
         // the keys were written with plain stores by the kernel in front, the copies read them through the async proxy
         asm volatile("fence.proxy.async.global;" ::: "memory");
         first_tiles();
@@ -1165,7 +1171,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
             softmax_tile(wt, live ? max(0, min(min(TK, klim), qi - wt * TK + 1)) : 0);
         }
         for (int t = 0; t < my_tiles; ++t)
-            softmax_tile(n_wt + t, live ? min(TK, (prefill ? min(base + qi + 1, ctx) : ctx) - (t0 + t) * TK) : 0);
+            softmax_tile(n_wt + t, live ? min(TK, (PRE ? min(base + qi + 1, ctx) : ctx) - (t0 + t) * TK) : 0);
     }
     if (t_done > 0) wait_on(&bar_o[(t_done - 1) & 1], (unsigned)((t_done - 1) >> 1) & 1u, 9);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -1360,8 +1366,8 @@ static T5Kernel t5_kernel(int dh, int rows, int *G_out)
 {
     const int G = rows > 64 ? 1 : rows > 32 ? 2 : 4;              // column groups: 128 / G query rows per CTA
     *G_out = G;
-    return dh == 128 ? (G == 1 ? attention_t5_kernel<128, 1> : G == 2 ? attention_t5_kernel<128, 2> : attention_t5_kernel<128, 4>)
-                     : (G == 1 ? attention_t5_kernel<64, 1> : G == 2 ? attention_t5_kernel<64, 2> : attention_t5_kernel<64, 4>);
+    return dh == 128 ? (G == 1 ? attention_t5_kernel<128, 1, false> : G == 2 ? attention_t5_kernel<128, 2, false> : attention_t5_kernel<128, 4, false>)
+                     : (G == 1 ? attention_t5_kernel<64, 1, false> : G == 2 ? attention_t5_kernel<64, 2, false> : attention_t5_kernel<64, 4, false>);
 }
 
 // the tcgen05 kernel's shared-memory opt-in, once per device
@@ -1372,12 +1378,14 @@ static int t5_prepare()
     const int rc = current_device(&dev);
     if (rc != SCD_OK) return rc;
     return once.run(dev, []() -> int {
-        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<128, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
-        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<128, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
-        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<128, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
-        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<64, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
-        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<64, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
-        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<64, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<128, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<128, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<128, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<64, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<64, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<64, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<128, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_t5_kernel<64, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T5_SMEM));
         return SCD_OK;
     });
 }
@@ -1449,7 +1457,8 @@ static int attention_t5(scd_session *s, AttnParams &p, int C, cudaStream_t st)
     const int units = s->Q * c.n_kv_heads * q_tiles;
     const int rows = p.Mq * p.n_rep;
     int G = 1;
-    const T5Kernel fn = t5_kernel(dh, rows, &G);
+    const T5Kernel fn = p.chunk_rows > 0 ? dh == 128 ? attention_t5_kernel<128, 1, true> : attention_t5_kernel<64, 1, true>
+                                         : t5_kernel(dh, rows, &G);
     const size_t tile_bytes = (size_t)TK * dh * 2;                // one K or V slot
     const size_t merge_bytes = (size_t)128 * (dh + 4 + 4) * sizeof(float);
     // All the shared memory a CTA can have: no CTA of another kernel fits beside this one, so the tensor
