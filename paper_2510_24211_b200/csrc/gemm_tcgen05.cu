@@ -21,7 +21,7 @@
 //
 // CTAs are small (a ring of ~72 KB, so that three fit on an SM) and the grid is ONE wave of them:
 // the shape rule picks the number of K slices so that every SM has two or three CTAs streaming
-// (grids of at most two CTAs per SM get a deeper ring). The kernel is launched with programmatic
+// (grids that fit with two CTAs per SM get a deeper ring). The kernel is launched with programmatic
 // stream serialisation: the weight tiles of the ring are requested before griddepcontrol.wait, so the
 // weight stream of this GEMM starts while the kernel in front of it drains; everything that
 // depends on that kernel (the x operand, the residual stream, the norm statistics) is touched
@@ -63,7 +63,7 @@ constexpr int MAX_SEG = 3;
 constexpr int MAX_STAGES = 12;
 constexpr int MAX_CLUSTER = 8;
 constexpr int MAX_ROWS = 256;        // window rows one launch may carry (scd_gemm_bf16)
-constexpr int WS_ROWS = 128;         // ... and up to which a session uses this kernel
+constexpr int WS_ROWS = 128;         // ... and up to which a session always uses this kernel (see choose_shape)
 constexpr int GEMM_THREADS = 192;
 
 enum { EPI_BF16 = 0, EPI_F32 = 1, EPI_RESID = 2, EPI_SWIGLU = 3 };
@@ -617,35 +617,12 @@ int tiles_for(const Segment *segs, int n_seg, bool pair, int h)
     return t;
 }
 
-// Launch shape of one GEMM: K slices C (= cluster size, at most 8, the portable limit) and tile
-// height h. Measured on B200: one wave of CTAs streams best (three CTAs fit per SM, clusters
-// leave some slots unused; a second wave costs 30-50 %), full-height tiles beat lower ones (the x
-// tile is re-read per weight tile), and a CTA should stream at most ~32 K blocks. So: full-height
-// tiles and the smallest C that gives every SM two CTAs.
-void choose_shape(const Segment *segs, int n_seg, bool pair, int k_blocks, int sm_count, int *C_out, int *h_out,
-                  int *tiles_out, int tuned = 0, int forced = 0)
-{
-    const int h = pair ? TILE_N / 2 : TILE_N;
-    const int tiles = tiles_for(segs, n_seg, pair, h);
-    int C;
-    if (forced > 0) C = forced;
-    else if (tuned > 0) C = tuned;
-    else {
-        C = (k_blocks + 31) / 32;
-        while (C < MAX_CLUSTER && tiles * C < 2 * sm_count && k_blocks / (C + 1) >= 2) ++C;
-    }
-    *C_out = std::max(1, std::min(std::min(C, k_blocks), MAX_CLUSTER));
-    *h_out = h;
-    *tiles_out = tiles;
-}
-
-// Ring slots: about 72 KB per CTA so that three CTAs share an SM - or about 100 KB when the grid has
-// at most two CTAs per SM anyway (measured: the deeper ring then wins a few percent) - and never
-// less than the partial-tile staging.
-int choose_stages(int nbox, int planes, int k_blocks_per_cta, bool two_per_sm, int forced = 0)
+// Ring slots: about 72 KB per CTA so that three CTAs share an SM - or up to 109 KB (`deep`) when the grid fits two
+// CTAs per SM anyway (measured: the deeper ring then wins a few percent) - and never less than the partial-tile staging.
+int choose_stages(int nbox, int planes, int k_blocks_per_cta, bool deep, int forced = 0)
 {
     const int stage_bytes = (int)stage_bytes_of(nbox, planes);
-    int st = std::max(2, ((two_per_sm ? 100 : 73) * 1024) / stage_bytes);
+    int st = std::max(2, ((deep ? 109 : 73) * 1024) / stage_bytes);
     if (forced > 0) st = forced;
     st = std::min(st, (int)((SMEM_LIMIT - 1024) / stage_bytes));
     st = std::min(st, MAX_STAGES);
@@ -653,23 +630,132 @@ int choose_stages(int nbox, int planes, int k_blocks_per_cta, bool two_per_sm, i
     return std::max(st, 1);
 }
 
-int launch(GemmParams &p, int tiles, cudaStream_t st)
+// dynamic shared memory of one CTA
+size_t smem_of(int nbox, int planes, int rows, int C, int stages)
 {
-    const size_t ring = std::max((size_t)p.stages * stage_bytes_of(p.nbox, p.x_planes), staging_bytes_of(p.nbox));
-    p.aux_offset = (int)ring;
-    const size_t rows_per_cta = (size_t)(p.M + p.k_splits - 1) / p.k_splits;
-    size_t smem = ring + 5 * rows_per_cta * sizeof(float) + 1024;
-    SCD_REQUIRE(smem <= SMEM_LIMIT, SCD_ERR_SHAPE, "GEMM needs %zu bytes of shared memory", smem);
-    SCD_REQUIRE(p.M <= MAX_ROWS, SCD_ERR_SHAPE, "GEMM carries at most %d window rows", MAX_ROWS);
+    const size_t ring = std::max((size_t)stages * stage_bytes_of(nbox, planes), staging_bytes_of(nbox));
+    return ring + 5 * (size_t)((rows + C - 1) / C) * sizeof(float) + 1024;
+}
+
+// Clusters of C CTAs that the device holds at once, n CTAs per SM: a GPC keeps whole clusters only, so 6 x 48 CTAs,
+// for instance, need more than two CTAs on each of 148 SMs.
+__global__ void __launch_bounds__(GEMM_THREADS) slots_kernel() {}   // (never launched: for the GEMM kernel itself, which
+                                     // allocates tensor memory, the occupancy query answers one CTA per SM at any size)
+
+struct Resident {
+    int sm_smem, cta_smem;           // shared memory of an SM; what a CTA takes beyond its dynamic part
+    int clusters[4][MAX_CLUSTER + 1];
+};
+
+int resident_clusters(Resident *out)
+{
+    static Resident table[DeviceOnce::kSlots];
     static DeviceOnce once;
     int dev = 0;
     int rc = current_device(&dev);
     if (rc != SCD_OK) return rc;
+    const bool slot = dev >= 0 && dev < DeviceOnce::kSlots;
     rc = once.run(dev, [&]() -> int {
+        Resident r;
+        int reserved = 0;
+        cudaFuncAttributes fa;
+        SCD_CUDA_TRY(cudaDeviceGetAttribute(&r.sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+        SCD_CUDA_TRY(cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev));
+        SCD_CUDA_TRY(cudaFuncGetAttributes(&fa, gemm_ws_kernel));
         SCD_CUDA_TRY(cudaFuncSetAttribute(gemm_ws_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(slots_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT));
+        r.cta_smem = reserved + (int)fa.sharedSizeBytes;
+        for (int n = 1; n <= 3; ++n)
+            for (int C = 1; C <= MAX_CLUSTER; ++C) {
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3((unsigned)(C * 256), 1, 1);
+                cfg.blockDim = dim3(GEMM_THREADS, 1, 1);
+                cfg.dynamicSmemBytes = std::min(SMEM_LIMIT, (size_t)(r.sm_smem / n - r.cta_smem) & ~(size_t)127);
+                cudaLaunchAttribute attr;
+                attr.id = cudaLaunchAttributeClusterDimension;
+                attr.val.clusterDim.x = (unsigned)C;
+                attr.val.clusterDim.y = 1;
+                attr.val.clusterDim.z = 1;
+                cfg.attrs = &attr;
+                cfg.numAttrs = 1;
+                SCD_CUDA_TRY(cudaOccupancyMaxActiveClusters(&r.clusters[n][C], slots_kernel, &cfg));
+            }
+        if (slot) table[dev] = r;
+        *out = r;
         return SCD_OK;
     });
+    if (rc == SCD_OK && slot) *out = table[dev];
+    return rc;
+}
+
+// Launch shape of one GEMM: K slices C (= cluster size, at most 8, the portable limit), tile height h and ring slots.
+// Measured on B200: one wave of CTAs streams best (a second wave costs 30-50 %), full-height tiles beat lower ones
+// (the x tile is re-read per weight tile), and a CTA should stream at most ~32 K blocks. So: full-height tiles and the
+// smallest C that gives every SM two CTAs, among those whose clusters are all resident at once (counting CTAs instead
+// put 6 x 48, 3 x 96 and 8 x 36 of them into a second wave: 12 layers of 3072 with 6 of 24 KV heads 1.100 -> 1.025 ms
+// at 64 rows), with a deep ring where they are with two CTAs per SM. Up to 64 rows three CTAs may share an SM; beyond,
+// their rings of two slots are slower than two CTAs with three (12 layers of 3072 at 80 rows: 1.577 and 1.070 ms; of
+// 1280: 0.760 and 0.646). Past 32 rows the sum over the slices is what more of them cost: once every SM has a CTA a
+// slice keeps five K blocks (K = 1280, 64 rows: 3840 columns 7.5 us with 5 slices, 8.8 with 8; 6912 gate and up
+// columns 9.8 with 4, 11.5 with 6; at 128 rows 13.7 and 23.3), two where K has less than 16 (768: 0.592 and 0.599 ms).
+// A grid of two waves takes the slices with the fewest K blocks one after the other, waves x blocks of a slice (22016 x
+// 4096 gate and up in 4 layers at 128 rows: 3 slices 0.668 ms, 2 slices 0.722; 28672 x 4096: 1 slice 0.692, 2 0.728).
+//
+// *streams: whether this kernel should take the GEMM at more than WS_ROWS rows, or the CTA-pair kernel, whose time
+// hardly depends on the rows. It should if its grid is one wave and either two CTAs fit per SM or a CTA streams at
+// most 24 K blocks. Both measured, here and there, in us at 256 rows: 3840 x 1280 13.5, 23.8; 4096 x 4096 29.2, 32.0
+// (16 blocks); 9216 x 3072 28.5, 28.5 (24); 16384 x 2048 35.6, 31.1 (32); two waves of 22016 x 4096 117, 66; at 144
+// rows 16384 x 3072 (two per SM) 31.8, 43.9. At most WS_ROWS rows this kernel is faster throughout (12 layers of 4096 at
+// 128 rows 1.99 and 2.46 ms, of 1280 0.79 and 1.35).
+constexpr int LONE_BLOCKS = 24;
+int choose_shape(const Segment *segs, int n_seg, bool pair, int rows, int sm_count, GemmParams *p, int *tiles_out, bool *streams,
+                 int tuned, int forced, int forced_stages)
+{
+    Resident res;
+    int rc = resident_clusters(&res);
     if (rc != SCD_OK) return rc;
+    const int h = pair ? TILE_N / 2 : TILE_N, nbox = round16(rows), k_blocks = p->k_blocks;
+    const int tiles = tiles_for(segs, n_seg, pair, h);
+    auto stages = [&](int C, bool deep) { return choose_stages(nbox, p->x_planes, (k_blocks + C - 1) / C, deep, forced_stages); };
+    auto per_sm = [&](int C, bool deep) {
+        const int smem = res.cta_smem + (int)smem_of(nbox, p->x_planes, rows, C, stages(C, deep));
+        return std::min(rows > 64 ? 2 : 3, res.sm_smem / smem);
+    };
+    auto waves = [&](int C, bool deep) { const int at_once = res.clusters[per_sm(C, deep)][C]; return (tiles + at_once - 1) / at_once; };
+    auto fits = [&](int C) { return waves(C, true) == 1 || waves(C, false) == 1; };
+    int C = forced > 0 ? forced : tuned;
+    if (C <= 0) {
+        const int C0 = std::min(MAX_CLUSTER, (k_blocks + 31) / 32);
+        C = C0;
+        for (int c = C + 1; c <= MAX_CLUSTER && tiles * C < 2 * sm_count; ++c) {
+            if (k_blocks / c < (rows > 32 && k_blocks >= 16 && tiles * C >= sm_count ? 5 : 2)) break;
+            if (fits(c)) C = c;
+        }
+        if (waves(C, rows > 64) == 2 && !fits(C)) {
+            auto at = [&](int c) { return waves(c, rows > 64); };
+            auto span = [&](int c) { return at(c) * ((k_blocks + c - 1) / c); };
+            for (int c = 1; c <= MAX_CLUSTER && k_blocks / c >= 5; ++c)
+                if ((c < C0 ? at(c) == 1 : at(c) <= 2) && (span(c) < span(C) || (span(c) == span(C) && at(c) < at(C)))) C = c;
+        }
+    }
+    C = std::max(1, std::min(std::min(C, k_blocks), MAX_CLUSTER));
+    const bool deep = rows > 64 || waves(C, true) == 1;
+    const int n = per_sm(C, deep);
+    p->k_splits = C;
+    p->tile_rows = h;
+    p->nbox = nbox;
+    p->stages = stages(C, deep);
+    *tiles_out = tiles;
+    *streams = n >= 2 || (waves(C, deep) == 1 && (k_blocks + C - 1) / C <= LONE_BLOCKS);
+    return SCD_OK;
+}
+
+int launch(GemmParams &p, int tiles, cudaStream_t st)
+{
+    p.aux_offset = (int)std::max((size_t)p.stages * stage_bytes_of(p.nbox, p.x_planes), staging_bytes_of(p.nbox));
+    const size_t smem = smem_of(p.nbox, p.x_planes, p.M, p.k_splits, p.stages);
+    SCD_REQUIRE(smem <= SMEM_LIMIT, SCD_ERR_SHAPE, "GEMM needs %zu bytes of shared memory", smem);
+    SCD_REQUIRE(p.M <= MAX_ROWS, SCD_ERR_SHAPE, "GEMM carries at most %d window rows", MAX_ROWS);
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)(tiles * p.k_splits), 1, 1);
@@ -804,18 +890,22 @@ int run_gemm_pair(scd_session *s, const Segment *segs, int n_seg, int epi, const
 int run_gemm(scd_session *s, int kind, const Segment *segs, int n_seg, int epi, const void *x, int K, int rows,
              void *out, int ldo, const NormIn *nin, const NormOut *nout, int x_planes, int *parts_out, cudaStream_t st)
 {
-    if (rows > WS_ROWS) return run_gemm_pair(s, segs, n_seg, epi, x, K, rows, out, ldo, nin, nout, x_planes, parts_out, st);
+    if (rows > MAX_ROWS) return run_gemm_pair(s, segs, n_seg, epi, x, K, rows, out, ldo, nin, nout, x_planes, parts_out, st);
     GemmPlan *plan = (GemmPlan *)s->model->gemm_plan;
     const bool pair = epi == EPI_SWIGLU;
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
     p.k_blocks = K / BLOCK_K;
     int tiles = 0;
-    choose_shape(segs, n_seg, pair, p.k_blocks, plan->sm_count, &p.k_splits, &p.tile_rows, &tiles,
-                 plan->kind_splits[kind], plan->forced_splits);
+    p.x_planes = x_planes;
+    bool streams = true;
+    int rc = choose_shape(segs, n_seg, pair, rows, plan->sm_count, &p, &tiles, &streams, plan->kind_splits[kind], plan->forced_splits,
+                          plan->forced_stages);
+    if (rc != SCD_OK) return rc;
+    if (rows > WS_ROWS && !streams) return run_gemm_pair(s, segs, n_seg, epi, x, K, rows, out, ldo, nin, nout, x_planes, parts_out, st);
     int t0 = 0;
     for (int i = 0; i < n_seg; ++i) {
-        int rc = w_map(plan, segs[i], p.tile_rows, &p.tmap_w[i]);
+        rc = w_map(plan, segs[i], p.tile_rows, &p.tmap_w[i]);
         if (rc != SCD_OK) return rc;
         p.seg_row0[i] = segs[i].row0;
         p.seg_nout[i] = segs[i].row_end;
@@ -825,11 +915,7 @@ int run_gemm(scd_session *s, int kind, const Segment *segs, int n_seg, int epi, 
     p.seg_tile0[pair ? 1 : n_seg] = tiles;
     p.n_seg = pair ? 1 : n_seg;
     p.M = rows;
-    p.nbox = round16(rows);
-    p.x_planes = x_planes;
     p.out_plane = (long long)s->rows_cap * ldo;           // (used by the outputs that are GEMM inputs themselves)
-    p.stages = choose_stages(p.nbox, p.x_planes, (p.k_blocks + p.k_splits - 1) / p.k_splits,
-                             tiles * p.k_splits <= 2 * plan->sm_count, plan->forced_stages);
     p.epi = epi;
     p.out = out;
     p.ldo = ldo;
@@ -845,7 +931,7 @@ int run_gemm(scd_session *s, int kind, const Segment *segs, int n_seg, int epi, 
         p.ss_out = nout->ss;
         *parts_out = tiles;                                // one partial sum of squares per output tile
     }
-    int rc = x_map(s, x, K, p.nbox, p.x_planes, &p.tmap_x);
+    rc = x_map(s, x, K, p.nbox, p.x_planes, &p.tmap_x);
     if (rc != SCD_OK) return rc;
     p.err = (int *)s->gemm_ws;
     p.skip = s->skip_now;
@@ -1027,17 +1113,17 @@ int scd_gemm_bf16_shaped(const void *x, const void *w, float *y, int32_t M, int3
     p.k_blocks = K / BLOCK_K;
     const Segment seg = {w, N, K, 0, N, 0};
     int tiles = 0;
-    choose_shape(&seg, 1, false, p.k_blocks, sms, &p.k_splits, &p.tile_rows, &tiles, 0, k_splits);
-    int rc = make_map(&p.tmap_w[0], w, (uint64_t)N, (uint64_t)K, (uint32_t)p.tile_rows);
+    bool streams;
+    p.x_planes = 1;                                       // the hook multiplies one bf16 matrix
+    int rc = choose_shape(&seg, 1, false, M, sms, &p, &tiles, &streams, 0, k_splits, stages);
     if (rc != SCD_OK) return rc;
-    p.nbox = round16(M);
+    rc = make_map(&p.tmap_w[0], w, (uint64_t)N, (uint64_t)K, (uint32_t)p.tile_rows);
+    if (rc != SCD_OK) return rc;
     // the x box may reach past row M: rows beyond the matrix are zero-filled by TMA
     rc = make_map(&p.tmap_x, x, (uint64_t)M, (uint64_t)K, (uint32_t)p.nbox);
     if (rc != SCD_OK) return rc;
     p.seg_tile0[0] = 0; p.seg_tile0[1] = tiles; p.seg_row0[0] = 0; p.seg_nout[0] = N; p.seg_col0[0] = 0; p.n_seg = 1;
     p.M = M;
-    p.x_planes = 1;                                       // the hook multiplies one bf16 matrix
-    p.stages = choose_stages(p.nbox, 1, (p.k_blocks + p.k_splits - 1) / p.k_splits, tiles * p.k_splits <= 2 * sms, stages);
     p.epi = EPI_F32;
     p.out = y;
     p.ldo = N;

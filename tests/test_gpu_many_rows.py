@@ -42,11 +42,12 @@ def test_many_rows_match_oracle(shape, page, P, B, M, min_ctx):
     assert torch.equal(again, logits)          # cut tiles are added up in a fixed order
 
 
-def test_step_of_many_rows_reads_only_the_sampled_ids():
-    """A decoding step of 160 rows computes the logits of the allowed ids and of the end-of-row id alone; they are
-    those of the explicit forward over the whole vocabulary. Only where a tile's sum over K is cut differs: fp32
+@pytest.mark.parametrize("L", [16, 32])
+def test_step_of_many_rows_reads_only_the_sampled_ids(L):
+    """A decoding step of 160 rows (the weight-streaming GEMM) and of 320 (CTA pairs) computes the logits of the
+    allowed ids and of the end-of-row id alone; they are those of the explicit forward over the whole vocabulary. Only where a tile's sum over K is cut differs: fp32
     sums of 576 terms in another order, 1e-5 of the largest logit."""
-    shape, B, L, P = WIDE_GQA4, 5, 16, 40
+    shape, B, P = WIDE_GQA4, 5, 40
     gm, _ = _models(shape, max_seq=P + 80, seed=5, std=0.06, page=64)
     rng = np.random.default_rng(2)
     cond = rng.integers(0, shape["vocab_in"], size=(B, P)).astype(np.int32)
