@@ -160,12 +160,10 @@ __device__ __forceinline__ Rope8 load_rope8(const float2 *cs)
     r.t0 = *(const float4 *)(cs); r.t1 = *(const float4 *)(cs + 2); r.t2 = *(const float4 *)(cs + 4); r.t3 = *(const float4 *)(cs + 6);
     return r;
 }
-__device__ __forceinline__ void rotate8(const float *xlo, const float *xhi, const Rope8 &rp,
+__device__ __forceinline__ void rotate8(const float4 a0, const float4 a1, const float4 b0, const float4 b1, const Rope8 &rp,
                                         float scale, uint4 &out_lo, uint4 &out_hi, uint4 *rest_lo = nullptr,
                                         uint4 *rest_hi = nullptr)
 {
-    const float4 a0 = *(const float4 *)xlo, a1 = *(const float4 *)(xlo + 4);
-    const float4 b0 = *(const float4 *)xhi, b1 = *(const float4 *)(xhi + 4);
     const float4 t0 = rp.t0, t1 = rp.t1, t2 = rp.t2, t3 = rp.t3;
     const float c[8] = {t0.x, t0.z, t1.x, t1.z, t2.x, t2.z, t3.x, t3.z};
     const float sn[8] = {t0.y, t0.w, t1.y, t1.w, t2.y, t2.w, t3.y, t3.w};
@@ -187,6 +185,13 @@ __device__ __forceinline__ void rotate8(const float *xlo, const float *xhi, cons
     out_hi = make_uint4(hi[0], hi[1], hi[2], hi[3]);
     if (rest_lo) { *rest_lo = make_uint4(rlo[0], rlo[1], rlo[2], rlo[3]); *rest_hi = make_uint4(rhi[0], rhi[1], rhi[2], rhi[3]); }
 }
+__device__ __forceinline__ void rotate8(const float *xlo, const float *xhi, const Rope8 &rp,
+                                        float scale, uint4 &out_lo, uint4 &out_hi, uint4 *rest_lo = nullptr,
+                                        uint4 *rest_hi = nullptr)
+{
+    rotate8(*(const float4 *)xlo, *(const float4 *)(xlo + 4), *(const float4 *)xhi, *(const float4 *)(xhi + 4), rp, scale,
+            out_lo, out_hi, rest_lo, rest_hi);
+}
 __device__ __forceinline__ void rotate8(const float *xlo, const float *xhi, const float2 *cs,
                                         float scale, uint4 &out_lo, uint4 &out_hi, uint4 *rest_lo = nullptr,
                                         uint4 *rest_hi = nullptr)
@@ -194,10 +199,17 @@ __device__ __forceinline__ void rotate8(const float *xlo, const float *xhi, cons
     rotate8(xlo, xhi, load_rope8(cs), scale, out_lo, out_hi, rest_lo, rest_hi);
 }
 // 8 consecutive fp32 values as bf16
-__device__ __forceinline__ uint4 round8(const float *x)
+__device__ __forceinline__ uint4 round8(const float4 a, const float4 b)
 {
-    const float4 a = *(const float4 *)x, b = *(const float4 *)(x + 4);
     return make_uint4(pack_bf16(a.x, a.y), pack_bf16(a.z, a.w), pack_bf16(b.x, b.y), pack_bf16(b.z, b.w));
+}
+__device__ __forceinline__ uint4 round8(const float *x) { return round8(*(const float4 *)x, *(const float4 *)(x + 4)); }
+// (a load that stays where it is written)
+__device__ __forceinline__ float4 ld_f32x4(const float *x)
+{
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(x) : "memory");
+    return v;
 }
 // the part of (lo, hi) that bf16 drops, as bf16: the second plane of a two-plane activation
 __device__ __forceinline__ uint32_t pack_bf16_rest(float lo, float hi)
@@ -332,8 +344,19 @@ __device__ __forceinline__ void process_tile(WarpState<DH> &w, uint32_t kbase, u
 // per query tile, each taking half of the keys of every tile; the two are folded together before
 // the cluster merge. That halves the tile loop; it pays from about four key tiles per CTA on
 // (measured on the 7B-shaped model: -0.12 ms per iteration at 2200 tokens of context, +0.03 ms at 120).
-template <int DH, int KS>
-__global__ void __launch_bounds__(256) attention_tc_kernel(const __grid_constant__ AttnParams p)
+//
+// PART: a part of more query rows than one launch takes. The parts in front of it are in the cache, the launch before this
+// one has just written the last of them: no tile is requested before the wait.
+//
+// A short context is a chain of latencies, and the CTA with the window rows has the longest: its K and V loads are under way
+// together with the queries' and it attends to them first, out of the ring slot that is not filled yet (after the
+// context, with loads of their own and in a copy of the tile routine of their own: 9.7 us a launch for 2 x 32 rows with 20
+// heads of 64 dims at 32 tokens of context, 8.5 so; 64 rows with 24 heads of 128 dims 16.9 and 14.6, at 400 tokens 17.6
+// and 16.6).
+// WARPS: 4 for up to 64 query rows, which leaves registers for the whole tile routine with as many CTAs per SM as grids of
+// one wave have (two of head dimension 128, three of 64); 8 for more.
+template <int DH, int KS, int WARPS, bool PART>
+__global__ void __launch_bounds__(32 * WARPS, WARPS == 4 ? (DH == 64 ? 3 : 2) : (DH == 64 ? 2 : 1)) attention_tc_kernel(const __grid_constant__ AttnParams p)
 {
     extern __shared__ __align__(1024) uint8_t smem_raw[];          // 128-byte swizzle: tiles start on 1024-byte boundaries
     __shared__ uint64_t full_bar[MAX_ATT_STAGES], empty_bar[MAX_ATT_STAGES];
@@ -369,14 +392,17 @@ __global__ void __launch_bounds__(256) attention_tc_kernel(const __grid_constant
 
     // n_known was written by the previous iteration, which is complete before any kernel of this
     // one starts; the cache entries below `base` are older still.
-    const int base = (p.pos_override >= 0 ? p.pos_override : p.n_known[b] - 1) + p.row_off;
-    const size_t row_base = (size_t)q * p.row_stride + p.row_off;
+    const int base = (p.pos_override >= 0 ? p.pos_override : p.n_known[b] - 1) + (PART ? p.row_off : 0);
+    const size_t row_base = PART ? (size_t)q * p.row_stride + p.row_off : (size_t)q * Mq;
     const int ctx = min(max(base, 0), p.max_seq);
     const int n_tiles = (ctx + TK - 1) / TK;
-    // The last CTA of the cluster also rotates, stores and attends to the window rows, which costs
-    // about as much as three context tiles: it takes that many fewer context tiles.
+    // (eight warps with 64 dims have 128 registers, too few for one loop over both kinds of tiles: there the window comes last)
+    constexpr bool FIRST = DH == 128 || WARPS == 4;
+    // The last CTA of the cluster also rotates, stores and attends to the window rows, which costs as much as a context
+    // tile (36 layers of 1280, 300 tokens: 1.667 ms a step, 1.696 when counted as three), as three where it comes last: it
+    // takes that many fewer.
     const bool has_window = rank == C - 1;
-    const int per = (n_tiles + 3 + C - 1) / C;                     // context tiles of the other CTAs
+    const int per = (n_tiles + (FIRST ? 1 : 3) + C - 1) / C;       // context tiles of the other CTAs
     const int t0 = min(n_tiles, rank * per);
     const int t1 = has_window ? n_tiles : min(n_tiles, (rank + 1) * per);
     const int my_tiles = t1 - t0;
@@ -405,10 +431,10 @@ __global__ void __launch_bounds__(256) attention_tc_kernel(const __grid_constant
         const int pre = min(p.stages - 1, my_tiles);
         for (int t = 0; t < pre; ++t) issue(t);
     };
-    if (tid == 0 && p.row_off == 0) first_tiles();
+    if (!PART && tid == 0) first_tiles();
 
     pdl_wait();                                                   // Q, K, V of the window come from the GEMM in front
-    if (tid == 0 && p.row_off > 0) {                              // the launch in front wrote the part before this one into the cache
+    if (PART && tid == 0) {
         asm volatile("fence.proxy.async.global;" ::: "memory");
         first_tiles();
     }
@@ -416,6 +442,56 @@ __global__ void __launch_bounds__(256) attention_tc_kernel(const __grid_constant
     // ---- Q: rotate, scale, stage in shared memory (8 dims of both halves per item, 16-byte accesses) ---
     const size_t qstride = (size_t)(p.H + 2 * p.Hkv) * DH;
     constexpr int CH = half / 8;                                  // 16-byte chunks per half row
+    // the window's K and V, tile by tile, in the slot that first_tiles() leaves free: requested, and once there rotated
+    // or rounded, stored to the cache and staged
+    uint8_t *const kt = stages + (size_t)(p.stages - 1) * stage_bytes, *const vt = kt + tile_bytes;
+    auto window_keep = [&](int pos, int j0, uint4 klo, uint4 khi, uint4 vlo, uint4 vhi) {
+        const int page = pt[pos >> p.page_shift];
+        const long long r = ((long long)page * p.Hkv + kvh) * p.page_tokens + (pos & (p.page_tokens - 1));
+        __nv_bfloat16 *kd = p.pool + (size_t)(p.row0_k + r) * DH, *vd = p.pool + (size_t)(p.row0_v + r) * DH;
+        *(uint4 *)(kd + j0) = klo; *(uint4 *)(kd + j0 + half) = khi;
+        *(uint4 *)(vd + j0) = vlo; *(uint4 *)(vd + j0 + half) = vhi;
+    };
+    auto window_stage = [&](int jr, int j0, uint4 klo, uint4 khi, uint4 vlo, uint4 vhi) {
+        *(uint4 *)(kt + sw_off(TK, jr, j0)) = klo;
+        *(uint4 *)(kt + sw_off(TK, jr, j0 + half)) = khi;
+        *(uint4 *)(vt + sw_off(TK, jr, j0)) = vlo;
+        *(uint4 *)(vt + sw_off(TK, jr, j0 + half)) = vhi;
+    };
+    constexpr int WI = DH / 64;                                   // items of a thread that are requested at once (32 rows by 128 threads)
+    float4 wk[WI][4], wv[WI][4];
+    auto window_row = [&](int e, int wt) { return wt * TK + e / CH; };
+    auto window_load = [&](int e0, int wt) {
+#pragma unroll
+        for (int n = 0; n < WI; ++n) {
+            const int e = e0 + n * (int)blockDim.x, i = window_row(e, wt), pos = base + i;
+            if (e >= TK * CH || i >= Mq || pos < 0 || pos >= p.max_seq) continue;
+            const float *src = p.qkv + (row_base + i) * qstride + (size_t)(p.H + kvh) * DH + (e % CH) * 8;
+            const float *vs = src + (size_t)p.Hkv * DH;
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                wk[n][h] = ld_f32x4(src + (h >> 1) * half + (h & 1) * 4);
+                wv[n][h] = ld_f32x4(vs + (h >> 1) * half + (h & 1) * 4);
+            }
+        }
+    };
+    auto window_store = [&](int e0, int wt) {
+#pragma unroll
+        for (int n = 0; n < WI; ++n) {
+            const int e = e0 + n * (int)blockDim.x, i = window_row(e, wt), pos = base + i;
+            if (e >= TK * CH) continue;
+            const int jr = e / CH, j0 = (e % CH) * 8;
+            uint4 klo = make_uint4(0u, 0u, 0u, 0u), khi = klo, vlo = klo, vhi = klo;
+            if (i < Mq && pos >= 0 && pos < p.max_seq) {
+                vlo = round8(wv[n][0], wv[n][1]);
+                vhi = round8(wv[n][2], wv[n][3]);
+                rotate8(wk[n][0], wk[n][1], wk[n][2], wk[n][3], load_rope8(p.rope + (size_t)pos * half + j0), 1.0f, klo, khi);
+                window_keep(pos, j0, klo, khi, vlo, vhi);
+            }
+            window_stage(jr, j0, klo, khi, vlo, vhi);
+        }
+    };
+    if (FIRST && has_window) window_load(tid, 0);
 #pragma unroll 4
     for (int e = tid; e < qrows_pad * CH; e += blockDim.x) {
         const int rr = e / CH, j0 = (e % CH) * 8;
@@ -430,6 +506,11 @@ __global__ void __launch_bounds__(256) attention_tc_kernel(const __grid_constant
         *(uint4 *)(q_s + sw_off(qrows_pad, rr, j0 + half)) = hi;
         *(uint4 *)(q_lo_s + sw_off(qrows_pad, rr, j0)) = rlo;
         *(uint4 *)(q_lo_s + sw_off(qrows_pad, rr, j0 + half)) = rhi;
+    }
+    if (FIRST && has_window) {
+        window_store(tid, 0);
+#pragma unroll 1
+        for (int e0 = tid + WI * blockDim.x; e0 < TK * CH; e0 += WI * blockDim.x) { window_load(e0, 0); window_store(e0, 0); }
     }
     __syncthreads();
 
@@ -458,67 +539,78 @@ __global__ void __launch_bounds__(256) attention_tc_kernel(const __grid_constant
         qi[h] = rr < rows ? rr % Mq : 0;
     }
 
-    // ---- committed context --------------------------------------------------------------------------
+    // ---- the window rows under the causal mask (t < 0), then the committed context: one loop, one copy of the code -----------
     bool ok = true;
-    for (int t = 0; compute && t < my_tiles; ++t) {
-        if (tid == 0 && t + p.stages - 1 < my_tiles) {
-            const int tn = t + p.stages - 1, s = tn % p.stages;
-            // the slot held tile tn - stages: every warp must have released it
-            if (tn >= p.stages && !mbar_wait(&empty_bar[s], ((tn / p.stages) - 1) & 1)) {
-                atomicExch(p.err, 4); abort_flag = 1;
-            } else {
-                issue(tn);
-            }
-        }
+    const int n_wt = has_window ? (Mq + TK - 1) / TK : 0;
+    const int klim = min(Mq, p.max_seq - base);                   // window keys that exist
+    for (int t = FIRST ? -n_wt : 0; t < my_tiles; ++t) {
+        if (t >= 0 && !compute) break;
+        const uint8_t *tile = kt;
+        int lim[2];                                               // keys of this tile that the thread's two rows see
         const int s = t % p.stages;
-        if (ok) {
-            ok = mbar_wait(&full_bar[s], (t / p.stages) & 1);
-            if (!ok) atomicExch(p.err, 5);
+        if (FIRST && t < 0) {
+            const int wt = t + n_wt;
+            if (WARPS > 4 && wt > 0) {                            // (more than 64 query rows)
+                __syncthreads();                                  // every warp is done with the tile before
+#pragma unroll 1
+                for (int e0 = tid; e0 < TK * CH; e0 += WI * blockDim.x) { window_load(e0, wt); window_store(e0, wt); }
+                __syncthreads();
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) lim[h] = min(klim, qi[h] + 1) - wt * TK;
+        } else {
+            if (tid == 0 && t + p.stages - 1 < my_tiles) {
+                const int tn = t + p.stages - 1, sn = tn % p.stages;
+                // the slot held tile tn - stages: every warp must have released it
+                if (tn >= p.stages && !mbar_wait(&empty_bar[sn], ((tn / p.stages) - 1) & 1)) {
+                    atomicExch(p.err, 4); abort_flag = 1;
+                } else {
+                    issue(tn);
+                }
+            }
+            if (ok) {
+                ok = mbar_wait(&full_bar[s], (t / p.stages) & 1);
+                if (!ok) atomicExch(p.err, 5);
+            }
+            tile = stages + (size_t)s * stage_bytes;
+            lim[0] = lim[1] = ctx - (t0 + t) * TK;                // below the context end
         }
-        if (ok) {
-            const uint32_t kb = smem_u32(stages + (size_t)s * stage_bytes);
-            const int valid = ctx - (t0 + t) * TK;                // keys of this tile below the context end
-            process_tile<DH, KS>(w, kb, kb + tile_bytes, lane, kh, valid < TK,
-                             [&](int, int key) { return key < valid; });
+        if (ok && compute) {
+            const uint32_t kb = smem_u32(tile);
+            process_tile<DH, KS>(w, kb, kb + tile_bytes, lane, kh, (FIRST && t < 0) || lim[0] < TK, [&](int h, int key) { return key < lim[h]; });
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&empty_bar[s]);
+        if (FIRST && t < -1) continue;
+        if (FIRST && t == -1) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the slot goes to the context tiles
+            __syncthreads();
+        } else {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&empty_bar[s]);
+        }
     }
 
-    // ---- the window rows: rotate K, store K and V into the cache, attend under the causal mask -------
-    if (has_window) {
-        for (int wt = 0; wt * TK < Mq; ++wt) {
+    if (!FIRST && has_window) {
+        for (int wt = 0; wt < n_wt; ++wt) {
             __syncthreads();                                      // every warp is done with the ring
-            uint8_t *kt = stages, *vt = stages + tile_bytes;
 #pragma unroll 4
             for (int e = tid; e < TK * CH; e += blockDim.x) {
-                const int jr = e / CH, j0 = (e % CH) * 8;
-                const int i = wt * TK + jr;
+                const int jr = e / CH, j0 = (e % CH) * 8, i = wt * TK + jr, pos = base + i;
                 uint4 klo = make_uint4(0u, 0u, 0u, 0u), khi = klo, vlo = klo, vhi = klo;
-                const int pos = base + i;
                 if (i < Mq && pos >= 0 && pos < p.max_seq) {
                     const float *src = p.qkv + (row_base + i) * qstride + (size_t)(p.H + kvh) * DH;
                     const float *vs = src + (size_t)p.Hkv * DH;
                     vlo = round8(vs + j0);
                     vhi = round8(vs + j0 + half);
                     rotate8(src + j0, src + j0 + half, p.rope + (size_t)pos * half + j0, 1.0f, klo, khi);
-                    const int page = pt[pos >> p.page_shift];
-                    const long long r = ((long long)page * p.Hkv + kvh) * p.page_tokens + (pos & (p.page_tokens - 1));
-                    __nv_bfloat16 *kd = p.pool + (size_t)(p.row0_k + r) * DH, *vd = p.pool + (size_t)(p.row0_v + r) * DH;
-                    *(uint4 *)(kd + j0) = klo; *(uint4 *)(kd + j0 + half) = khi;
-                    *(uint4 *)(vd + j0) = vlo; *(uint4 *)(vd + j0 + half) = vhi;
+                    window_keep(pos, j0, klo, khi, vlo, vhi);
                 }
-                *(uint4 *)(kt + sw_off(TK, jr, j0)) = klo;
-                *(uint4 *)(kt + sw_off(TK, jr, j0 + half)) = khi;
-                *(uint4 *)(vt + sw_off(TK, jr, j0)) = vlo;
-                *(uint4 *)(vt + sw_off(TK, jr, j0 + half)) = vhi;
+                window_stage(jr, j0, klo, khi, vlo, vhi);
             }
             __syncthreads();
-            const int klim = min(Mq, p.max_seq - base) - wt * TK; // window keys that exist
             const uint32_t kb = smem_u32(kt);
             if (compute)
                 process_tile<DH, KS>(w, kb, kb + tile_bytes, lane, kh, true,
-                                 [&](int h, int key) { return key < klim && wt * TK + key <= qi[h]; });
+                                     [&](int h, int key) { return wt * TK + key < klim && wt * TK + key <= qi[h]; });
         }
     }
 
@@ -1582,14 +1674,19 @@ static int attention_part(scd_session *s, int layer, int Mq, int row_stride, int
     if (rc != SCD_OK) return rc;
     rc = once.run(dev, [&]() -> int {
         const int lim = 227 * 1024 - 4096;
-        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel<128, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel<128, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel<64, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel<64, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel<128, 1, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel<128, 2, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel<128, 1, 8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel<128, 1, 8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel<64, 1, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel<64, 2, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel<64, 1, 8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+        SCD_CUDA_TRY(cudaFuncSetAttribute(attention_tc_kernel<64, 1, 8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
         return SCD_OK;
     });
     if (rc != SCD_OK) return rc;
-    const bool wide = (variant & 15) == 1;                        // two warps per query tile
+    const bool later = p.row_off > 0 || p.row_stride != Mq;      // one of several parts
+    const bool wide = !later && (variant & 15) == 1;              // two warps per query tile
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)(units * p.C), 1, 1);
@@ -1605,13 +1702,14 @@ static int attention_part(scd_session *s, int layer, int Mq, int row_stride, int
     attrs[1].val.clusterDim.z = 1;
     cfg.attrs = attrs;
     cfg.numAttrs = 2;
-    if (dh == 128) {
-        if (wide) SCD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attention_tc_kernel<128, 2>, p));
-        else SCD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attention_tc_kernel<128, 1>, p));
-    } else {
-        if (wide) SCD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attention_tc_kernel<64, 2>, p));
-        else SCD_CUDA_TRY(cudaLaunchKernelEx(&cfg, attention_tc_kernel<64, 1>, p));
-    }
+    auto pick = [&](auto of_dh) -> void (*)(const AttnParams) {
+        constexpr int DH = decltype(of_dh)::value;
+        if (later) return attention_tc_kernel<DH, 1, 8, true>;
+        if (wide) return attention_tc_kernel<DH, 2, 4, false>;
+        return p.n_mtiles <= 4 ? attention_tc_kernel<DH, 1, 4, false> : attention_tc_kernel<DH, 1, 8, false>;
+    };
+    void (*const fn)(const AttnParams) = dh == 128 ? pick(std::integral_constant<int, 128>{}) : pick(std::integral_constant<int, 64>{});
+    SCD_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, p));
     count_launches(1);
     return SCD_OK;
 }

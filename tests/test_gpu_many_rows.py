@@ -23,6 +23,9 @@ WIDE_GQA4 = dict(n_layers=2, d_model=576, n_heads=8, n_kv_heads=2, head_dim=64, 
     (WIDE_GQA4, 64, 161, 3, 43, 512),          # 480 prompt rows, 129 window rows of three sequences
     (WIDE_GQA4, 128, 2700, 1, 5, 512),         # two passes over the prompt (2560 rows at most), the second over a context
     (SMALL_BF16, 16, 150, 2, 70, 512),         # head_dim 32: no tensor-core attention
+    (MID_BF16_D64, 64, 70, 1, 65, 512),        # a second window tile with one row, eight warps, 64 dims: window last
+    (dict(MID_BF16_D128_GQA, n_kv_heads=MID_BF16_D128_GQA["n_heads"]), 64, 200, 1, 128, 512),   # 128 dims: window first
+    (MID_BF16_D64, 64, 300, 2, 64, 512),       # four warps, a full window tile, a ring that wraps
 ])
 def test_many_rows_match_oracle(shape, page, P, B, M, min_ctx):
     gm, om = _models(shape, max_seq=P + M + 9, seed=17, std=0.06, page=page, n_streams=B)
