@@ -27,8 +27,8 @@
 // only serial part: first rejection, commit, next window.
 //
 // us per scd_verify call on a B200, before (an exponential per id, four byte-wise passes over the cluster for the nucleus,
-// tickets for the commit, the race on one CTA per row) and now: 1 x 32 rows of 16384 ids, top-k 2000: 32.8, 26.6;
-// 8 x 32 with guidance: 107.8, 49.3; 64 rows of 64000 ids, top-p 0.8: 279, 78; 2 x 32 of 16384, Gumbel: 234, 39.
+// tickets for the commit, the race on one CTA per row) and now: 1 x 32 rows of 16384 ids, top-k 2000: 32.3, 24.3;
+// 8 x 32 with guidance: 108, 51; 64 rows of 64000 ids, top-p 0.8: 277, 83; 2 x 32 of 16384, Gumbel: 233, 36.6.
 //
 // Gumbel race (Algorithm 4): the winner is the smallest E_v / W_v of integers that take 40 squarings each. An fp32
 // estimate of every ratio first, the integers only for ids within RACE_SLACK of the smallest estimate. A row that
@@ -182,8 +182,14 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
     const int rank = blockIdx.x % C;                   // = rank in the cluster (cluster dims (C, 1, 1))
     const int k = blockIdx.x / C, b = blockIdx.y;
     pdl_trigger();
-    // (in a session this grid may have started early: up to pdl_wait() it reads only what earlier iterations left
-    // behind - the window counters, the draft ids, the drafts' stored weights)
+    auto zero_hist = [&]() {
+        for (int i = tid; i < 2 * 2 * NB / 4; i += CT) ((uint4 *)&xc.hist[0][0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
+    };
+    zero_hist();
+    // This grid may have started early. In a session it reads, up to the wait further down, only what earlier iterations left
+    // behind - the window counters, the draft ids, the drafts' stored weights. In a stand-alone call every input may come from
+    // the kernel in front.
+    if (!p.n_known) pdl_wait();
     const WindowState w = load_state(p, b);
     if (k >= w.Lw) { pdl_wait(); return; }             // (all CTAs of the cluster; no kernel ends before the one in front)
     const int L = p.L, V = p.V;
@@ -223,7 +229,7 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
             x[0] = t.x; x[1] = t.y; x[2] = t.z; x[3] = t.w;
         } else {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) x[i] = v + i >= hi ? 0.f : p.n_known ? __ldcg(src + v + i) : src[v + i];
+            for (int i = 0; i < 4; ++i) x[i] = v + i >= hi ? 0.f : __ldcg(src + v + i);
         }
     };
     auto has = [&](int v) { return v >= lo && v < hi; };
@@ -274,15 +280,11 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
     };
     auto all_cand = [&](int a) -> uint2 * { return (uint2 *)&xc.hist[a][0][0]; };
     static_assert(sizeof(uint2) * CAND_CAP <= sizeof(xc.hist[0]), "the candidates reuse the histograms");
-    auto zero_hist = [&]() {
-        for (int i = tid; i < 2 * 2 * NB / 4; i += CT) ((uint4 *)&xc.hist[0][0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
-    };
 
     const int X = p.draft_in[row];
     const bool x_in = X >= lo && X < hi;
     const float xq_raw = qr && x_in ? qr[X] : 0.f;     // raw logit, or stored integer weight (bit pattern), of the draft
     const unsigned long long Zq_stored = !fresh && !rawq ? p.stats[w.parity ^ 1][(size_t)b * L + qk].Z : 0ull;
-    zero_hist();
     if (tid < 2) { xc.cand_n[tid] = 0u; lc.sel[tid] = -1; lc.bound[tid] = -INFINITY; }
     __syncthreads();
     pdl_wait();                                        // the target logits come from the kernel in front
@@ -1092,9 +1094,11 @@ __global__ void __launch_bounds__(256) commit_kernel(const VerifyParams p)
 {
     __shared__ int redraft[256], entering_s[256], first_s;
     const int b = blockIdx.x, k = threadIdx.x, L = p.L;
+    if (!p.n_known) pdl_wait();                        // (the verify grid starts before its inputs are there, so does this one)
     const WindowState w = load_state(p, b);
     if (k == 0) first_s = w.Lw;
     pdl_wait();                                        // the rows come from the grid in front
+    pdl_trigger();                                     // (a caller's next call starts under the rest of this one)
     const size_t row = (size_t)b * L + k;
     const bool live = k < w.Lw;
     const int y = live ? __ldcg(&p.row_y[row]) : 0;
@@ -1152,7 +1156,7 @@ bool choose_cluster(const VerifyParams &p, int sm_count, int *C_out, int *ids_ou
 }
 
 template <class K, class... A>
-cudaError_t launch_ex(bool dependent, K kernel, dim3 grid, int threads, size_t smem, int C, cudaStream_t st, A... args)
+cudaError_t launch_ex(K kernel, dim3 grid, int threads, size_t smem, int C, cudaStream_t st, A... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -1167,10 +1171,8 @@ cudaError_t launch_ex(bool dependent, K kernel, dim3 grid, int threads, size_t s
         attr[n].val.clusterDim.y = 1;
         attr[n++].val.clusterDim.z = 1;
     }
-    if (dependent) {
-        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[n++].val.programmaticStreamSerializationAllowed = 1;
-    }
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
@@ -1204,18 +1206,19 @@ int launch_verify_rows(const VerifyParams &p, cudaStream_t stream)
     if (dev >= 0 && dev < DeviceOnce::kSlots) sms = sm_count[dev];
     int C = 1, ids = 1;
     SCD_REQUIRE(choose_cluster(p, sms, &C, &ids), SCD_ERR_SHAPE, "verify: rows of %d ids do not fit a cluster", p.allowed_hi - p.allowed_lo);
-    // (the stand-alone call takes its inputs from the caller's kernels: only a session's grid may start early)
-    const bool dep = p.n_known != nullptr;
+    // Always a programmatic launch: the kernel waits before it reads what the one in front may have written. Stand-alone
+    // calls one after the other otherwise paid a full launch each (1 x 32 rows of 16384 ids: 26.6 us a call, 24.3 so,
+    // 4 us less on the host included; Gumbel, 2 x 32: 39.5 and 36.6).
     const dim3 grid((unsigned)(p.L * C), (unsigned)p.B, 1);
-    if (ids <= 128) SCD_CUDA_TRY(launch_ex(dep, verify_rows_kernel<1, true>, grid, CT, (size_t)lists(128), C, stream, p, C, 1));
-    else if (ids <= 256) SCD_CUDA_TRY(launch_ex(dep, verify_rows_kernel<2, true>, grid, CT, (size_t)lists(256), C, stream, p, C, 1));
-    else SCD_CUDA_TRY(launch_ex(dep, verify_rows_kernel<2, false>, grid, CT, (size_t)lists(WCAP_LONG), C, stream, p, C, (ids + 255) / 256));
+    if (ids <= 128) SCD_CUDA_TRY(launch_ex(verify_rows_kernel<1, true>, grid, CT, (size_t)lists(128), C, stream, p, C, 1));
+    else if (ids <= 256) SCD_CUDA_TRY(launch_ex(verify_rows_kernel<2, true>, grid, CT, (size_t)lists(256), C, stream, p, C, 1));
+    else SCD_CUDA_TRY(launch_ex(verify_rows_kernel<2, false>, grid, CT, (size_t)lists(WCAP_LONG), C, stream, p, C, (ids + 255) / 256));
     return SCD_OK;
 }
 
 int launch_commit(const VerifyParams &p, cudaStream_t stream)
 {
-    SCD_CUDA_TRY(launch_ex(true, commit_kernel, dim3((unsigned)p.B, 1, 1), (p.L + 31) / 32 * 32, 0, 0, stream, p));
+    SCD_CUDA_TRY(launch_ex(commit_kernel, dim3((unsigned)p.B, 1, 1), (p.L + 31) / 32 * 32, 0, 0, stream, p));
     return SCD_OK;
 }
 

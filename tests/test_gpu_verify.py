@@ -223,3 +223,25 @@ def test_verify_bound_from_an_unlucky_sample(V, L, B, top_k, top_p):
     assert np.array_equal(next_drafts, want["next_drafts"])
     for b in range(B):
         assert np.array_equal(committed[b, :n_commit[b]], want["committed"][b, :n_commit[b]])
+
+
+@pytest.mark.parametrize("B,L,V,top_k", [(1, 32, 16384, 2000), (3, 8, 1001, 50)])
+def test_verify_reads_what_the_kernel_in_front_wrote(B, L, V, top_k):
+    """The call's kernels start before the caller's last kernel is done: inputs copied into the same buffers right in front
+    of every call give what each set gives by itself."""
+    cfg = scd.decode_config(mode=scd.SCD_MODE_SCD_MC, batch=B, window_L=L, top_k=top_k, seed=8, allowed_hi=V)
+    sets, want = [], []
+    for i in range(3):
+        p, q = synth.verify_logits(3 + i, 1, B, L, V, device="cuda")
+        sets.append((p, q, synth.draft_ids_from_logits(q, top_k, 5 + i), torch.arange(B, device="cuda", dtype=torch.int64) * 7 + 9 * i))
+        torch.cuda.synchronize()
+        want.append([t.clone() for t in scd.scd_verify(cfg, *sets[-1], 4)])
+        torch.cuda.synchronize()
+    into = [torch.empty_like(t) for t in sets[0]]
+    got = []
+    for n in range(30):
+        for a, b in zip(into, sets[n % 3]):
+            a.copy_(b)
+        got.append(scd.scd_verify(cfg, *into, 4))
+    for n in range(30):
+        assert all(torch.equal(a, b) for a, b in zip(got[n], want[n % 3]))
