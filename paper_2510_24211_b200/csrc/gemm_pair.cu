@@ -1,4 +1,5 @@
-// GEMM of a forward with more than 128 rows (prefill chunks, large batches): y[m, n] = sum_k x[m, k] * w[n, k],
+// GEMM of a forward with more than 128 rows (prefill chunks, large batches; up to 256 rows only where choose_shape in
+// gemm_tcgen05.cu finds it faster): y[m, n] = sum_k x[m, k] * w[n, k],
 // x in one or two bf16 planes, fp32 accumulation in tensor memory, output operations fused.
 //
 // Such a GEMM is bound by the tensor cores (two planes: 2 x 2 flop per weight and row), and next by the copies
@@ -20,6 +21,11 @@
 // and adds up its share of the columns in contributor order - the result does not depend on scheduling. A pair
 // that has work left never waits.
 // Every wait is bounded; on expiry the error word is raised, the roles run out and the outputs are not written.
+//
+// Measured on a B200 (before: 256 rows at a time through the weight-streaming kernel, or an earlier step of this one):
+// 2560 x 12288 x 3072, two planes: 247 us with one producer lane, 207 with one per operand;
+// 2560 x 9216 x 3072, one plane: 179, 111; 256 x 22016 x 4096 SwiGLU: 112 with parts loaded through registers, 65 by
+// bulk copies. 2560 tokens of prefill through 28 layers of 3072: 73 ms by passes of 128 rows, 32 ms.
 #include <algorithm>
 #include <cstring>
 

@@ -830,8 +830,7 @@ int w_map(GemmPlan *plan, const Segment &sg, int box_rows, CUtensorMap *out)
     return SCD_OK;
 }
 
-// Forwards of more than 128 rows go to the CTA-pair kernel, whatever the shape: there the tensor cores bound the
-// GEMM, and at 256 rows this file's kernel has a ring of two slots.
+// Forwards that the CTA-pair kernel takes (see choose_shape): there the tensor cores bound the GEMM.
 int run_gemm_pair(scd_session *s, const Segment *segs, int n_seg, int epi, const void *x, int K, int rows, void *out, int ldo,
                   const NormIn *nin, const NormOut *nout, int x_planes, int *parts_out, cudaStream_t st)
 {
