@@ -903,6 +903,7 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
 
     // Sum of `mass` over the row's entries, and the entry in which a running sum in id order first exceeds
     // (U * sum) >> 24. found(id) runs in one lane of the cluster; returns the sum. slot: of xc.u64, one per call.
+    // When it returns, other warps may still add up lc.red_a, lc.red_b and lc.peer: a barrier before these are written again.
     auto draw = [&](int slot, unsigned U, auto mass, auto found) -> u128 {
         Limbs s = {0ull, 0ull};
         for (int e0 = 0; e0 < n_e[0]; e0 += 32) s.add(mass(e0 + lane));
@@ -1064,6 +1065,7 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) fk = max(fk, __shfl_xor_sync(FULLM, fk, o));
         const float wbest = -warp_max(-best);
+        __syncthreads();                               // (an earlier user of these is done: the draw of a rejected row)
         if (lane == 0) { lc.red_f[0][warp] = wbest; lc.red_a[warp] = fk; }
         __syncthreads();
         if (warp == 0) {

@@ -245,3 +245,24 @@ def test_verify_reads_what_the_kernel_in_front_wrote(B, L, V, top_k):
         got.append(scd.scd_verify(cfg, *into, 4))
     for n in range(30):
         assert all(torch.equal(a, b) for a, b in zip(got[n], want[n % 3]))
+
+
+@pytest.mark.parametrize("V,top_k,top_p", [(300, 4, 0.0), (1000, 20, 0.0), (4000, 30, 0.0), (9000, 0, 0.3)])
+def test_verify_gumbel_after_many_rejections(V, top_k, top_p):
+    """A rejected row draws from its residual and then enters the Gumbel race, both through the same per-warp sums. Here
+    every row rejects (drafts without mass), the lists are short, and the rows that enter the window sit at forced
+    end-of-row positions, so that the race follows the draw at once; the same call again and again gives the oracle's answer."""
+    B, L, seed, eol = 4, 15, 61, 299                   # L odd, row_period 2: ordinary rows at even positions enter odd ones
+    p, q = synth.verify_logits(seed, 0, B, L, V, device="cuda")
+    drafts = torch.argmin(p[0][..., :290] + q[..., :290], dim=-1).to(torch.int32)
+    positions = torch.arange(B, device="cuda", dtype=torch.int64) * 10 + 100
+    cfg = scd.decode_config(mode=scd.SCD_MODE_SCD_GS, batch=B, window_L=L, top_k=top_k, top_p=top_p, seed=seed, allowed_hi=V,
+                            row_period=2, eol_id=eol)
+    for it in range(4):
+        want = oracle_verify("gs", p.cpu().numpy(), q.cpu().numpy(), drafts.cpu().numpy(), positions.cpu().numpy(), it, seed,
+                             top_k=top_k, top_p=top_p, row_period=2, eol_id=eol)
+        assert (want["flags"][:, ::2] == 0).all()      # (the forced positions have the one id, which is not the draft)
+        for n_commit, committed, next_drafts, flags in [scd.scd_verify(cfg, p, q, drafts, positions, it) for _ in range(50)]:
+            assert np.array_equal(n_commit.cpu().numpy(), want["n_commit"]) and np.array_equal(flags.cpu().numpy(), want["flags"])
+            assert np.array_equal(next_drafts.cpu().numpy(), want["next_drafts"])
+            assert np.array_equal(committed.cpu().numpy()[:, 0], want["committed"][:, 0])
