@@ -114,6 +114,10 @@ __device__ __forceinline__ uint4 ld_peer_u32x4(const void *local, uint32_t rank)
     return v;
 }
 
+// order-preserving key of a logit for the selection of the threshold. -0 takes the key of +0: the ids at the threshold are
+// those that compare equal to it as floats (with a key of its own -0 lost its weight here and kept it in the accept test)
+__device__ __forceinline__ unsigned logit_key(float x) { return float_key(__fadd_rn(x, 0.0f)); }
+
 // step of the live range an id falls into: 0 at the maximum, NB - 1 at m - 22; -1: not live
 __device__ __forceinline__ int live_step(float x, float m)
 {
@@ -678,7 +682,7 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
                 if (cand) {
                     const unsigned at = atomicAdd(&xc.cand_n[a], 1u);
                     if (at < CAND_CAP) {
-                        xc.cand[a][at] = make_uint2(float_key(x), wv);
+                        xc.cand[a][at] = make_uint2(logit_key(x), wv);
                         lc.cand_at[a][at] = (unsigned short)(whole[a] ? 0xFFFF : warp * WCAP + e);
                     }
                 }
@@ -774,7 +778,7 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
                     bool in;
                     const float x = entry_x(A_, e0 + lane, in);
                     if (!in || live_step(x, m[a]) != sb[a]) continue;
-                    const unsigned key = float_key(x);
+                    const unsigned key = logit_key(x);
                     if ((key & mask) == prefix) atomicAdd(&xc.hist[a][0][(key >> shift) & 255u], 1u);
                 }
                 csync();

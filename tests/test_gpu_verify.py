@@ -141,6 +141,36 @@ def test_verify_ties_and_topk_edges():
         _run_case("scd", 1, 6, 600, it, seed=14, top_k=5000)       # k > n
 
 
+@pytest.mark.parametrize("B,L,V,top_k,top_p,lam", [
+    (2, 8, 300, 20, 0.0, 0.0), (3, 5, 2634, 20, 0.0, 2.0), (1, 12, 1643, 1, 0.0, 0.0), (2, 8, 800, 150, 0.5, 0.0),
+    (2, 80, 9000, 900, 0.0, 0.0),                                        # more candidates than are selected by counting
+    (1, 3, 131073, 500, 0.0, 0.0),
+])
+def test_verify_threshold_at_signed_zeros(B, L, V, top_k, top_p, lam):
+    """+0 and -0 are one logit: both are at the threshold, or neither is. Half of the ids at -1, the rest at zero, with the
+    minus sign on most of them in the target rows and on few in the draft rows."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    S = 2 if lam else 1
+    r = torch.rand(B, L, V, generator=g, device="cuda")
+    at_zero = torch.rand(B, L, V, generator=g, device="cuda") < 0.5
+    def row(minus):
+        return torch.where(at_zero, torch.where(r < minus, -0.0, 0.0), -1.0)
+    q = row(0.2)
+    for it, p0 in enumerate((row(0.8), row(0.0), row(1.0))):
+        p = p0[None].repeat(S, 1, 1, 1).contiguous()
+        drafts = torch.argmax((q + r * at_zero > -1.0).to(torch.int32), dim=-1).to(torch.int32)
+        positions = torch.arange(B, device="cuda", dtype=torch.int64) * 300 + 9
+        cfg = scd.decode_config(mode=scd.SCD_MODE_SCD_MC, batch=B, window_L=L, top_k=top_k, top_p=top_p, cfg_lambda=lam, seed=8,
+                                allowed_hi=V)
+        n_commit, committed, next_drafts, flags = [t.cpu().numpy() for t in scd.scd_verify(cfg, p, q, drafts, positions, it)]
+        want = oracle_verify("scd", p.cpu().numpy(), q.cpu().numpy(), drafts.cpu().numpy(), positions.cpu().numpy(), it, 8,
+                             top_k=top_k, top_p=top_p, cfg_lambda=lam)
+        assert (want["flags"] == 1).all()              # the same distribution twice
+        assert np.array_equal(n_commit, want["n_commit"]) and np.array_equal(flags, want["flags"])
+        assert np.array_equal(next_drafts, want["next_drafts"]) and np.array_equal(committed, want["committed"])
+
+
 def test_verify_large_vocab_and_max_window():
     _run_case("scd", 1, 64, 64000, 0, seed=15, top_k=1000)
     _run_case("scd", 1, 256, 512, 1, seed=16, top_k=20)
