@@ -172,14 +172,16 @@ __device__ __noinline__ float post_logit(const float *c, const float *u, int v, 
 }
 
 // A warp's ids come in groups of NS x 128: lane l holds ids 4 l .. 4 l + 3 of each 128 (16-byte loads where rows are
-// aligned). REG: one group, which stays in registers. range: ids of a warp, a multiple of 32. (As a multiple of a group it
-// left half of the warps without ids where a warp's share is just above one group, and the others with more than a list
-// takes: 8 x 32 rows of 4371 ids, top-k 4000, 82.9 us, 42.4 so.)
+// aligned). REG: one group, which stays in registers. Else long_range: ids of a warp, a multiple of 32. (As a multiple of a
+// group it left half of the warps without ids where a warp's share is just above one group, and the others with more than
+// a list takes: 8 x 32 rows of 4371 ids, top-k 4000, 82.9 us, 42.4 so. In registers there is no such limit, and shares
+// that are no whole groups are 5 % slower: 6 rows of 24774 ids 26.1 and 27.3 us.)
 template <int NS, bool REG>
-__global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p, int C, int range)
+__global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p, int C, int long_range)
 {
     constexpr int N = 4 * NS;                          // ids per lane and group
     constexpr int WCAP = REG ? 32 * N : WCAP_LONG;     // entries of a warp's list
+    const int range = REG ? 32 * N : long_range;       // ids of a warp
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ __align__(16) Xchg xc;
     __shared__ Local lc;
@@ -1252,10 +1254,9 @@ int launch_verify_rows(const VerifyParams &p, cudaStream_t stream)
     // calls one after the other otherwise paid a full launch each (1 x 32 rows of 16384 ids: 26.6 us a call, 24.3 so,
     // 4 us less on the host included; Gumbel, 2 x 32: 39.5 and 36.6).
     const dim3 grid((unsigned)(p.L * C), (unsigned)p.B, 1);
-    const int range = (ids + 31) / 32 * 32;
-    if (ids <= 128) SCD_CUDA_TRY(launch_ex(verify_rows_kernel<1, true>, grid, CT, (size_t)lists(128), C, stream, p, C, range));
-    else if (ids <= 256) SCD_CUDA_TRY(launch_ex(verify_rows_kernel<2, true>, grid, CT, (size_t)lists(256), C, stream, p, C, range));
-    else SCD_CUDA_TRY(launch_ex(verify_rows_kernel<2, false>, grid, CT, (size_t)lists(WCAP_LONG), C, stream, p, C, range));
+    if (ids <= 128) SCD_CUDA_TRY(launch_ex(verify_rows_kernel<1, true>, grid, CT, (size_t)lists(128), C, stream, p, C, 0));
+    else if (ids <= 256) SCD_CUDA_TRY(launch_ex(verify_rows_kernel<2, true>, grid, CT, (size_t)lists(256), C, stream, p, C, 0));
+    else SCD_CUDA_TRY(launch_ex(verify_rows_kernel<2, false>, grid, CT, (size_t)lists(WCAP_LONG), C, stream, p, C, (ids + 31) / 32 * 32));
     return SCD_OK;
 }
 
