@@ -16,7 +16,7 @@
 //                                                                                                     -> exchange
 //      Nucleus without top-k: maximum and weights take a sweep each; the bound is one on W, from a sample as well, the
 //      mass below it is only summed. The step (logarithmic, of W) in which the mass from the top reaches top_p of the
-//      row is divided again, NB ways, until it is one value of W.
+//      row is divided again, NB ways, until it is one value of W or holds few ids, which are selected by counting.
 //   5. accept test in 128-bit integers; on rejection the residual masses max(0, Wp_v Zq - Wq_v Zp)   -> exchange
 //      and the inverse-CDF walk in the one warp that holds the target
 // Rows of up to 256 ids per warp stay in registers (REG): there the histogram counts every id and the lists come after
@@ -52,10 +52,12 @@ constexpr int NB = 1024;           // steps of a histogram
 constexpr int MAXC = 8;
 constexpr int MAXG = 4;            // groups of 256 ids per warp: a CTA takes up to 16384 ids
 constexpr int CAND_CAP = 1024;     // candidates of a row that are selected by counting
+constexpr int NUC_CAP = 256;       // ... and weights of the nucleus' last step
 constexpr int WCAP_LONG = 384;     // list entries of a warp of up to 1024 ids (two CTAs share an SM's memory)
 constexpr float LIVE_SPAN = 22.0f; // scd_exp(x) = 0 below -22
 constexpr unsigned W_TAIL = 1u << 14;   // nucleus: lighter ids are only summed at first
 constexpr float LIST_SHARE = 0.28f;     // ... and so are those beyond this share of the ids (a list takes 384 of 1024)
+constexpr float TAIL_WIDE = 0.6f, TAIL_TIGHT = 0.85f, LIST_FILL = 0.8f, FAR = 1.6f;   // (where the lists are built)
 constexpr float RACE_SLACK = 2e-4f;
 constexpr unsigned FULLM = 0xffffffffu;
 
@@ -82,7 +84,7 @@ struct Local {
     unsigned long long peer[4][MAXC];
     unsigned peer_n[2][MAXC];
     int sel[2];
-    float bound[2];
+    float bound[2], cuts[2][5];
     unsigned sel_k[2], tau_key[2];
     unsigned long long above[2], kept[2], total[2];
 };
@@ -169,6 +171,45 @@ __device__ __noinline__ float post_logit(const float *c, const float *u, int v, 
     float x = __ldcg(c + v);
     if (u) x = __fsub_rn(__fmul_rn(one_plus_lam, x), __fmul_rn(lam, __ldcg(u + v)));
     return T != 1.0f ? __fdiv_rn(x, T) : x;
+}
+
+// Nucleus: the candidates of every CTA (up to NUC_CAP weights of each row's last step) to this one, and among them the largest
+// weight whose ids, with the mass above the step, hold top_p of the mass Z: into lc.tau_key, the mass into lc.kept. Half the
+// threads per row, a candidate each. (Off the main path: inlined it cost every call registers)
+__device__ __noinline__ void nucleus_among(Xchg &xc, Local &lc, int C, unsigned p24, unsigned long long Z0, unsigned long long Z1,
+                                           unsigned long long above0, unsigned long long above1)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, a = tid >> 8;
+    const unsigned t = tid & 255;
+    if (warp < 2 && lane < MAXC) lc.peer_n[warp][lane] = lane < C ? ld_peer_u32(&xc.cand_n[warp], (uint32_t)lane) : 0u;
+    __syncthreads();
+    unsigned n = 0;
+#pragma unroll
+    for (int r = 0; r < MAXC; ++r) n += lc.peer_n[a][r];
+    unsigned *const all = &xc.hist[a][0][0];           // (the tables are done with)
+    if (t < n) {
+        unsigned off = 0;
+        int rr = 0;
+#pragma unroll
+        for (int r = 0; r < MAXC - 1; ++r) {
+            const unsigned end = off + lc.peer_n[a][r];
+            if (rr == r && t >= end) { off = end; rr = r + 1; }
+        }
+        all[t] = ld_peer_u32(&xc.cand[a][t - off].x, (uint32_t)rr);
+    }
+    __syncthreads();
+    if (t < n) {
+        const unsigned wv = all[t];
+        unsigned long long gt = a ? above1 : above0, ge = gt;
+        for (unsigned i = 0; i < n; ++i) {
+            const unsigned o = all[i];
+            gt += o > wv ? o : 0u;
+            ge += o >= wv ? o : 0u;
+        }
+        const u128 need = (u128)p24 * (a ? Z1 : Z0);
+        if (((u128)ge << 24) >= need && ((u128)gt << 24) < need) { lc.tau_key[a] = wv; lc.kept[a] = ge; }   // (equal weights write the same)
+    }
+    __syncthreads();
 }
 
 // A warp's ids come in groups of NS x 128: lane l holds ids 4 l .. 4 l + 3 of each 128 (16-byte loads where rows are
@@ -291,7 +332,7 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
     const bool x_in = X >= lo && X < hi;
     const float xq_raw = qr && x_in ? qr[X] : 0.f;     // raw logit, or stored integer weight (bit pattern), of the draft
     const unsigned long long Zq_stored = !fresh && !rawq ? p.stats[w.parity ^ 1][(size_t)b * L + qk].Z : 0ull;
-    if (tid < 2) { xc.cand_n[tid] = 0u; lc.sel[tid] = -1; lc.bound[tid] = -INFINITY; }
+    if (tid < 2) { xc.cand_n[tid] = 0u; lc.sel[tid] = -1; lc.bound[tid] = -INFINITY; lc.above[tid] = lc.kept[tid] = 0ull; }
     __syncthreads();
     pdl_wait();                                        // the target logits come from the kernel in front
     const float xX = x_in ? load_p(X) : 0.f;           // the draft's own logit: every CTA weighs X itself
@@ -336,33 +377,36 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
             if (ib) { body(0, pb); if (rawq) body(1, qb); }
         }
     };
-    // After a sample's histogram (2 NB bins per row in the tables of the masses, the smallest sample in bin 0): the highest
-    // bin from which on at least `want(samples)` of them lie, if there is one. Thread t of row a looks at 8 bins.
-    auto sample_bin = [&](auto want, auto found) {
+    // After a sample's histogram (2 NB bins per row in the tables of the masses, the smallest sample in bin 0): visits the
+    // bins that hold something, with want(sum of value(bin, count) over all) and the sums over the bins above and from this
+    // one on.
+    // Thread t of row a looks at 8 bins. The tables are cleared.
+    auto sample_bins = [&](auto value, auto want, auto visit) {
+        using T = decltype(value(0, 0u));
         const int a = tid >> 8, t = tid & 255, wi = warp & 7;
-        unsigned cnt[8], mine = 0, inc = 0;
+        T val[8], mine = 0, inc = 0;
         const unsigned *h = &xc.hist[a][0][0] + 2 * NB - 8 - 8 * t;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) { cnt[j] = h[j]; mine += cnt[j]; }
+        for (int j = 0; j < 8; ++j) { val[j] = value(2 * NB - 8 - 8 * t + j, h[j]); mine += val[j]; }
         inc = mine;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const unsigned v = __shfl_up_sync(FULLM, inc, o);
+            const T v = __shfl_up_sync(FULLM, inc, o);
             if (lane >= o) inc += v;
         }
         if (lane == 31) lc.scan[a][wi] = inc;
         __syncthreads();
-        unsigned acc = inc - mine, all = 0;
+        T acc = inc - mine, all = 0;
 #pragma unroll
         for (int i = 0; i < NWARP / 2; ++i) {
-            if (i < wi) acc += (unsigned)lc.scan[a][i];
-            all += (unsigned)lc.scan[a][i];
+            if (i < wi) acc += (T)lc.scan[a][i];
+            all += (T)lc.scan[a][i];
         }
-        const unsigned need = want(all);
+        const auto need = want(all);
 #pragma unroll
         for (int j = 7; j >= 0; --j) {
-            if (acc < need && need <= acc + cnt[j]) found(a, 2 * NB - 8 - 8 * t + j);
-            acc += cnt[j];
+            if (val[j] != 0) visit(a, 2 * NB - 8 - 8 * t + j, need, acc, acc + val[j]);
+            acc += val[j];
         }
         __syncthreads();
         zero_hist();
@@ -497,11 +541,13 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
             // (a share of top_k / n of the samples lies above the k-th largest, give or take; four deviations more are
             // listed. Without that many samples the list takes everything.)
             const float share = (float)p.top_k / (float)(hi - lo);
-            sample_bin([&](unsigned all) { const float e = share * (float)all; return (unsigned)(e + 4.0f * sqrtf(e)) + 4u; },
-                       [&](int a, int bin) {
-                           const float t = key_float((unsigned)bin << 21);
-                           lc.bound[a] = t > -INFINITY ? t : -INFINITY;      // (the bin of -inf begins among the NaNs)
-                       });
+            sample_bins([](int, unsigned n) { return n; },
+                        [&](unsigned all) { const float e = share * (float)all; return (unsigned)(e + 4.0f * sqrtf(e)) + 4u; },
+                        [&](int a, int bin, unsigned need, unsigned above, unsigned sum) {
+                if (above >= need || sum < need) return;
+                const float t = key_float((unsigned)bin << 21);
+                lc.bound[a] = t > -INFINITY ? t : -INFINITY;                 // (the bin of -inf begins among the NaNs)
+            });
         }
         for (bool again = false;; again = true) {
             const float bound[2] = {again ? -INFINITY : lc.bound[0], again ? -INFINITY : lc.bound[1]};
@@ -598,10 +644,34 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
             const unsigned wv = weight_of(x, a ? m[1] : m[0], -INFINITY);
             atomicAdd(&xc.hist[a][0][0] + (wv ? NB - 1 - weight_step(wv) : 0), 1u);
         });
-        if (tid < 2) lc.bound[tid] = (float)W_TAIL;
+        // The bound lists the heaviest LIST_SHARE of the ids, and in flat rows more: until the sample's mass reaches top_p and
+        // TAIL_WIDE of the rest, so that the nucleus ends inside the lists (without it such rows had them built twice: 175
+        // rows of 12991 ids, guidance, top-p 0.95, 226 us, 65 so), but not more than fit a list (LIST_FILL: some warps have
+        // more ids above the bound than others). Only where the nucleus itself is far from fitting (top_p and TAIL_TIGHT of the rest take
+        // FAR times as much) the lists are given up at once (128 rows of 30000 ids, top-p 0.99: 138 us after a try, 109 so).
+        if (tid < 10) (&lc.cuts[0][0])[tid] = (float)W_TAIL;
         __syncthreads();
-        sample_bin([&](unsigned all) { return (unsigned)(LIST_SHARE * (float)all) + 1u; },
-                   [&](int a, int bin) { lc.bound[a] = fmaxf((float)W_TAIL, bin > 0 ? (float)weight_step_lo(NB - 1 - bin) : 0.f); });
+        auto cut_at = [&](int bin) { return fmaxf((float)W_TAIL, bin > 0 ? (float)weight_step_lo(NB - 1 - bin) : 0.f); };
+        const float rest = 1.0f - (float)p.top_p24 * 0x1p-24f, fit = LIST_FILL * (float)WCAP / (float)range;
+        // (number and mass of a bin's ids in one word: up to 1024 of them, weights below 2^31)
+        sample_bins([](int bin, unsigned n) { return ((unsigned long long)n << 48) + (bin > 0 ? (unsigned long long)n * weight_step_lo(NB - 1 - bin) : 0ull); },
+                    [](unsigned long long all) { return all; },
+                    [&](int a, int bin, unsigned long long all, unsigned long long above, unsigned long long sum) {
+            const unsigned long long mass = 0xFFFFFFFFFFFFull;
+            const float n = (float)(all >> 48), m_ = (float)(all & mass);
+            auto ids = [&](float share) { const unsigned need = (unsigned)(share * n) + 1u; return (unsigned)(above >> 48) < need && need <= (unsigned)(sum >> 48); };
+            auto tail = [&](float share) { const unsigned long long need = (all & mass) - (unsigned long long)(share * rest * m_); return (above & mass) < need && need <= (sum & mass); };
+            if (ids(LIST_SHARE)) lc.cuts[a][0] = cut_at(bin);
+            if (ids(fit)) lc.cuts[a][1] = cut_at(bin + 1);
+            if (ids(FAR * fit)) lc.cuts[a][2] = cut_at(bin + 1);
+            if (tail(TAIL_WIDE)) lc.cuts[a][3] = cut_at(bin);
+            if (tail(TAIL_TIGHT)) lc.cuts[a][4] = cut_at(bin);
+        });
+        if (tid < 2) {
+            const float *c_ = lc.cuts[tid];
+            lc.bound[tid] = c_[4] < c_[2] ? fminf(c_[0], c_[4]) : fmaxf(fminf(c_[0], c_[3]), c_[1]);
+        }
+        __syncthreads();
         for (bool again = false;; again = true) {
             // (a bound is the smallest weight of a step: exact in fp32)
             const unsigned cut[2] = {again ? 1u : (unsigned)lc.bound[0], again ? 1u : (unsigned)lc.bound[1]};
@@ -863,6 +933,7 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         if (use_topk) {                                // (the histogram tables hold the counts of top-k)
             csync();
             zero_hist();
+            if (tid < 2) xc.cand_n[tid] = 0u;
             __syncthreads();
             level([&](int, unsigned wv) { return weight_step(wv); });
         } else {
@@ -871,25 +942,55 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         }
         EACH_ROW([&](auto A_) {
             constexpr int a = decltype(A_)::value;
+            if (Zall[a] == 0ull) return;               // no id has a weight: no step, nothing to divide
             range_lo[a] = weight_step_lo(sb[a]);
             bits[a] = max(0, ((NB - 1 - sb[a]) >> 5) - 5);           // a step is 2^(e - 5) weights wide
         });
+        auto in_range = [&](int a, unsigned wv) { return wv >= range_lo[a] && ((wv - range_lo[a]) >> bits[a]) == 0u; };
         while (bits[0] > 0 || (rawq && bits[1] > 0)) {
-            const int sh[2] = {max(0, bits[0] - 10), max(0, bits[1] - 10)};
-            level([&](int a, unsigned wv) -> int {
-                const unsigned d = (wv - range_lo[a]) >> sh[a];
-                return wv >= range_lo[a] && ((wv - range_lo[a]) >> bits[a]) == 0u ? NB - 1 - (int)d : -1;
-            });
+            // the range's mass over its smallest weight bounds the number of its ids
+            bool few = true;
             EACH_ROW([&](auto A_) {
                 constexpr int a = decltype(A_)::value;
-                range_lo[a] += (unsigned)(NB - 1 - sb[a]) << sh[a];
-                bits[a] = sh[a];
+                if (bits[a] > 0 && lc.kept[a] - lc.above[a] > (unsigned long long)NUC_CAP * range_lo[a]) few = false;
             });
+            if (!few) {
+                const int sh[2] = {max(0, bits[0] - 10), max(0, bits[1] - 10)};
+                level([&](int a, unsigned wv) -> int {
+                    const unsigned d = (wv - range_lo[a]) >> sh[a];
+                    return in_range(a, wv) ? NB - 1 - (int)d : -1;
+                });
+                EACH_ROW([&](auto A_) {
+                    constexpr int a = decltype(A_)::value;
+                    range_lo[a] += (unsigned)(NB - 1 - sb[a]) << sh[a];
+                    bits[a] = sh[a];
+                });
+                continue;
+            }
+            // few: every CTA takes them all and selects among them by counting, one exchange for what takes up to three
+            // divisions of two each (16 rows of 21458 ids, top-k 1000 and top-p 0.8: 84 us, 48 so)
+            EACH_ROW([&](auto A_) {
+                constexpr int a = decltype(A_)::value;
+                if (bits[a] == 0) return;
+                for (int e = lane; e < n_e[a]; e += 32) {
+                    const unsigned wv = entry_w(A_, e);
+                    if (wv == 0u || !in_range(a, wv)) continue;
+                    const unsigned at = atomicAdd(&xc.cand_n[a], 1u);
+                    if (at < CAND_CAP) xc.cand[a][at].x = wv;
+                }
+            });
+            csync();                                                                  // ---- exchange: candidates
+            nucleus_among(xc, lc, C, (unsigned)p.top_p24, Zall[0], Zall[1], above[0], above[1]);
+            EACH_ROW([&](auto A_) {
+                constexpr int a = decltype(A_)::value;
+                if (bits[a] > 0) range_lo[a] = lc.tau_key[a];
+            });
+            break;
         }
         EACH_ROW([&](auto A_) {
             constexpr int a = decltype(A_)::value;
             theta[a] = range_lo[a];
-            Zall[a] = lc.kept[a];
+            if (Zall[a] != 0ull) Zall[a] = lc.kept[a];
         });
     }
     const unsigned long long Zp = Zall[0];

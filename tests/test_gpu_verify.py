@@ -231,6 +231,47 @@ def test_verify_rows_at_the_edges_of_the_dispatch(mode, B, L, V, kw):
     _run_case(mode, B, L, V, iteration=2, seed=21, **kw)
 
 
+@pytest.mark.parametrize("n", [1, 255, 256, 257, 1000])
+@pytest.mark.parametrize("L,V,top_k", [(3, 3000, 0), (3, 3000, 2500), (80, 3000, 0), (80, 9000, 0), (3, 20000, 4000)])
+def test_verify_nucleus_that_ends_among_close_weights(L, V, top_k, n):
+    """The nucleus ends in a run of n ids whose weights lie within 1 % of each other (one step of the search), distinct or in
+    pairs: up to 256 are selected by counting, more are divided again."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    def row():
+        x = torch.rand(2, L, V, generator=g, device="cuda") * 4.0 - 12.0
+        at = torch.rand(2, L, V, generator=g, device="cuda").argsort(dim=-1)
+        x.scatter_(-1, at[..., :n + 20], torch.cat([torch.linspace(-3.0, -2.99, n, device="cuda"), torch.linspace(-1.0, 0.0, 20, device="cuda")]).expand(2, L, -1).contiguous())
+        return x
+    p, q = row()[None].contiguous(), row()
+    p[0, 1, :, 1::2] = p[0, 1, :, 0::2]                # sequence 1: weights in pairs
+    drafts = torch.argmax(q, dim=-1).to(torch.int32)
+    positions = torch.arange(2, device="cuda", dtype=torch.int64) * 300 + 9
+    for mode, top_p in (("scd", 0.5 if n < 200 else 0.75), ("sjd", 0.9)):
+        cfg = scd.decode_config(mode=MODES[mode], batch=2, window_L=L, top_k=top_k, top_p=top_p, seed=8, allowed_hi=V)
+        got = [t.cpu().numpy() for t in scd.scd_verify(cfg, p, q, drafts, positions, 4)]
+        want = oracle_verify(mode, p.cpu().numpy(), q.cpu().numpy(), drafts.cpu().numpy(), positions.cpu().numpy(), 4, 8, top_k=top_k, top_p=top_p)
+        assert np.array_equal(got[0], want["n_commit"]) and np.array_equal(got[3], want["flags"])
+        assert np.array_equal(got[2], want["next_drafts"]) and np.array_equal(got[1], want["committed"])
+
+
+@pytest.mark.parametrize("B,L,V", [(1, 5, 2303), (1, 3, 20000), (2, 80, 9000), (4, 20, 40)])
+@pytest.mark.parametrize("top_k,top_p", [(0, 0.8), (30, 0.8), (30, 0.0), (0, 0.0)])
+def test_verify_rows_without_mass(B, L, V, top_k, top_p):
+    """Rows whose logits are all -inf, in the target, in the draft, or in both, between ordinary ones: nothing is drawn from
+    them and nothing depends on what the nucleus leaves undefined there."""
+    p, q = synth.verify_logits(9, 1, B, L, V, device="cuda")
+    p[0, :, 1::3] = float("-inf")
+    q[:, 1::2] = float("-inf")
+    drafts = torch.argmax(torch.where(torch.isinf(q), p[0], q), dim=-1).to(torch.int32)
+    positions = torch.arange(B, device="cuda", dtype=torch.int64) * 300 + 9
+    cfg = scd.decode_config(mode=scd.SCD_MODE_SCD_MC, batch=B, window_L=L, top_k=top_k, top_p=top_p, seed=8, allowed_hi=V)
+    got = [t.cpu().numpy() for t in scd.scd_verify(cfg, p, q, drafts, positions, 4)]
+    want = oracle_verify("scd", p.cpu().numpy(), q.cpu().numpy(), drafts.cpu().numpy(), positions.cpu().numpy(), 4, 8, top_k=top_k, top_p=top_p)
+    assert np.array_equal(got[0], want["n_commit"]) and np.array_equal(got[3], want["flags"])
+    assert np.array_equal(got[2], want["next_drafts"]) and np.array_equal(got[1], want["committed"])
+
+
 @pytest.mark.parametrize("V,L,B,top_k,top_p", [(9000, 80, 2, 700, 0.0), (9000, 80, 2, 0, 0.8), (9001, 80, 2, 300, 0.0), (4000, 6, 1, 300, 0.0)])
 def test_verify_bound_from_an_unlucky_sample(V, L, B, top_k, top_p):
     """The bound that the lists start from is estimated from ids at fixed places of each warp's range: here exactly those
