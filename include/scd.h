@@ -138,7 +138,10 @@ int scd_free_model(scd_model_t *model);
  * and iteration counters - all resident on the device) and scratch activations for one decode
  * batch. Allocates device memory (cudaMalloc); free with scd_session_free. bf16 models: a forward
  * carries S*B*L window rows in one pass over the weights; at most 1024 rows are accepted
- * (SCD_ERR_CAPACITY beyond). */
+ * (SCD_ERR_CAPACITY beyond). The activation buffers are for the window (or 128 to 256 rows, whichever is more); a
+ * prompt that long is fed in passes of up to 2560 rows, and the first one brings the buffers for them: per row
+ * 8 (d_model + (n_heads + n_kv_heads) head_dim) + 4 d_ffn bytes and a little, and 39 MB once. They stay until
+ * the session is freed, and so do the smaller ones. */
 int scd_session_create(scd_model_t *model, const scd_decode_config_t *cfg, scd_session_t **out);
 int scd_session_free(scd_session_t *session);
 
@@ -147,7 +150,9 @@ int scd_session_free(scd_session_t *session);
  * that the first iteration feeds. Afterwards n = P, kv_len = P-1, t = 0 and the window holds
  * L fresh rows (draft distribution uniform over the allowed ids, draft X ~ it: the
  * initialisation of Algorithm 6). n_total = P + n_new is the final sequence length (window rows beyond it stay
- * inert). Errors: SCD_ERR_CAPACITY if P + n_new > max_seq. Synchronises the stream. */
+ * inert). A prompt longer than any before may allocate device memory (see scd_session_create); without
+ * room for it the prompt is fed in narrower passes. Errors: SCD_ERR_CAPACITY if P + n_new > max_seq.
+ * Synchronises the stream. */
 int scd_prefill(scd_session_t *session, const int32_t *prompt_ids, int32_t P, int32_t n_new,
                 void *stream);
 

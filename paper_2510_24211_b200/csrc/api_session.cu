@@ -146,11 +146,59 @@ int launch_step(scd_session *s, cudaStream_t st)
     return SCD_OK;
 }
 
+// Activation buffers for `rows` rows of one forward, in place of the present ones. Nothing changes if there is no
+// memory for them.
+int set_rows(scd_session *s, int rows)
+{
+    const scd_model_config_t &c = s->model->cfg;
+    const size_t es = elem_size(c.dtype), n = (size_t)rows;
+    const size_t d = c.d_model, dq = c.n_heads * c.head_dim, dkv = c.n_kv_heads * c.head_dim, F = c.d_ffn;
+    // bf16 sessions: GEMM inputs (xn, att, act) in two bf16 planes [2][rows][K], projections (qkv) in fp32
+    const size_t wide = c.dtype == SCD_BF16 ? 2 : 1;
+    const size_t bytes[6] = {n * d * sizeof(float), wide * n * d * es, wide * n * (dq + 2 * dkv) * es, wide * n * dq * es, wide * n * F * es,
+                             (size_t)s->ss_parts_cap * n * sizeof(float)};
+    void **const slot[6] = {(void **)&s->h, &s->xn, &s->qkv, &s->att, &s->act, (void **)&s->ss};
+    constexpr int most_retired = (int)(sizeof(s->retired) / sizeof(s->retired[0]));
+    SCD_REQUIRE(!s->h || s->n_retired + 6 <= most_retired, SCD_ERR_CAPACITY, "activation buffers have grown %d times", s->n_retired / 6);
+    void *fresh[6] = {};
+    for (int i = 0; i < 6; ++i) {
+        const cudaError_t e = cudaMalloc(&fresh[i], std::max<size_t>(bytes[i], 1));
+        if (e == cudaSuccess) continue;
+        for (int j = 0; j < i; ++j) cudaFree(fresh[j]);
+        cudaGetLastError();                              // (an allocation that failed leaves the context as it was)
+        return cuda_fail(e, "cudaMalloc of the activation buffers");
+    }
+    for (int i = 0; i < 6; ++i) {
+        if (*slot[i]) s->retired[s->n_retired++] = *slot[i];
+        *slot[i] = fresh[i];
+    }
+    s->rows_cap = rows;
+    gemm_session_rows_changed(s);
+    drop_step_graph(s);
+    return SCD_OK;
+}
+
+// Rows per stream-sequence of a pass over the first n tokens of the prompts. Long prompts go in few wide passes, the
+// buffers for them at least doubling each time; if there is no memory for that, in passes of what every session holds.
+int prefill_pass(scd_session *s, int n)
+{
+    if (n < 1) return 1;
+    const int passes = (n + s->prefill_chunk - 1) / s->prefill_chunk;
+    const int len = std::min(n, std::min(s->prefill_chunk, ((n + passes - 1) / passes + 127) / 128 * 128));
+    const int rows = s->Q * len;
+    const bool wide = s->model->cfg.dtype == SCD_BF16 && len > s->chunk;
+    if (!wide) return len;
+    if (gemm_pair_scratch(s) != SCD_OK) return s->chunk;
+    if (rows > s->rows_cap && set_rows(s, std::min(s->Q * s->prefill_chunk, std::max(rows, 2 * s->rows_cap))) != SCD_OK) return s->chunk;
+    return len;
+}
+
 void free_session_memory(scd_session *s)
 {
     if (s->step_graph) cudaGraphExecDestroy(s->step_graph);
+    for (int i = 0; i < s->n_retired; ++i) cudaFree(s->retired[i]);
     void *ptrs[] = {s->kv_pool, s->page_table, s->n_known, s->n_total, s->shift, s->prev_lw, s->drafts,
-                    s->n_commit, s->tokens, s->tokens_u, s->row_y, s->row_y_indep, s->ids_buf, s->iter,
+                    s->n_commit, s->tokens, s->tokens_u, s->row_y, s->row_y_indep, s->iter,
                     s->accept_flags, s->xbuf[0], s->xbuf[1], s->stats[0], s->stats[1],
                     s->dev_stats, s->finished, s->h, s->ss, s->xn, s->qkv, s->att, s->act, s->logits, s->gemm_ws, s->gemm_scratch, s->stamps};
     for (void *p : ptrs) if (p) cudaFree(p);
@@ -264,14 +312,14 @@ int scd_session_create(scd_model_t *m, const scd_decode_config_t *cfg, scd_sessi
     // layers of 3072: 32 ms in one pass, 73 ms in passes of 128 rows).
     s->prefill_chunk = s->chunk;
     if (c.dtype == SCD_BF16) s->prefill_chunk = std::max(s->chunk, std::min(c.max_seq - 1, PREFILL_ROWS / s->Q));
-    s->rows_cap = s->Q * s->prefill_chunk;
+    // (the buffers for it come with the first prompt that long)
     s->pages_per_seq = (c.max_seq + c.kv_page_tokens - 1) / c.kv_page_tokens;
     const size_t es = elem_size(c.dtype);
-    const int d = c.d_model, dq = c.n_heads * c.head_dim, dkv = c.n_kv_heads * c.head_dim, F = c.d_ffn, V = c.vocab_out;
+    const int V = c.vocab_out;
     const size_t page_elems = (size_t)c.n_kv_heads * c.kv_page_tokens * c.head_dim;
     s->kv_kind_stride = (size_t)s->Q * s->pages_per_seq * page_elems;
     s->kv_layer_stride = 2 * s->kv_kind_stride;
-    const size_t rows = (size_t)s->rows_cap, wrows = (size_t)s->B * s->L;
+    const size_t wrows = (size_t)s->B * s->L;
 
 #define TRY_ALLOC(expr) do { rc = (expr); if (rc != SCD_OK) { free_session_memory(s); delete s; return rc; } } while (0)
     {
@@ -292,22 +340,14 @@ int scd_session_create(scd_model_t *m, const scd_decode_config_t *cfg, scd_sessi
     TRY_ALLOC(dev_alloc(&s->accept_flags, wrows));
     TRY_ALLOC(dev_alloc(&s->tokens, (size_t)s->B * c.max_seq));
     TRY_ALLOC(dev_alloc(&s->tokens_u, (size_t)s->B * c.max_seq));
-    TRY_ALLOC(dev_alloc(&s->ids_buf, rows));
     TRY_ALLOC(dev_alloc(&s->xbuf[0], wrows * V));
     TRY_ALLOC(dev_alloc(&s->xbuf[1], wrows * V));
     TRY_ALLOC(dev_alloc(&s->stats[0], wrows));
     TRY_ALLOC(dev_alloc(&s->stats[1], wrows));
     TRY_ALLOC(dev_alloc(&s->dev_stats, 1));
     TRY_ALLOC(dev_alloc(&s->finished, 2));
-    TRY_ALLOC(dev_alloc(&s->h, rows * d));
-    // bf16 sessions: GEMM inputs (xn, att, act) in two bf16 planes [2][rows][K], projections (qkv) in fp32
-    const size_t wide = c.dtype == SCD_BF16 ? 2 : 1;
-    { char *p; TRY_ALLOC(dev_alloc(&p, wide * rows * d * es)); s->xn = p; }
-    { char *p; TRY_ALLOC(dev_alloc(&p, wide * rows * (dq + 2 * dkv) * es)); s->qkv = p; }
-    { char *p; TRY_ALLOC(dev_alloc(&p, wide * rows * dq * es)); s->att = p; }
-    { char *p; TRY_ALLOC(dev_alloc(&p, wide * rows * F * es)); s->act = p; }
     s->ss_parts_cap = c.dtype == SCD_BF16 && m->gemm_plan ? gemm_norm_parts_cap(s) : 1;
-    TRY_ALLOC(dev_alloc(&s->ss, (size_t)s->ss_parts_cap * rows));
+    TRY_ALLOC(set_rows(s, s->Q * s->chunk));
     TRY_ALLOC(dev_alloc(&s->logits, (size_t)s->Q * s->L * V));
     s->host_pinned_ints = std::max<size_t>((size_t)s->Q * c.max_seq, 4096);
     {
@@ -366,8 +406,7 @@ int scd_prefill(scd_session_t *s, const int32_t *prompt_ids, int32_t P, int32_t 
                                        (size_t)P * sizeof(int), s->B, cudaMemcpyHostToDevice, st));
     // chunks of the prompt (all but its last token) through the forward, no logits; the kernels read the
     // prompt from the token records just copied, so the chunks are enqueued back to back
-    const int passes = (P - 1 + s->prefill_chunk - 1) / s->prefill_chunk;
-    const int per_pass = passes > 0 ? std::min(s->prefill_chunk, ((P - 1 + passes - 1) / passes + 127) / 128 * 128) : 0;
+    const int per_pass = prefill_pass(s, P - 1);
     for (int p0 = 0; p0 < P - 1; p0 += per_pass) {
         const int len = std::min(per_pass, P - 1 - p0);
         ForwardArgs a;

@@ -46,6 +46,11 @@ int attention_tc_variant(const scd_session *s, int Mq, long long ctx);
 // per-session state (activation tensor maps, device error word); bf16 sessions only
 int gemm_session_prepare(scd_session *s);
 void gemm_session_release(scd_session *s);
+// forget the maps of the activation buffers (they are others now)
+void gemm_session_rows_changed(scd_session *s);
+// the CTA-pair kernel's partial tiles, allocated unless they are there. Forwards of more than 256 rows need it; up to 256
+// the weight-streaming kernel takes over if there is no room for them.
+int gemm_pair_scratch(scd_session *s);
 // reads the device error word that a bounded wait sets when it gives up (0 = healthy). Blocking.
 int gemm_error_word(scd_session *s, int *host_value, cudaStream_t st);
 

@@ -889,7 +889,11 @@ int run_gemm_pair(scd_session *s, const Segment *segs, int n_seg, int epi, const
 int run_gemm(scd_session *s, int kind, const Segment *segs, int n_seg, int epi, const void *x, int K, int rows,
              void *out, int ldo, const NormIn *nin, const NormOut *nout, int x_planes, int *parts_out, cudaStream_t st)
 {
-    if (rows > MAX_ROWS) return run_gemm_pair(s, segs, n_seg, epi, x, K, rows, out, ldo, nin, nout, x_planes, parts_out, st);
+    if (rows > MAX_ROWS) {
+        const int rc = gemm_pair_scratch(s);
+        if (rc != SCD_OK) return rc;
+        return run_gemm_pair(s, segs, n_seg, epi, x, K, rows, out, ldo, nin, nout, x_planes, parts_out, st);
+    }
     GemmPlan *plan = (GemmPlan *)s->model->gemm_plan;
     const bool pair = epi == EPI_SWIGLU;
     GemmParams p;
@@ -901,7 +905,7 @@ int run_gemm(scd_session *s, int kind, const Segment *segs, int n_seg, int epi, 
     int rc = choose_shape(segs, n_seg, pair, rows, plan->sm_count, &p, &tiles, &streams, plan->kind_splits[kind], plan->forced_splits,
                           plan->forced_stages);
     if (rc != SCD_OK) return rc;
-    if (rows > WS_ROWS && !streams) return run_gemm_pair(s, segs, n_seg, epi, x, K, rows, out, ldo, nin, nout, x_planes, parts_out, st);
+    if (rows > WS_ROWS && !streams && gemm_pair_scratch(s) == SCD_OK) return run_gemm_pair(s, segs, n_seg, epi, x, K, rows, out, ldo, nin, nout, x_planes, parts_out, st);
     int t0 = 0;
     for (int i = 0; i < n_seg; ++i) {
         rc = w_map(plan, segs[i], p.tile_rows, &p.tmap_w[i]);
@@ -1037,21 +1041,41 @@ void gemm_set_kind_splits(scd_model *m, int kind, int k_splits)
 int gemm_norm_parts_cap(const scd_session *s) { return (s->model->cfg.d_model + PAIR_UNIT - 1) / PAIR_UNIT; }
 
 // Per-session state: the activation-side tensor maps, the device error word and, when a forward can have more
-// rows than one weight-streaming launch takes, the CTA-pair kernel's tile counters and partial tiles.
+// rows than one weight-streaming launch takes, the CTA-pair kernel's tile counters (its partial tiles, 39 MB, only
+// when a window or a prompt asks for them).
 int gemm_session_prepare(scd_session *s)
 {
     s->gemm_state = new SessionGemm();
     s->gemm_ws_bytes = 256;
-    if (s->rows_cap > WS_ROWS) {
+    const int most = s->Q * s->prefill_chunk;
+    if (most > WS_ROWS) {
         const scd_model_config_t &c = s->model->cfg;
         const int widest = std::max(std::max((c.n_heads + 2 * c.n_kv_heads) * c.head_dim, 2 * c.d_ffn), std::max(c.vocab_out, c.d_model));
-        s->gemm_counters = pair_counter_count(widest / PAIR_COLS + PAIR_MAX_SEG + 1, (s->rows_cap + PAIR_ROWS - 1) / PAIR_ROWS);
+        s->gemm_counters = pair_counter_count(widest / PAIR_COLS + PAIR_MAX_SEG + 1, (most + PAIR_ROWS - 1) / PAIR_ROWS);
         s->gemm_ws_bytes += s->gemm_counters * sizeof(unsigned);
-        SCD_CUDA_TRY(cudaMalloc(&s->gemm_scratch, pair_scratch_bytes(((GemmPlan *)s->model->gemm_plan)->pairs)));
     }
     SCD_CUDA_TRY(cudaMalloc(&s->gemm_ws, s->gemm_ws_bytes));
     SCD_CUDA_TRY(cudaMemset(s->gemm_ws, 0, s->gemm_ws_bytes));
-    return SCD_OK;
+    return s->Q * s->L > WS_ROWS ? gemm_pair_scratch(s) : SCD_OK;
+}
+
+int gemm_pair_scratch(scd_session *s)
+{
+    if (s->gemm_scratch) return SCD_OK;
+    // (an explicit forward may run under the caller's stream capture: the allocation is no part of it)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    SCD_CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
+    const cudaError_t e = cudaMalloc(&s->gemm_scratch, pair_scratch_bytes(((GemmPlan *)s->model->gemm_plan)->pairs));
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e == cudaSuccess) return SCD_OK;
+    s->gemm_scratch = nullptr;
+    cudaGetLastError();                                  // (an allocation that failed leaves the context as it was)
+    return cuda_fail(e, "cudaMalloc of the GEMM's partial tiles");
+}
+
+void gemm_session_rows_changed(scd_session *s)
+{
+    if (s->gemm_state) ((SessionGemm *)s->gemm_state)->xmaps.clear();
 }
 
 void gemm_session_release(scd_session *s)

@@ -19,8 +19,10 @@ struct scd_session {
     scd_decode_config_t cfg;
     int B, S, Q, L;           // sequences, streams per sequence, stream-sequences, window rows
     int chunk;                // rows per stream-sequence that one explicit forward may carry
-    int prefill_chunk;        // ... that one pass over the prompt carries (>= chunk)
-    int rows_cap;             // Q * prefill_chunk
+    int prefill_chunk;        // ... that one pass over a prompt may carry (>= chunk)
+    int rows_cap;             // rows the activation buffers hold: Q * chunk, after a longer prompt up to Q * prefill_chunk
+    void *retired[36];        // activation buffers that larger ones have taken the place of (a caller's captured launches
+    int n_retired;            // may still use them)
     int pages_per_seq;
     int prompt_len, n_new;
     bool prefilled;
@@ -33,7 +35,7 @@ struct scd_session {
 
     // window state (device)
     int *n_known, *n_total, *shift, *prev_lw, *drafts, *n_commit, *tokens, *tokens_u;
-    int *row_y, *row_y_indep, *ids_buf;
+    int *row_y, *row_y_indep;
     unsigned *iter;
     unsigned char *accept_flags;
     float *xbuf[2];
@@ -54,7 +56,7 @@ struct scd_session {
     void *stamps;             // device time stamps of scd_step_timeline (allocated on first use)
     void *gemm_ws;            // device error word of the tcgen05 kernels, then the CTA-pair GEMM's tile counters
     size_t gemm_ws_bytes, gemm_counters;
-    float *gemm_scratch;      // partial tiles of the CTA-pair GEMM
+    float *gemm_scratch;      // partial tiles of the CTA-pair GEMM (allocated when a forward first takes that kernel)
     void *gemm_state;         // activation-side tensor maps
     void *attn_plan;          // tensor map of the KV pool for the tensor-core attention (bf16 sessions)
 
