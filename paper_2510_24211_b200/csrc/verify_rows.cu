@@ -39,6 +39,7 @@
 // every CTA of a cluster reaches the same number of times (branches that hold one are taken on values that all
 // CTAs of the cluster compute from the same data).
 #include <algorithm>
+#include <type_traits>
 
 #include "verify.cuh"
 
@@ -217,7 +218,9 @@ __device__ __noinline__ void nucleus_among(Xchg &xc, Local &lc, int C, unsigned 
 // group it left half of the warps without ids where a warp's share is just above one group, and the others with more than
 // a list takes: 8 x 32 rows of 4371 ids, top-k 4000, 82.9 us, 42.4 so. In registers there is no such limit, and shares
 // that are no whole groups are 5 % slower: 6 rows of 24774 ids 26.1 and 27.3 us.)
-template <int NS, bool REG>
+// TOP_P: with nucleus truncation. (A kernel of its own: in one with the rest it cost the other calls spilled registers, 32
+// rows of 16384 ids 24.0 us, 21.1 so; 256 rows with guidance 48.9 and 44.9.)
+template <int NS, bool REG, bool TOP_P>
 __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p, int C, int long_range)
 {
     constexpr int N = 4 * NS;                          // ids per lane and group
@@ -337,7 +340,7 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
     pdl_wait();                                        // the target logits come from the kernel in front
     const float xX = x_in ? load_p(X) : 0.f;           // the draft's own logit: every CTA weighs X itself
     unsigned *wstore = p.keep_x ? (unsigned *)(p.xbuf[w.parity] + row * V) : nullptr;
-    const bool nucleus = p.top_p24 != 0u && !use_topk; // the nucleus is taken of the whole row
+    const bool nucleus = TOP_P && !use_topk;           // the nucleus is taken of the whole row
     float m[2] = {-INFINITY, 0.f};
 
     // maxima (and bounds) of the CTAs -> of the row
@@ -906,7 +909,7 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
     }
     // ---- nucleus: theta = the largest weight whose ids {W >= theta} hold at least top_p of the mass. The selected step
     // is a range [range_lo, range_lo + 2^bits) of weights, divided NB ways until it is one value. -------------------
-    if (p.top_p24) {
+    if (TOP_P) {
         unsigned range_lo[2] = {0u, 0u};
         int bits[2] = {0, 0};
         unsigned long long above[2] = {0ull, 0ull};    // mass of the weights above the range
@@ -1342,9 +1345,13 @@ int launch_verify_rows(const VerifyParams &p, cudaStream_t stream)
     rc = once.run(dev, [&]() -> int {
         SCD_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         if (dev >= 0 && dev < DeviceOnce::kSlots) sm_count[dev] = sms;
-        SCD_CUDA_TRY(cudaFuncSetAttribute(verify_rows_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lists(128)));
-        SCD_CUDA_TRY(cudaFuncSetAttribute(verify_rows_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lists(256)));
-        SCD_CUDA_TRY(cudaFuncSetAttribute(verify_rows_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lists(WCAP_LONG)));
+        auto opt_in = [&](auto kernel, int wcap) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lists(wcap)); };
+        SCD_CUDA_TRY(opt_in(verify_rows_kernel<1, true, false>, 128));
+        SCD_CUDA_TRY(opt_in(verify_rows_kernel<1, true, true>, 128));
+        SCD_CUDA_TRY(opt_in(verify_rows_kernel<2, true, false>, 256));
+        SCD_CUDA_TRY(opt_in(verify_rows_kernel<2, true, true>, 256));
+        SCD_CUDA_TRY(opt_in(verify_rows_kernel<2, false, false>, WCAP_LONG));
+        SCD_CUDA_TRY(opt_in(verify_rows_kernel<2, false, true>, WCAP_LONG));
         return SCD_OK;
     });
     if (rc != SCD_OK) return rc;
@@ -1355,9 +1362,14 @@ int launch_verify_rows(const VerifyParams &p, cudaStream_t stream)
     // calls one after the other otherwise paid a full launch each (1 x 32 rows of 16384 ids: 26.6 us a call, 24.3 so,
     // 4 us less on the host included; Gumbel, 2 x 32: 39.5 and 36.6).
     const dim3 grid((unsigned)(p.L * C), (unsigned)p.B, 1);
-    if (ids <= 128) SCD_CUDA_TRY(launch_ex(verify_rows_kernel<1, true>, grid, CT, (size_t)lists(128), C, stream, p, C, 0));
-    else if (ids <= 256) SCD_CUDA_TRY(launch_ex(verify_rows_kernel<2, true>, grid, CT, (size_t)lists(256), C, stream, p, C, 0));
-    else SCD_CUDA_TRY(launch_ex(verify_rows_kernel<2, false>, grid, CT, (size_t)lists(WCAP_LONG), C, stream, p, C, (ids + 31) / 32 * 32));
+    auto launch = [&](auto kernel, int wcap, int range) { return launch_ex(kernel, grid, CT, (size_t)lists(wcap), C, stream, p, C, range); };
+    auto pick = [&](auto with_top_p) {
+        constexpr bool TOP_P = decltype(with_top_p)::value;
+        return ids <= 128 ? launch(verify_rows_kernel<1, true, TOP_P>, 128, 0)
+             : ids <= 256 ? launch(verify_rows_kernel<2, true, TOP_P>, 256, 0)
+                          : launch(verify_rows_kernel<2, false, TOP_P>, WCAP_LONG, (ids + 31) / 32 * 32);
+    };
+    SCD_CUDA_TRY(p.top_p24 ? pick(std::true_type{}) : pick(std::false_type{}));
     return SCD_OK;
 }
 
