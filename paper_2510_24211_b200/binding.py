@@ -154,7 +154,10 @@ def _stream(stream=None):
     if not torch.cuda.is_initialized():
         return torch.cuda.current_stream().cuda_stream
     # (the handle alone: torch.cuda.current_stream() looks the device up and builds an object, 4 us of a 21 us call)
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    try:
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    except AttributeError:                             # names of torch's own, which another version may lack
+        return torch.cuda.current_stream().cuda_stream
 
 
 def _ptr(t):

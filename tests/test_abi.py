@@ -75,3 +75,17 @@ def test_calls_that_need_no_device():
     with pytest.raises(scd.ScdError):
         scd._check(lib.scd_prefill(None, None, 1, 1, None))
     assert lib.scd_session_attention_min_ctx(None, 0) < 0           # null session
+
+
+@pytest.mark.parametrize("gone", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_current_stream_without_the_private_names(monkeypatch, gone):
+    import types
+
+    import torch
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=4711))
+    monkeypatch.delattr(torch._C, gone, raising=False)
+    other = "_cuda_getDevice" if gone == "_cuda_getCurrentRawStream" else "_cuda_getCurrentRawStream"
+    monkeypatch.setattr(torch._C, other, lambda *a: 0, raising=False)
+    assert scd._stream() == 4711
+    assert scd._stream(types.SimpleNamespace(cuda_stream=5)) == 5
