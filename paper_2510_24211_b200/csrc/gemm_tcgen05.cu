@@ -66,7 +66,7 @@ constexpr int MAX_ROWS = 256;        // window rows one launch may carry (scd_ge
 constexpr int WS_ROWS = 128;         // ... and up to which a session always uses this kernel (see choose_shape)
 constexpr int GEMM_THREADS = 192;
 
-enum { EPI_BF16 = 0, EPI_F32 = 1, EPI_RESID = 2, EPI_SWIGLU = 3 };
+enum { EPI_F32 = 0, EPI_RESID, EPI_SWIGLU };
 
 struct GemmParams {
     CUtensorMap tmap_w[MAX_SEG];     // weight segments; SwiGLU: [0] gate, [1] up, boxes of 64 rows
@@ -86,7 +86,7 @@ struct GemmParams {
     int stages;
     int aux_offset;                  // byte offset (from the aligned ring base) of the small per-row scratch
     int epi;
-    void *out;                       // bf16 or fp32 [M][ldo]
+    void *out;                       // fp32 [M][ldo]; SwiGLU: two bf16 planes of [M][ldo]
     int ldo;
     // RMSNorm of the x rows (optional): ss_in [ss_parts][ss_stride] partial sums of squares
     const float *ss_in;
@@ -231,8 +231,7 @@ __device__ __forceinline__ void reduce_rows(const GemmParams &p, uint32_t base, 
             }
             if (scale) { const float is = inv_s[m - m_lo]; v.x *= is; v.y *= is; v.z *= is; v.w *= is; }
             const size_t o = (size_t)m * p.ldo + oc.col;
-            if (p.epi == EPI_BF16) store_bf16x4((__nv_bfloat16 *)p.out + o, v, oc.n_ok, oc.vec);
-            else if (p.epi == EPI_F32) store_f32x4((float *)p.out + o, v, oc);
+            if (p.epi == EPI_F32) store_f32x4((float *)p.out + o, v, oc);
             else {
                 float4 hn = h[j];
                 hn.x += v.x; hn.y += v.y; hn.z += v.z; hn.w += v.w;

@@ -11,11 +11,9 @@
 // and 7) as an integer exponential race with noise keyed by position and id only. Top-p after
 // top-k as a threshold on the integer weights.
 //
-// Data flow of a row: logits -> x (registers when the row has at most 16 ids per thread, else the
-// row's cells) -> radix selection of the top-k threshold -> integer weights W, written once into
-// the row's cells (shared memory when the row fits, else global memory); every later pass (sum,
-// accept test, residual search, race) reads integers. A session stores W as the next iteration's
-// draft distribution.
+// Data flow of a row: logits -> x, in the row's cells (its row of xbuf, global memory) -> radix selection of the top-k
+// threshold -> integer weights W, in the same cells; every later pass (sum, accept test, residual search, race) reads
+// integers. A session keeps W there as the next iteration's draft distribution.
 //
 // Exactness: a distribution is the integer vector W_v = trunc(scd_exp(x_v - max x) * 2^30) over
 // the ids whose post-processed logit x_v reaches the top-k threshold; every decision is an
@@ -44,13 +42,12 @@ struct Smem {
 
 // Post-processed logit of id v of a stored row; raw draft logits still need the temperature.
 struct XRow {
-    const float *row;      // global row (off = 0) or its copy in shared memory (off = first allowed id)
-    int off;
+    const float *row;
     float T;
     bool div;
     __device__ __forceinline__ float operator()(int v) const
     {
-        const float x = row[v - off];
+        const float x = row[v];
         return div ? __fdiv_rn(x, T) : x;
     }
 };
@@ -153,116 +150,6 @@ __device__ float kth_largest(const XRow &x, int lo, int hi, int k, Smem &sm)
     }
     __syncthreads();
     return key_float(prefix);
-}
-
-// A row whose ids fit EPT per thread, kept in registers from the logits to the weights: thread t
-// owns ids lo + t + i VT. Loads are issued as a batch; the radix selection works on the registers
-// (a bit per element says whether it still matches the selected prefix) and the exponential runs
-// once per id. Writes the integer weights to wcell[v - lo] (and to wglob[v] when given) and returns
-// the row maximum, the top-k threshold and the sum of the weights.
-template <int EPT>
-__device__ __forceinline__ void row_in_registers(const float *c, const float *u, float one_plus_lam, float lam,
-                                                 bool div, float T, int lo, int hi, int top_k, unsigned *wcell,
-                                                 unsigned *wglob, unsigned *scratch, int scratch_words, Smem &sm,
-                                                 float &m_out, float &tau_out, unsigned long long &Z_out)
-{
-    const int tid = threadIdx.x, lane = tid & 31;
-    float x[EPT];
-    {
-        float a[EPT], bu[EPT];
-#pragma unroll
-        for (int i = 0; i < EPT; ++i) {
-            const int v = lo + tid + i * VT;
-            a[i] = v < hi ? c[v] : 0.f;
-            bu[i] = (u && v < hi) ? u[v] : 0.f;
-        }
-#pragma unroll
-        for (int i = 0; i < EPT; ++i) {
-            float t = a[i];
-            if (u) t = __fsub_rn(__fmul_rn(one_plus_lam, t), __fmul_rn(lam, bu[i]));
-            if (div) t = __fdiv_rn(t, T);
-            x[i] = t;
-        }
-    }
-    unsigned mine = 0;                             // bit i: element i exists
-    float mx = -INFINITY;
-#pragma unroll
-    for (int i = 0; i < EPT; ++i)
-        if (lo + tid + i * VT < hi) { mine |= 1u << i; mx = fmaxf(mx, x[i]); }
-    const bool ragged = (hi - lo) != EPT * VT;     // (uniform) some threads own fewer than EPT ids
-    const float m = block_max(mx, sm);
-    float tau = -INFINITY;
-    if (top_k > 0 && top_k < hi - lo) {
-        // radix selection, 8 bits per pass, on order-preserving keys held in the registers of x
-        unsigned key[EPT];
-#pragma unroll
-        for (int i = 0; i < EPT; ++i) key[i] = float_key(x[i]);
-        unsigned prefix = 0, mask = 0, kk = (unsigned)top_k;
-        bool any = true;                           // this thread still owns a candidate
-        for (int shift = 24; shift >= 0; shift -= 8) {
-            for (int i = tid; i < 256; i += VT) sm.hist[i] = 0;
-            __syncthreads();
-            if (shift == 24 && scratch_words >= 256 * 32) {
-                // sign and high exponent bits: a handful of bins take almost every element. One
-                // histogram per lane (scratch[bin][lane]) keeps a warp's atomics apart; a warp
-                // then adds the 32 copies of a bin with one reduction.
-                for (int i = tid; i < 256 * 32; i += VT) scratch[i] = 0u;
-                __syncthreads();
-#pragma unroll
-                for (int i = 0; i < EPT; ++i)
-                    if (!ragged || ((mine >> i) & 1u)) atomicAdd(&scratch[(key[i] >> 24) * 32u + lane], 1u);
-                __syncthreads();
-                for (int bin = tid >> 5; bin < 256; bin += NW) {
-                    const unsigned cnt = __reduce_add_sync(FULL, scratch[bin * 32 + lane]);
-                    if (lane == 0) sm.hist[bin] = cnt;
-                }
-            } else if (shift == 24) {
-                // (no scratch: count the lanes of each bin once; every thread takes part in the votes)
-#pragma unroll
-                for (int i = 0; i < EPT; ++i) {
-                    const bool on = !ragged || ((mine >> i) & 1u);
-                    const unsigned bin = key[i] >> 24;
-                    const unsigned active = __ballot_sync(FULL, on);
-                    if (on) {
-                        const unsigned peers = __match_any_sync(active, bin);
-                        if (lane == __ffs(peers) - 1) atomicAdd(&sm.hist[bin], (unsigned)__popc(peers));
-                    }
-                }
-            } else if (any) {
-                // the candidates thin out by a factor of the bin count per pass: most threads skip
-                any = false;
-#pragma unroll
-                for (int i = 0; i < EPT; ++i) {
-                    if ((key[i] & mask) == prefix && (!ragged || ((mine >> i) & 1u))) {
-                        atomicAdd(&sm.hist[(key[i] >> shift) & 255u], 1u);
-                        any = true;
-                    }
-                }
-            }
-            __syncthreads();
-            select_bin(sm, kk);
-            __syncthreads();
-            prefix |= sm.sel_bin << shift;
-            mask |= 0xFFu << shift;
-            kk = sm.sel_k;
-        }
-        __syncthreads();
-        tau = key_float(prefix);
-    }
-    unsigned long long z = 0;
-#pragma unroll
-    for (int i = 0; i < EPT; ++i) {
-        if ((mine >> i) & 1u) {
-            const int v = lo + tid + i * VT;
-            const unsigned wv = weight_of(x[i], m, tau);
-            wcell[v - lo] = wv;
-            if (wglob) wglob[v] = wv;
-            z += wv;
-        }
-    }
-    Z_out = block_sum_u64(z, sm);
-    m_out = m;
-    tau_out = tau;
 }
 
 // Nucleus (top-p) threshold on the integer weights of ids [lo, hi): the largest weight value theta
@@ -413,11 +300,8 @@ __device__ int block_fresh_race(int lo, int hi, const VerifyParams &p, int b, lo
     return fresh_key_id(best);
 }
 
-// Rows are staged in shared memory when they fit (stage_cap floats per row; stage_q: a second
-// buffer for the draft row), so that the selection, sum and search passes read HBM only once.
-__global__ void __launch_bounds__(VT, 1) verify_kernel(const VerifyParams p, int stage_cap, int stage_q)
+__global__ void __launch_bounds__(VT, 1) verify_kernel(const VerifyParams p)
 {
-    extern __shared__ float staged[];
     __shared__ Smem sm;
     const int tid = threadIdx.x;
     const int k = blockIdx.x, b = blockIdx.y;
@@ -431,17 +315,11 @@ __global__ void __launch_bounds__(VT, 1) verify_kernel(const VerifyParams p, int
         const size_t row = (size_t)b * L + k;
 
         // ---- target distribution p = post-process(logits) ------------------------------------
-        // The row's cells (shared memory when the row fits, else its row of xbuf in global memory)
-        // first hold the post-processed logits x and then, in place, the integer weights W: the
-        // exponential is evaluated once per id and every later pass reads integers. In a session
-        // the weights also go to xbuf[t & 1]: they are the next iteration's draft distribution.
-        float *xp = p.xbuf[w.parity] + row * V;
-        const bool in_smem = hi - lo <= stage_cap;           // this row fits the staging buffer
-        float *xs_q = in_smem && stage_q ? staged + stage_cap : nullptr;
-        float *prow = in_smem ? staged : xp;
-        const int poff = in_smem ? lo : 0;
-        unsigned *wp = (unsigned *)prow;
-        const bool store_w = p.keep_x && in_smem;            // (cells in global memory are xbuf itself)
+        // The row's cells first hold the post-processed logits x and then, in place, the integer weights W: the exponential
+        // is evaluated once per id and every later pass reads integers. In a session they are the next iteration's draft
+        // distribution.
+        float *const xp = p.xbuf[w.parity] + row * V;
+        unsigned *const wp = (unsigned *)xp;
         const float *c = p.p_logits + row * V;
         const float *u = p.S == 2 ? p.p_logits + ((size_t)(p.B + b) * L + k) * V : nullptr;
         const bool mix = (p.S == 2);
@@ -449,15 +327,8 @@ __global__ void __launch_bounds__(VT, 1) verify_kernel(const VerifyParams p, int
         const bool use_topk = p.top_k > 0 && p.top_k < hi - lo;
         float m_p, tau_p;
         unsigned long long Zp;
-        unsigned *const wstore = (store_w && !p.top_p24) ? (unsigned *)xp : nullptr;
-        if (in_smem && hi - lo <= 8 * VT) {
-            row_in_registers<8>(c, mix ? u : nullptr, p.one_plus_lam, p.lam, div, p.temperature, lo, hi, p.top_k,
-                                wp, wstore, (unsigned *)xs_q, xs_q ? stage_cap : 0, sm, m_p, tau_p, Zp);
-        } else if (in_smem && hi - lo <= 16 * VT) {
-            row_in_registers<16>(c, mix ? u : nullptr, p.one_plus_lam, p.lam, div, p.temperature, lo, hi, p.top_k,
-                                 wp, wstore, (unsigned *)xs_q, xs_q ? stage_cap : 0, sm, m_p, tau_p, Zp);
-        } else {
-            // long rows: the cells live in global memory; loads go out four at a time
+        {
+            // loads go out four at a time
             float mx = -INFINITY;
             for (int v0 = lo + tid; v0 < hi; v0 += 4 * VT) {
                 float xc[4], xu[4];
@@ -474,25 +345,24 @@ __global__ void __launch_bounds__(VT, 1) verify_kernel(const VerifyParams p, int
                         float x = xc[j];
                         if (mix) x = __fsub_rn(__fmul_rn(p.one_plus_lam, x), __fmul_rn(p.lam, xu[j]));
                         if (div) x = __fdiv_rn(x, p.temperature);
-                        prow[v - poff] = x;
+                        xp[v] = x;
                         mx = fmaxf(mx, x);
                     }
                 }
             }
             m_p = block_max(mx, sm);       // barrier inside: the row is visible to the CTA
-            tau_p = use_topk ? kth_largest(XRow{prow, poff, 1.0f, false}, lo, hi, p.top_k, sm) : -INFINITY;
+            tau_p = use_topk ? kth_largest(XRow{xp, 1.0f, false}, lo, hi, p.top_k, sm) : -INFINITY;
             unsigned long long zp = 0;
             for (int v0 = lo + tid; v0 < hi; v0 += 4 * VT) {     // x -> W, each thread on its own cells
                 float xv[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) xv[j] = v0 + j * VT < hi ? prow[v0 + j * VT - poff] : -INFINITY;
+                for (int j = 0; j < 4; ++j) xv[j] = v0 + j * VT < hi ? xp[v0 + j * VT] : -INFINITY;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int v = v0 + j * VT;
                     if (v < hi) {
                         const unsigned wv = weight_of(xv[j], m_p, tau_p);
-                        wp[v - poff] = wv;
-                        if (wstore) wstore[v] = wv;
+                        wp[v] = wv;
                         zp += wv;
                     }
                 }
@@ -501,34 +371,28 @@ __global__ void __launch_bounds__(VT, 1) verify_kernel(const VerifyParams p, int
         }
         unsigned theta_p = 0u;
         if (p.top_p24) {
-            auto fw = [&](int v) -> unsigned { return wp[v - poff]; };
+            auto fw = [&](int v) -> unsigned { return wp[v]; };
             unsigned long long kept;
             theta_p = nucleus_threshold(fw, lo, hi, Zp, p.top_p24, sm, &kept);
             Zp = kept;
-            for (int v = lo + tid; v < hi; v += VT) {
-                unsigned wv = wp[v - poff];
-                if (wv < theta_p) { wv = 0u; wp[v - poff] = 0u; }
-                if (store_w) ((unsigned *)xp)[v] = wv;
-            }
+            for (int v = lo + tid; v < hi; v += VT)
+                if (wp[v] < theta_p) wp[v] = 0u;
             __syncthreads();
         }
         if (tid == 0) {
             RowStats st; st.m = m_p; st.tau = tau_p; st.Z = Zp; st.theta = theta_p; st.pad_ = 0u;
             p.stats[w.parity][row] = st;
         }
-        auto WP = [&](int v) -> unsigned { return wp[v - poff]; };
+        auto WP = [&](int v) -> unsigned { return wp[v]; };
 
         // ---- draft distribution q: the previous iteration's p of the same position -----------
         // session: its integer weights, as stored by that iteration; stand-alone: raw logits that
-        // go through the same steps here (cached in shared memory when the row fits, else
-        // recomputed per visit); fresh rows: uniform weights 1 on the allowed ids.
+        // go through the same steps here (recomputed per visit); fresh rows: uniform weights 1 on the allowed ids.
         const int qk = k + w.shift;
         const bool fresh = !(qk < w.prev_lw);
         unsigned long long Zq = (unsigned long long)(hi - lo);
-        const unsigned *qcache = nullptr;                     // cached integer weights, id v at qcache[v - qoff]
-        int qoff = 0;
-        bool q_in_smem = false;
-        XRow XQ = {nullptr, 0, p.temperature, false};         // recompute path only
+        const unsigned *q_weights = nullptr;                  // the stored weights
+        XRow XQ = {nullptr, p.temperature, false};            // the raw logits
         float m_q = 0.f, tau_q = -INFINITY;
         unsigned theta_q = 0u;
         if (!fresh) {
@@ -536,65 +400,27 @@ __global__ void __launch_bounds__(VT, 1) verify_kernel(const VerifyParams p, int
             if (p.q_is_raw) {
                 XQ.row = p.xbuf[w.parity ^ 1] + qrow * V;
                 XQ.div = div;
-                if (xs_q) {
-                    unsigned *wq = (unsigned *)xs_q;
-                    if (hi - lo <= 8 * VT) {
-                        row_in_registers<8>(XQ.row, nullptr, 0.f, 0.f, div, p.temperature, lo, hi, p.top_k, wq, nullptr,
-                                            wq, stage_cap, sm, m_q, tau_q, Zq);
-                    } else if (hi - lo <= 16 * VT) {
-                        row_in_registers<16>(XQ.row, nullptr, 0.f, 0.f, div, p.temperature, lo, hi, p.top_k, wq, nullptr,
-                                             wq, stage_cap, sm, m_q, tau_q, Zq);
-                    } else {
-                        float mq = -INFINITY;
-                        for (int v = lo + tid; v < hi; v += VT) {
-                            const float x = XQ(v);
-                            xs_q[v - lo] = x;
-                            mq = fmaxf(mq, x);
-                        }
-                        m_q = block_max(mq, sm);
-                        tau_q = use_topk ? kth_largest(XRow{xs_q, lo, 1.0f, false}, lo, hi, p.top_k, sm) : -INFINITY;
-                        unsigned long long zq = 0;
-                        for (int v = lo + tid; v < hi; v += VT) {
-                            const unsigned wv = weight_of(xs_q[v - lo], m_q, tau_q);
-                            wq[v - lo] = wv;
-                            zq += wv;
-                        }
-                        Zq = block_sum_u64(zq, sm);
-                    }
-                    if (p.top_p24) {
-                        auto fq = [&](int v) -> unsigned { return wq[v - lo]; };
-                        unsigned long long kept;
-                        theta_q = nucleus_threshold(fq, lo, hi, Zq, p.top_p24, sm, &kept);
-                        Zq = kept;
-                        for (int v = lo + tid; v < hi; v += VT)
-                            if (wq[v - lo] < theta_q) wq[v - lo] = 0u;
-                        __syncthreads();
-                    }
-                    qcache = wq; qoff = lo; q_in_smem = true;
-                } else {
-                    float mq = -INFINITY;
-                    for (int v = lo + tid; v < hi; v += VT) mq = fmaxf(mq, XQ(v));
-                    m_q = block_max(mq, sm);
-                    tau_q = use_topk ? kth_largest(XQ, lo, hi, p.top_k, sm) : -INFINITY;
-                    unsigned long long zq = 0;
-                    for (int v = lo + tid; v < hi; v += VT) zq += weight_of(XQ(v), m_q, tau_q);
-                    Zq = block_sum_u64(zq, sm);
-                    if (p.top_p24) {
-                        auto fq = [&](int v) -> unsigned { return weight_of(XQ(v), m_q, tau_q); };
-                        unsigned long long kept;
-                        theta_q = nucleus_threshold(fq, lo, hi, Zq, p.top_p24, sm, &kept);
-                        Zq = kept;
-                    }
+                float mq = -INFINITY;
+                for (int v = lo + tid; v < hi; v += VT) mq = fmaxf(mq, XQ(v));
+                m_q = block_max(mq, sm);
+                tau_q = use_topk ? kth_largest(XQ, lo, hi, p.top_k, sm) : -INFINITY;
+                unsigned long long zq = 0;
+                for (int v = lo + tid; v < hi; v += VT) zq += weight_of(XQ(v), m_q, tau_q);
+                Zq = block_sum_u64(zq, sm);
+                if (p.top_p24) {
+                    auto fq = [&](int v) -> unsigned { return weight_of(XQ(v), m_q, tau_q); };
+                    unsigned long long kept;
+                    theta_q = nucleus_threshold(fq, lo, hi, Zq, p.top_p24, sm, &kept);
+                    Zq = kept;
                 }
             } else {
                 Zq = p.stats[w.parity ^ 1][qrow].Z;
-                qcache = (const unsigned *)(p.xbuf[w.parity ^ 1] + qrow * V);
-                qoff = 0;
+                q_weights = (const unsigned *)(p.xbuf[w.parity ^ 1] + qrow * V);
             }
         }
         auto WQ = [&](int v) -> unsigned {
             if (fresh) return 1u;
-            if (qcache) return qcache[v - qoff];
+            if (q_weights) return q_weights[v];
             return weight_of(XQ(v), m_q, tau_q, theta_q);
         };
 
@@ -628,20 +454,6 @@ __global__ void __launch_bounds__(VT, 1) verify_kernel(const VerifyParams p, int
             if (!accept) {
                 // Y ~ norm(max(0, p - q)): R_v = max(0, Wp_v Zq - Wq_v Zp)
                 const unsigned Ur = noise_u24(p.seed, NOISE_RESIDUAL, (unsigned)b, pos, w.t, 0);
-                if (!fresh && !q_in_smem && qcache && xs_q) {
-                    // rejected: the residual needs the whole draft row, twice; read it from HBM once
-                    unsigned *wq = (unsigned *)xs_q;
-                    for (int v0 = lo + tid; v0 < hi; v0 += 8 * VT) {        // loads issued as a batch
-                        unsigned t[8];
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) t[j] = v0 + j * VT < hi ? qcache[v0 + j * VT - qoff] : 0u;
-#pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            if (v0 + j * VT < hi) wq[v0 + j * VT - lo] = t[j];
-                    }
-                    __syncthreads();
-                    qcache = wq; qoff = lo; q_in_smem = true;
-                }
                 auto fr = [&](int v) -> u128 {
                     const u128 a = mul_32x64(WP(v), Zq);
                     const u128 bq = mul_32x64(WQ(v), Zp);
@@ -721,24 +533,7 @@ int launch_verify(const VerifyParams &p, cudaStream_t stream)
         const int rc = launch_verify_rows(p, stream);
         return rc == SCD_OK ? launch_commit(p, stream) : rc;
     }
-    dim3 grid((unsigned)p.L, (unsigned)p.B);
-    // shared-memory staging: both rows if they fit, else the target row alone, else none
-    const int n = p.allowed_hi - p.allowed_lo;
-    const size_t budget = 200 * 1024;
-    int stage_cap = 0, stage_q = 0;
-    if ((size_t)n * 8 <= budget) { stage_cap = n; stage_q = 1; }
-    else if ((size_t)n * 4 <= budget) { stage_cap = n; }
-    const size_t smem = (size_t)stage_cap * 4 * (stage_q ? 2 : 1);
-    static DeviceOnce once;
-    int dev = 0;
-    int rc = current_device(&dev);
-    if (rc != SCD_OK) return rc;
-    rc = once.run(dev, [&]() -> int {
-        SCD_CUDA_TRY(cudaFuncSetAttribute(verify_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
-        return SCD_OK;
-    });
-    if (rc != SCD_OK) return rc;
-    verify_kernel<<<grid, VT, smem, stream>>>(p, stage_cap, stage_q);
+    verify_kernel<<<dim3((unsigned)p.L, (unsigned)p.B), VT, 0, stream>>>(p);
     SCD_CUDA_TRY(cudaGetLastError());
     return launch_commit(p, stream);
 }

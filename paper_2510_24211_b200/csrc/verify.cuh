@@ -35,7 +35,7 @@ struct VerifyParams {
     // integer weights W (uint32 in the float-typed cells) of the window rows' target distributions,
     // two buffers [B][L][V] used in ping-pong by iteration parity: this iteration writes
     // xbuf[t & 1] and reads the drafts' distributions from xbuf[(t & 1) ^ 1]. Stand-alone use:
-    // xbuf[0] = scratch (rows that do not fit in shared memory), xbuf[1] = raw draft logits.
+    // xbuf[0] = scratch (rows too long for a cluster), xbuf[1] = raw draft logits.
     float *xbuf[2];
     RowStats *stats[2];    // [B][L] each; stats of xbuf[i] rows
     int keep_x;            // 1: write the target row's weights to xbuf[t & 1] (the next iteration reads them)
