@@ -28,6 +28,7 @@
 
 #include "model.cuh"
 #include "gemm.cuh"
+#include "ptx.cuh"
 
 namespace scd {
 
@@ -35,7 +36,6 @@ namespace {
 
 constexpr int TK = 64;                 // keys per tile
 constexpr int MAX_ATT_STAGES = 8;
-constexpr unsigned ATT_SPIN_LIMIT = 1u << 22;
 
 struct AttnParams {
     CUtensorMap kv_map;                // the whole pool as a 2-D bf16 matrix [rows][head_dim]
@@ -61,42 +61,15 @@ struct AttnParams {
     unsigned long long *stamp;         // optional [2][STAMP_CTAS]: %globaltimer at CTA entry and exit
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, unsigned count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, unsigned bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity)
-{
-    const uint32_t a = smem_u32(bar);
-    for (unsigned i = 0; i < ATT_SPIN_LIMIT; ++i) {
-        unsigned ok;
-        asm volatile("{\n\t.reg .pred p;\n\t"
-                     "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                     "selp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(ok) : "r"(a), "r"(parity) : "memory");
-        if (ok) return true;
-    }
-    return false;
 }
 __device__ __forceinline__ void tma_load_2d(const CUtensorMap *map, uint64_t *bar, void *dst, int x, int y)
 {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
                  " [%0], [%1, {%3, %4}], [%2];"
                  ::"r"(smem_u32(dst)), "l"((uint64_t)map), "r"(smem_u32(bar)), "r"(x), "r"(y) : "memory");
-}
-__device__ __forceinline__ void cluster_sync_all()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ uint32_t map_peer(uint32_t local_smem_addr, uint32_t peer)
 {
@@ -793,7 +766,7 @@ __device__ __forceinline__ uint64_t t5_desc_mn(uint32_t smem_addr, uint32_t lbo_
 __device__ __forceinline__ bool t5_wait(uint64_t *bar, unsigned parity, volatile int *failed)
 {
     const uint32_t a = smem_u32(bar);
-    for (unsigned i = 0; i < ATT_SPIN_LIMIT; ++i) {
+    for (unsigned i = 0; i < SPIN_LIMIT; ++i) {
         unsigned ok;
         asm volatile("{\n\t.reg .pred p;\n\t"
                      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
@@ -811,33 +784,6 @@ __device__ __forceinline__ void t5_mma_ts(uint32_t tmem_d, uint32_t tmem_a, uint
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                  "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
                  ::"r"(tmem_d), "r"(tmem_a), "l"(db), "r"(idesc), "r"(acc) : "memory");
-}
-__device__ __forceinline__ void t5_commit(uint64_t *bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-// 32 consecutive columns of this thread's tensor-memory lane
-__device__ __forceinline__ void t5_ld32(uint32_t taddr, float *v)
-{
-    uint32_t r[32];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-                 : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ void t5_ld16(uint32_t taddr, float *v)
-{
-    uint32_t r[16];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                 : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 __device__ __forceinline__ float t5_ex2(float x)
 {
@@ -1143,7 +1089,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
             const uint32_t koff = (uint32_t)(ks >> 2) * (uint32_t)(TK * 128) + (uint32_t)(ks & 3) * 32u;
             t5_mma_ts(d, tmem_q + 64u + (uint32_t)ks * 8u, dk + (koff >> 4), idesc_s, 1u);
         }
-        t5_commit(&bar_s[t & 1]);
+        umma_commit(&bar_s[t & 1]);
     };
     // O lane: O += P[t & 1] V(t) once the threads have written P(t)
     auto mma_o = [&](int t, uint32_t vaddr) {
@@ -1154,7 +1100,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
 #pragma unroll
         for (int kk = 0; kk < TK / 16; ++kk)                      // 16 keys = 8 columns of P, 16 rows of V
             t5_mma_ts(tmem_o, pa + (uint32_t)kk * 8u, dv + (uint32_t)(kk * 2048 >> 4), idesc_o, (t > 0 || kk > 0) ? 1u : 0u);
-        t5_commit(&bar_o[t & 1]);
+        umma_commit(&bar_o[t & 1]);
     };
 
     float m_used = -INFINITY, l_run = 0.f;                        // softmax threads: the state of the lane's row
@@ -1166,10 +1112,10 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         float v[NC];
         const uint32_t s_addr = tmem_s + lane_base + (uint32_t)(t & 1) * 64u + (uint32_t)c_lo;
-        if (NC == 16) t5_ld16(s_addr, v);
+        if (NC == 16) tmem_ld16(s_addr, v);
         else {
 #pragma unroll
-            for (int c0 = 0; c0 < NC; c0 += 32) t5_ld32(s_addr + (uint32_t)c0, v + c0);
+            for (int c0 = 0; c0 < NC; c0 += 32) tmem_ld32(s_addr + (uint32_t)c0, v + c0);
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         mbar_arrive(&bar_sc[t & 1]);                              // S[t & 1] may be overwritten
@@ -1192,7 +1138,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
 #pragma unroll 1
             for (int c0 = 0; c0 < DH; c0 += 32) {
                 float ov[32];
-                t5_ld32(tmem_o + lane_base + (uint32_t)c0, ov);
+                tmem_ld32(tmem_o + lane_base + (uint32_t)c0, ov);
 #pragma unroll
                 for (int j = 0; j < 32; ++j) ov[j] *= alpha;
                 t5_st32(tmem_o + lane_base + (uint32_t)c0, ov);
@@ -1228,7 +1174,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
         for (int t = 0; t < my_tiles; ++t) {
             wait_on(&kfull[s], ph, 5);
             mma_s(n_wt + t, smem_u32(kring + (size_t)s * tile_bytes));
-            t5_commit(&kempty[s]);
+            umma_commit(&kempty[s]);
             if (++s == NK) { s = 0; ph ^= 1u; }
         }
     } else if (o_lane) {
@@ -1238,7 +1184,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
         for (int t = 0; t < my_tiles; ++t) {
             wait_on(&vfull[s], ph, 5);
             mma_o(n_wt + t, smem_u32(vring + (size_t)s * tile_bytes));
-            t5_commit(&vempty[s]);
+            umma_commit(&vempty[s]);
             if (++s == NV) { s = 0; ph ^= 1u; }
         }
     } else if (k_lane) {
@@ -1281,7 +1227,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) attention_t5_kernel(const __gri
 #pragma unroll 1
         for (int c0 = 0; c0 < DH; c0 += 32) {
             float ov[32];
-            t5_ld32(tmem_o + lane_base + (uint32_t)c0, ov);       // (warp-wide: dead rows read along)
+            tmem_ld32(tmem_o + lane_base + (uint32_t)c0, ov);       // (warp-wide: dead rows read along)
             const bool keep = live && t_done > 0;
 #pragma unroll
             for (int j = 0; j < 32; j += 4)

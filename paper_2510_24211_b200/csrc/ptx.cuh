@@ -1,5 +1,5 @@
-// Thin wrappers of the sm_100a instructions that the GEMM kernels share: mbarriers, TMA copies, tcgen05 MMA
-// and tensor-memory loads.
+// Thin wrappers of the sm_100a instructions that the GEMM and attention kernels share: mbarriers, TMA copies, tcgen05
+// MMA and tensor-memory loads.
 #pragma once
 #include <cuda.h>
 
@@ -77,6 +77,7 @@ __device__ __forceinline__ void umma_commit(uint64_t *bar)
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                  ::"r"(smem_u32(bar)) : "memory");
 }
+// 32 consecutive columns of this thread's tensor-memory lane
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v)
 {
     uint32_t r[32];
