@@ -97,3 +97,77 @@ def test_fp32_layers_match_oracle(over, P, B, M):
         ref_logits, ref_hidden = om.forward(ids[b], P - 1, stream=b, want_hidden=True)
         assert _rel(hidden[b].cpu().numpy(), ref_hidden) <= 2e-5
         assert _rel(logits[b].cpu().numpy(), ref_logits) <= 2e-5
+
+
+@pytest.mark.parametrize("B,M", [(1, 40), (2, 256)])
+def test_swiglu_where_the_exponential_is_large(B, M):
+    """silu(g) u with g down to -88.5, where 1 + exp(-g) passes 2^126, and u large enough for the product to matter: the
+    weight-streaming kernel (40 rows) and the CTA-pair kernel (512). One layer without attention output, embeddings of +-1.
+    Bound 1e-4 of the largest value: g is good to 2e-5 absolute (64 fp32 terms), the product is kept in two bf16 planes."""
+    d, F = 64, 128
+    shape = dict(n_layers=1, d_model=d, n_heads=1, n_kv_heads=1, head_dim=64, d_ffn=F, vocab_out=64, vocab_in=64, dtype="bf16",
+                 rope_base=10000.0, rms_eps=1e-5)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    bf = dict(device="cuda", dtype=torch.bfloat16)
+    gate = torch.linspace(-20.0, 20.0, F, device="cuda")
+    gate[::16] = torch.tensor([-87.5, -88.0, -88.5, -87.5, -80.0, -88.0, -88.5, -60.0], device="cuda")
+    up = torch.where(gate < -50.0, torch.full_like(gate, 3e37), torch.ones_like(gate))
+    w = {"tok_emb": torch.ones(64, d, **bf), "final_norm": torch.ones(d, **bf), "lm_head": torch.zeros(64, d, **bf)}
+    w["tok_emb"][1::2, d // 2:] = -1.0                 # odd tokens: g = u = 0
+    w.update(attn_norm=[torch.ones(d, **bf)], ffn_norm=[torch.ones(d, **bf)], wo=[torch.zeros(d, 64, **bf)])
+    for k in ("wq", "wk", "wv"):
+        w[k] = [torch.zeros(64, d, **bf)]
+    w["w_gate"] = [(gate / d).to(torch.bfloat16)[:, None].expand(F, d).contiguous()]
+    w["w_up"] = [(up / d).to(torch.bfloat16)[:, None].expand(F, d).contiguous()]
+    w["w_down"] = [(torch.rand(d, F, generator=g, device="cuda") * 0.2 - 0.1).to(torch.bfloat16)]
+    model = scd.Model(shape, w, max_seq=M + 8)
+    sess = scd.Session(model, scd.decode_config(batch=B, window_L=M, allowed_hi=64))
+    sess.scd_prefill(np.zeros((B, 1), dtype=np.int32), n_new=M)
+    ids = (torch.arange(B * M, device="cuda", dtype=torch.int32) % 64).reshape(B, M)
+    _, hidden = sess.scd_forward_window(ids, want_hidden=True)
+    h = w["tok_emb"][ids.long()].double()
+    n = h / (h.square().mean(-1, keepdim=True) + 1e-5).sqrt()
+    gd, ud = n @ w["w_gate"][0].double().T, n @ w["w_up"][0].double().T
+    want = h + (gd / (1.0 + torch.exp(-gd)) * ud) @ w["w_down"][0].double().T
+    assert (hidden.double() - want).abs().max() <= 1e-4 * want.abs().max()
+
+
+@pytest.mark.parametrize("d,F,V,B,M", [
+    (576, 832, 1000, 3, 86),        # 258 rows: a second x tile with two; weight tiles that end inside a run of 32 columns
+    (1024, 2816, 4000, 4, 256),     # 1024 rows: every tile of the layer cut between pairs
+    (256, 512, 40000, 2, 200),      # LM head of more tiles than pairs: whole ones and cut ones
+    (4096, 256, 64, 2, 150),        # two tiles, each cut into many parts
+    (64, 64, 8, 2, 129),            # one K block
+])
+def test_pair_gemm_against_64_bits(d, F, V, B, M):
+    """One layer without attention output, so that the forward is the norm and the three GEMMs of the CTA-pair kernel in
+    front of and behind known values. Gate, up and down multiply both bf16 planes of their input: 16 bits, 7.6e-6 of a value,
+    which sums of many terms average; one plane alone would be off by 1e-3. Bound 1e-4 of the largest sum. The logits take
+    the hidden state that came out, rounded to bf16 once: only fp32 sums differ, 2e-6 of the sum of magnitudes."""
+    shape = dict(n_layers=1, d_model=d, n_heads=1, n_kv_heads=1, head_dim=64, d_ffn=F, vocab_out=V, vocab_in=512, dtype="bf16",
+                 rope_base=10000.0, rms_eps=1e-5)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d)
+    def mat(*dims, std=0.05):
+        return (torch.randn(*dims, generator=g, device="cuda") * std).to(torch.bfloat16)
+    def gain():
+        return (1.0 + 0.4 * (torch.rand(d, generator=g, device="cuda") - 0.5)).to(torch.bfloat16)
+    w = dict(tok_emb=mat(512, d, std=1.0), final_norm=gain(), lm_head=mat(V, d), attn_norm=[gain()], ffn_norm=[gain()],
+             wq=[mat(64, d)], wk=[mat(64, d)], wv=[mat(64, d)], wo=[torch.zeros(d, 64, device="cuda", dtype=torch.bfloat16)],
+             w_gate=[mat(F, d)], w_up=[mat(F, d)], w_down=[mat(d, F)])
+    sess = scd.Session(scd.Model(shape, w, max_seq=M + 8), scd.decode_config(batch=B, window_L=M, allowed_hi=V))
+    sess.scd_prefill(np.zeros((B, 1), dtype=np.int32), n_new=M)
+    ids = torch.randint(0, 512, (B, M), generator=g, device="cuda", dtype=torch.int32)
+    logits, hidden = sess.scd_forward_window(ids, want_hidden=True)
+    h = w["tok_emb"][ids.long()].double()
+    n = h / (h.square().mean(-1, keepdim=True) + 1e-5).sqrt() * w["ffn_norm"][0].double()
+    gd, ud = n @ w["w_gate"][0].double().T, n @ w["w_up"][0].double().T
+    down = (gd / (1.0 + torch.exp(-gd)) * ud) @ w["w_down"][0].double().T
+    assert (hidden.double() - h - down).abs().max() <= 1e-4 * down.abs().max()
+    x = (hidden * w["final_norm"].float()).to(torch.bfloat16).double()
+    inv = 1.0 / (hidden.double().square().mean(-1, keepdim=True) + 1e-5).sqrt()
+    head = w["lm_head"].double().T
+    assert (logits.double() - (x @ head) * inv).abs().max() <= 2e-6 * ((x.abs() @ head.abs()) * inv).max()
+    again, hidden2 = sess.scd_forward_window(ids, want_hidden=True)
+    assert torch.equal(again, logits) and torch.equal(hidden2, hidden)
