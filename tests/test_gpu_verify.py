@@ -337,3 +337,57 @@ def test_verify_gumbel_after_many_rejections(V, top_k, top_p):
             assert np.array_equal(n_commit.cpu().numpy(), want["n_commit"]) and np.array_equal(flags.cpu().numpy(), want["flags"])
             assert np.array_equal(next_drafts.cpu().numpy(), want["next_drafts"])
             assert np.array_equal(committed.cpu().numpy()[:, 0], want["committed"][:, 0])
+
+
+def _dispatch(rows, n):
+    """CTAs per row and ids per warp, as the launcher chooses them."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ids = lambda C: -(-max(n, 4) // (C * 16))
+    C = 1
+    while C < 8 and ids(C) > 128 and (rows * C * 2 <= sms or (rows * C * 2 <= 2 * sms and ids(C) > 256)):
+        C *= 2
+    while C < 8 and ids(C) > 1024:
+        C *= 2
+    return C, -(-ids(C) // 32) * 32
+
+
+@pytest.mark.parametrize("B,L,V,C_want", [(1, 64, 64000, 4), (1, 8, 65536, 8), (2, 40, 20000, 2), (2, 80, 9000, 1)])
+@pytest.mark.parametrize("unlucky", ["all", "one"])
+@pytest.mark.parametrize("top_p", [0.0, 0.9])
+def test_verify_lists_built_again_in_clusters(B, L, V, C_want, unlucky, top_p):
+    """The bound of the lists comes from ids at fixed places of each warp's range. Here exactly those (of every CTA of a row, or
+    of its first one) hold the largest logits, too few of them for the truncation: the bound is above the threshold, and all
+    CTAs of the cluster build their lists again."""
+    C, ids = _dispatch(B * L, V)
+    assert C == C_want and ids > 256                   # read again from L2, not kept in registers
+    g = torch.Generator(device="cuda")
+    g.manual_seed(V)
+    v = torch.arange(V, device="cuda")
+    n, at = ids // 128, v % ids
+    sampled = (at // 128 == n // 4) & (v % 4 == 1) | (at // 128 == n - 1 - n // 4) & (v % 4 == 2)
+    sampled &= at < 128 * n
+    if unlucky == "one":
+        sampled &= v < 16 * ids
+    n_sampled = int(sampled.sum())
+    p = torch.rand(1, B, L, V, generator=g, device="cuda")
+    q = (p[0] + 0.2 * torch.rand(B, L, V, generator=g, device="cuda")).contiguous()
+    p[..., sampled] += 3.0
+    q[..., sampled] += 3.0
+    top_k = 0 if top_p else 2 * n_sampled
+    # the bound of an unlucky CTA against the threshold of the row
+    mine = p[0, 0, 0, : 16 * ids][sampled[: 16 * ids]].sort(descending=True).values
+    if top_p:
+        w = torch.exp(p[0, 0, 0].double())
+        order = w.sort(descending=True).values
+        theta = order[int((order.cumsum(0) < top_p * w.sum()).sum())]
+        assert torch.exp(mine[int(0.28 * len(mine))].double()) > theta and torch.exp(mine[-1].double()) > 2.0 * theta
+    else:
+        e = top_k / V * len(mine)
+        assert mine[min(len(mine) - 1, int(e + 4 * e ** 0.5) + 4)] > p[0, 0, 0].sort(descending=True).values[top_k - 1]
+    drafts = torch.argmax(q, dim=-1).to(torch.int32)
+    positions = torch.arange(B, device="cuda", dtype=torch.int64) * 300 + 9
+    cfg = scd.decode_config(mode=scd.SCD_MODE_SCD_MC, batch=B, window_L=L, top_k=top_k, top_p=top_p, seed=8, allowed_hi=V)
+    got = [t.cpu().numpy() for t in scd.scd_verify(cfg, p, q, drafts, positions, 4)]
+    want = oracle_verify("scd", p.cpu().numpy(), q.cpu().numpy(), drafts.cpu().numpy(), positions.cpu().numpy(), 4, 8, top_k=top_k, top_p=top_p)
+    assert np.array_equal(got[0], want["n_commit"]) and np.array_equal(got[3], want["flags"])
+    assert np.array_equal(got[2], want["next_drafts"]) and np.array_equal(got[1], want["committed"])
