@@ -18,9 +18,11 @@
 // [p U / P, (p + 1) U / P) of the U = tiles x k_blocks, whatever tile borders they cross, so that no last wave is
 // half empty. A tile that is cut is finished from partial tiles in global memory (they stay in L2): every
 // contributor stores its part and counts itself in; a pair whose LAST segment the tile is waits for the others
-// and adds up its share of the columns in contributor order - the result does not depend on scheduling. A pair
-// that has work left never waits.
-// Every wait is bounded; on expiry the error word is raised, the roles run out and the outputs are not written.
+// and adds up its share of the columns, its own part first and the others' in order - the result does not depend on
+// scheduling. A pair that has work left never waits, and none waits for long: with the kernels of other streams on the
+// device the pairs that are waited for may have no SM while these hold them. One that has waited PATIENCE polls stores
+// its share too, says so and leaves; who is counted in last adds up the shares left to it, in the same order.
+// Every other wait is bounded; on expiry the error word is raised, the roles run out and the outputs are not written.
 //
 // Measured on a B200 (before: 256 rows at a time through the weight-streaming kernel, or an earlier step of this one):
 // 2560 x 12288 x 3072, two planes: 247 us with one producer lane, 207 with one per operand;
@@ -46,6 +48,7 @@ constexpr int PAIR_UNITS = PAIR_COLS / PAIR_UNIT;                    // 8 runs o
 constexpr size_t RUN_FLOATS = (size_t)128 * PAIR_UNIT;               // 32 columns of the CTA's 128 rows: [column / 8][row][8]
 constexpr size_t SLOT_FLOATS = PAIR_UNITS * RUN_FLOATS;              // one CTA's part of a cut tile
 constexpr int RED_SLOTS = 12;                                        // runs of other pairs' parts in flight (in the ring's memory)
+constexpr unsigned PATIENCE = 1u << 11;                              // polls for the other parts of a tile: a millisecond or two
 
 __device__ __forceinline__ uint32_t cluster_rank()
 {
@@ -125,6 +128,18 @@ __device__ __forceinline__ void st_run(float *run, int row, const float *v)
                      ::"l"(run + (size_t)(j >> 3) * 1024 + row * 8), "f"(v[j]), "f"(v[j + 1]), "f"(v[j + 2]), "f"(v[j + 3]),
                        "f"(v[j + 4]), "f"(v[j + 5]), "f"(v[j + 6]), "f"(v[j + 7]) : "memory");
 }
+__device__ __forceinline__ void add_run_global(const float *run, int row, float *v)
+{
+#pragma unroll
+    for (int j = 0; j < 32; j += 8) {
+        float t[8];
+        asm volatile("ld.relaxed.gpu.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=f"(t[0]), "=f"(t[1]), "=f"(t[2]), "=f"(t[3]), "=f"(t[4]), "=f"(t[5]), "=f"(t[6]), "=f"(t[7])
+                     : "l"(run + (size_t)(j >> 3) * 1024 + row * 8) : "memory");
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[j + i] += t[i];
+    }
+}
 __device__ __forceinline__ void add_run(const float *run, int row, float *v)   // (in shared memory)
 {
 #pragma unroll
@@ -197,6 +212,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) gemm_pair_kernel(const __grid
     __shared__ uint64_t full_bar[MAX_PAIR_STAGES], empty_bar[MAX_PAIR_STAGES], tfull[2], tempty[2], red_bar[RED_SLOTS];
     __shared__ float scale_s[PAIR_MAX_X_TILES][128];                 // 1 / rms of this CTA's rows of each x tile
     __shared__ uint32_t tmem_base_s;
+    __shared__ unsigned ticket_s;
     __shared__ volatile int failed;
 
     if (p.skip && *p.skip) return;
@@ -426,48 +442,99 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) gemm_pair_kernel(const __grid
             const long long U = (long long)p.w_tiles * p.x_tiles * p.k_blocks;
             const long long tile_u0 = (long long)w.tile * w.kb, tile_u1 = tile_u0 + w.kb;
             const int q1 = pair_of(p, tile_u1 - 1), n_parts = q1 - q0 + 1;
-            const int n_red = U * (q1 + 1) / p.pairs == tile_u1 ? n_parts : n_parts - 1;   // contributors that end on this tile
-            const bool reduces = w.last();
+            // contributors that end on this tile, as many as there are runs of columns to add up
+            const int n_red = min(limit_units, U * (q1 + 1) / p.pairs == tile_u1 ? n_parts : n_parts - 1), me = pair - q0;
+            const bool reduces = w.last() && me < n_red;
+            auto part_of = [&](int q) -> const float * {             // (its second slot if it had a tile in front of this one)
+                return p.scratch + ((size_t)(q * 2 + (U * q / p.pairs >= tile_u0 ? 0 : 1)) * 2 + rank) * SLOT_FLOATS;
+            };
             float *slot = p.scratch + ((size_t)(pair * 2 + (seg_i == 0 ? 0 : 1)) * 2 + rank) * SLOT_FLOATS;
 #pragma unroll 1
             for (int u = 0; u < PAIR_UNITS; ++u) {
-                if (reduces && (u % limit_units) % n_red == pair - q0) continue;
+                if (reduces && (u % limit_units) % n_red == me) continue;
                 tmem_ld32(acc + 32u * u, v);
                 st_run(slot + u * RUN_FLOATS, row, v);
             }
+            // counters of a tile: [0] parts that are there, from bit 16 on the shares that were left; [1] shares that are done
             unsigned *cnt = p.counters + (size_t)w.tile * 4 + rank * 2;
-            __threadfence();
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            asm volatile("bar.sync 1, 128;" ::: "memory");
-            if (tid == 64) atomicAdd(cnt, 1u);
+            auto count_in = [&](unsigned what) -> unsigned {         // (what was there before, in all four warps)
+                __threadfence();
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+                if (tid == 64) ticket_s = atomicAdd(cnt, what);
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+                return ticket_s;
+            };
+            auto done = [&](unsigned shares) {                       // the last one clears the tile's counters for the next launch
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+                if (tid == 64 && atomicAdd(cnt + 1, shares) + shares == (unsigned)n_red) { cnt[0] = 0u; cnt[1] = 0u; }
+            };
+            auto add_left = [&](unsigned left) {                     // shares that their pairs left to the last one to come
+                __threadfence();
+#pragma unroll 1
+                for (int sh = 0; sh < n_red; ++sh) {
+                    if (!(left >> sh & 1u)) continue;
+                    auto sum_parts = [&](int u, float *sum) {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) sum[j] = 0.f;
+                        add_run_global(part_of(q0 + sh) + (size_t)u * RUN_FLOATS, row, sum);
+#pragma unroll 1
+                        for (int q = q0; q <= q1; ++q)
+                            if (q != q0 + sh) add_run_global(part_of(q) + (size_t)u * RUN_FLOATS, row, sum);
+                    };
+#pragma unroll 1
+                    for (int u = sh; u < limit_units; u += n_red) {
+                        if (p.epi == PAIR_EPI_RESID) load_resid(u, g);
+                        if (swiglu) sum_parts(u, g);
+                        sum_parts(swiglu ? u + PAIR_UNITS / 2 : u, v);
+                        finish(u, v, g);
+                    }
+                }
+                done((unsigned)__popc(left));
+            };
+            const unsigned ticket = count_in(1u);
+            const bool all_here = (ticket & 0xFFFFu) + 1u == (unsigned)n_parts;
+            const unsigned left = all_here ? ticket >> 16 : 0u;
             if (!reduces) {
                 if (lane == 0) arrive_cluster(tempty_leader[b]);
+                if (left) add_left(left);
                 continue;
             }
-            // (a wait that gives up here is met by all four warps at the barrier behind it)
-            if (tid == 64) {
-                unsigned seen = 0;
-                for (unsigned i = 0; i < SPIN_LIMIT && seen < (unsigned)n_parts; ++i) {
-                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(cnt) : "memory");
-                    if ((i & 1023u) == 1023u && failed) break;
+            if (!all_here) {
+                unsigned seen = (unsigned)n_parts;
+                if (tid == 64) {
+                    seen = 0;
+                    for (unsigned i = 0; i < PATIENCE && seen < (unsigned)n_parts; ++i) {
+                        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(cnt) : "memory");
+                        seen &= 0xFFFFu;
+                        if ((i & 1023u) == 1023u && failed) break;
+                    }
                 }
-                if (seen < (unsigned)n_parts) { atomicExch(p.err, 3); failed = 1; }
+                if (!all_epilogue(!failed)) break;
+                if (!all_epilogue(seen == (unsigned)n_parts)) {
+#pragma unroll 1
+                    for (int u = me; u < PAIR_UNITS; ++u) {
+                        if ((u % limit_units) % n_red != me) continue;
+                        tmem_ld32(acc + 32u * u, v);
+                        st_run(slot + u * RUN_FLOATS, row, v);
+                    }
+                    // (unless the last one has come meanwhile, and found nothing left to it)
+                    if ((count_in(0x10000u << me) & 0xFFFFu) != (unsigned)n_parts) break;
+                }
             }
-            if (!all_epilogue(!failed)) break;
             __threadfence();
             // The runs to add, in order: for each of this pair's runs of columns (SwiGLU: gate, then up) the parts of the
             // other contributors. They come by bulk copies into the ring, which this CTA's MMAs no longer need, twelve
             // at a time: with register loads, one or two in flight, a tile took 8 to 27 us.
-            const int me = pair - q0, n_oth = n_parts - 1, per_unit = swiglu ? 2 * n_oth : n_oth;
+            const int n_oth = n_parts - 1, per_unit = swiglu ? 2 * n_oth : n_oth;
             const int my_units = (limit_units - me + n_red - 1) / n_red, n_runs = my_units * per_unit;
             auto request = [&](int first) {
                 asm volatile("fence.proxy.async;" ::: "memory");
                 for (int r = first; r < min(n_runs, first + RED_SLOTS); ++r) {
                     const int k = r % per_unit, i = k % n_oth;
                     const int u = me + (r / per_unit) * n_red + (k >= n_oth ? PAIR_UNITS / 2 : 0);
-                    const int q = q0 + i + (i >= me ? 1 : 0);        // its second slot if it had a tile in front of this one
-                    const float *src = p.scratch + ((size_t)(q * 2 + (U * q / p.pairs >= tile_u0 ? 0 : 1)) * 2 + rank) * SLOT_FLOATS +
-                                       (size_t)u * RUN_FLOATS;
+                    const int q = q0 + i + (i >= me ? 1 : 0);
+                    const float *src = part_of(q) + (size_t)u * RUN_FLOATS;
                     uint64_t *bar = &red_bar[r - first];
                     mbar_expect_tx(bar, (unsigned)(RUN_FLOATS * sizeof(float)));
                     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -501,9 +568,8 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) gemm_pair_kernel(const __grid
                 __syncwarp();
                 if (good) finish(u, v, g);
             }
-            // the last reader clears the tile's counters for the next launch
-            asm volatile("bar.sync 1, 128;" ::: "memory");
-            if (tid == 64 && atomicAdd(cnt + 1, 1u) == (unsigned)n_red - 1u) { cnt[0] = 0u; cnt[1] = 0u; }
+            done(1u);
+            if (left) add_left(left);
         }
     }
     __syncwarp();
@@ -520,9 +586,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) gemm_pair_kernel(const __grid
 size_t pair_scratch_bytes(int pairs) { return (size_t)pairs * 4 * SLOT_FLOATS * sizeof(float); }
 size_t pair_counter_count(int w_tiles, int x_tiles) { return (size_t)w_tiles * x_tiles * 4; }
 
-// The pairs of one cut tile wait for each other, so the grid never has more pairs than fit at once. (Kernels of
-// other streams may delay some of them: a tile's pairs have neighbouring indices and are dispatched in order,
-// and the pairs of complete tiles leave without waiting, so the rest always finds room.)
+// The pairs of one cut tile wait for each other, for a while, so the grid never has more pairs than fit at once.
 int pair_grid_limit(int *pairs)
 {
     SCD_CUDA_TRY(cudaFuncSetAttribute(gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PAIR_SMEM));
