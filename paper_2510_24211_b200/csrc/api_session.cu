@@ -159,18 +159,20 @@ int set_rows(scd_session *s, int rows)
                              (size_t)s->ss_parts_cap * n * sizeof(float)};
     void **const slot[6] = {(void **)&s->h, &s->xn, &s->qkv, &s->att, &s->act, (void **)&s->ss};
     constexpr int most_retired = (int)(sizeof(s->retired) / sizeof(s->retired[0]));
-    SCD_REQUIRE(!s->h || s->n_retired + 6 <= most_retired, SCD_ERR_CAPACITY, "activation buffers have grown %d times", s->n_retired / 6);
-    void *fresh[6] = {};
-    for (int i = 0; i < 6; ++i) {
-        const cudaError_t e = cudaMalloc(&fresh[i], std::max<size_t>(bytes[i], 1));
-        if (e == cudaSuccess) continue;
-        for (int j = 0; j < i; ++j) cudaFree(fresh[j]);
+    SCD_REQUIRE(s->n_retired < most_retired, SCD_ERR_CAPACITY, "activation buffers have grown %d times", s->n_retired);
+    size_t total = 0;
+    for (size_t b : bytes) total += (b + 1023) & ~(size_t)1023;
+    char *fresh = nullptr;
+    const cudaError_t e = cudaMalloc((void **)&fresh, total);
+    if (e != cudaSuccess) {
         cudaGetLastError();                              // (an allocation that failed leaves the context as it was)
         return cuda_fail(e, "cudaMalloc of the activation buffers");
     }
+    if (s->rows_mem) s->retired[s->n_retired++] = s->rows_mem;
+    s->rows_mem = fresh;
     for (int i = 0; i < 6; ++i) {
-        if (*slot[i]) s->retired[s->n_retired++] = *slot[i];
-        *slot[i] = fresh[i];
+        *slot[i] = fresh;
+        fresh += (bytes[i] + 1023) & ~(size_t)1023;
     }
     s->rows_cap = rows;
     gemm_session_rows_changed(s);
@@ -200,7 +202,7 @@ void free_session_memory(scd_session *s)
     void *ptrs[] = {s->kv_pool, s->page_table, s->n_known, s->n_total, s->shift, s->prev_lw, s->drafts,
                     s->n_commit, s->tokens, s->tokens_u, s->row_y, s->row_y_indep, s->iter,
                     s->accept_flags, s->xbuf[0], s->xbuf[1], s->stats[0], s->stats[1],
-                    s->dev_stats, s->finished, s->h, s->ss, s->xn, s->qkv, s->att, s->act, s->logits, s->gemm_ws, s->gemm_scratch, s->stamps};
+                    s->dev_stats, s->finished, s->rows_mem, s->logits, s->gemm_ws, s->gemm_scratch, s->stamps};
     for (void *p : ptrs) if (p) cudaFree(p);
     if (s->host_pinned) cudaFreeHost(s->host_pinned);
     if (s->gemm_state) gemm_session_release(s);

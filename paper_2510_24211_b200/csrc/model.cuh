@@ -21,8 +21,9 @@ struct scd_session {
     int chunk;                // rows per stream-sequence that one explicit forward may carry
     int prefill_chunk;        // ... that one pass over a prompt may carry (>= chunk)
     int rows_cap;             // rows the activation buffers hold: Q * chunk, after a longer prompt up to Q * prefill_chunk
-    void *retired[36];        // activation buffers that larger ones have taken the place of (a caller's captured launches
-    int n_retired;            // may still use them)
+    void *rows_mem;           // their memory
+    void *retired[8];         // ... of buffers that larger ones have taken the place of (a caller's captured launches may
+    int n_retired;            // still use them)
     int pages_per_seq;
     int prompt_len, n_new;
     bool prefilled;
