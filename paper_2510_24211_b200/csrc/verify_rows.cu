@@ -23,12 +23,12 @@
 // it, without a sample (28.9 us against 30.7 for 32 rows of 16384 ids). Longer ones are read again from L2 where a sweep
 // repeats (three sweeps, one for the histogram: 63.7 us against 53.8 for 256 rows of 16384 ids).
 // A warp whose list would overflow (a row that hardly is truncated) works on its whole range instead, reading x
-// again: entry e is then simply its e-th id. commit_kernel, one CTA per sequence behind this grid, does the
+// again (the nucleus leaves its weights in the list's place): entry e is then simply its e-th id. commit_kernel, one CTA per sequence behind this grid, does the
 // only serial part: first rejection, commit, next window.
 //
 // us per scd_verify call on a B200, before (an exponential per id, four byte-wise passes over the cluster for the nucleus,
-// tickets for the commit, the race on one CTA per row) and now: 1 x 32 rows of 16384 ids, top-k 2000: 32.3, 24.3;
-// 8 x 32 with guidance: 108, 51; 64 rows of 64000 ids, top-p 0.8: 277, 83; 2 x 32 of 16384, Gumbel: 233, 36.6.
+// tickets for the commit, the race on one CTA per row) and now: 1 x 32 rows of 16384 ids, top-k 2000: 32.8, 21.9;
+// 8 x 32 with guidance: 107, 45.0; 64 rows of 64000 ids, top-p 0.8: 280, 66.2; 2 x 32 of 16384, Gumbel: 235, 34.2.
 //
 // Gumbel race (Algorithm 4): the winner is the smallest E_v / W_v of integers that take 40 squarings each. An fp32
 // estimate of every ratio first, the integers only for ids within RACE_SLACK of the smallest estimate. A row that
@@ -86,6 +86,7 @@ struct Local {
     unsigned peer_n[2][MAXC];
     int sel[2];
     float bound[2], cuts[2][5];
+    bool give_up[2];
     unsigned sel_k[2], tau_key[2];
     unsigned long long above[2], kept[2], total[2];
 };
@@ -461,6 +462,8 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
     };
     // entry e of this warp: of its list, or of its whole range when the list did not fit
     bool whole[2] = {false, false};
+    bool dense = false;                                // whole[0], and the weights of the range lie where the lists were
+    auto dense_at = [&](int e) -> unsigned * { return e < 2 * WCAP ? (unsigned *)list_p + e : list_q + (e - 2 * WCAP); };
     int n_e[2] = {0, 0};
     auto close_lists = [&]() {
         __syncwarp();
@@ -481,6 +484,7 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         constexpr int a = decltype(A_)::value;
         if (!entry_in(a, e)) return 0u;
         if (!whole[a]) return a == 0 ? list_p[e].x : list_q[e];
+        if (TOP_P && !REG && a == 0 && dense) return *dense_at(e);
         return weight_of(a == 0 ? load_p(wbase + e) : load_q(wbase + e), m[a], tau[a]);
     };
     auto entry_id = [&](int e) -> int { return whole[0] ? wbase + e : (int)list_p[e].y; };
@@ -651,7 +655,7 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         // TAIL_WIDE of the rest, so that the nucleus ends inside the lists (without it such rows had them built twice: 175
         // rows of 12991 ids, guidance, top-p 0.95, 226 us, 65 so), but not more than fit a list (LIST_FILL: some warps have
         // more ids above the bound than others). Only where the nucleus itself is far from fitting (top_p and TAIL_TIGHT of the rest take
-        // FAR times as much) the lists are given up at once (128 rows of 30000 ids, top-p 0.99: 138 us after a try, 109 so).
+        // FAR times as much) the lists are given up at once (128 rows of 30000 ids, top-p 0.99: 138 us after a try, 111 so).
         if (tid < 10) (&lc.cuts[0][0])[tid] = (float)W_TAIL;
         __syncthreads();
         auto cut_at = [&](int bin) { return fmaxf((float)W_TAIL, bin > 0 ? (float)weight_step_lo(NB - 1 - bin) : 0.f); };
@@ -672,14 +676,34 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
         });
         if (tid < 2) {
             const float *c_ = lc.cuts[tid];
+            lc.give_up[tid] = c_[4] < c_[2];
             lc.bound[tid] = c_[4] < c_[2] ? fminf(c_[0], c_[4]) : fmaxf(fminf(c_[0], c_[3]), c_[1]);
         }
         __syncthreads();
+        // A warp whose target list is given up, or overflows, keeps the weights of its whole range where the lists were: up to
+        // 2 x 384 words over the target row's, up to 1024 where the draft row leaves its own free. Weighed again from L2 in
+        // every pass instead, 64 rows of 64000 ids of a random decoder took 212 us inside a session, 155 so; 64 rows of 64000
+        // ids, top-p 0.95, both rows raw, 161 us, 139 so. A list that fits is the shorter one to go over (128 rows of 20000
+        // ids, guidance, top-p 0.99: 82 us, 94 with the weights of whole ranges).
+        const bool give_up[2] = {!REG && range > WCAP && lc.give_up[0], !REG && range > WCAP && lc.give_up[1]};
+        auto fill = [&](int v) {
+#pragma unroll
+            for (int h = 0; h < NS; ++h) {
+                const int e = v + 128 * h - wbase;
+                if (e >= range) continue;
+                unsigned wv[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) wv[i] = weight_of(xr[0][4 * h + i], m[0], -INFINITY);
+                *(uint4 *)dense_at(e) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
+            }
+        };
         for (bool again = false;; again = true) {
             // (a bound is the smallest weight of a step: exact in fp32)
             const unsigned cut[2] = {again ? 1u : (unsigned)lc.bound[0], again ? 1u : (unsigned)lc.bound[1]};
             unsigned long long z[2] = {0ull, 0ull};
-            n_list[0] = n_list[1] = 0;
+            dense = give_up[0] && (range <= 2 * WCAP || !rawq || give_up[1]);
+            n_list[0] = dense ? WCAP + 1 : 0;
+            n_list[1] = dense && give_up[1] ? WCAP + 1 : 0;
             sweep([&](int v) {
                 unsigned keep[2] = {0u, 0u};
                 float val[2][N];
@@ -694,9 +718,18 @@ __global__ void __launch_bounds__(CT, 2) verify_rows_kernel(const VerifyParams p
                         val[a][j] = __uint_as_float(wv);
                     }
                 }
-                append(v, keep, val);
+                if (!REG && dense) {
+                    keep[0] = 0u;
+                    fill(v);
+                }
+                if (!dense || (rawq && !give_up[1]) || wstore) append(v, keep, val);
             });
             close_lists();
+            if (!REG && whole[0] && !dense && (range <= 2 * WCAP || !rawq || whole[1])) {
+                dense = true;
+                sweep(fill);
+                __syncwarp();
+            }
             EACH_ROW([&](auto A_) {
                 constexpr int a = decltype(A_)::value;
                 const unsigned long long t = warp_sum64(z[a]);

@@ -225,6 +225,12 @@ def test_step_replay_nucleus_truncation():
     _replay_case(SMALL, oracle.MODE_SCD_GS, B=1, L=6, P=5, n_new=40, top_k=30, seed=15, top_p=0.6)
 
 
+@pytest.mark.parametrize("L,V,n_new", [(12, 40000, 24), (64, 64000, 20)])
+def test_step_replay_nucleus_of_flat_rows(L, V, n_new):
+    # rows whose nucleus no list holds: the weights that the next iteration reads are left by the other route
+    _replay_case(dict(SMALL, vocab_out=V, vocab_in=V + 8), oracle.MODE_SCD_MC, B=1, L=L, P=5, n_new=n_new, top_k=0, seed=16, top_p=0.8, std=0.05)
+
+
 def test_step_replay_wide_window_ragged_batch_bf16():
     # L = 48 through the tensor-core path with three sequences that progress at different speeds
     _replay_case(MID_BF16_D64, oracle.MODE_SCD_MC, B=3, L=48, P=66, n_new=120, top_k=60, seed=17, page=64)

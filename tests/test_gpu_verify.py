@@ -391,3 +391,30 @@ def test_verify_lists_built_again_in_clusters(B, L, V, C_want, unlucky, top_p):
     want = oracle_verify("scd", p.cpu().numpy(), q.cpu().numpy(), drafts.cpu().numpy(), positions.cpu().numpy(), 4, 8, top_k=top_k, top_p=top_p)
     assert np.array_equal(got[0], want["n_commit"]) and np.array_equal(got[3], want["flags"])
     assert np.array_equal(got[2], want["next_drafts"]) and np.array_equal(got[1], want["committed"])
+
+
+@pytest.mark.parametrize("B,L,V", [(1, 64, 64000), (1, 8, 65536), (1, 64, 45001), (2, 80, 9000)])
+@pytest.mark.parametrize("draft", ["none", "flat", "peaked"])
+@pytest.mark.parametrize("top_p", [0.8, 0.99])
+def test_verify_nucleus_of_flat_rows(B, L, V, draft, top_p):
+    """Rows so flat that no list holds the nucleus (1000, 512, 704 and 576 ids per warp, lists of 384): the target row's weights
+    take the place of the lists, unless the list of a peaked draft row is in the way of more than 768. Row 1 is peaked."""
+    C, ids = _dispatch(B * L, V)
+    assert ids > 384 + 100
+    g = torch.Generator(device="cuda")
+    g.manual_seed(V + L)
+    p = 0.3 * torch.randn(1, B, L, V, generator=g, device="cuda")
+    p[:, :, 1] *= 20.0
+    q = (p[0] + 0.1 * torch.randn(B, L, V, generator=g, device="cuda")) * (20.0 if draft == "peaked" else 1.0)
+    drafts = torch.argmax(q, dim=-1).to(torch.int32)
+    positions = torch.arange(B, device="cuda", dtype=torch.int64) * 300 + 9
+    for mode in ("scd", "sjd"):
+        cfg = scd.decode_config(mode=MODES[mode], batch=B, window_L=L, top_p=top_p, seed=8, allowed_lo=3, allowed_hi=V - 2)
+        qx = None if draft == "none" else q
+        got = [t.cpu().numpy() for t in scd.scd_verify(cfg, p, qx, drafts, positions, 4)]
+        want = oracle_verify(mode, p.cpu().numpy(), None if qx is None else q.cpu().numpy(), drafts.cpu().numpy(),
+                             positions.cpu().numpy(), 4, 8, top_p=top_p, lo=3, hi=V - 2)
+        assert np.array_equal(got[0], want["n_commit"]) and np.array_equal(got[3], want["flags"])
+        assert np.array_equal(got[2], want["next_drafts"])
+        for b in range(B):
+            assert np.array_equal(got[1][b, :got[0][b]], want["committed"][b, :got[0][b]])
