@@ -71,8 +71,9 @@ int scd_noise_u24(uint64_t seed, uint32_t noise_stream, uint32_t batch, const in
 /* The workspace must be zero-filled before its first use (it holds an error word that every call leaves
  * at zero unless a bounded wait gave up). scd_gemm_bf16_shaped is the same GEMM with the number of K
  * slices (= cluster size, 1..8) and ring slots given by the caller (0 = the built-in rule), for tests
- * that walk through the launch shapes. scd_model_gemm_tune does that for every later GEMM launch of one
- * model (all its sessions), for benchmarking; 0, 0 restores the rule. */
+ * that walk through the launch shapes. scd_model_gemm_tune does that for every later launch of this kernel by one
+ * model (all its sessions; forwards of more than 128 rows may take the CTA-pair kernel, which has no such shape),
+ * for benchmarking; 0, 0 restores the rule. */
 int64_t scd_gemm_workspace_bytes(int32_t M, int32_t N, int32_t K);
 int scd_model_gemm_tune(scd_model_t *model, int32_t k_splits, int32_t stages);
 int scd_gemm_bf16_shaped(const void *x, const void *w, float *y, int32_t M, int32_t N, int32_t K,
